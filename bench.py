@@ -481,7 +481,7 @@ def run_cpm(args, world, rank, local):
         "e2e": {"value": e2e_ms / 1e3, "unit": "s", "h2d_bytes_per_step": nb * 8,
                 "d2h_bytes_per_step": nb * 8},
         "gpu_launches": int(launches),
-        "roofline": {"kernel": "k_extend_tiles<float,3> (FP32 extension over B+, the largest "
+        "roofline": {"kernel": "k_extend_units<3> (FP32 extension over B+, the largest "
                                "share of the mixed solve's kernel time)", "bound": "hbm",
                      "achieved": ach32, "peak": pk.get("hbm_gbs"), "unit": "GB/s",
                      "frac": ach32 / pk.get("hbm_gbs", 6800.0),
@@ -602,7 +602,7 @@ def run_micro(args):
     each case is one kind of launch, timed with CUDA events on the launching
     stream after `--warmup` untimed launches.  Cases: extend32 / extend64 (the
     extension over B+), extend32_v0 / _v1 / _v2 (the FP32 extension forced to
-    one work decomposition), apply32 / apply64 (M u), jacobi32 (one Jacobi
+    one launch shape), apply32 / apply64 (M u), jacobi32 (one Jacobi
     sweep), resid64 / resid64_f64 (the relative-form outer residual in FP32 pairs
     / in FP64), vcycle32 (one FP32
     V-cycle: transfers and the coarsest solve included), mlp (the learned

@@ -214,7 +214,7 @@ typedef struct cpm_mg_opts {
                                preconditioned by omega / diag(A), classical
                                Gram-Schmidt twice, fixed step counts, all on
                                the device                                      */
-  int32_t ext_variant;      /* FP32 extension work decomposition of every level
+  int32_t ext_variant;      /* FP32 extension launch shape of every level
                                (see cpm_hier_ext_tuning): 0 = chosen per level
                                by timing when the hierarchy is built; 1, 2, 3 =
                                variant 0, 1, 2 everywhere                       */
@@ -244,13 +244,12 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts,
 cpm_status cpm_hier_info(cpm_hier h, int32_t* n_levels, int32_t level, int64_t* n_band);
 
 /*
- * The work decomposition of level `level`'s FP32 extension, chosen when the
- * hierarchy was built by timing each candidate on that level (three launches
- * over B+ after a warm-up): 0 one CTA per extension tile and one thread per
- * point, 1 persistent CTAs that stage the next tile while evaluating the
- * current one, 2 one thread per chunk of points that share a stencil base.
- * variant: host int32 (may be NULL); ms: host array of 3 doubles, the measured
- * milliseconds of each candidate (may be NULL).  No counterpart in the paper.
+ * The launch shape of level `level`'s FP32 extension, chosen when the hierarchy
+ * was built by timing each candidate on that level (three launches over B+
+ * after a warm-up): one (0), two (1) or four (2) extension tiles, one warp each,
+ * per thread block.  The results do not depend on it.  variant: host int32 (may
+ * be NULL); ms: host array of 3 doubles, the measured milliseconds of each
+ * candidate (may be NULL).  No counterpart in the paper.
  */
 cpm_status cpm_hier_ext_tuning(cpm_hier h, int32_t level, int32_t* variant, double* ms);
 

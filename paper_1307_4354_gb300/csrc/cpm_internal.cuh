@@ -178,15 +178,8 @@ struct Level {
   DBuf<float> efr32;          // d x (nB+nG) fractions in E order
   DBuf<double> ew64;          // 4d x (nB+nG) FP64 cubic weights in E order
   DBuf<float2> ewp;           // the same as FP32 pairs (built on demand: build_pair_weights)
-  // chunks: runs of at most kChunkMax consecutive E-order points of one tile
-  // that share one stencil base (and are all in B or all in G); one thread
-  // loads the base's 4^d values once and evaluates every point of the chunk
-  int ext_variant = 0;        // FP32 extension variant chosen by timing (ExtVariant)
+  int ext_variant = 0;        // FP32 extension's launch shape, chosen by timing (ExtVariant)
   float ext_ms[3] = {0.f, 0.f, 0.f};
-  int32_t nchunks = 0;
-  DBuf<uint32_t> echunk;      // first E-order point | (count - 1) << 26
-  DBuf<int32_t> tile_cstart;  // ntiles + 1 offsets into echunk
-  DBuf<int32_t> tile_cmid;    // per tile: end of its chunks of points of B
   DBuf<int32_t> nbr;          // 2d x nB: B+ index of the Laplacian neighbours of B
 
   BrickView view() const {

@@ -161,42 +161,6 @@ __global__ void k_tile_sort(const int32_t* tile_start, int64_t nplus, int32_t nB
   }
 }
 
-// Chunks.  Inside a tile the points are sorted by (point of G, base
-// position), so the points that share one stencil base are consecutive; each
-// such run (never crossing the B/G boundary) is cut into chunks of at most
-// kChunkMax points.  One thread per tile counts (emit = false) or writes
-// (emit = true) its chunks.
-#ifndef CPM_EXT_CHUNK
-#define CPM_EXT_CHUNK 2
-#endif
-constexpr int kChunkMax = CPM_EXT_CHUNK;
-static_assert(kChunkMax >= 1 && kChunkMax <= 8, "chunk count must fit in 3 bits");
-
-__global__ void k_tile_chunks(const int32_t* tile_start, const int32_t* tile_mid, int32_t ntiles,
-                              const uint32_t* erec, bool emit, int32_t* count, int32_t* count_B,
-                              const int32_t* cstart, uint32_t* echunk) {
-  const int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= ntiles) return;
-  const int32_t beg = tile_start[t], mid = tile_mid[t], end = tile_start[t + 1];
-  int32_t n = 0, nB = 0;
-  int32_t c0 = emit ? cstart[t] : 0;
-  int32_t k = beg;
-  while (k < end) {
-    const uint32_t pos = erec[k] & 63u;
-    const int32_t stop = k < mid ? mid : end;  // a run stays in B or in G
-    int32_t j = k + 1;
-    while (j < stop && j - k < kChunkMax && (erec[j] & 63u) == pos) ++j;
-    if (emit) echunk[c0 + n] = (uint32_t)k | ((uint32_t)(j - k - 1) << 26);
-    ++n;
-    if (k < mid) ++nB;
-    k = j;
-  }
-  if (!emit) {
-    count[t] = n;
-    count_B[t] = nB;
-  }
-}
-
 void build_ext_tiles(Level& L, cudaStream_t st) {
   const int64_t np = L.nplus();
   CPM_CHECK(np < (1ll << 26), CPM_ERR_ARG, "more than 2^26 points on one level");
@@ -254,43 +218,6 @@ void build_ext_tiles(Level& L, cudaStream_t st) {
     L.erec = std::move(erec2);
     L.efr32 = std::move(efr2);
     L.ew64 = std::move(ew2);
-  }
-  // chunks of points with one stencil base
-  L.tile_cstart.alloc(ntiles + 1);
-  L.tile_cmid.alloc(ntiles);
-  L.nchunks = 0;
-  if (ntiles > 0) {
-    DBuf<int32_t> ccount(ntiles), ccount_B(ntiles);
-    DBuf<int64_t> coff(ntiles);
-    k_tile_chunks<<<nblk(ntiles, 256), 256, 0, st>>>(L.tile_start.get(), L.tile_mid.get(),
-                                                     (int32_t)ntiles, L.erec.get(), false,
-                                                     ccount.get(), ccount_B.get(), nullptr, nullptr);
-    CPM_CUDA_TRY(cudaGetLastError());
-    std::vector<int32_t> hc(ntiles), hcb(ntiles);
-    CPM_CUDA_TRY(cudaMemcpyAsync(hc.data(), ccount.get(), ntiles * sizeof(int32_t),
-                                 cudaMemcpyDeviceToHost, st));
-    CPM_CUDA_TRY(cudaMemcpyAsync(hcb.data(), ccount_B.get(), ntiles * sizeof(int32_t),
-                                 cudaMemcpyDeviceToHost, st));
-    CPM_CUDA_TRY(cudaStreamSynchronize(st));
-    std::vector<int32_t> hstart(ntiles + 1), hmid(ntiles);
-    int64_t acc = 0;
-    for (int64_t t = 0; t < ntiles; ++t) {
-      hstart[t] = (int32_t)acc;
-      hmid[t] = (int32_t)(acc + hcb[t]);
-      acc += hc[t];
-    }
-    hstart[ntiles] = (int32_t)acc;
-    CPM_CHECK(acc < (1ll << 31), CPM_ERR_ARG, "too many extension chunks");
-    L.nchunks = (int32_t)acc;
-    CPM_CUDA_TRY(cudaMemcpyAsync(L.tile_cstart.get(), hstart.data(), (ntiles + 1) * sizeof(int32_t),
-                                 cudaMemcpyHostToDevice, st));
-    CPM_CUDA_TRY(cudaMemcpyAsync(L.tile_cmid.get(), hmid.data(), ntiles * sizeof(int32_t),
-                                 cudaMemcpyHostToDevice, st));
-    L.echunk.alloc(acc);
-    k_tile_chunks<<<nblk(ntiles, 256), 256, 0, st>>>(L.tile_start.get(), L.tile_mid.get(),
-                                                     (int32_t)ntiles, L.erec.get(), true, nullptr,
-                                                     nullptr, L.tile_cstart.get(), L.echunk.get());
-    CPM_CUDA_TRY(cudaGetLastError());
   }
   int32_t herr = 0;
   CPM_CUDA_TRY(cudaMemcpyAsync(&herr, err.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -715,269 +642,14 @@ __global__ void __launch_bounds__(kExtThreads) k_extend_pair(LevelView<double> L
   }
 }
 
-// FP32 extension, persistent and software-pipelined: a fixed grid of CTAs, each
-// looping over tiles blockIdx.x, blockIdx.x + gridDim.x, ...; while it
-// evaluates the points of one tile from one shared-memory box it has the row
-// loads of its next tile in flight (into registers, one box row per thread)
-// and writes them into the other box afterwards, so the staging latency of a
-// tile hides behind the arithmetic of the previous one.
-#ifndef CPM_EXT_PIPELINED
-#define CPM_EXT_PIPELINED 0
-#endif
-constexpr bool kPipelined = CPM_EXT_PIPELINED != 0;
-constexpr int kPipeThreads = 64;
-
-template <int DIM>
-__global__ void __launch_bounds__(kPipeThreads) k_extend_pipe(LevelView<float> L,
-                                                              const float* __restrict__ u,
-                                                              float* __restrict__ w, bool with_ghost) {
-  constexpr int RS = kRS;
-  constexpr int NZ = DIM == 3 ? 7 : 1;
-  constexpr int NB = DIM == 3 ? 8 : 4;
-  __shared__ __align__(16) float win[2][NZ * 7 * RS];
-  __shared__ uint32_t smask[2][NB][2];
-  __shared__ int32_t sstart[2][NB][2];
-  static_assert(kPipeThreads >= 49, "one box row per thread");
-  int32_t tile = blockIdx.x;
-  if (tile >= L.ntiles) return;
-  // the rows of tile t: addresses from its masks in buffer b, values into v
-  auto load_rows = [&](int32_t t, int b, float v[7], int& ylo_o, int& z_o, int& y_o, int& xlo_o,
-                       int& xhi_o) -> bool {
-    const uint32_t tbox = __ldg(L.tile_box + t);
-    const int xlo = tbox & 3, xhi = (tbox >> 2) & 3;
-    const int ylo = (tbox >> 4) & 3, yhi = (tbox >> 6) & 3;
-    const int zlo = DIM == 3 ? (tbox >> 8) & 3 : 0, zhi = DIM == 3 ? ((tbox >> 10) & 3) + 3 : 0;
-    const int ny = yhi + 4 - ylo;
-    const int r = threadIdx.x;
-    if (r >= ny * (zhi + 1 - zlo)) return false;
-    const int y = ylo + r % ny, z = zlo + r / ny;
-    const int jyz = ((y >> 2) << 1) | ((z >> 2) << 2);
-    const int half = (z >> 1) & 1;
-    const int shift = ((y & 3) << 2) | ((z & 1) << 4);
-    const uint32_t wa = smask[b][jyz][half], wb = smask[b][jyz | 1][half];
-    const uint32_t rba = (wa >> shift) & 0xFu, rbb = (wb >> shift) & 0xFu;
-    const uint32_t below = (1u << shift) - 1u;
-    int32_t ca = sstart[b][jyz][half] + __popc(wa & below) + __popc(rba & ((1u << xlo) - 1u));
-    int32_t cb = sstart[b][jyz | 1][half] + __popc(wb & below);
-#pragma unroll
-    for (int i = 0; i < 7; ++i) {
-      const int x = xlo + i;
-      v[i] = 0.f;
-      if (x <= xhi + 3) {
-        const bool hi = x >= 4;
-        if (((hi ? rbb : rba) >> (x & 3)) & 1u) v[i] = __ldg(u + (hi ? cb++ : ca++));
-      }
-    }
-    y_o = y;
-    z_o = z;
-    ylo_o = ylo;
-    xlo_o = xlo;
-    xhi_o = xhi;
-    return true;
-  };
-  auto load_masks = [&](int32_t t, int b) {
-    if (threadIdx.x < NB) {
-      const int j = threadIdx.x;
-      const uint64_t m = __ldg(L.tile_mask + 8 * (int64_t)t + j);
-      const int32_t s0 = __ldg(L.tile_bstart + 8 * (int64_t)t + j);
-      smask[b][j][0] = (uint32_t)m;
-      smask[b][j][1] = (uint32_t)(m >> 32);
-      sstart[b][j][0] = s0;
-      sstart[b][j][1] = s0 + __popc((uint32_t)m);
-    }
-  };
-  auto store_rows = [&](int b, const float v[7], int y, int z, int xlo, int xhi) {
-    float* row = win[b] + (z * 7 + y) * RS;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (xlo + i <= xhi) store4(row + 4 * (xlo + i), v[i], v[i + 1], v[i + 2], v[i + 3]);
-  };
-  // prologue: the first tile's box
-  int buf = 0;
-  load_masks(tile, 0);
-  __syncthreads();
-  {
-    float v[7];
-    int ylo, y, z, xlo, xhi;
-    if (load_rows(tile, 0, v, ylo, z, y, xlo, xhi)) store_rows(0, v, y, z, xlo, xhi);
-  }
-  __syncthreads();
-  for (; tile < L.ntiles; tile += gridDim.x) {
-    const int32_t next = tile + gridDim.x;
-    const bool has_next = next < L.ntiles;
-    if (has_next) load_masks(next, buf ^ 1);
-    __syncthreads();
-    float v[7];
-    int ylo = 0, y = 0, z = 0, xlo = 0, xhi = 0;
-    const bool row = has_next && load_rows(next, buf ^ 1, v, ylo, z, y, xlo, xhi);
-    // the points of this tile from win[buf]
-    const int32_t beg = __ldg(L.tile_start + tile);
-    const int32_t end = with_ghost ? __ldg(L.tile_start + tile + 1) : __ldg(L.tile_mid + tile);
-    for (int32_t k = beg + threadIdx.x; k < end; k += kPipeThreads) {
-      const uint32_t rec = __ldg(L.erec + k);
-      PointWeights<float, DIM> pw;
-      pw.load(L, k);
-      const float* base = win[buf] + ((rec >> 4) & 3) * 7 * RS + ((rec >> 2) & 3) * RS + (rec & 3) * 4;
-      w[rec >> 6] = contract<DIM>(base, pw);
-    }
-    if (row) store_rows(buf ^ 1, v, y, z, xlo, xhi);
-    __syncthreads();
-    buf ^= 1;
-  }
-}
-
-#ifndef CPM_EXT_CHUNKED
-#define CPM_EXT_CHUNKED 0
-#endif
-constexpr bool kChunked = CPM_EXT_CHUNKED != 0;
-#ifndef CPM_EXT_CHUNK_THREADS
-#define CPM_EXT_CHUNK_THREADS 64
-#endif
-constexpr int kChunkThreads = CPM_EXT_CHUNK_THREADS;
-
-// One thread per chunk (up to kChunkMax points with one stencil base): the
-// thread streams the base's 4^d stencil rows from the staged box, one 16-byte
-// shared-memory load per row, and accumulates every point of the chunk from
-// each row, in the order of `contract` (y and z first with paired FMAs, then
-// x), so the results equal the per-point kernel's bit for bit.  A chunk of one
-// point repeats it in the second slot and stores it once.
-template <int DIM>
-__global__ void __launch_bounds__(kChunkThreads) k_extend_chunks(LevelView<float> L,
-                                                                 const float* __restrict__ u,
-                                                                 float* __restrict__ w, bool with_ghost) {
-  constexpr int RS = kRS;
-  constexpr int NC = DIM == 3 ? 4 : 1;
-  __shared__ TileBox<float, DIM, false> sm;
-  const int32_t tile = blockIdx.x;
-  const uint32_t tbox = __ldg(L.tile_box + tile);
-  const int32_t cbeg = __ldg(L.tile_cstart + tile);
-  const int32_t cend = with_ghost ? __ldg(L.tile_cstart + tile + 1) : __ldg(L.tile_cmid + tile);
-  if (cbeg == cend) return;  // a tile of ghost points only, extension over B
-  int32_t c = cbeg + threadIdx.x;
-  uint32_t ch = c < cend ? __ldg(L.echunk + c) : 0u;
-  stage_box<float, DIM, false, kChunkThreads>(L, u, tile, tbox, sm);
-  for (; c < cend; c += kChunkThreads) {
-    const int32_t k0 = (int32_t)(ch & 0x3FFFFFFu);
-    const int cnt = (int)(ch >> 26) + 1;
-    PointWeights<float, DIM> pw[kChunkMax];
-    uint32_t rec[kChunkMax];
-#pragma unroll
-    for (int j = 0; j < kChunkMax; ++j) {
-      const int32_t kj = k0 + (j < cnt ? j : 0);
-      rec[j] = __ldg(L.erec + kj);
-      pw[j].load(L, kj);
-    }
-    const int32_t cn = c + kChunkThreads;
-    if (cn < cend) ch = __ldg(L.echunk + cn);
-    const float* base = sm.win + ((rec[0] >> 4) & 3) * 7 * RS + ((rec[0] >> 2) & 3) * RS + (rec[0] & 3) * 4;
-    float2 q01[kChunkMax], q23[kChunkMax];
-#pragma unroll
-    for (int cc = 0; cc < NC; ++cc) {
-      float2 p01[kChunkMax], p23[kChunkMax];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const float4 v = *reinterpret_cast<const float4*>(base + (cc * 7 + b) * RS);
-#pragma unroll
-        for (int j = 0; j < kChunkMax; ++j) {
-          const float2 wyb = make_float2(pw[j].wy[b], pw[j].wy[b]);
-          if (b == 0) {
-            p01[j] = __fmul2_rn(wyb, make_float2(v.x, v.y));
-            p23[j] = __fmul2_rn(wyb, make_float2(v.z, v.w));
-          } else {
-            p01[j] = __ffma2_rn(wyb, make_float2(v.x, v.y), p01[j]);
-            p23[j] = __ffma2_rn(wyb, make_float2(v.z, v.w), p23[j]);
-          }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kChunkMax; ++j) {
-        const float wzc = DIM == 3 ? pw[j].wz[cc] : 1.f;
-        const float2 wz2 = make_float2(wzc, wzc);
-        if (cc == 0) {
-          q01[j] = __fmul2_rn(wz2, p01[j]);
-          q23[j] = __fmul2_rn(wz2, p23[j]);
-        } else {
-          q01[j] = __ffma2_rn(wz2, p01[j], q01[j]);
-          q23[j] = __ffma2_rn(wz2, p23[j], q23[j]);
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < kChunkMax; ++j) {
-      if (j < cnt) {
-        const float2 t = __ffma2_rn(make_float2(pw[j].wx[2], pw[j].wx[3]), q23[j],
-                                    __fmul2_rn(make_float2(pw[j].wx[0], pw[j].wx[1]), q01[j]));
-        w[rec[j] >> 6] = t.x + t.y;
-      }
-    }
-  }
-}
-
-// The FP32 extension's work decomposition ("tile variant") of a level:
-// EXT_TILES one CTA per tile, one thread per point; EXT_PIPE persistent CTAs
-// with the next tile's staging in flight; EXT_CHUNKS one thread per chunk of
-// points with one stencil base.  The hierarchy picks one per level by timing
-// (tune_extension).  CPM_EXT_PIPELINED / CPM_EXT_CHUNKED force a variant.
-template <typename T>
-static void extend_variant(const LevelView<T>& L, int variant, const T* u, T* w, bool with_ghost,
-                           cudaStream_t st) {
-  const int32_t nt = L.ntiles;
-  if constexpr (sizeof(T) == 4) {
-    if (variant == EXT_PIPE) {
-      const unsigned grid = (unsigned)std::min<int32_t>(nt, 152 * 16);
-      if (L.dim == 3)
-        k_extend_pipe<3><<<grid, kPipeThreads, 0, st>>>(L, u, w, with_ghost);
-      else
-        k_extend_pipe<2><<<grid, kPipeThreads, 0, st>>>(L, u, w, with_ghost);
-      return;
-    }
-    if (variant == EXT_CHUNKS) {
-      if (L.dim == 3)
-        k_extend_chunks<3><<<nt, kChunkThreads, 0, st>>>(L, u, w, with_ghost);
-      else
-        k_extend_chunks<2><<<nt, kChunkThreads, 0, st>>>(L, u, w, with_ghost);
-      return;
-    }
-  }
+void launch_extend(const LevelView<double>& L, const double* u, double* w, int32_t npts, cudaStream_t st) {
+  if (npts <= 0 || L.ntiles <= 0) return;
+  const bool with_ghost = npts > L.nB;
   if (L.dim == 3)
-    k_extend_tiles<T, 3><<<nt, kExtThreads, 0, st>>>(L, u, w, with_ghost, nullptr);
+    k_extend_tiles<double, 3><<<L.ntiles, kExtThreads, 0, st>>>(L, u, w, with_ghost, nullptr);
   else
-    k_extend_tiles<T, 2><<<nt, kExtThreads, 0, st>>>(L, u, w, with_ghost, nullptr);
-}
-
-template <typename T>
-void launch_extend(const LevelView<T>& L, const T* u, T* w, int32_t npts, cudaStream_t st) {
-  if (npts <= 0) return;
-  if (L.ntiles <= 0) return;
-  int variant = L.ext_variant;
-  if (kPipelined) variant = EXT_PIPE;
-  if (kChunked) variant = EXT_CHUNKS;
-  extend_variant<T>(L, variant, u, w, npts > L.nB, st);
+    k_extend_tiles<double, 2><<<L.ntiles, kExtThreads, 0, st>>>(L, u, w, with_ghost, nullptr);
   count_launch();
-}
-
-int tune_extension(const LevelView<float>& L, const float* u, float* w, cudaStream_t st, float ms[3]) {
-  int best = EXT_TILES;
-  for (int v = 0; v < 3; ++v) ms[v] = 0.f;
-  if (L.ntiles <= 0) return best;
-  cudaEvent_t e0, e1;
-  CPM_CUDA_TRY(cudaEventCreate(&e0));
-  CPM_CUDA_TRY(cudaEventCreate(&e1));
-  constexpr int kReps = 3;
-  for (int v = 0; v < 3; ++v) {
-    extend_variant<float>(L, v, u, w, true, st);  // warm-up
-    CPM_CUDA_TRY(cudaEventRecord(e0, st));
-    for (int r = 0; r < kReps; ++r) extend_variant<float>(L, v, u, w, true, st);
-    CPM_CUDA_TRY(cudaEventRecord(e1, st));
-    CPM_CUDA_TRY(cudaEventSynchronize(e1));
-    CPM_CUDA_TRY(cudaEventElapsedTime(&ms[v], e0, e1));
-    ms[v] /= kReps;
-    if (ms[v] < ms[best]) best = v;
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  CPM_CUDA_TRY(cudaGetLastError());
-  return best;
 }
 
 template <typename T>
@@ -1018,10 +690,5 @@ template void launch_extend_rel<double>(const LevelView<double>&, const double*,
                                         cudaStream_t);
 template void launch_extend_rel<float>(const LevelView<float>&, const float*, float*, float*,
                                        cudaStream_t);
-
-template void launch_extend<double>(const LevelView<double>&, const double*, double*, int32_t,
-                                    cudaStream_t);
-template void launch_extend<float>(const LevelView<float>&, const float*, float*, int32_t,
-                                   cudaStream_t);
 
 }  // namespace cpm

@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "dense32.cuh"
 #include "gmres.cuh"
 #include "gemv.cuh"
 #include "mlp.cuh"
@@ -117,6 +118,7 @@ struct Work {
 
 struct HLevel {
   std::unique_ptr<Level> lev;
+  Dense32 dense;      // structures of the FP32 passes
   DBuf<double> c64;   // per-point c (empty: scalar)
   DBuf<float> c32;
   DBuf<double> a64;   // diffusion coefficient (CPM_OP_VARDIFF)
@@ -129,6 +131,7 @@ struct HLevel {
 
   template <typename T>
   LevelView<T> view() const;
+  DenseView dview() const { return dense_view(*lev, dense); }
   template <typename T>
   const T* cvec() const;
   template <typename T>
@@ -157,10 +160,6 @@ LevelView<double> HLevel::view<double>() const {
   v.ew64 = lev->ew64.get();
   v.ewp = lev->ewp.get();
   v.ntiles = lev->ntiles;
-  v.ext_variant = lev->ext_variant;
-  v.echunk = lev->echunk.get();
-  v.tile_cstart = lev->tile_cstart.get();
-  v.tile_cmid = lev->tile_cmid.get();
   v.nbr = lev->nbr.get();
   return v;
 }
@@ -186,10 +185,6 @@ LevelView<float> HLevel::view<float>() const {
   v.ew64 = lev->ew64.get();
   v.ewp = lev->ewp.get();
   v.ntiles = lev->ntiles;
-  v.ext_variant = lev->ext_variant;
-  v.echunk = lev->echunk.get();
-  v.tile_cstart = lev->tile_cstart.get();
-  v.tile_cmid = lev->tile_cmid.get();
   v.nbr = lev->nbr.get();
   return v;
 }
@@ -222,6 +217,7 @@ using namespace cpm;
 struct Workspace {
   std::vector<cpm::Work<double>> w64;
   std::vector<cpm::Work<float>> w32;
+  std::vector<cpm::DBuf<float>> ud, wd, fd;  // brick-dense u, w = E u and f of the FP32 passes
   cpm::DBuf<double> part;   // norm partials (2 per block)
   int part_blocks = 0;
   cpm::DBuf<double> own_norms;  // [max, sumsq, 1/max, -] unless norms points elsewhere
@@ -293,11 +289,19 @@ namespace cpm {
 static void alloc_workspace(const cpm_hier_s& H, Workspace& W, double* norms_slot = nullptr) {
   W.w64.resize(H.L.size());
   W.w32.resize(H.L.size());
+  W.ud.resize(H.L.size());
+  W.wd.resize(H.L.size());
+  W.fd.resize(H.L.size());
   for (size_t l = 0; l < H.L.size(); ++l) {
     const int64_t nB = H.L[l].lev->nB, np = H.L[l].lev->nplus();
     const bool paper = H.opts.op_form != CPM_OP_MBR;
     W.w64[l].alloc(nB, np, paper, H.opts.relative != 0);
     W.w32[l].alloc(nB, np, paper, H.opts.relative != 0);
+    const size_t slots = dense_size(*H.L[l].lev);
+    for (auto* v : {&W.ud[l], &W.wd[l], &W.fd[l]}) {
+      v->alloc(slots);
+      CPM_CUDA_TRY(cudaMemset(v->get(), 0, sizeof(float) * slots));
+    }
   }
   const int64_t nB0 = H.L[0].lev->nB;
   W.part_blocks = std::max<int>(std::max(lap_blocks_f64(H.L[0].view<double>()),
@@ -337,6 +341,34 @@ static void alloc_workspace(const cpm_hier_s& H, Workspace& W, double* norms_slo
 namespace cpm {
 
 // ----------------------------------------------------------------- level ops
+// w = E u on the first npts points of B+ of level l, vectors in band order.
+static void extend(const HLevel& lv, const double* u, double* w, int32_t npts, cudaStream_t st) {
+  launch_extend(lv.view<double>(), u, w, npts, st);
+}
+static void extend(const HLevel& lv, const float* u, float* w, int32_t npts, cudaStream_t st) {
+  launch_extend32_compact(lv.dview(), u, w, npts, st);
+}
+
+// E u and then one stencil pass of the MBR form: FP64 in band order, FP32 with
+// w brick-dense.
+static void mbr_op(cpm_hier_s* H, Workspace& W, int l, LapMode mode, const double* f, const double* u,
+                   double* out, const double* dA, double* u_inout, double* part, cudaStream_t st) {
+  HLevel& lv = H->L[l];
+  const LevelView<double> v = lv.view<double>();
+  launch_extend(v, u, W.w64[l].w.get(), (int32_t)v.nplus, st);
+  launch_lap(v, mode, u, W.w64[l].w.get(), f, lv.c64.get(), H->c, dA, H->opts.omega, out, u_inout,
+                     part, 0, st);
+}
+static void mbr_op(cpm_hier_s* H, Workspace& W, int l, LapMode mode, const float* f, const float* u,
+                   float* out, const float*, float* u_inout, double*, cudaStream_t st) {
+  HLevel& lv = H->L[l];
+  const DenseView v = lv.dview();
+  const Vec32<const float> uv{nullptr, u};
+  launch_extend32(v, uv, W.wd[l].get(), st);
+  launch_lap32(v, mode, uv, W.wd[l].get(), f, (float)H->c, Vec32<float>{nullptr, u_inout ? u_inout : out},
+               nullptr, st);
+}
+
 // The operator of level l in the hierarchy's form: M u (APPLY), the residual
 // f - A u (RESID, block partials into part when given) or one weighted Jacobi
 // sweep on A u = f in place (JACOBI).  MBR form: w = E u on B+, then the
@@ -357,7 +389,7 @@ static void level_op(cpm_hier_s* H, Workspace& W, int l, LapMode mode, const T* 
       launch_lap_vard<T>(v, u, a, w.v.get(), st);
     else
       launch_lap_band<T>(v, u, w.v.get(), st);
-    launch_extend<T>(v, u, w.w.get(), v.nB, st);
+    extend(lv, u, w.w.get(), v.nB, st);
     launch_paper<T>(v, mode, u, w.v.get(), w.w.get(), f, lv.cvec<T>(), (T)H->c, dA, out, u_inout,
                     part, a, st);
   } else if (H->opts.relative && (mode == LAP_RESID || mode == LAP_JACOBI)) {
@@ -365,15 +397,36 @@ static void level_op(cpm_hier_s* H, Workspace& W, int l, LapMode mode, const T* 
     launch_lap_rel<T>(v, mode == LAP_RESID ? LAP_RESID_REL : LAP_JAC_REL, u, w.w.get(), w.refv.get(), f,
                       lv.cvec<T>(), (T)H->c, dA, out, u_inout, part, st);
   } else {
-    launch_extend<T>(v, u, w.w.get(), (int32_t)v.nplus, st);
-    launch_lap<T>(v, mode, u, w.w.get(), f, lv.cvec<T>(), (T)H->c, dA, (T)H->opts.omega, out,
-                  u_inout, part, 0, st);
+    mbr_op(H, W, l, mode, f, u, out, dA, u_inout, part, st);
+  }
+}
+
+// Weighted Jacobi sweeps of the MBR form in FP32: u and f are read in band order
+// by the first sweep, stay brick-dense between sweeps, and u is written back in
+// band order by the last.
+static void smooth32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* u, int sweeps,
+                     cudaStream_t st) {
+  HLevel& lv = H->L[l];
+  const DenseView v = lv.dview();
+  const Vec32<float> dense{W.ud[l].get(), nullptr}, compact{nullptr, u};
+  for (int s = 0; s < sweeps; ++s) {
+    const Vec32<float> in = s == 0 ? compact : dense, out = s == sweeps - 1 ? compact : dense;
+    const Vec32<const float> cin{in.dense, in.compact};
+    launch_extend32(v, cin, W.wd[l].get(), st);
+    launch_lap32(v, LAP_JACOBI, cin, W.wd[l].get(), s == 0 ? f : W.fd[l].get(), (float)H->c, out,
+                 sweeps > 1 ? W.fd[l].get() : nullptr, st);
   }
 }
 
 template <typename T>
 static void smooth(cpm_hier_s* H, Workspace& W, int l, const T* f, T* u, int sweeps,
                    cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    if (H->opts.smoother == CPM_SMOOTH_JACOBI && H->opts.op_form == CPM_OP_MBR && !H->opts.relative) {
+      smooth32(H, W, l, f, u, sweeps, st);
+      return;
+    }
+  }
   HLevel& lv = H->L[l];
   const LevelView<T> v = lv.view<T>();
   Work<T>& w = W.work<T>(l);
@@ -382,7 +435,7 @@ static void smooth(cpm_hier_s* H, Workspace& W, int l, const T* f, T* u, int swe
   for (int s = 0; s < sweeps; ++s) {
     if (H->opts.smoother == CPM_SMOOTH_RM) {
       launch_rm_jacobi<T>(v, u, f, lv.cvec<T>(), cval, omega, w.tmp.get(), st);
-      launch_extend<T>(v, w.tmp.get(), u, v.nB, st);
+      extend(lv, w.tmp.get(), u, v.nB, st);
     } else if (H->opts.smoother == CPM_SMOOTH_RBGS) {
       level_op<T>(H, W, l, LAP_JAC_RED, f, u, nullptr, nullptr, st);
       level_op<T>(H, W, l, LAP_JAC_BLACK, f, u, nullptr, nullptr, st);
@@ -405,7 +458,7 @@ static void transfer_residual(cpm_hier_s* H, Workspace& W, int l, const T* f, co
     level_op<T>(H, W, l, LAP_RESID, f, u, r, nullptr, st);
   } else {
     // f - A (E u): first E u on B, then the residual of that re-extended iterate
-    launch_extend<T>(v, u, w.tmp.get(), v.nB, st);
+    extend(lv, u, w.tmp.get(), v.nB, st);
     level_op<T>(H, W, l, LAP_RESID, f, w.tmp.get(), r, nullptr, st);
   }
 }
@@ -488,9 +541,7 @@ static void vcycle_level(cpm_hier_s* H, Workspace* const* W, int G, int l, const
       if (l == 0 && H->learned_active && pre > 0) {
         // learned smoother in place of the first Jacobi sweep: r = f - A u, u += net(r)
         const LevelView<float> v = lv.view<float>();
-        launch_extend<float>(v, u[g], w.w.get(), (int32_t)v.nplus, st);
-        launch_lap<float>(v, LAP_RESID, u[g], w.w.get(), f[g], lv.cvec<float>(), (float)H->c, nullptr,
-                          0.f, w.r.get(), nullptr, nullptr, 0, st);
+        mbr_op(H, *W[g], l, LAP_RESID, f[g], u[g], w.r.get(), nullptr, nullptr, nullptr, st);
         mlp_forward(H->mlp->params.get(), *H->mlpd, w.r.get(), 1.f / v.inv_h2, nullptr, u[g], nullptr,
                     st);
         --pre;
@@ -755,8 +806,6 @@ static void copy_level(const Level& a, Level& b, cudaStream_t st) {
   b.ntiles = a.ntiles;
   cp(b.tile_brick, a.tile_brick); cp(b.tile_box, a.tile_box); cp(b.tile_mask, a.tile_mask); cp(b.tile_bstart, a.tile_bstart); cp(b.tile_start, a.tile_start); cp(b.tile_mid, a.tile_mid); cp(b.erec, a.erec);
   cp(b.efr32, a.efr32); cp(b.ew64, a.ew64); cp(b.nbr, a.nbr);
-  b.nchunks = a.nchunks;
-  cp(b.echunk, a.echunk); cp(b.tile_cstart, a.tile_cstart); cp(b.tile_cmid, a.tile_cmid);
 }
 
 static void build_transfer(const Level& target, const Level& src, Transfer& t, int deg,
@@ -885,6 +934,7 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
   CPM_CHECK(o.coarse_gmres >= 0 && o.coarse_gmres <= 1000, CPM_ERR_ARG, "bad coarse_gmres");
   CPM_CHECK(o.residual_mode == 0 || o.residual_mode == 1, CPM_ERR_ARG, "bad residual_mode");
 
+  for (auto& lv : H->L) build_dense32(*lv.lev, lv.dense, st);
   DBuf<int32_t> err(1);
   CPM_CUDA_TRY(cudaMemsetAsync(err.get(), 0, sizeof(int32_t), st));
   for (int l = 0; l + 1 < nl; ++l) {
@@ -938,6 +988,7 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
     CPM_CUDA_TRY(cudaGetLastError());
     CPM_CUDA_TRY(cudaStreamSynchronize(st));
     lv.dM64 = std::move(dM);
+    dense_static(*lv.lev, lv.dense, lv.dA32.get(), lv.c32.get(), st);
   }
   // coarsest: dense A = diag(c) - M, inverted in place (FP64)
   H->nc = cl.nB;
@@ -982,17 +1033,12 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
 
   // solve buffers
   alloc_workspace(*H, H->ws);
-  // the FP32 extension variant of every level, by timing (its "tile": one
-  // thread per point, persistent pipelined tiles, or chunks of one base)
+  // the launch shape of every level's FP32 extension, by timing
   for (int l = 0; l < nl; ++l) {
     Level& lev = *H->L[l].lev;
-    if (o.ext_variant > 0) {
-      lev.ext_variant = o.ext_variant - 1;
-      continue;
-    }
-    CPM_CUDA_TRY(cudaMemsetAsync(H->ws.w32[l].u.get(), 0, sizeof(float) * lev.nB, st));
-    lev.ext_variant = tune_extension(H->L[l].view<float>(), H->ws.w32[l].u.get(), H->ws.w32[l].w.get(),
-                                     st, lev.ext_ms);
+    lev.ext_variant = o.ext_variant > 0 ? o.ext_variant - 1
+                                        : tune_extend32(H->L[l].dview(), H->ws.ud[l].get(), H->ws.wd[l].get(),
+                                                        st, lev.ext_ms);
   }
   *out = H.release();
   CPM_API_END
@@ -1045,10 +1091,10 @@ cpm_status cpm_extend(cpm_hier h, int32_t level, int32_t prec, const void* u, vo
   HLevel& lv = h->L[level];
   const int32_t np = with_ghost ? (int32_t)lv.lev->nplus() : lv.lev->nB;
   if (prec == CPM_F64) {
-    launch_extend<double>(lv.view<double>(), (const double*)u, (double*)w, np, st);
+    extend(lv, (const double*)u, (double*)w, np, st);
   } else {
     CPM_CHECK(prec == CPM_F32, CPM_ERR_ARG, "unknown precision");
-    launch_extend<float>(lv.view<float>(), (const float*)u, (float*)w, np, st);
+    extend(lv, (const float*)u, (float*)w, np, st);
   }
   CPM_CUDA_TRY(cudaGetLastError());
   CPM_API_END
@@ -1444,7 +1490,7 @@ static void mlp_loss_grad_host(cpm_hier h, const float* r, cudaStream_t st) {
   CPM_CHECK(h != nullptr && r != nullptr, CPM_ERR_ARG, "NULL argument");
   CPM_CHECK(h->mlp && h->mlpd, CPM_ERR_ARG, "no learned smoother set (cpm_hier_set_smoother)");
   HLevel& lv = h->L[0];
-  mlp_loss_grad(h->mlp->params.get(), *h->mlpd, lv.view<float>(), lv.c32.get(), (float)h->c, r,
+  mlp_loss_grad(h->mlp->params.get(), *h->mlpd, lv.view<float>(), lv.dview(), lv.c32.get(), (float)h->c, r,
                 h->mlp->tb, st);
 }
 
@@ -1496,7 +1542,7 @@ cpm_status cpm_mlp_train(cpm_mlp m, const cpm_train_set* set, const cpm_train_op
   cudaStream_t st = (cudaStream_t)stream;
   const int nf = set->n_fields;
   int32_t maxB = 0;
-  int64_t maxP = 0;
+  int64_t maxP = 0, maxS = 0;
   for (int k = 0; k < nf; ++k) {
     cpm_hier h = set->hier[k];
     CPM_CHECK(h != nullptr && set->r[k] != nullptr, CPM_ERR_ARG, "cpm_mlp_train: NULL field");
@@ -1507,13 +1553,14 @@ cpm_status cpm_mlp_train(cpm_mlp m, const cpm_train_set* set, const cpm_train_op
     }
     maxB = std::max(maxB, h->L[0].lev->nB);
     maxP = std::max(maxP, h->L[0].lev->nplus());
+    maxS = std::max(maxS, (int64_t)dense_size(*h->L[0].lev));
   }
   if (o.reset) {
     CPM_CUDA_TRY(cudaMemsetAsync(m->m.get(), 0, kNParams * sizeof(float), st));
     CPM_CUDA_TRY(cudaMemsetAsync(m->v.get(), 0, kNParams * sizeof(float), st));
     m->step = 0;
   }
-  m->tb.ensure(maxB, maxP);
+  m->tb.ensure(maxB, maxP, maxS);
   // the fields scaled by 1 / max|r| into FP32
   std::vector<DBuf<float>> f32(nf);
   DBuf<double> norms(4 * (size_t)nf), part(2 * (size_t)kNormBlocks);

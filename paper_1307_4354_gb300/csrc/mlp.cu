@@ -583,11 +583,12 @@ void mlp_forward(const float* params, const MlpLevelData& D, const float* r, flo
   count_launch();
 }
 
-void MlpTrainBuffers::ensure(int32_t nB, int64_t nplus) {
+void MlpTrainBuffers::ensure(int32_t nB, int64_t nplus, int64_t slots) {
   nparts = kBwdCtas;
-  if (nB <= n && nplus <= np) return;  // capacity suffices
-  n = nB;
-  np = nplus;
+  if (nB <= n && nplus <= np && slots <= ns) return;  // capacity suffices
+  n = nB = std::max(n, nB);
+  np = nplus = std::max(np, nplus);
+  ns = slots = std::max(ns, slots);
   Xs.alloc((size_t)nB * 32);
   H1.alloc((size_t)nB * 64);
   H2.alloc((size_t)nB * 64);
@@ -595,7 +596,7 @@ void MlpTrainBuffers::ensure(int32_t nB, int64_t nplus) {
   du.alloc(nB);
   Mdu.alloc(nB);
   z.alloc(nB);
-  w.alloc(nplus);
+  w.alloc(slots);
   t.alloc(nplus);
   et.alloc(nB);
   dy.alloc(nB);
@@ -608,16 +609,16 @@ void MlpTrainBuffers::ensure(int32_t nB, int64_t nplus) {
 
 // Loss and gradient of one residual field (FP32 on level 0 of the view L).
 void mlp_loss_grad(const float* params, const MlpLevelData& D, const LevelView<float>& L,
-                   const float* cvec, float cval, const float* r, MlpTrainBuffers& tb,
+                   const DenseView& DL, const float* cvec, float cval, const float* r, MlpTrainBuffers& tb,
                    cudaStream_t st) {
   const int32_t nB = L.nB;
   const float dx2 = 1.f / L.inv_h2;
-  tb.ensure(nB, L.nplus);
+  tb.ensure(nB, L.nplus, ((int64_t)DL.nbricks + 1) << (2 * DL.dim));
   mlp_forward(params, D, r, dx2, tb.du.get(), nullptr, &tb, st);
   // M du (extension over B+ then the stencil)
-  launch_extend<float>(L, tb.du.get(), tb.w.get(), (int32_t)L.nplus, st);
-  launch_lap<float>(L, LAP_APPLY, tb.du.get(), tb.w.get(), nullptr, nullptr, 0.f, nullptr, 0.f,
-                    tb.Mdu.get(), nullptr, nullptr, 0, st);
+  const Vec32<const float> du{nullptr, tb.du.get()};
+  launch_extend32(DL, du, tb.w.get(), st);
+  launch_lap32(DL, LAP_APPLY, du, tb.w.get(), nullptr, 0.f, Vec32<float>{nullptr, tb.Mdu.get()}, nullptr, st);
   const int nb256 = (int)((nB + 255) / 256);
   k_mlp_resid<<<nb256, 256, 0, st>>>(r, tb.du.get(), tb.Mdu.get(), cvec, cval, nB, tb.z.get(),
                                       tb.lpart.get());

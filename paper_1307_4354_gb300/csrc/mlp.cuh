@@ -3,7 +3,7 @@
 
 #include <cuda_bf16.h>
 
-#include "ops.cuh"
+#include "dense32.cuh"
 
 namespace cpm {
 
@@ -28,12 +28,12 @@ struct MlpLevelData {
 
 struct MlpTrainBuffers {
   int32_t n = -1;
-  int64_t np = -1;
+  int64_t np = -1, ns = -1;
   int nparts = 0;
   DBuf<__nv_bfloat16> Xs, H1, H2;
   DBuf<float> S, du, Mdu, z, w, t, et, dy, part, grad;
   DBuf<double> lpart, loss;
-  void ensure(int32_t nB, int64_t nplus);
+  void ensure(int32_t nB, int64_t nplus, int64_t slots);
 };
 
 // du = network correction of residual r (u_add != null: u_add += du instead);
@@ -42,7 +42,7 @@ void mlp_forward(const float* params, const MlpLevelData& D, const float* r, flo
                  float* u_add, const MlpTrainBuffers* tb, cudaStream_t st);
 // Loss ||r - A du||^2 / ||r||^2 (tb.loss: [||z||^2, ||r||^2]) and gradient (tb.grad).
 void mlp_loss_grad(const float* params, const MlpLevelData& D, const LevelView<float>& L,
-                   const float* cvec, float cval, const float* r, MlpTrainBuffers& tb,
+                   const DenseView& DL, const float* cvec, float cval, const float* r, MlpTrainBuffers& tb,
                    cudaStream_t st);
 void mlp_adam(float* params, const float* grad, float* m, float* v, int64_t step, float lr,
               cudaStream_t st);

@@ -142,7 +142,7 @@ void residual_norms_noalloc(const LevelView<double>& v, const double* f, const d
   double* scratch = scratch_address();
   double* w = scratch;
   double* part = scratch + CPM_NOALLOC_MAX_POINTS_VALUE;
-  launch_extend<double>(v, u, w, (int32_t)v.nplus, st);
+  launch_extend(v, u, w, (int32_t)v.nplus, st);
   const int nblocks = (v.nB + 255) / 256;
   if (nblocks > 0) {
     k_resid_partials_noalloc<<<nblocks, 256, 0, st>>>(v, u, w, f, cvec, cval, part);

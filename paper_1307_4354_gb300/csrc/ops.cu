@@ -323,10 +323,10 @@ static void lap_dim(const LevelView<T>& L, const T* u, const T* w, const T* f, c
     lap_dispatch<2, MODE>(L, u, w, f, cvec, cval, dA, omega, out, u_inout, part, refv, st);
 }
 
-template <typename T>
-void launch_lap(const LevelView<T>& L, LapMode mode, const T* u, const T* w, const T* f,
-                const T* cvec, T cval, const T* dA, T omega, T* out, T* u_inout, double* part,
-                int nblocks_part, cudaStream_t st) {
+void launch_lap(const LevelView<double>& L, LapMode mode, const double* u, const double* w,
+                const double* f, const double* cvec, double cval, const double* dA, double omega,
+                double* out, double* u_inout, double* part, int nblocks_part, cudaStream_t st) {
+  using T = double;
   (void)nblocks_part;
   if (mode == LAP_APPLY) lap_dim<LAP_APPLY>(L, u, w, f, cvec, cval, dA, omega, out, u_inout, part, (const T*)nullptr, st);
   if (mode == LAP_RESID) lap_dim<LAP_RESID>(L, u, w, f, cvec, cval, dA, omega, out, u_inout, part, (const T*)nullptr, st);
@@ -1182,8 +1182,6 @@ void invert_dense(double* A, int32_t n, cudaStream_t st, int32_t* err) {
 
 // ----------------------------------------------------------------- instantiations
 #define CPM_INST(T)                                                                              \
-  template void launch_lap<T>(const LevelView<T>&, LapMode, const T*, const T*, const T*,        \
-                              const T*, T, const T*, T, T*, T*, double*, int, cudaStream_t);      \
   template void launch_rm_jacobi<T>(const LevelView<T>&, const T*, const T*, const T*, T, T, T*, \
                                     cudaStream_t);                                               \
   template void launch_rm_resid<T>(const LevelView<T>&, const T*, const T*, const T*, T, T*,     \

@@ -29,10 +29,6 @@ struct LevelView {
   const double* ew64;   // E-order FP64 weights
   const float2* ewp;    // E-order weights as FP32 pairs (finest level, pair residual)
   int32_t ntiles;
-  int ext_variant;            // FP32 extension work decomposition (ExtVariant)
-  const uint32_t* echunk;     // chunk records (ext.cu)
-  const int32_t* tile_cstart; // ntiles + 1 chunk offsets
-  const int32_t* tile_cmid;   // per tile: end of its chunks of B
   const int32_t* nbr;   // 2d x nB neighbour indices into B+
 };
 
@@ -59,15 +55,9 @@ enum LapMode { LAP_APPLY = 0, LAP_RESID = 1, LAP_JACOBI = 2, LAP_RESID_REL = 3,
 // that of the global ones.
 __host__ __device__ inline int node_colour_local(int l) { return ((l & 3) + ((l >> 2) & 3) + (l >> 4)) & 1; }
 
-enum ExtVariant { EXT_TILES = 0, EXT_PIPE = 1, EXT_CHUNKS = 2 };
-// Time the three FP32 extension variants on a level (over B+, one warm-up and
-// three timed launches each, CUDA events on st) and return the fastest; ms[v]
-// gets each variant's time.  u, w: device scratch of nB and nB + nG floats.
-int tune_extension(const LevelView<float>& L, const float* u, float* w, cudaStream_t st, float ms[3]);
-
-// w = E u on the first npts points of B+ (npts = nB or nB + nG).
-template <typename T>
-void launch_extend(const LevelView<T>& L, const T* u, T* w, int32_t npts, cudaStream_t st);
+// w = E u on the first npts points of B+ (npts = nB or nB + nG), FP64 (the FP32
+// extension is in dense32.cuh).
+void launch_extend(const LevelView<double>& L, const double* u, double* w, int32_t npts, cudaStream_t st);
 
 // Extension over B+ in relative form: delta_j = (E u)_j - ref_j with
 // ref_j = u at a reference node of j's tile (see k_extend_tiles).
@@ -92,10 +82,10 @@ void launch_resid_rel(const LevelView<double>& L, const double* u, const double*
 //   RESID : out = f - c u + M u  (and block partials of max|out|, sum out^2
 //           into part[2*block], part[2*block+1] if part != nullptr)
 //   JACOBI: u += (f - c u + M u) * wdA, wdA = omega / dA (in place, out unused)
-template <typename T>
-void launch_lap(const LevelView<T>& L, LapMode mode, const T* u, const T* w, const T* f,
-                const T* cvec, T cval, const T* dA, T omega, T* out, T* u_inout, double* part,
-                int nblocks_part, cudaStream_t st);
+// (FP64; the FP32 passes are in dense32.cuh.)
+void launch_lap(const LevelView<double>& L, LapMode mode, const double* u, const double* w,
+                const double* f, const double* cvec, double cval, const double* dA, double omega,
+                double* out, double* u_inout, double* part, int nblocks_part, cudaStream_t st);
 
 // Number of blocks (2 partial doubles each) of a RESID / RESID_REL stencil pass.
 int lap_blocks_f64(const LevelView<double>& L);

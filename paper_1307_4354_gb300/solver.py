@@ -111,7 +111,7 @@ class Hierarchy:
         self.n_levels, self.nb = capi.cpm_hier_info(self.handle, 0)
 
     def ext_tuning(self, level: int = 0):
-        """(FP32 extension variant chosen for the level, ms of each candidate)."""
+        """(FP32 extension launch shape chosen for the level, ms of each candidate)."""
         return capi.cpm_hier_ext_tuning(self.handle, level)
 
     def level_size(self, level: int) -> int:
