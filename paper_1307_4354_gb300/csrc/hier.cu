@@ -266,7 +266,7 @@ struct cpm_hier_s {
   double c = 1.0;
   std::vector<HLevel> L;
   DBuf<double> Ainv;     // coarse_mode 0: FP64 inverse
-  DBuf<float> Ainv32;    // coarse_mode 1: FP32 inverse
+  DBuf<float> Ainv32;    // coarse_mode 1: FP32 inverse, rows of ld_f32 floats
   DBuf<float> Ainv_f32;  // coarse_mode 0: the FP64 inverse rounded to FP32, for FP32
                          // V-cycles (FP32 GEMV at twice the bandwidth and off the FP64
                          // pipe); built when it takes at most kCoarseF32CopyMax points;
@@ -477,7 +477,7 @@ static void coarse_solve(cpm_hier_s* H, Workspace* const* W, int G, const T* con
   if (H->coarse_mode == 0) {
     if constexpr (sizeof(T) == 4) {
       if (H->Ainv_f32.n > 0) {
-        launch_dense_gemv_v4<T>(H->Ainv_f32.get(), H->ld_f32, f, u, G, H->nc, st);
+        launch_dense_gemv_v4<T, false>(H->Ainv_f32.get(), H->ld_f32, f, u, G, H->nc, st);
         count_launch((G + kGemvMaxVectors - 1) / kGemvMaxVectors);
         return;
       }
@@ -486,7 +486,7 @@ static void coarse_solve(cpm_hier_s* H, Workspace* const* W, int G, const T* con
     return;
   }
   if (H->coarse_mode == 1) {
-    launch_coarse_gemv32<T>(H->Ainv32.get(), f, u, G, H->nc, false, st);
+    launch_coarse_gemv32<T>(H->Ainv32.get(), H->ld_f32, f, u, G, H->nc, false, st);
     if constexpr (sizeof(T) == 8) {
       // two steps of iterative refinement with the FP64 residual of the level
       HLevel& lv = H->L[l];
@@ -496,7 +496,7 @@ static void coarse_solve(cpm_hier_s* H, Workspace* const* W, int G, const T* con
       for (int it = 0; it < 2; ++it) {
         for (int g = 0; g < G; ++g)
           level_op<double>(H, *W[g], l, LAP_RESID, f[g], u[g], W[g]->w64[l].r.get(), nullptr, st);
-        launch_coarse_gemv32<double>(H->Ainv32.get(), r, u, G, H->nc, true, st);
+        launch_coarse_gemv32<double>(H->Ainv32.get(), H->ld_f32, r, u, G, H->nc, true, st);
       }
     }
     return;
@@ -1022,8 +1022,9 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
       launch_assemble_A<float>(H->L[nl - 1].view<double>(), H->L[nl - 1].c64.get(), H->c,
                                A32.get(), st);
     CPM_CUDA_TRY(cudaGetLastError());
-    H->Ainv32.alloc(nn);
-    invert_dense_f32(A32.get(), H->Ainv32.get(), H->nc, st, err.get());
+    H->ld_f32 = (H->nc + 3) / 4 * 4;
+    H->Ainv32.alloc((size_t)H->nc * H->ld_f32);
+    invert_dense_f32(A32.get(), H->Ainv32.get(), H->nc, H->ld_f32, st, err.get());
   }
   int32_t herr = 0;
   CPM_CUDA_TRY(cudaMemcpyAsync(&herr, err.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, st));

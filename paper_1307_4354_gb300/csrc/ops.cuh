@@ -183,10 +183,10 @@ void residual_norms_noalloc(const LevelView<double>& v, const double* f, const d
 
 // Coarsest solve with an FP32 explicit inverse (coarse32.cu): x_g (+)= Ainv b_g.
 template <typename T>
-void launch_coarse_gemv32(const float* Ainv, const T* const* b, T* const* x, int G, int32_t n, bool add,
-                          cudaStream_t st);
-// A (row-major FP32, overwritten) -> X = A^-1 (library LU, setup only).
-void invert_dense_f32(float* A, float* X, int32_t n, cudaStream_t st, int32_t* err);
+void launch_coarse_gemv32(const float* Ainv, int32_t ld, const T* const* b, T* const* x, int G, int32_t n,
+                          bool add, cudaStream_t st);
+// A (row-major FP32, overwritten) -> X = A^-1 in rows of ld floats (library LU, setup only).
+void invert_dense_f32(float* A, float* X, int32_t n, int32_t ld, cudaStream_t st, int32_t* err);
 
 // Setup kernels.
 void launch_diag_M(const LevelView<double>& L, double* diagM, cudaStream_t st);
