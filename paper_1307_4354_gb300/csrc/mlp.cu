@@ -9,7 +9,7 @@
 // relu(W1^T x + b1) + b2) + b3.
 //
 // Forward: BF16 weights and features, FP32 accumulation on the tensor cores
-// (warp-level mma.sync m16n8k16, one warp per 16 points).  Training: the loss
+// (warp-level mma.sync m16n8k16, one warp per 32 points).  Training: the loss
 // of a residual field r is ||r - A du||^2 / ||r||^2; its gradient with
 // respect to du is -2 A^T (r - A du) / ||r||^2 (A^T through a transposed
 // neighbour gather and a transposed extension scatter over the extension
@@ -76,22 +76,26 @@ struct MlpFwdArgs {
   const float* stat;
   int32_t nB;
   float dx2;
-  float* du;             // out: correction (mode 0) ...
-  float* u;              // ... or u += correction (mode 1)
-  // training outputs (mode 0, may be null)
+  float* du;             // out: correction ...
+  float* u;              // ... or u += correction
+  // training outputs
   __nv_bfloat16* Xs;     // nB x 32
   __nv_bfloat16* H1;     // nB x 64
   __nv_bfloat16* H2;     // nB x 64
   float* S;              // nB
 };
 
+// MODE: 0 du = correction, 1 u += correction, 2 du and the training outputs.
+// Bound by the latency of the feature gather (27 indices, then 27 values, all in
+// flight per lane): 1.63 M points 113 us with a point per lane and three CTAs
+// on an SM, against 170 us with a point per lane of a half warp.
 template <int MODE>
-__global__ void __launch_bounds__(kFwdWarps * 32) k_mlp_forward(MlpFwdArgs A) {
+__global__ void __launch_bounds__(kFwdWarps * 32, MODE == 2 ? 2 : 3) k_mlp_forward(MlpFwdArgs A) {
   __shared__ __align__(16) __nv_bfloat16 w1t[64 * kW1S];  // w1t[n][k] = W1[k][n]
   __shared__ __align__(16) __nv_bfloat16 w2t[64 * kW2S];
   __shared__ float bias1[64], bias2[64], w3s[64];
-  __shared__ __align__(16) __nv_bfloat16 xs[kFwdWarps][16 * kXS];
-  __shared__ float ss[kFwdWarps][16];
+  __shared__ __align__(16) __nv_bfloat16 xs[kFwdWarps][32 * kXS];
+  __shared__ float ss[kFwdWarps][32];
   for (int q = threadIdx.x; q < 64 * 32; q += blockDim.x) {
     const int n = q & 63, k = q >> 6;
     w1t[n * kW1S + k] = __float2bfloat16_rn(A.params[kOffW1 + k * 64 + n]);
@@ -109,45 +113,51 @@ __global__ void __launch_bounds__(kFwdWarps * 32) k_mlp_forward(MlpFwdArgs A) {
   const float b3 = A.params[kOffB3];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
-  __nv_bfloat16* xw = xs[warp];
-  const int64_t ngroups = ((int64_t)A.nB + 15) / 16;
-  for (int64_t grp = (int64_t)blockIdx.x * kFwdWarps + warp; grp < ngroups;
-       grp += (int64_t)gridDim.x * kFwdWarps) {
-    const int64_t p0 = grp * 16;
-    // features: lanes 0..15 one point each
-    if (lane < 16) {
-      const int64_t p = p0 + lane;
+  const int64_t nsteps = ((int64_t)A.nB + 31) / 32;
+  for (int64_t step = (int64_t)blockIdx.x * kFwdWarps + warp; step < nsteps;
+       step += (int64_t)gridDim.x * kFwdWarps) {
+    // features: one point per lane
+    {
+      const int64_t p = step * 32 + lane;
+      __nv_bfloat16* xw = xs[warp];
       float f[32];
       float smax = 0.f;
       if (p < A.nB) {
+        int32_t j[27];
 #pragma unroll
-        for (int q = 0; q < 27; ++q) {
-          const int32_t j = __ldg(A.nbr27 + (int64_t)q * A.nB + p);
-          f[q] = j >= 0 ? __ldg(A.r + j) : 0.f;
-          smax = fmaxf(smax, fabsf(f[q]));
-        }
+        for (int q = 0; q < 27; ++q) j[q] = __ldg(A.nbr27 + (int64_t)q * A.nB + p);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) f[27 + q] = __ldg(A.stat + (int64_t)q * A.nB + p);
+#pragma unroll
+        for (int q = 0; q < 27; ++q) f[q] = j[q] >= 0 ? __ldg(A.r + j[q]) : 0.f;
+#pragma unroll
+        for (int q = 0; q < 27; ++q) smax = fmaxf(smax, fabsf(f[q]));
         const float inv = smax > 0.f ? 1.f / smax : 0.f;
 #pragma unroll
         for (int q = 0; q < 27; ++q) f[q] *= inv;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) f[27 + q] = __ldg(A.stat + (int64_t)q * A.nB + p);
       } else {
 #pragma unroll
         for (int q = 0; q < 31; ++q) f[q] = 0.f;
       }
       f[31] = 0.f;
 #pragma unroll
-      for (int q = 0; q < 32; q += 2)
-        *reinterpret_cast<uint32_t*>(&xw[lane * kXS + q]) = pack_bf16(f[q], f[q + 1]);
-      ss[warp][lane] = smax;
-      if (MODE == 0 && A.Xs && p < A.nB) {
-        uint4* dst = reinterpret_cast<uint4*>(A.Xs + p * 32);
-        const uint4* src = reinterpret_cast<const uint4*>(&xw[lane * kXS]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) dst[q] = src[q];
+      for (int q = 0; q < 32; q += 8) {
+        uint4 v;
+        v.x = pack_bf16(f[q], f[q + 1]);
+        v.y = pack_bf16(f[q + 2], f[q + 3]);
+        v.z = pack_bf16(f[q + 4], f[q + 5]);
+        v.w = pack_bf16(f[q + 6], f[q + 7]);
+        *reinterpret_cast<uint4*>(&xw[lane * kXS + q]) = v;
+        if (MODE == 2 && A.Xs && p < A.nB) reinterpret_cast<uint4*>(A.Xs + p * 32)[q / 8] = v;
       }
+      ss[warp][lane] = smax;
     }
     __syncwarp();
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+    const int64_t p0 = step * 32 + 16 * half;
+    const __nv_bfloat16* xw = xs[warp] + 16 * half * kXS;
+    const float* sw = ss[warp] + 16 * half;
     // layer 1: [16 x 32] x [32 x 64]
     uint32_t a[2][4];
 #pragma unroll
@@ -181,7 +191,7 @@ __global__ void __launch_bounds__(kFwdWarps * 32) k_mlp_forward(MlpFwdArgs A) {
       a2[kc][2] = pack_bf16(h[2 * kc + 1][0], h[2 * kc + 1][1]);
       a2[kc][3] = pack_bf16(h[2 * kc + 1][2], h[2 * kc + 1][3]);
     }
-    if (MODE == 0 && A.H1) {
+    if (MODE == 2 && A.H1) {
 #pragma unroll
       for (int kc = 0; kc < 4; ++kc) {
         const int64_t r0 = p0 + g, r1 = p0 + g + 8;
@@ -210,7 +220,7 @@ __global__ void __launch_bounds__(kFwdWarps * 32) k_mlp_forward(MlpFwdArgs A) {
       }
 #pragma unroll
       for (int e = 0; e < 4; ++e) c[e] = fmaxf(c[e], 0.f);
-      if (MODE == 0 && A.H2) {
+      if (MODE == 2 && A.H2) {
         const int64_t r0 = p0 + g, r1 = p0 + g + 8;
         if (r0 < A.nB) *reinterpret_cast<uint32_t*>(A.H2 + r0 * 64 + n) = pack_bf16(c[0], c[1]);
         if (r1 < A.nB) *reinterpret_cast<uint32_t*>(A.H2 + r1 * 64 + n) = pack_bf16(c[2], c[3]);
@@ -225,15 +235,16 @@ __global__ void __launch_bounds__(kFwdWarps * 32) k_mlp_forward(MlpFwdArgs A) {
     if (t == 0) {
       const int64_t r0 = p0 + g, r1 = p0 + g + 8;
       if (r0 < A.nB) {
-        const float d = ss[warp][g] * A.dx2 * (y0 + b3);
+        const float d = sw[g] * A.dx2 * (y0 + b3);
         if (MODE == 1) A.u[r0] += d; else A.du[r0] = d;
-        if (MODE == 0 && A.S) A.S[r0] = ss[warp][g];
+        if (MODE == 2 && A.S) A.S[r0] = sw[g];
       }
       if (r1 < A.nB) {
-        const float d = ss[warp][g + 8] * A.dx2 * (y1 + b3);
+        const float d = sw[g + 8] * A.dx2 * (y1 + b3);
         if (MODE == 1) A.u[r1] += d; else A.du[r1] = d;
-        if (MODE == 0 && A.S) A.S[r1] = ss[warp][g + 8];
+        if (MODE == 2 && A.S) A.S[r1] = sw[g + 8];
       }
+    }
     }
     __syncwarp();
   }
@@ -244,182 +255,235 @@ __global__ void __launch_bounds__(kFwdWarps * 32) k_mlp_forward(MlpFwdArgs A) {
 // partial gradient (kBwdCtas x 25 KB whatever the band size).
 constexpr int kBwdCtas = 2 * 152;
 
-// Tensor-core backward.  A CTA of 4 warps loops over groups of 16 points;
-// per group the three contractions run as BF16 mma.sync.m16n8k16 with FP32
-// accumulation:
-//   dz1 = (dz2 W2^T) [h1 > 0]    M = 16 points, N = 64, K = 64  (warp w: dz1 columns 16w..16w+15)
-//   dW2 += H1^T dz2              M = 64, N = 64, K = 16 points (warp w: rows 16w..16w+15)
-//   dW1 += X^T dz1               M = 32, N = 64, K = 16 points (warp w: columns 16w..16w+15)
-// with dz2 = dy w3 [h2 > 0].  The operands sit in shared memory transposed so
-// that the K index (the points) is contiguous; the dW accumulators stay in
-// registers across all the CTA's groups; bias gradients are FP32 sums by 65
-// threads.  Each CTA writes one partial gradient, summed by k_grad_reduce.
-constexpr int kTcWarps = 4;
-constexpr int kTcS = 24;   // row stride (bf16) of the transposed 16-point tiles
-constexpr int kTcW2 = 72;  // row stride (bf16) of W2 in shared memory
+// Tensor-core backward.  A CTA of 8 warps loops over groups of kBwdPts points,
+// copied to shared memory (two CTAs on an SM: one waits for its copies while the
+// other contracts); BF16 mma.sync.m16n8k16, FP32 accumulation:
+//   dz1 = (dz2 W2^T) [h1 > 0]    M = points, N = 64, K = 64       (warp w: points 16 w .. 16 w + 15)
+//   dW2 += H1^T dz2              M = 64, N = 64, K = points       (warp w: rows 16 (w / 2), columns 32 (w % 2))
+//   dW1 += X^T dz1               M = 32, N = 64, K = points       (warp w: rows 16 (w / 4), columns 16 (w % 4))
+// with dz2 = dy w3 [h2 > 0].  All operands lie in shared memory point by point;
+// the contractions over points read them with transposing matrix loads.  The
+// dW accumulators and the FP32 bias sums stay in registers over all the CTA's
+// groups; each CTA writes one partial gradient, summed by k_grad_reduce.
+// Bound by the reads of the stored activations (324 bytes per point) and three
+// barriers per group: 342 thousand points 56 us, against 528 us with 16 points
+// per step copied value by value.
+constexpr int kBwdWarps = 8;
+constexpr int kBwdPts = 16 * kBwdWarps;
+constexpr int kRowX = 40;  // row strides (bf16) in shared memory
+constexpr int kRowH = 72;
 
-__global__ void __launch_bounds__(kTcWarps * 32) k_mlp_backward_tc(const float* params, const float* dy,
-                                                                   const __nv_bfloat16* Xs,
-                                                                   const __nv_bfloat16* H1,
-                                                                   const __nv_bfloat16* H2, int32_t nB,
-                                                                   float* part) {
-  __shared__ __align__(16) __nv_bfloat16 w2s[64 * kTcW2];   // w2s[k][j] = W2[k][j]
-  __shared__ __align__(16) __nv_bfloat16 xT[32 * kTcS];     // xT[f][p]
-  __shared__ __align__(16) __nv_bfloat16 h1T[64 * kTcS];    // h1T[k][p]
-  __shared__ __align__(16) __nv_bfloat16 dz2T[64 * kTcS];   // dz2T[j][p]
-  __shared__ __align__(16) __nv_bfloat16 dz1T[64 * kTcS];   // dz1T[k][p]
-  __shared__ __align__(16) __nv_bfloat16 dz2r[16 * kTcW2];  // dz2r[p][j] (A operand of dz1)
-  __shared__ float h1f[16][65], h2f[16][65], dz1f[16][65], w3s[64], dys[16];
+struct BwdStage {
+  __nv_bfloat16 x[kBwdPts * kRowX];
+  __nv_bfloat16 h1[kBwdPts * kRowH];
+  __nv_bfloat16 h2[kBwdPts * kRowH];
+  float dy[kBwdPts];
+};
+struct BwdShared {
+  BwdStage st;
+  __nv_bfloat16 dz1[kBwdPts * kRowH];
+  __nv_bfloat16 w2[64 * kRowH];  // w2[k][j] = W2[k][j]
+  float w3[64];
+  float red[3][kBwdWarps][64];
+};
+
+__device__ __forceinline__ void copy16_or_zero(void* smem, const void* gmem, bool ok) {
+  const uint32_t n = ok ? 16 : 0;  // bytes read; the rest is zero-filled
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
+               "l"(gmem), "r"(n)
+               : "memory");
+}
+template <bool TRANS>
+__device__ __forceinline__ void ldmatrix4(uint32_t (&d)[4], const __nv_bfloat16* p) {
+  if (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+
+// Copies of one group (zero rows past the last point).
+__device__ __forceinline__ void bwd_fetch(BwdStage& s, const float* dy, const __nv_bfloat16* Xs,
+                                          const __nv_bfloat16* H1, const __nv_bfloat16* H2, int64_t p0,
+                                          int32_t nB) {
+  for (int q = threadIdx.x; q < kBwdPts * 20; q += blockDim.x) {  // 16-byte words: 4 of x, 8 of h1, 8 of h2
+    const int p = q / 20, c = q - 20 * p;
+    const bool ok = p0 + p < nB;
+    const int64_t gp = ok ? p0 + p : 0;
+    if (c < 4) copy16_or_zero(s.x + p * kRowX + 8 * c, Xs + gp * 32 + 8 * c, ok);
+    else if (c < 12) copy16_or_zero(s.h1 + p * kRowH + 8 * (c - 4), H1 + gp * 64 + 8 * (c - 4), ok);
+    else copy16_or_zero(s.h2 + p * kRowH + 8 * (c - 12), H2 + gp * 64 + 8 * (c - 12), ok);
+  }
+  for (int p = threadIdx.x; p < kBwdPts; p += blockDim.x) s.dy[p] = p0 + p < nB ? __ldg(dy + p0 + p) : 0.f;
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kBwdWarps * 32, 2) k_mlp_backward_tc(const float* params, const float* dy,
+                                                                    const __nv_bfloat16* Xs,
+                                                                    const __nv_bfloat16* H1,
+                                                                    const __nv_bfloat16* H2, int32_t nB,
+                                                                    float* part) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  BwdShared& S = *reinterpret_cast<BwdShared*>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, t = lane & 3;
+  const int64_t ngroups = ((int64_t)nB + kBwdPts - 1) / kBwdPts;
+  if (blockIdx.x < ngroups) bwd_fetch(S.st, dy, Xs, H1, H2, (int64_t)blockIdx.x * kBwdPts, nB);
   for (int q = tid; q < 64 * 64; q += blockDim.x)
-    w2s[(q >> 6) * kTcW2 + (q & 63)] = __float2bfloat16_rn(params[kOffW2 + q]);
-  for (int q = tid; q < 64; q += blockDim.x) w3s[q] = params[kOffW3 + q];
-  float acc2[8][4], acc1[2][2][4];  // dW2 rows 16w.., dW1 (m-tile, n-tile of the warp)
-#pragma unroll
-  for (int a = 0; a < 8; ++a)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc2[a][e] = 0.f;
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc1[a][b][e] = 0.f;
-  float sb1 = 0.f, sb2 = 0.f, sw3 = 0.f, sb3 = 0.f;  // bias sums of threads 0..64
-  const int64_t ngroups = ((int64_t)nB + 15) / 16;
+    S.w2[(q >> 6) * kRowH + (q & 63)] = __float2bfloat16_rn(params[kOffW2 + q]);
+  if (tid < 64) S.w3[tid] = params[kOffW3 + tid];
   __syncthreads();
+  const int j2 = 2 * lane;  // column pair of the elementwise step
+  const float w3a = S.w3[j2], w3b = S.w3[j2 + 1];
+  float acc2[4][4], acc1[2][4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a) acc2[a][e] = 0.f;
+#pragma unroll
+    for (int a = 0; a < 2; ++a) acc1[a][e] = 0.f;
+  }
+  float sb2[2] = {0.f, 0.f}, sw3[2] = {0.f, 0.f}, sb3 = 0.f, sb1[8][2];
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt) sb1[nt][0] = sb1[nt][1] = 0.f;
+  BwdStage& s = S.st;
   for (int64_t grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
-    const int64_t p0 = grp * 16;
-    // operands of this group
-    for (int q = tid; q < 16 * 64; q += blockDim.x) {
-      const int p = q >> 6, j = q & 63;
-      const int64_t gp = p0 + p;
-      const bool ok = gp < nB;
-      const float h1v = ok ? __bfloat162float(H1[gp * 64 + j]) : 0.f;
-      const float h2v = ok ? __bfloat162float(H2[gp * 64 + j]) : 0.f;
-      const float dyv = ok ? dy[gp] : 0.f;
-      const float d2 = h2v > 0.f ? dyv * w3s[j] : 0.f;
-      h1f[p][j] = h1v;
-      h2f[p][j] = h2v;
-      h1T[j * kTcS + p] = __float2bfloat16_rn(h1v);
-      dz2T[j * kTcS + p] = __float2bfloat16_rn(d2);
-      dz2r[p * kTcW2 + j] = __float2bfloat16_rn(d2);
-      if (j < 32) xT[j * kTcS + p] = ok ? Xs[gp * 32 + j] : __float2bfloat16_rn(0.f);
-      if (j == 0) dys[p] = dyv;
+    __nv_bfloat16* dz2 = s.h2;  // takes h2's place, element by element
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // this group has arrived
+    // dz2 and the column sums: warp w the points 16 w .. 16 w + 15, a column pair per lane
+#pragma unroll 4
+    for (int i = 0; i < 16; ++i) {
+      const int p = 16 * warp + i;
+      const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(s.h2 + p * kRowH + j2);
+      const float ha = __low2float(h), hb = __high2float(h), d = s.dy[p];
+      const float da = ha > 0.f ? d * w3a : 0.f, db = hb > 0.f ? d * w3b : 0.f;
+      sb2[0] += da;
+      sb2[1] += db;
+      sw3[0] += d * ha;
+      sw3[1] += d * hb;
+      sb3 += d;
+      *reinterpret_cast<uint32_t*>(dz2 + p * kRowH + j2) = pack_bf16(da, db);
     }
-    __syncthreads();
-    // dz1 columns 16 warp .. 16 warp + 15: A = dz2 (points x j), B[j][k] = W2[k][j]
+    __syncwarp();
+    // dz1 of the warp's 16 points
     {
-      float c[2][4];
+      uint32_t a[4][4];
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) c[nt][e] = 0.f;
-#pragma unroll
-      for (int kc = 0; kc < 4; ++kc) {
-        uint32_t a[4];
-        a[0] = *reinterpret_cast<const uint32_t*>(&dz2r[g * kTcW2 + kc * 16 + 2 * t]);
-        a[1] = *reinterpret_cast<const uint32_t*>(&dz2r[(g + 8) * kTcW2 + kc * 16 + 2 * t]);
-        a[2] = *reinterpret_cast<const uint32_t*>(&dz2r[g * kTcW2 + kc * 16 + 8 + 2 * t]);
-        a[3] = *reinterpret_cast<const uint32_t*>(&dz2r[(g + 8) * kTcW2 + kc * 16 + 8 + 2 * t]);
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          const int n = 16 * warp + 8 * nt + g;
-          const __nv_bfloat16* wb = &w2s[n * kTcW2 + kc * 16 + 2 * t];
-          mma_bf16(c[nt], a, *reinterpret_cast<const uint32_t*>(wb),
-                   *reinterpret_cast<const uint32_t*>(wb + 8));
-        }
-      }
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const int k0 = 16 * warp + 8 * nt + 2 * t;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int p = g + (e >> 1) * 8, k = k0 + (e & 1);
-          const float v = h1f[p][k] > 0.f ? c[nt][e] : 0.f;
-          dz1f[p][k] = v;
-          dz1T[k * kTcS + p] = __float2bfloat16_rn(v);
-        }
-      }
-    }
-    __syncthreads();
-    // dW2 rows 16 warp ..: A[k][p] = h1T, B[p][j] = dz2T (as [j][p])
-    {
-      uint32_t a[4];
-      const int m0 = 16 * warp;
-      a[0] = *reinterpret_cast<const uint32_t*>(&h1T[(m0 + g) * kTcS + 2 * t]);
-      a[1] = *reinterpret_cast<const uint32_t*>(&h1T[(m0 + g + 8) * kTcS + 2 * t]);
-      a[2] = *reinterpret_cast<const uint32_t*>(&h1T[(m0 + g) * kTcS + 8 + 2 * t]);
-      a[3] = *reinterpret_cast<const uint32_t*>(&h1T[(m0 + g + 8) * kTcS + 8 + 2 * t]);
+      for (int kc = 0; kc < 4; ++kc)
+        ldmatrix4<false>(a[kc], dz2 + (16 * warp + (lane & 15)) * kRowH + 16 * kc + 8 * (lane >> 4));
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt) {
-        const __nv_bfloat16* bb = &dz2T[(nt * 8 + g) * kTcS + 2 * t];
-        mma_bf16(acc2[nt], a, *reinterpret_cast<const uint32_t*>(bb),
-                 *reinterpret_cast<const uint32_t*>(bb + 8));
-      }
-    }
-    // dW1 columns 16 warp ..: A[f][p] = xT, B[p][k] = dz1T (as [k][p])
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      uint32_t a[4];
-      a[0] = *reinterpret_cast<const uint32_t*>(&xT[(16 * mt + g) * kTcS + 2 * t]);
-      a[1] = *reinterpret_cast<const uint32_t*>(&xT[(16 * mt + g + 8) * kTcS + 2 * t]);
-      a[2] = *reinterpret_cast<const uint32_t*>(&xT[(16 * mt + g) * kTcS + 8 + 2 * t]);
-      a[3] = *reinterpret_cast<const uint32_t*>(&xT[(16 * mt + g + 8) * kTcS + 8 + 2 * t]);
+        for (int k2 = 0; k2 < 2; ++k2) {
+          uint32_t b[4];
+          ldmatrix4<false>(b, S.w2 + (8 * nt + (lane & 7)) * kRowH + 32 * k2 + 8 * (lane >> 3));
+          mma_bf16(c, a[2 * k2], b[0], b[1]);
+          mma_bf16(c, a[2 * k2 + 1], b[2], b[3]);
+        }
+        const int k0 = 8 * nt + 2 * t;
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const __nv_bfloat16* bb = &dz1T[(16 * warp + 8 * nt + g) * kTcS + 2 * t];
-        mma_bf16(acc1[mt][nt], a, *reinterpret_cast<const uint32_t*>(bb),
-                 *reinterpret_cast<const uint32_t*>(bb + 8));
+        for (int r = 0; r < 2; ++r) {
+          const int p = 16 * warp + g + 8 * r;
+          const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(s.h1 + p * kRowH + k0);
+          const float va = __low2float(h) > 0.f ? c[2 * r] : 0.f, vb = __high2float(h) > 0.f ? c[2 * r + 1] : 0.f;
+          sb1[nt][0] += va;
+          sb1[nt][1] += vb;
+          *reinterpret_cast<uint32_t*>(S.dz1 + p * kRowH + k0) = pack_bf16(va, vb);
+        }
       }
-    }
-    // bias gradients (FP32)
-    if (tid < 64) {
-      for (int p = 0; p < 16; ++p) {
-        sb1 += dz1f[p][tid];
-        const float d2 = h2f[p][tid] > 0.f ? dys[p] * w3s[tid] : 0.f;
-        sb2 += d2;
-        sw3 += dys[p] * h2f[p][tid];
-      }
-    } else if (tid == 64) {
-      for (int p = 0; p < 16; ++p) sb3 += dys[p];
     }
     __syncthreads();
+    // dW2 and dW1 over the group's points
+    const int m2 = 16 * (warp >> 1), n2 = 32 * (warp & 1), m1 = 16 * (warp >> 2), n1 = 16 * (warp & 3);
+#pragma unroll 2
+    for (int kc = 0; kc < kBwdPts / 16; ++kc) {
+      // transposed 8 x 8 blocks: rows are points, so a lane's address is a point's row
+      const int ra = 16 * kc + (lane & 7) + 8 * (lane >> 4), ca = 8 * ((lane >> 3) & 1);
+      const int rb = 16 * kc + (lane & 15), cb = 8 * (lane >> 4);
+      uint32_t a[4], b[4];
+      ldmatrix4<true>(a, s.h1 + ra * kRowH + m2 + ca);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        ldmatrix4<true>(b, dz2 + rb * kRowH + n2 + 16 * h + cb);
+        mma_bf16(acc2[2 * h], a, b[0], b[1]);
+        mma_bf16(acc2[2 * h + 1], a, b[2], b[3]);
+      }
+      ldmatrix4<true>(a, s.x + ra * kRowX + m1 + ca);
+      ldmatrix4<true>(b, S.dz1 + rb * kRowH + n1 + cb);
+      mma_bf16(acc1[0], a, b[0], b[1]);
+      mma_bf16(acc1[1], a, b[2], b[3]);
+    }
+    __syncthreads();  // every warp has left the group
+    if (grp + gridDim.x < ngroups) bwd_fetch(s, dy, Xs, H1, H2, (grp + gridDim.x) * kBwdPts, nB);
   }
   float* out = part + (int64_t)blockIdx.x * kNParams;
 #pragma unroll
-  for (int nt = 0; nt < 8; ++nt)
+  for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int k = 16 * warp + g + (e >> 1) * 8, j = nt * 8 + 2 * t + (e & 1);
+      const int k = 16 * (warp >> 1) + g + (e >> 1) * 8, j = 32 * (warp & 1) + 8 * nt + 2 * t + (e & 1);
       out[kOffW2 + k * 64 + j] = acc2[nt][e];
     }
 #pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
+  for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
+    for (int e = 0; e < 4; ++e) {
+      const int f = 16 * (warp >> 2) + g + (e >> 1) * 8, k = 16 * (warp & 3) + 8 * nt + 2 * t + (e & 1);
+      out[kOffW1 + f * 64 + k] = acc1[nt][e];
+    }
+  // bias sums: over the lanes of a column, then over the warps in order
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int f = 16 * mt + g + (e >> 1) * 8, k = 16 * warp + 8 * nt + 2 * t + (e & 1);
-        out[kOffW1 + f * 64 + k] = acc1[mt][nt][e];
-      }
-  if (tid < 64) {
-    out[kOffB1 + tid] = sb1;
-    out[kOffB2 + tid] = sb2;
-    out[kOffW3 + tid] = sw3;
-  } else if (tid == 64) {
-    out[kOffB3] = sb3;
+  for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      float v = sb1[nt][e];
+      v += __shfl_xor_sync(0xffffffffu, v, 4);
+      v += __shfl_xor_sync(0xffffffffu, v, 8);
+      v += __shfl_xor_sync(0xffffffffu, v, 16);
+      if (g == 0) S.red[0][warp][8 * nt + 2 * t + e] = v;
+    }
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    S.red[1][warp][j2 + e] = sb2[e];
+    S.red[2][warp][j2 + e] = sw3[e];
+  }
+  __syncthreads();
+  if (tid < 192) {
+    const int which = tid >> 6, q = tid & 63;
+    float v = 0.f;
+    for (int w = 0; w < kBwdWarps; ++w) v += S.red[which][w][q];
+    out[(which == 0 ? kOffB1 : which == 1 ? kOffB2 : kOffW3) + q] = v;
+  }
+  __syncthreads();
+  if (lane == 0) S.red[0][warp][0] = sb3;
+  __syncthreads();
+  if (tid == 0) {
+    float v = 0.f;
+    for (int w = 0; w < kBwdWarps; ++w) v += S.red[0][w][0];
+    out[kOffB3] = v;
   }
 }
 
 // grad[q] = sum over CTAs of part[c][q] (fixed order).
-__global__ void k_grad_reduce(const float* part, int nparts, float* grad) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= kNParams) return;
+// A block takes 32 parameters, its 8 warps every eighth partial.
+__global__ void __launch_bounds__(256) k_grad_reduce(const float* part, int nparts, float* grad) {
+  __shared__ float red[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int q = blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int c = 0; c < nparts; ++c) s += part[(int64_t)c * kNParams + q];
-  grad[q] = s;
+  if (q < kNParams)
+    for (int c = warp; c < nparts; c += 8) s += part[(int64_t)c * kNParams + q];
+  red[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && q < kNParams) {
+    for (int w = 1; w < 8; ++w) s += red[w][lane];
+    grad[q] = s;
+  }
 }
 
 // Adam (Kingma & Ba) on the FP32 master parameters.
@@ -453,51 +517,86 @@ __global__ void k_nbr_transpose(BrickView v, const uint64_t* key, int64_t nplus,
   t[k] = s;
 }
 
-// out[j] += sum_k E_{kj} t[k]: each extension tile scatters its points'
-// weighted values into its shared-memory box, then adds the box to out.
-__global__ void __launch_bounds__(64) k_extend_transpose(LevelView<float> L, const float* t,
-                                                         float* out) {
-  __shared__ float box[7 * 7 * 7];
-  __shared__ uint64_t sm_mask[8];
-  __shared__ int32_t sm_start[8];
-  const int32_t tile = blockIdx.x;
-  for (int q = threadIdx.x; q < 343; q += blockDim.x) box[q] = 0.f;
-  if (threadIdx.x < 8) {
-    sm_mask[threadIdx.x] = L.tile_mask[8 * (int64_t)tile + threadIdx.x];
-    sm_start[threadIdx.x] = L.tile_bstart[8 * (int64_t)tile + threadIdx.x];
+// out[j] += sum_k E_{kj} t[k], one warp per extension tile.  Each lane takes a
+// base and sums its points' 4^3 weighted values in registers (6.6 points share
+// a base on a smooth surface), then adds them to the tile's box in shared
+// memory; the box is added to out.  342 thousand points: 36 us, against 148 us
+// with one shared-memory addition per point and node.
+constexpr int kExtTWarps = 2;
+__global__ void __launch_bounds__(32 * kExtTWarps) k_extend_transpose(LevelView<float> L, const float* t,
+                                                                      float* out) {
+  __shared__ float boxes[kExtTWarps][344];
+  __shared__ int32_t runs[kExtTWarps][64][4];  // per base: its points of B and of G, begin and end
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int32_t tile = blockIdx.x * kExtTWarps + warp;
+  if (tile >= L.ntiles) return;
+  float* box = boxes[warp];
+  for (int q = lane; q < 343; q += 32) box[q] = 0.f;
+  for (int q = lane; q < 256; q += 32) runs[warp][q >> 2][q & 3] = 0;
+  __syncwarp();
+  const int32_t beg = L.tile_start[tile], mid = L.tile_mid[tile], end = L.tile_start[tile + 1];
+  for (int32_t k = beg + lane; k < end; k += 32) {
+    const uint32_t pos = L.erec[k] & 63u;
+    const int part = k < mid ? 0 : 2;
+    if (k == beg || k == mid || (L.erec[k - 1] & 63u) != pos) runs[warp][pos][part] = k;
+    if (k + 1 == end || k + 1 == mid || (L.erec[k + 1] & 63u) != pos) runs[warp][pos][part + 1] = k + 1;
   }
-  __syncthreads();
-  const int32_t beg = L.tile_start[tile], end = L.tile_start[tile + 1];
+  __syncwarp();
   const int64_t np = L.nplus;
-  for (int32_t k = beg + threadIdx.x; k < end; k += blockDim.x) {
-    const uint32_t rec = L.erec[k];
-    const int lx = rec & 3, ly = (rec >> 2) & 3, lz = (rec >> 4) & 3;
-    float wx[4], wy[4], wz[4];
-    const float s3[3] = {L.efr[k], L.efr[np + k], L.efr[2 * np + k]};
-    float* ws[3] = {wx, wy, wz};
-    for (int a = 0; a < 3; ++a) {
-      const float s = s3[a], sm1 = s - 1.f, sm2 = s - 2.f, sp1 = s + 1.f;
-      const float p = s * sm1, q = sp1 * sm2;
-      ws[a][0] = (p * sm2) * (-1.f / 6.f);
-      ws[a][1] = (q * sm1) * 0.5f;
-      ws[a][2] = (q * s) * -0.5f;
-      ws[a][3] = (p * sp1) * (1.f / 6.f);
+  // the bases that have points, dealt to the lanes in turn
+  uint32_t has0 = __ballot_sync(0xffffffffu, runs[warp][lane][1] + runs[warp][lane][3] > 0);
+  uint32_t has1 = __ballot_sync(0xffffffffu, runs[warp][lane + 32][1] + runs[warp][lane + 32][3] > 0);
+  const int n0 = __popc(has0), nbase = n0 + __popc(has1);
+  for (int q = lane; q < nbase; q += 32) {
+    const int pos = q < n0 ? (int)__fns(has0, 0, q + 1) : 32 + (int)__fns(has1, 0, q - n0 + 1);
+    float acc[64];
+#pragma unroll
+    for (int e = 0; e < 64; ++e) acc[e] = 0.f;
+#pragma unroll 1
+    for (int part = 0; part < 4; part += 2) {
+      const int32_t k1 = runs[warp][pos][part + 1];
+#pragma unroll 1
+      for (int32_t k = runs[warp][pos][part]; k < k1; ++k) {
+        const float tv = t[L.erec[k] >> 6];
+        const float s3[3] = {L.efr[k], L.efr[np + k], L.efr[2 * np + k]};
+        float w[3][4];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const float s = s3[a], sm1 = s - 1.f, sm2 = s - 2.f, sp1 = s + 1.f;
+          const float p = s * sm1, qq = sp1 * sm2;
+          w[a][0] = (p * sm2) * (-1.f / 6.f);
+          w[a][1] = (qq * sm1) * 0.5f;
+          w[a][2] = (qq * s) * -0.5f;
+          w[a][3] = (p * sp1) * (1.f / 6.f);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const float v = w[2][c] * w[1][b] * tv;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) acc[(c * 4 + b) * 4 + a] += w[0][a] * v;
+          }
+      }
     }
-    const float tv = t[rec >> 6];
+    const int lx = pos & 3, ly = (pos >> 2) & 3, lz = pos >> 4;
+#pragma unroll
     for (int c = 0; c < 4; ++c)
+#pragma unroll
       for (int b = 0; b < 4; ++b)
+#pragma unroll
         for (int a = 0; a < 4; ++a)
-          atomicAdd(&box[((lz + c) * 7 + ly + b) * 7 + lx + a], wx[a] * wy[b] * wz[c] * tv);
+          atomicAdd(&box[((lz + c) * 7 + ly + b) * 7 + lx + a], acc[(c * 4 + b) * 4 + a]);
   }
-  __syncthreads();
-  for (int q = threadIdx.x; q < 343; q += blockDim.x) {
+  __syncwarp();
+  for (int q = lane; q < 343; q += 32) {
     const float val = box[q];
     if (val == 0.f) continue;
     const int x = q % 7, y = (q / 7) % 7, z = q / 49;
     const int j = (x >> 2) | ((y >> 2) << 1) | ((z >> 2) << 2);
     const uint64_t bit = 1ull << ((x & 3) | ((y & 3) << 2) | ((z & 3) << 4));
-    const uint64_t m = sm_mask[j];
-    if (m & bit) atomicAdd(out + sm_start[j] + __popcll(m & (bit - 1)), val);
+    const uint64_t m = __ldg(L.tile_mask + 8 * (int64_t)tile + j);
+    if (m & bit) atomicAdd(out + __ldg(L.tile_bstart + 8 * (int64_t)tile + j) + __popcll(m & (bit - 1)), val);
   }
 }
 
@@ -539,12 +638,33 @@ __global__ void k_mlp_resid(const float* r, const float* du, const float* Mdu, c
   }
 }
 
-__global__ void k_mlp_loss_final(const double* part, int nblocks, double* out) {
-  if (threadIdx.x != 0) return;
-  double a = 0, b = 0;
-  for (int q = 0; q < nblocks; ++q) { a += part[2 * q]; b += part[2 * q + 1]; }
-  out[0] = a;  // ||z||^2
-  out[1] = b;  // ||r||^2
+// out[0] = ||z||^2, out[1] = ||r||^2 (fixed order).
+__global__ void __launch_bounds__(1024) k_mlp_loss_final(const double* part, int nblocks, double* out) {
+  double a = 0.0, b = 0.0;
+  for (int q = threadIdx.x; q < nblocks; q += blockDim.x) {
+    a += part[2 * q];
+    b += part[2 * q + 1];
+  }
+  __shared__ double sa[32], sb[32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sa[threadIdx.x >> 5] = a;
+    sb[threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    a = b = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      a += sa[w];
+      b += sb[w];
+    }
+    out[0] = a;
+    out[1] = b;
+  }
 }
 
 // ----------------------------------------------------------------- host side
@@ -574,10 +694,12 @@ void mlp_forward(const float* params, const MlpLevelData& D, const float* r, flo
     a.H2 = tb->H2.get();
     a.S = tb->S.get();
   }
-  const int64_t groups = ((int64_t)D.nB + 15) / 16;
-  const unsigned grid = (unsigned)std::min<int64_t>((groups + kFwdWarps - 1) / kFwdWarps, 152 * 8);
+  const int64_t steps = ((int64_t)D.nB + 31) / 32;
+  const unsigned grid = (unsigned)std::min<int64_t>((steps + kFwdWarps - 1) / kFwdWarps, 152 * 6);
   if (u_add)
     k_mlp_forward<1><<<grid, kFwdWarps * 32, 0, st>>>(a);
+  else if (tb)
+    k_mlp_forward<2><<<grid, kFwdWarps * 32, 0, st>>>(a);
   else
     k_mlp_forward<0><<<grid, kFwdWarps * 32, 0, st>>>(a);
   count_launch();
@@ -613,6 +735,9 @@ void mlp_loss_grad(const float* params, const MlpLevelData& D, const LevelView<f
                    cudaStream_t st) {
   const int32_t nB = L.nB;
   const float dx2 = 1.f / L.inv_h2;
+  // (per call: the attribute belongs to the device that is current)
+  CPM_CUDA_TRY(cudaFuncSetAttribute(k_mlp_backward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)sizeof(BwdShared)));
   tb.ensure(nB, L.nplus, ((int64_t)DL.nbricks + 1) << (2 * DL.dim));
   mlp_forward(params, D, r, dx2, tb.du.get(), nullptr, &tb, st);
   // M du (extension over B+ then the stencil)
@@ -622,17 +747,17 @@ void mlp_loss_grad(const float* params, const MlpLevelData& D, const LevelView<f
   const int nb256 = (int)((nB + 255) / 256);
   k_mlp_resid<<<nb256, 256, 0, st>>>(r, tb.du.get(), tb.Mdu.get(), cvec, cval, nB, tb.z.get(),
                                       tb.lpart.get());
-  k_mlp_loss_final<<<1, 32, 0, st>>>(tb.lpart.get(), nb256, tb.loss.get());
+  k_mlp_loss_final<<<1, 1024, 0, st>>>(tb.lpart.get(), nb256, tb.loss.get());
   // A^T z = (c + gamma) z - E^T (N^T z) / dx^2
   k_nbr_transpose<<<nblk(L.nplus, 256), 256, 0, st>>>(L.bv, L.key, L.nplus, L.dim, tb.z.get(),
                                                        tb.t.get());
   CPM_CUDA_TRY(cudaMemsetAsync(tb.et.get(), 0, sizeof(float) * nB, st));
-  k_extend_transpose<<<L.ntiles, 64, 0, st>>>(L, tb.t.get(), tb.et.get());
+  k_extend_transpose<<<nblk(L.ntiles, kExtTWarps), 32 * kExtTWarps, 0, st>>>(L, tb.t.get(), tb.et.get());
   k_mlp_dy<<<nb256, 256, 0, st>>>(tb.z.get(), tb.et.get(), cvec, cval, L.gamma, L.inv_h2, tb.S.get(),
                                    dx2, tb.loss.get() + 1, nB, tb.dy.get());
-  k_mlp_backward_tc<<<tb.nparts, kTcWarps * 32, 0, st>>>(params, tb.dy.get(), tb.Xs.get(), tb.H1.get(),
+  k_mlp_backward_tc<<<tb.nparts, kBwdWarps * 32, sizeof(BwdShared), st>>>(params, tb.dy.get(), tb.Xs.get(), tb.H1.get(),
                                                          tb.H2.get(), nB, tb.part.get());
-  k_grad_reduce<<<nblk(kNParams, 256), 256, 0, st>>>(tb.part.get(), tb.nparts, tb.grad.get());
+  k_grad_reduce<<<nblk(kNParams, 32), 256, 0, st>>>(tb.part.get(), tb.nparts, tb.grad.get());
   count_launch(9);
   CPM_CUDA_TRY(cudaGetLastError());
 }
