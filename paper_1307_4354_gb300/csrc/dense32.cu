@@ -195,6 +195,17 @@ void build_dense32(const Level& L, Dense32& D, cudaStream_t st) {
   build_units(L, D, nullptr, D.all, st);
 }
 
+UnitsView units_view(const ExtUnits& U) {
+  UnitsView v;
+  v.tiles = U.tiles.get();
+  v.ntiles = U.ntiles;
+  for (int h = 0; h < 2; ++h) {
+    v.pts[h] = U.pts[h].get();
+    v.cidx[h] = U.cidx[h].get();
+  }
+  return v;
+}
+
 DenseView dense_view(const Level& L, const Dense32& D) {
   DenseView v;
   v.bmask = L.bmask.get();
@@ -208,12 +219,7 @@ DenseView dense_view(const Level& L, const Dense32& D) {
   v.dim = L.dim;
   v.inv_h2 = (float)(1.0 / (L.dx * L.dx));
   v.gamma = (float)(2.0 * L.dim / (L.dx * L.dx));
-  v.tiles = D.all.tiles.get();
-  for (int h = 0; h < 2; ++h) {
-    v.pts[h] = D.all.pts[h].get();
-    v.cidx[h] = D.all.cidx[h].get();
-  }
-  v.ntiles = D.all.ntiles;
+  v.all = units_view(D.all);
   v.variant = L.ext_variant;
   v.dA = D.dA.get();
   v.c = D.c.get();
@@ -267,22 +273,22 @@ __device__ __forceinline__ float4 load_row_ordered(const DenseView& L, const flo
 // loads again but leave 13 warps on an SM: 111 us.
 template <int DIM, bool CIN, bool COUT, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, kExtThreadsSM / (32 * WARPS))
-    k_extend_units(DenseView L, const float* __restrict__ u, float* __restrict__ w, int32_t npts) {
+    k_extend_units(DenseView L, UnitsView S, const float* __restrict__ u, float* __restrict__ w, int32_t npts) {
   constexpr int NC = DIM == 3 ? 4 : 1, RS = kRowStride, NH = DIM == 3 ? 2 : 1;
   __shared__ __align__(16) float box[WARPS][DIM == 3 ? 7 * kPlaneStride : 8 * RS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* win = box[warp];
   const int32_t tile = blockIdx.x * WARPS + warp;
-  if (tile >= L.ntiles) return;
-  const uint32_t hdr = __ldg(L.tiles + (size_t)tile * kTileWords + min(lane, kTileWords - 1));
+  if (tile >= S.ntiles) return;
+  const uint32_t hdr = __ldg(S.tiles + (size_t)tile * kTileWords + min(lane, kTileWords - 1));
     const uint32_t tbox = __shfl_sync(0xffffffffu, hdr, kTileBox);
     const int32_t beg = (int32_t)__shfl_sync(0xffffffffu, hdr, kTileBeg);
     const int32_t end = (int32_t)__shfl_sync(0xffffffffu, hdr, kTileEnd);
     int32_t k = beg + lane;
     float4 ra, rb;
     if (k < end) {
-      ra = __ldg(L.pts[0] + k);
-      rb = __ldg(L.pts[1] + k);
+      ra = __ldg(S.pts[0] + k);
+      rb = __ldg(S.pts[1] + k);
     }
     // row r = lane + 32 h of the 2^(d-1) columns of bricks along x: column r / 4^(d-1),
     // row r mod 4^(d-1) of its bricks
@@ -373,7 +379,7 @@ __global__ void __launch_bounds__(32 * WARPS, kExtThreadsSM / (32 * WARPS))
     const float va = (wa[0].x * qa01.x + wa[2].x * qa23.x) + (wa[1].x * qa01.y + wa[3].x * qa23.y);
     const float vb = (wb[0].x * qb01.x + wb[2].x * qb23.x) + (wb[1].x * qb01.y + wb[3].x * qb23.y);
     if (COUT) {
-      const int32_t ia = (int32_t)__ldg(L.cidx[0] + k), ib = (int32_t)__ldg(L.cidx[1] + k);
+      const int32_t ia = (int32_t)__ldg(S.cidx[0] + k), ib = (int32_t)__ldg(S.cidx[1] + k);
       if (ia < npts) w[ia] = va;
       if (ib < npts) w[ib] = vb;
     } else {
@@ -381,59 +387,60 @@ __global__ void __launch_bounds__(32 * WARPS, kExtThreadsSM / (32 * WARPS))
       w[sb & kSlotMask] = vb;
     }
     if (k + 32 < end) {
-      ra = __ldg(L.pts[0] + k + 32);
-      rb = __ldg(L.pts[1] + k + 32);
+      ra = __ldg(S.pts[0] + k + 32);
+      rb = __ldg(S.pts[1] + k + 32);
     }
     }
 }
 
 // Launch shapes (variant 0, 1, 2): one, two or four tiles (warps) per CTA.
 template <int DIM, bool CIN, bool COUT>
-static void extend_units(const DenseView& L, int variant, const float* u, float* w, int32_t npts,
-                         cudaStream_t st) {
-  if (L.ntiles <= 0) return;
+static void extend_units(const DenseView& L, const UnitsView& S, int variant, const float* u, float* w,
+                         int32_t npts, cudaStream_t st) {
+  if (S.ntiles <= 0) return;
   if (variant == 2)
-    k_extend_units<DIM, CIN, COUT, 4><<<nblk(L.ntiles, 4), 128, 0, st>>>(L, u, w, npts);
+    k_extend_units<DIM, CIN, COUT, 4><<<nblk(S.ntiles, 4), 128, 0, st>>>(L, S, u, w, npts);
   else if (variant == 1)
-    k_extend_units<DIM, CIN, COUT, 2><<<nblk(L.ntiles, 2), 64, 0, st>>>(L, u, w, npts);
+    k_extend_units<DIM, CIN, COUT, 2><<<nblk(S.ntiles, 2), 64, 0, st>>>(L, S, u, w, npts);
   else
-    k_extend_units<DIM, CIN, COUT, 1><<<L.ntiles, 32, 0, st>>>(L, u, w, npts);
+    k_extend_units<DIM, CIN, COUT, 1><<<S.ntiles, 32, 0, st>>>(L, S, u, w, npts);
 }
 
-static void extend32(const DenseView& L, int variant, Vec32<const float> u, float* w, cudaStream_t st) {
+static void extend32(const DenseView& L, const UnitsView& S, int variant, Vec32<const float> u, float* w,
+                     cudaStream_t st) {
   if (L.dim == 3) {
-    if (u.dense) extend_units<3, false, false>(L, variant, u.dense, w, 0, st);
-    else extend_units<3, true, false>(L, variant, u.compact, w, 0, st);
+    if (u.dense) extend_units<3, false, false>(L, S, variant, u.dense, w, 0, st);
+    else extend_units<3, true, false>(L, S, variant, u.compact, w, 0, st);
   } else {
-    if (u.dense) extend_units<2, false, false>(L, variant, u.dense, w, 0, st);
-    else extend_units<2, true, false>(L, variant, u.compact, w, 0, st);
+    if (u.dense) extend_units<2, false, false>(L, S, variant, u.dense, w, 0, st);
+    else extend_units<2, true, false>(L, S, variant, u.compact, w, 0, st);
   }
 }
 
-void launch_extend32(const DenseView& L, Vec32<const float> u, float* w, cudaStream_t st) {
-  extend32(L, L.variant, u, w, st);
+void launch_extend32(const DenseView& L, const UnitsView& S, Vec32<const float> u, float* w, cudaStream_t st) {
+  extend32(L, S, L.variant, u, w, st);
   count_launch();
 }
 
 void launch_extend32_compact(const DenseView& L, const float* u, float* w, int32_t npts, cudaStream_t st) {
-  if (L.dim == 3) extend_units<3, true, true>(L, L.variant, u, w, npts, st);
-  else extend_units<2, true, true>(L, L.variant, u, w, npts, st);
+  if (L.dim == 3) extend_units<3, true, true>(L, L.all, L.variant, u, w, npts, st);
+  else extend_units<2, true, true>(L, L.all, L.variant, u, w, npts, st);
   count_launch();
 }
 
 int tune_extend32(const DenseView& L, const float* u, float* w, cudaStream_t st, float ms[3]) {
   int best = 0;
   for (int v = 0; v < 3; ++v) ms[v] = 0.f;
-  if (L.ntiles <= 0) return best;
+  if (L.all.ntiles <= 0) return best;
   cudaEvent_t e0, e1;
   CPM_CUDA_TRY(cudaEventCreate(&e0));
   CPM_CUDA_TRY(cudaEventCreate(&e1));
   constexpr int kReps = 3;
   const Vec32<const float> uv{u, nullptr};
   for (int v = 0; v < 3; ++v) {
-    extend32(L, v, uv, w, st);  // warm-up
+    extend32(L, L.all, v, uv, w, st);  // warm-up
     CPM_CUDA_TRY(cudaEventRecord(e0, st));
-    for (int r = 0; r < kReps; ++r) extend32(L, v, uv, w, st);
+    for (int r = 0; r < kReps; ++r) extend32(L, L.all, v, uv, w, st);
     CPM_CUDA_TRY(cudaEventRecord(e1, st));
     CPM_CUDA_TRY(cudaEventSynchronize(e1));
     CPM_CUDA_TRY(cudaEventElapsedTime(&ms[v], e0, e1));
@@ -462,12 +469,13 @@ int tune_extend32(const DenseView& L, const float* u, float* w, cudaStream_t st,
 template <int DIM, int MODE, bool CIN>
 __global__ void __launch_bounds__(256) k_lap_rows(DenseView L, const float* u, const float* __restrict__ w,
                                                   const float* __restrict__ f, float cval, Vec32<float> out,
-                                                  float* __restrict__ fd) {
+                                                  float* __restrict__ fd, RowsView rows) {
   constexpr int ROWS = DIM == 3 ? 16 : 4, SH = 2 * DIM;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= rows.n) return;
+  if (rows.list) t = __ldg(rows.list + t);
   const int32_t b = (int32_t)(t / ROWS);
   const int row = (int)(t % ROWS);
-  if (b >= L.nbricks) return;
   const int y = row & 3, z = row >> 2;
   const size_t s0 = ((size_t)b << SH) + 4 * row;
   auto load4 = [](const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); };
@@ -543,32 +551,335 @@ __global__ void __launch_bounds__(256) k_lap_rows(DenseView L, const float* u, c
 
 template <int MODE>
 static void lap32(const DenseView& L, Vec32<const float> u, const float* w, const float* f, float cval,
-                  Vec32<float> out, float* fd, cudaStream_t st) {
-  if (L.nbricks <= 0) return;
-  const unsigned g = nblk((int64_t)L.nbricks * (L.dim == 3 ? 16 : 4), 256);
+                  Vec32<float> out, float* fd, RowsView rows, cudaStream_t st) {
+  if (rows.n == 0) return;
+  const unsigned g = nblk(rows.n, 256);
   if (L.dim == 3) {
-    if (u.dense) k_lap_rows<3, MODE, false><<<g, 256, 0, st>>>(L, u.dense, w, f, cval, out, nullptr);
-    else k_lap_rows<3, MODE, true><<<g, 256, 0, st>>>(L, u.compact, w, f, cval, out, fd);
+    if (u.dense) k_lap_rows<3, MODE, false><<<g, 256, 0, st>>>(L, u.dense, w, f, cval, out, nullptr, rows);
+    else k_lap_rows<3, MODE, true><<<g, 256, 0, st>>>(L, u.compact, w, f, cval, out, fd, rows);
   } else {
-    if (u.dense) k_lap_rows<2, MODE, false><<<g, 256, 0, st>>>(L, u.dense, w, f, cval, out, nullptr);
-    else k_lap_rows<2, MODE, true><<<g, 256, 0, st>>>(L, u.compact, w, f, cval, out, fd);
+    if (u.dense) k_lap_rows<2, MODE, false><<<g, 256, 0, st>>>(L, u.dense, w, f, cval, out, nullptr, rows);
+    else k_lap_rows<2, MODE, true><<<g, 256, 0, st>>>(L, u.compact, w, f, cval, out, fd, rows);
   }
   count_launch();
 }
 
 void launch_lap32(const DenseView& L, LapMode mode, Vec32<const float> u, const float* w, const float* f,
-                  float cval, Vec32<float> out, float* fd, cudaStream_t st) {
-  if (mode == LAP_APPLY) lap32<LAP_APPLY>(L, u, w, f, cval, out, fd, st);
-  if (mode == LAP_RESID) lap32<LAP_RESID>(L, u, w, f, cval, out, fd, st);
-  if (mode == LAP_JACOBI) lap32<LAP_JACOBI>(L, u, w, f, cval, out, fd, st);
-  if (mode == LAP_JAC_RED) lap32<LAP_JAC_RED>(L, u, w, f, cval, out, fd, st);
-  if (mode == LAP_JAC_BLACK) lap32<LAP_JAC_BLACK>(L, u, w, f, cval, out, fd, st);
+                  float cval, Vec32<float> out, float* fd, const RowsView& rows, cudaStream_t st) {
+  if (mode == LAP_APPLY) lap32<LAP_APPLY>(L, u, w, f, cval, out, fd, rows, st);
+  if (mode == LAP_RESID) lap32<LAP_RESID>(L, u, w, f, cval, out, fd, rows, st);
+  if (mode == LAP_JACOBI) lap32<LAP_JACOBI>(L, u, w, f, cval, out, fd, rows, st);
+  if (mode == LAP_JAC_RED) lap32<LAP_JAC_RED>(L, u, w, f, cval, out, fd, rows, st);
+  if (mode == LAP_JAC_BLACK) lap32<LAP_JAC_BLACK>(L, u, w, f, cval, out, fd, rows, st);
 }
 
+// The first Jacobi sweep from u = 0: E u and M u vanish, u = f dA.
+__global__ void __launch_bounds__(256) k_jacobi_zero(const float* __restrict__ f, const float* __restrict__ dA,
+                                                     float* __restrict__ u, RowsView rows) {
+  uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= rows.n) return;
+  if (rows.list) t = __ldg(rows.list + t);
+  const float4 a = __ldg(reinterpret_cast<const float4*>(f) + t), d = __ldg(reinterpret_cast<const float4*>(dA) + t);
+  reinterpret_cast<float4*>(u)[t] = make_float4(a.x * d.x, a.y * d.y, a.z * d.z, a.w * d.w);
+}
+void launch_jacobi_zero32(const DenseView& L, const float* f, float* u, const RowsView& rows, cudaStream_t st) {
+  if (rows.n == 0) return;
+  k_jacobi_zero<<<nblk(rows.n, 256), 256, 0, st>>>(f, L.dA, u, rows);
+  count_launch();
+}
+
+// ----------------------------------------------------------------- transfers
+// Linear closest-point interpolation (Sec. 4.3) at a list of targets from a
+// brick-dense source: a record holds the slot of the cell's first node and the
+// fractions, the other nodes follow from the slot (and, across a face, from
+// the brick's forward neighbours), so a target reads 20 bytes instead of 44
+// with a table of the eight node indices.
+template <int DIM, bool ADD>
+__global__ void __launch_bounds__(256) k_transfer_dense(const float4* __restrict__ rec,
+                                                        const uint32_t* __restrict__ dst, int32_t n,
+                                                        const int32_t* __restrict__ bfwd,
+                                                        const float* __restrict__ src, float* __restrict__ out) {
+  const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const float4 r = __ldg(rec + j);
+  const uint32_t d = __ldg(dst + j);
+  const float old = ADD ? out[d] : 0.f;
+  const uint32_t s = __float_as_uint(r.x);
+  const int32_t b = (int32_t)(s >> (2 * DIM));
+  const int x = s & 3, y = (s >> 2) & 3, z = DIM == 3 ? (s >> 4) & 3 : 0;
+  const float wx[2] = {1.f - r.y, r.y}, wy[2] = {1.f - r.z, r.z}, wz[2] = {1.f - r.w, r.w};
+  float acc = 0.f;
+#pragma unroll
+  for (int c = 0; c < (DIM == 3 ? 2 : 1); ++c) {
+    float accy = 0.f;
+#pragma unroll
+    for (int bb = 0; bb < 2; ++bb) {
+      const int q = (((y + bb) >> 2) << 1) | (((z + c) >> 2) << 2);
+      const int row = ((y + bb) & 3) * 4 + (DIM == 3 ? ((z + c) & 3) * 16 : 0);
+      const int32_t b0 = q ? __ldg(bfwd + 8 * (int64_t)b + q) : b;
+      const int32_t b1 = x == 3 ? __ldg(bfwd + 8 * (int64_t)b + q + 1) : b0;
+      const float v0 = __ldg(src + ((size_t)b0 << (2 * DIM)) + row + x);
+      const float v1 = __ldg(src + ((size_t)b1 << (2 * DIM)) + row + ((x + 1) & 3));
+      accy += wy[bb] * (wx[0] * v0 + wx[1] * v1);
+    }
+    acc += (DIM == 3 ? wz[c] : 1.f) * accy;
+  }
+  out[d] = ADD ? old + acc : acc;
+}
+void launch_transfer32(const DenseTransfer& T, const DenseView& source, const float* src, float* out, bool add,
+                       cudaStream_t st) {
+  if (T.n <= 0) return;
+  const unsigned g = nblk(T.n, 256);
+  const float4* r = T.rec.get();
+  const uint32_t* d = T.dst.get();
+  if (source.dim == 3) {
+    if (add) k_transfer_dense<3, true><<<g, 256, 0, st>>>(r, d, T.n, source.bfwd, src, out);
+    else k_transfer_dense<3, false><<<g, 256, 0, st>>>(r, d, T.n, source.bfwd, src, out);
+  } else {
+    if (add) k_transfer_dense<2, true><<<g, 256, 0, st>>>(r, d, T.n, source.bfwd, src, out);
+    else k_transfer_dense<2, false><<<g, 256, 0, st>>>(r, d, T.n, source.bfwd, src, out);
+  }
+  count_launch();
+}
+
+// Prolongation from the coarsest level, whose solution is in band order.
+template <int DIM>
+__global__ void __launch_bounds__(256) k_prolong_coarsest(TransferView<float> tv, const uint32_t* __restrict__ slot,
+                                                          const float* __restrict__ src, float* __restrict__ out) {
+  const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= tv.n) return;
+  const float sx = __ldg(tv.fr + j), sy = __ldg(tv.fr + tv.n + j);
+  const float sz = DIM == 3 ? __ldg(tv.fr + 2 * (int64_t)tv.n + j) : 0.f;
+  const float wx[2] = {1.f - sx, sx}, wy[2] = {1.f - sy, sy}, wz[2] = {1.f - sz, sz};
+  const uint32_t d = __ldg(slot + j);
+  float acc = 0.f;
+#pragma unroll
+  for (int c = 0; c < (DIM == 3 ? 2 : 1); ++c) {
+    float accy = 0.f;
+#pragma unroll
+    for (int bb = 0; bb < 2; ++bb) {
+      const int q = 4 * c + 2 * bb;
+      const float v0 = __ldg(src + __ldg(tv.idx + (int64_t)q * tv.n + j));
+      const float v1 = __ldg(src + __ldg(tv.idx + (int64_t)(q + 1) * tv.n + j));
+      accy += wy[bb] * (wx[0] * v0 + wx[1] * v1);
+    }
+    acc += (DIM == 3 ? wz[c] : 1.f) * accy;
+  }
+  out[d] += acc;
+}
+void launch_prolong_coarsest32(const TransferView<float>& tv, const uint32_t* slot, const float* src, float* out,
+                               cudaStream_t st) {
+  if (tv.n <= 0) return;
+  if (tv.dim == 3) k_prolong_coarsest<3><<<nblk(tv.n, 256), 256, 0, st>>>(tv, slot, src, out);
+  else k_prolong_coarsest<2><<<nblk(tv.n, 256), 256, 0, st>>>(tv, slot, src, out);
+  count_launch();
+}
+
+// ----------------------------------------------------------------- needed points
+// Inside a cycle a coarse level's u is read only at the nodes of the stencils
+// (interpolation at its own closest points and at the finer level's), its
+// residual only at the nodes that the restriction reads.  A sweep there has to
+// update the former, which takes w = E u at them and their Laplacian
+// neighbours; the residual of any level takes w at the latter and their
+// neighbours.  On a sphere these are 0.73 and 0.36 of B, with w at 0.77 and
+// 0.47 of B+ (the band keeps a margin on both sides of the stencils).
+
+// bit of grid node (x, y, z) in per-brick masks
+__device__ __forceinline__ bool mask_bit(const BrickView& v, const uint64_t* mask, int x, int y, int z) {
+  if ((unsigned)x >= (unsigned)v.n || (unsigned)y >= (unsigned)v.n || (unsigned)z >= (unsigned)v.n) return false;
+  const int32_t b = v.map[((size_t)(z >> 2) * v.nby + (y >> 2)) * v.nbx + (x >> 2)];
+  return b >= 0 && ((mask[b] >> ((x & 3) | ((y & 3) << 2) | ((z & 3) << 4))) & 1ull);
+}
+__device__ __forceinline__ void set_mask_bit(const BrickView& v, uint64_t* mask, int x, int y, int z) {
+  const int32_t b = v.map[((size_t)(z >> 2) * v.nby + (y >> 2)) * v.nbx + (x >> 2)];
+  if (b < 0) return;
+  const unsigned long long bit = 1ull << ((x & 3) | ((y & 3) << 2) | ((z & 3) << 4));
+  if (!(mask[b] & bit)) atomicOr(reinterpret_cast<unsigned long long*>(mask + b), bit);
+}
+// the 2^d nodes of each target's cell
+__global__ void k_mark_cells(const uint64_t* base, int32_t n, int dim, BrickView src, uint64_t* mask) {
+  const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const uint64_t k = base[j];
+  const int x = (int)(k & 0xffffu), y = (int)((k >> 16) & 0xffffu), z = (int)((k >> 32) & 0xffffu);
+  for (int q = 0; q < (dim == 3 ? 8 : 4); ++q)
+    set_mask_bit(src, mask, x + (q & 1), y + ((q >> 1) & 1), z + (q >> 2));
+}
+// the 4^d nodes of every stencil, one warp per tile
+__global__ void __launch_bounds__(32) k_mark_stencils(BrickView v, const uint32_t* tile_brick,
+                                                      const int32_t* tile_start, const uint32_t* erec, int dim,
+                                                      const int32_t* bfwd, uint64_t* mask) {
+  __shared__ uint32_t has[2], box[8][2];
+  const int lane = threadIdx.x;
+  const int32_t tile = blockIdx.x;
+  if (lane < 2) has[lane] = 0u;
+  if (lane < 8) box[lane][0] = box[lane][1] = 0u;
+  __syncwarp();
+  for (int32_t k = tile_start[tile] + lane; k < tile_start[tile + 1]; k += 32)
+    atomicOr(has + ((erec[k] >> 5) & 1u), 1u << (erec[k] & 31u));
+  __syncwarp();
+  for (int b = lane; b < 64; b += 32) {
+    if (!((has[b >> 5] >> (b & 31)) & 1u)) continue;
+    const int lx = b & 3, ly = (b >> 2) & 3, lz = b >> 4;
+    const uint32_t lo = (0xFu << lx) & 0xFu, hi = 0xFu >> (4 - lx);
+    for (int c = 0; c < (dim == 3 ? 4 : 1); ++c)
+      for (int a = 0; a < 4; ++a) {
+        const int y = ly + a, z = lz + c, q = ((y >> 2) << 1) | ((z >> 2) << 2);
+        const int sh = 4 * (y & 3) + 16 * (z & 3);
+        atomicOr(&box[q][sh >> 5], lo << (sh & 31));
+        if (hi) atomicOr(&box[q + 1][sh >> 5], hi << (sh & 31));
+      }
+  }
+  __syncwarp();
+  const uint32_t tb = tile_brick[tile];
+  const int32_t home = v.map[((size_t)((tb >> 20) & 1023) * v.nby + ((tb >> 10) & 1023)) * v.nbx + (tb & 1023)];
+  if (lane < 8) {
+    const int32_t b = bfwd[8 * (int64_t)home + lane];
+    const unsigned long long m = box[lane][0] | ((unsigned long long)box[lane][1] << 32);
+    if (b < v.nbricks && (mask[b] & m) != m) atomicOr(reinterpret_cast<unsigned long long*>(mask + b), m);
+  }
+}
+// keep[i]: point i of B+ is a marked node or a Laplacian neighbour of one
+__global__ void k_keep_near(BrickView v, const uint64_t* key, int64_t nplus, int dim, const uint64_t* mask,
+                            uint8_t* keep) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nplus) return;
+  const uint64_t k = key[i];
+  const int x = key_x(k), y = key_y(k), z = dim == 3 ? key_z(k) : 0;
+  bool in = mask_bit(v, mask, x, y, z) || mask_bit(v, mask, x - 1, y, z) || mask_bit(v, mask, x + 1, y, z) ||
+            mask_bit(v, mask, x, y - 1, z) || mask_bit(v, mask, x, y + 1, z);
+  if (dim == 3) in = in || mask_bit(v, mask, x, y, z - 1) || mask_bit(v, mask, x, y, z + 1);
+  keep[i] = in;
+}
+__global__ void k_or_masks(uint64_t* a, const uint64_t* b, int32_t n) {
+  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) a[i] |= b[i];
+}
+__global__ void k_row_flags(const uint64_t* mask, int64_t nrows, int per, int64_t* flag) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < nrows) flag[t] = ((mask[t / per] >> (4 * (t % per))) & 15ull) != 0;
+}
+__global__ void k_row_emit(const uint64_t* mask, int64_t nrows, int per, const int64_t* pos, uint32_t* rows) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < nrows && ((mask[t / per] >> (4 * (t % per))) & 15ull)) rows[pos[t]] = (uint32_t)t;
+}
+
+static void build_need(const Level& L, const Dense32& D, const uint64_t* mask, NeedSet& S, cudaStream_t st) {
+  DBuf<uint8_t> keep(L.nplus());
+  k_keep_near<<<nblk(L.nplus(), 256), 256, 0, st>>>(L.view(), L.key.get(), L.nplus(), L.dim, mask, keep.get());
+  CPM_CUDA_TRY(cudaGetLastError());
+  build_units(L, D, keep.get(), S.units, st);
+  const int per = L.dim == 3 ? 16 : 4;
+  const int64_t nrows = (int64_t)L.nbricks * per;
+  DBuf<int64_t> pos(nrows);
+  k_row_flags<<<nblk(nrows, 256), 256, 0, st>>>(mask, nrows, per, pos.get());
+  S.nrows = (int32_t)scan_exclusive_i64(pos.get(), nrows, st);
+  S.rows.alloc((size_t)S.nrows);
+  k_row_emit<<<nblk(nrows, 256), 256, 0, st>>>(mask, nrows, per, pos.get(), S.rows.get());
+  CPM_CUDA_TRY(cudaGetLastError());
+  CPM_CUDA_TRY(cudaStreamSynchronize(st));  // the scratch arrays go out of scope
+}
+
+void build_need_sets(const Level& L, Dense32& D, const TransferCells* restrict_from, const TransferCells* prolong_from,
+                     cudaStream_t st) {
+  DBuf<uint64_t> mr(L.nbricks), mu(L.nbricks);
+  const size_t bytes = sizeof(uint64_t) * L.nbricks;
+  CPM_CUDA_TRY(cudaMemsetAsync(mr.get(), 0, bytes, st));
+  k_mark_cells<<<nblk(restrict_from->n, 256), 256, 0, st>>>(restrict_from->base, restrict_from->n, L.dim, L.view(),
+                                                            mr.get());
+  build_need(L, D, mr.get(), D.resid, st);
+  if (prolong_from) {  // a coarse level: its sweeps can be restricted too
+    CPM_CUDA_TRY(cudaMemsetAsync(mu.get(), 0, bytes, st));
+    k_mark_cells<<<nblk(prolong_from->n, 256), 256, 0, st>>>(prolong_from->base, prolong_from->n, L.dim, L.view(),
+                                                             mu.get());
+    k_mark_stencils<<<L.ntiles, 32, 0, st>>>(L.view(), L.tile_brick.get(), L.tile_start.get(), L.erec.get(), L.dim,
+                                             D.bfwd.get(), mu.get());
+    k_or_masks<<<nblk(L.nbricks, 256), 256, 0, st>>>(mu.get(), mr.get(), L.nbricks);
+    build_need(L, D, mu.get(), D.sweep, st);
+    D.mask_sweep = std::move(mu);
+  }
+  CPM_CUDA_TRY(cudaGetLastError());
+}
+
+// flag[j]: target j (a point of B of the target level) is wanted
+__global__ void k_target_flags(const uint32_t* slot, int32_t n, int dim, const uint64_t* mask, int64_t* flag) {
+  const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const uint32_t s = slot[j];
+  flag[j] = !mask || ((mask[s >> (2 * dim)] >> (s & ((1u << (2 * dim)) - 1u))) & 1ull);
+}
+__global__ void k_transfer_emit(const uint64_t* base, const float* fr, int32_t n, int dim, BrickView src,
+                                const uint32_t* slot, bool dense_dst, const uint64_t* mask, const int64_t* pos,
+                                float4* rec, uint32_t* dst) {
+  const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const uint32_t sj = slot[j];
+  if (mask && !((mask[sj >> (2 * dim)] >> (sj & ((1u << (2 * dim)) - 1u))) & 1ull)) return;
+  const uint64_t k = base[j];
+  const int x = (int)(k & 0xffffu), y = (int)((k >> 16) & 0xffffu), z = (int)((k >> 32) & 0xffffu);
+  const int32_t b = src.map[((size_t)(z >> 2) * src.nby + (y >> 2)) * src.nbx + (x >> 2)];
+  const uint32_t s = ((uint32_t)max(b, 0) << (2 * dim)) | (uint32_t)((x & 3) | ((y & 3) << 2) | ((z & 3) << 4));
+  const int64_t p = pos[j];
+  rec[p] = make_float4(__uint_as_float(s), fr[j], fr[n + j], dim == 3 ? fr[2 * (int64_t)n + j] : 0.f);
+  dst[p] = dense_dst ? sj : (uint32_t)j;
+}
+
+void build_transfer32(const Level& target, const Dense32& TD, const Level& source, const TransferCells& cells,
+                      bool dense_dst, bool pruned, DenseTransfer& T, cudaStream_t st) {
+  const uint64_t* mask = pruned ? TD.mask_sweep.get() : nullptr;
+  DBuf<int64_t> pos(cells.n);
+  k_target_flags<<<nblk(cells.n, 256), 256, 0, st>>>(TD.slot.get(), cells.n, target.dim, mask, pos.get());
+  CPM_CUDA_TRY(cudaGetLastError());
+  T.n = (int32_t)scan_exclusive_i64(pos.get(), cells.n, st);
+  T.rec.alloc((size_t)T.n);
+  T.dst.alloc((size_t)T.n);
+  k_transfer_emit<<<nblk(cells.n, 256), 256, 0, st>>>(cells.base, cells.fr, cells.n, target.dim, source.view(),
+                                                      TD.slot.get(), dense_dst, mask, pos.get(), T.rec.get(),
+                                                      T.dst.get());
+  CPM_CUDA_TRY(cudaGetLastError());
+  CPM_CUDA_TRY(cudaStreamSynchronize(st));
+}
+
+// ----------------------------------------------------------------- layout changes
 __global__ void k_scatter32(const float* __restrict__ x, const uint32_t* __restrict__ slot, int32_t n, float* d) {
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) d[slot[i]] = x[i];
 }
+void launch_scatter32(const DenseView& L, const float* x, float* d, cudaStream_t st) {
+  if (L.nB <= 0) return;
+  k_scatter32<<<nblk(L.nB, 256), 256, 0, st>>>(x, L.slot, L.nB, d);
+  count_launch();
+}
+__global__ void k_gather32(const float* __restrict__ d, const uint32_t* __restrict__ slot, int32_t n, float* x) {
+  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) x[i] = d[slot[i]];
+}
+void launch_gather32(const DenseView& L, const float* d, float* x, cudaStream_t st) {
+  if (L.nB <= 0) return;
+  k_gather32<<<nblk(L.nB, 256), 256, 0, st>>>(d, L.slot, L.nB, x);
+  count_launch();
+}
+// fd = r / max|r|, brick-dense.
+__global__ void k_scale_dense(const double* __restrict__ r, const double* __restrict__ norms,
+                              const uint32_t* __restrict__ slot, int32_t n, float* __restrict__ fd) {
+  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) fd[slot[i]] = (float)(r[i] * norms[2]);
+}
+void launch_scale_dense(const DenseView& L, const double* r, const double* norms, float* fd, cudaStream_t st) {
+  k_scale_dense<<<nblk(L.nB, 256), 256, 0, st>>>(r, norms, L.slot, L.nB, fd);
+  count_launch();
+}
+// u += max|r| d
+__global__ void k_axpy_dense(double* __restrict__ u, const float* __restrict__ d, const uint32_t* __restrict__ slot,
+                             const double* __restrict__ norms, int32_t n) {
+  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) u[i] += norms[0] * (double)d[slot[i]];
+}
+void launch_axpy_dense(const DenseView& L, double* u, const float* d, const double* norms, cudaStream_t st) {
+  k_axpy_dense<<<nblk(L.nB, 256), 256, 0, st>>>(u, d, L.slot, norms, L.nB);
+  count_launch();
+}
+
 void dense_static(const Level& L, Dense32& D, const float* dA, const float* c, cudaStream_t st) {
   const size_t n = dense_size(L);
   auto put = [&](DBuf<float>& d, const float* x) {

@@ -15,6 +15,21 @@
 
 namespace cpm {
 
+// Extension units of a set of points (see ExtUnits).
+struct UnitsView {
+  const uint32_t* tiles;
+  const float4* pts[2];
+  const uint32_t* cidx[2];
+  int32_t ntiles;
+};
+
+// Brick rows of a set of nodes (row = brick * 4^(d-1) + row of the brick):
+// a list, or all n rows of the level.
+struct RowsView {
+  const uint32_t* list;
+  uint32_t n;
+};
+
 // Plain-pointer view of a level's brick-dense structures.
 struct DenseView {
   const uint64_t* bmask;   // band occupancy per brick
@@ -27,11 +42,7 @@ struct DenseView {
   int64_t nplus;
   int dim;
   float inv_h2, gamma;
-  // units of the extension over B+ (ExtUnits)
-  const uint32_t* tiles;
-  const float4* pts[2];
-  const uint32_t* cidx[2];
-  int32_t ntiles;
+  UnitsView all;           // the extension over B+
   int variant;             // launch shape of the extension (0, 1, 2)
   const float* dA;         // brick-dense omega / diag(A)
   const float* c;          // brick-dense c, or null (constant)
@@ -44,6 +55,13 @@ struct ExtUnits {
   DBuf<float4> pts[2];   // a unit's first and second point: slot (bits) and cp fractions
   DBuf<uint32_t> cidx[2];  // their band indices
 };
+// The nodes of a level that a pass inside a cycle has to visit: rows of the
+// stencil, and the points whose w = E u they take (dense32.cu).
+struct NeedSet {
+  ExtUnits units;
+  DBuf<uint32_t> rows;
+  int32_t nrows = 0;
+};
 // Brick-dense structures of one level.
 struct Dense32 {
   DBuf<int4> bface;
@@ -51,7 +69,36 @@ struct Dense32 {
   DBuf<uint32_t> slot;
   ExtUnits all;          // every point of B+
   DBuf<float> dA, c;     // brick-dense omega / diag(A) and c
+  // levels of a V-cycle (build_need_sets)
+  NeedSet resid;         // residual that is restricted (every level but the coarsest)
+  NeedSet sweep;         // sweeps (levels between the finest and the coarsest)
+  DBuf<uint64_t> mask_sweep;
 };
+// Targets of a linear transfer: base nodes of their cells in the source grid
+// (packed), fractions (SoA, d x n).
+struct TransferCells {
+  const uint64_t* base;
+  const float* fr;
+  int32_t n;
+};
+// Linear transfer from a brick-dense source: per target the slot (bits) of the
+// cell's first node and the fractions, and where the result goes.
+struct DenseTransfer {
+  DBuf<float4> rec;
+  DBuf<uint32_t> dst;
+  int32_t n = 0;
+};
+UnitsView units_view(const ExtUnits& U);
+inline RowsView rows_view(const NeedSet& S) { return {S.rows.get(), (uint32_t)S.nrows}; }
+inline RowsView all_rows(const DenseView& L) { return {nullptr, (uint32_t)L.nbricks << (2 * (L.dim - 1))}; }
+// D.resid from the cells of the restriction to the next level; D.sweep too where
+// the level is prolonged from (prolong_from: the cells of the finer level's points).
+void build_need_sets(const Level& L, Dense32& D, const TransferCells* restrict_from,
+                     const TransferCells* prolong_from, cudaStream_t st);
+// Records of a transfer to the points of B of `target` (only those in its sweep set if
+// pruned), written brick-dense or in band order.
+void build_transfer32(const Level& target, const Dense32& TD, const Level& source, const TransferCells& cells,
+                      bool dense_dst, bool pruned, DenseTransfer& T, cudaStream_t st);
 inline size_t dense_size(const Level& L) { return (size_t)(L.nbricks + 1) << (2 * L.dim); }
 void build_dense32(const Level& L, Dense32& D, cudaStream_t st);
 // D.dA (and D.c) from the band-order vectors.
@@ -65,15 +112,28 @@ struct Vec32 {
   T* compact;  // band order (used when dense is null)
 };
 
-// w (brick-dense) = E u over B+.  u brick-dense or in band order.
-void launch_extend32(const DenseView& L, Vec32<const float> u, float* w, cudaStream_t st);
+// w (brick-dense) = E u over the set S.  u brick-dense or in band order.
+void launch_extend32(const DenseView& L, const UnitsView& S, Vec32<const float> u, float* w, cudaStream_t st);
 // w (band order, the first npts points of B+) = E u, u in band order.
 void launch_extend32_compact(const DenseView& L, const float* u, float* w, int32_t npts, cudaStream_t st);
 // Stencil pass of `mode` (APPLY, RESID, JACOBI, JAC_RED, JAC_BLACK) from w = E u (brick-dense):
 // out = M u, out = f - c u + M u, or out = u + (f - c u + M u) dA (out may be u).  f has u's layout;
 // where that is band order and fd is given, f is also written there brick-dense.
 void launch_lap32(const DenseView& L, LapMode mode, Vec32<const float> u, const float* w, const float* f,
-                  float cval, Vec32<float> out, float* fd, cudaStream_t st);
+                  float cval, Vec32<float> out, float* fd, const RowsView& rows, cudaStream_t st);
+// u = f dA, the first Jacobi sweep from u = 0 (all brick-dense).
+void launch_jacobi_zero32(const DenseView& L, const float* f, float* u, const RowsView& rows, cudaStream_t st);
+// out[dst] (+)= linear interpolation of the brick-dense src (a vector of level `source`).
+void launch_transfer32(const DenseTransfer& T, const DenseView& source, const float* src, float* out, bool add,
+                       cudaStream_t st);
+// out[slot[j]] += linear interpolation of src in band order (tv.idx set).
+void launch_prolong_coarsest32(const TransferView<float>& tv, const uint32_t* slot, const float* src, float* out,
+                               cudaStream_t st);
+// Layout changes of vectors on B.
+void launch_scatter32(const DenseView& L, const float* x, float* d, cudaStream_t st);
+void launch_gather32(const DenseView& L, const float* d, float* x, cudaStream_t st);
+void launch_scale_dense(const DenseView& L, const double* r, const double* norms, float* fd, cudaStream_t st);
+void launch_axpy_dense(const DenseView& L, double* u, const float* d, const double* norms, cudaStream_t st);
 // Time the extension's launch shapes (as tune_extension).
 int tune_extend32(const DenseView& L, const float* u, float* w, cudaStream_t st, float ms[3]);
 

@@ -128,6 +128,7 @@ struct HLevel {
   DBuf<double> dM64;  // diag(M)
   Transfer R;  // restriction: targets = B of level l+1, source = this level
   Transfer P;  // prolongation: targets = B of this level, source = level l+1
+  DenseTransfer R32, P32;  // the same for brick-dense FP32 vectors (P32 not from the coarsest level)
 
   template <typename T>
   LevelView<T> view() const;
@@ -217,7 +218,8 @@ using namespace cpm;
 struct Workspace {
   std::vector<cpm::Work<double>> w64;
   std::vector<cpm::Work<float>> w32;
-  std::vector<cpm::DBuf<float>> ud, wd, fd;  // brick-dense u, w = E u and f of the FP32 passes
+  std::vector<cpm::DBuf<float>> ud, wd, fd, rd;  // brick-dense u, w = E u, f and r of the FP32 passes
+  std::vector<cpm::DBuf<float>> td;  // brick-dense E u where the residual of E u is restricted
   cpm::DBuf<double> part;   // norm partials (2 per block)
   int part_blocks = 0;
   cpm::DBuf<double> own_norms;  // [max, sumsq, 1/max, -] unless norms points elsewhere
@@ -277,6 +279,7 @@ struct cpm_hier_s {
                               // 3: GMRES
   int32_t coarse_sweeps = 0;
   int32_t coarse_restarts = 3;
+  bool dense_cycle = false;   // FP32 V-cycles on brick-dense vectors (vcycle32)
   bool pair_resid = false;    // outer residual in FP32 pairs (k_extend_pair + k_resid_pair)
   cpm_mlp mlp = nullptr;
   std::unique_ptr<cpm::MlpLevelData> mlpd;
@@ -292,13 +295,18 @@ static void alloc_workspace(const cpm_hier_s& H, Workspace& W, double* norms_slo
   W.ud.resize(H.L.size());
   W.wd.resize(H.L.size());
   W.fd.resize(H.L.size());
+  W.rd.resize(H.L.size());
+  W.td.resize(H.L.size());
   for (size_t l = 0; l < H.L.size(); ++l) {
     const int64_t nB = H.L[l].lev->nB, np = H.L[l].lev->nplus();
     const bool paper = H.opts.op_form != CPM_OP_MBR;
     W.w64[l].alloc(nB, np, paper, H.opts.relative != 0);
     W.w32[l].alloc(nB, np, paper, H.opts.relative != 0);
     const size_t slots = dense_size(*H.L[l].lev);
-    for (auto* v : {&W.ud[l], &W.wd[l], &W.fd[l]}) {
+    for (auto* v : {&W.ud[l], &W.wd[l], &W.fd[l], &W.rd[l], &W.td[l]}) {
+      const bool cycle_only = v == &W.rd[l] || v == &W.td[l];
+      if (cycle_only && (!H.dense_cycle || l + 1 == H.L.size())) continue;
+      if (v == &W.td[l] && H.opts.residual_mode == 1) continue;
       v->alloc(slots);
       CPM_CUDA_TRY(cudaMemset(v->get(), 0, sizeof(float) * slots));
     }
@@ -364,9 +372,9 @@ static void mbr_op(cpm_hier_s* H, Workspace& W, int l, LapMode mode, const float
   HLevel& lv = H->L[l];
   const DenseView v = lv.dview();
   const Vec32<const float> uv{nullptr, u};
-  launch_extend32(v, uv, W.wd[l].get(), st);
+  launch_extend32(v, v.all, uv, W.wd[l].get(), st);
   launch_lap32(v, mode, uv, W.wd[l].get(), f, (float)H->c, Vec32<float>{nullptr, u_inout ? u_inout : out},
-               nullptr, st);
+               nullptr, all_rows(v), st);
 }
 
 // The operator of level l in the hierarchy's form: M u (APPLY), the residual
@@ -412,9 +420,9 @@ static void smooth32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* 
   for (int s = 0; s < sweeps; ++s) {
     const Vec32<float> in = s == 0 ? compact : dense, out = s == sweeps - 1 ? compact : dense;
     const Vec32<const float> cin{in.dense, in.compact};
-    launch_extend32(v, cin, W.wd[l].get(), st);
+    launch_extend32(v, v.all, cin, W.wd[l].get(), st);
     launch_lap32(v, LAP_JACOBI, cin, W.wd[l].get(), s == 0 ? f : W.fd[l].get(), (float)H->c, out,
-                 sweeps > 1 ? W.fd[l].get() : nullptr, st);
+                 sweeps > 1 ? W.fd[l].get() : nullptr, all_rows(v), st);
   }
 }
 
@@ -520,6 +528,112 @@ static void coarse_solve(cpm_hier_s* H, Workspace* const* W, int G, const T* con
   }
 }
 
+// What a level's FP32 iterate is at a point of the cycle: zero, brick-dense (in
+// Workspace::ud) or in band order.
+enum class State32 { zero, dense, compact };
+
+// Weighted Jacobi sweeps of level l on brick-dense vectors, f in Workspace::fd
+// (where u is in band order, so is f, and the first sweep fills fd).  Only the
+// rows and points of `need`, if given.  The last sweep writes u_out (band
+// order) where that is given.
+static void sweeps32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* u, State32& state, int sweeps,
+                     const NeedSet* need, float* u_out, cudaStream_t st) {
+  const DenseView v = H->L[l].dview();
+  const UnitsView units = need ? units_view(need->units) : v.all;
+  const RowsView rows = need ? rows_view(*need) : all_rows(v);
+  float* ud = W.ud[l].get();
+  float* fd = W.fd[l].get();
+  for (int s = 0; s < sweeps; ++s) {
+    const Vec32<float> out = u_out && s == sweeps - 1 ? Vec32<float>{nullptr, u_out} : Vec32<float>{ud, nullptr};
+    if (state == State32::zero && out.dense) {
+      launch_jacobi_zero32(v, fd, ud, rows, st);
+    } else {
+      if (state == State32::zero)
+        CPM_CUDA_TRY(cudaMemsetAsync(ud, 0, W.ud[l].n * sizeof(float), st));
+      const bool band = state == State32::compact;
+      const Vec32<const float> in{band ? nullptr : ud, band ? u : nullptr};
+      launch_extend32(v, units, in, W.wd[l].get(), st);
+      launch_lap32(v, LAP_JACOBI, in, W.wd[l].get(), band ? f : fd, (float)H->c, out, band ? fd : nullptr, rows,
+                   st);
+    }
+    state = out.dense ? State32::dense : State32::compact;
+  }
+}
+
+// FP32 V-cycle of the MBR form with Jacobi smoothing and linear transfers, all
+// vectors brick-dense between the levels; the coarsest solve is in band order.
+// Level 0: state says how u[g] and f[g] come (zero and dense: f in
+// Workspace::fd; band order: u[g], f[g], and fd is filled); u_out, if given,
+// receives the result in band order, else it is left in Workspace::ud.  Below
+// level 0 only the needed points are visited (NeedSet).
+static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const float* const* f, float* const* u,
+                     State32 state0, bool band_out, cudaStream_t st) {
+  const int nl = (int)H->L.size();
+  HLevel& lv = H->L[l];
+  const DenseView v = lv.dview();
+  const bool last = l + 1 == nl - 1;  // the next level is the coarsest
+  const NeedSet* need = l > 0 ? &lv.dense.sweep : nullptr;
+  State32 state[kMaxGroup];
+  const float* cf[kMaxGroup];
+  float* cu[kMaxGroup];
+  for (int g = 0; g < G; ++g) {
+    Workspace& w = *W[g];
+    float* ud = w.ud[l].get();
+    float* fd = w.fd[l].get();
+    state[g] = state0;
+    int pre = H->opts.nu1;
+    auto make_dense = [&]() {
+      if (state[g] == State32::zero) CPM_CUDA_TRY(cudaMemsetAsync(ud, 0, w.ud[l].n * sizeof(float), st));
+      if (state[g] == State32::compact) {
+        launch_scatter32(v, u[g], ud, st);
+        launch_scatter32(v, f[g], fd, st);
+      }
+      state[g] = State32::dense;
+    };
+    if (l == 0 && H->learned_active && pre > 0) {
+      // learned smoother in place of the first Jacobi sweep: r = f - A u, u += net(r)
+      make_dense();
+      launch_extend32(v, v.all, {ud, nullptr}, w.wd[0].get(), st);
+      launch_lap32(v, LAP_RESID, {ud, nullptr}, w.wd[0].get(), fd, (float)H->c, {nullptr, w.w32[0].r.get()},
+                   nullptr, all_rows(v), st);
+      mlp_forward(H->mlp->params.get(), *H->mlpd, w.w32[0].r.get(), 1.f / v.inv_h2, nullptr, ud, v.slot, nullptr,
+                  st);
+      --pre;
+    }
+    sweeps32(H, w, l, f ? f[g] : nullptr, u ? u[g] : nullptr, state[g], pre, need, nullptr, st);
+    if (state[g] != State32::dense) make_dense();
+    // the residual of u (or of E u) where the restriction reads it
+    const NeedSet& rs = lv.dense.resid;
+    const float* uu = ud;
+    if (H->opts.residual_mode == 0) {
+      launch_extend32(v, need ? units_view(need->units) : v.all, {ud, nullptr}, w.td[l].get(), st);
+      uu = w.td[l].get();
+    }
+    launch_extend32(v, units_view(rs.units), {uu, nullptr}, w.wd[l].get(), st);
+    launch_lap32(v, LAP_RESID, {uu, nullptr}, w.wd[l].get(), fd, (float)H->c, {w.rd[l].get(), nullptr}, nullptr,
+                 rows_view(rs), st);
+    cf[g] = last ? w.w32[l + 1].f.get() : w.fd[l + 1].get();
+    cu[g] = w.w32[l + 1].u.get();
+    launch_transfer32(lv.R32, v, w.rd[l].get(), const_cast<float*>(cf[g]), false, st);
+  }
+  if (last) {
+    coarse_solve<float>(H, W, G, cf, cu, st);
+  } else {
+    // W-cycle: a second cycle from the first's result
+    for (int q = 0; q < H->opts.cycle; ++q)
+      vcycle32(H, W, G, l + 1, nullptr, nullptr, q == 0 ? State32::zero : State32::dense, false, st);
+  }
+  for (int g = 0; g < G; ++g) {
+    Workspace& w = *W[g];
+    if (last)
+      launch_prolong_coarsest32(tview<float>(lv.P, lv.lev->dim), v.slot, cu[g], w.ud[l].get(), st);
+    else
+      launch_transfer32(lv.P32, H->L[l + 1].dview(), w.ud[l + 1].get(), w.ud[l].get(), true, st);
+    sweeps32(H, w, l, nullptr, nullptr, state[g], H->opts.nu2, need, band_out ? u[g] : nullptr, st);
+    if (band_out && H->opts.nu2 == 0) launch_gather32(v, w.ud[l].get(), u[g], st);
+  }
+}
+
 // V-cycle of Algorithm 4.1 from level l for G systems in lockstep.
 template <typename T>
 static void vcycle_level(cpm_hier_s* H, Workspace* const* W, int G, int l, const T* const* f,
@@ -528,6 +642,12 @@ static void vcycle_level(cpm_hier_s* H, Workspace* const* W, int G, int l, const
   if (l == nl - 1) {
     coarse_solve<T>(H, W, G, f, u, st);
     return;
+  }
+  if constexpr (sizeof(T) == 4) {
+    if (H->dense_cycle && l == 0) {
+      vcycle32(H, W, G, 0, f, u, State32::compact, true, st);
+      return;
+    }
   }
   HLevel& lv = H->L[l];
   HLevel& cv = H->L[l + 1];
@@ -543,7 +663,7 @@ static void vcycle_level(cpm_hier_s* H, Workspace* const* W, int G, int l, const
         const LevelView<float> v = lv.view<float>();
         mbr_op(H, *W[g], l, LAP_RESID, f[g], u[g], w.r.get(), nullptr, nullptr, nullptr, st);
         mlp_forward(H->mlp->params.get(), *H->mlpd, w.r.get(), 1.f / v.inv_h2, nullptr, u[g], nullptr,
-                    st);
+                    nullptr, st);
         --pre;
       }
     }
@@ -637,6 +757,14 @@ static void outer_step(cpm_hier_s* H, Workspace* const* W, int G, int mode, int 
     else
       vcycle_level<double>(H, W, G, 0, r, d, st);
     for (int g = 0; g < G; ++g) launch_axpy64(W[g]->u_own.get(), W[g]->d64.get(), nB, st);
+  } else if (H->dense_cycle && !first_fmg) {
+    const DenseView v = H->L[0].dview();
+    for (int g = 0; g < G; ++g)
+      launch_scale_dense(v, W[g]->r64.get(), W[g]->norms, W[g]->fd[0].get(), st);
+    for (int j = 0; j < inner; ++j)
+      vcycle32(H, W, G, 0, nullptr, nullptr, j == 0 ? State32::zero : State32::dense, false, st);
+    for (int g = 0; g < G; ++g)
+      launch_axpy_dense(v, W[g]->u_own.get(), W[g]->ud[0].get(), W[g]->norms, st);
   } else {
     const float* r[kMaxGroup];
     float* d[kMaxGroup];
@@ -940,6 +1068,22 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
   for (int l = 0; l + 1 < nl; ++l) {
     build_transfer(*H->L[l + 1].lev, *H->L[l].lev, H->L[l].R, o.transfer_deg, st, err.get());
     build_transfer(*H->L[l].lev, *H->L[l + 1].lev, H->L[l].P, o.transfer_deg, st, err.get());
+  }
+  H->dense_cycle = o.op_form == CPM_OP_MBR && o.smoother == CPM_SMOOTH_JACOBI && !o.relative &&
+                   o.transfer_deg == 1 && nl > 1;
+  if (H->dense_cycle) {
+    auto cells = [](const Transfer& t) { return TransferCells{t.base.get(), t.fr32.get(), t.n}; };
+    for (int l = 0; l + 1 < nl; ++l) {
+      const TransferCells r = cells(H->L[l].R);
+      const TransferCells p = l > 0 ? cells(H->L[l - 1].P) : TransferCells{};
+      build_need_sets(*H->L[l].lev, H->L[l].dense, &r, l > 0 ? &p : nullptr, st);
+    }
+    for (int l = 0; l + 1 < nl; ++l) {
+      const bool last = l + 1 == nl - 1;
+      HLevel &a = H->L[l], &b = H->L[l + 1];
+      build_transfer32(*b.lev, b.dense, *a.lev, cells(a.R), !last, !last, a.R32, st);
+      if (!last) build_transfer32(*a.lev, a.dense, *b.lev, cells(a.P), true, l > 0, a.P32, st);
+    }
   }
   // per-point c on every level (restricted from the finest band)
   if (o.c_device) {
@@ -1481,7 +1625,7 @@ cpm_status cpm_mlp_correction(cpm_hier h, const float* r, float* du, cpm_stream 
   CPM_CHECK(h != nullptr && r != nullptr && du != nullptr, CPM_ERR_ARG, "NULL argument");
   CPM_CHECK(h->mlp && h->mlpd, CPM_ERR_ARG, "no learned smoother set (cpm_hier_set_smoother)");
   const double dx = h->L[0].lev->dx;
-  mlp_forward(h->mlp->params.get(), *h->mlpd, r, (float)(dx * dx), du, nullptr, nullptr,
+  mlp_forward(h->mlp->params.get(), *h->mlpd, r, (float)(dx * dx), du, nullptr, nullptr, nullptr,
               (cudaStream_t)stream);
   CPM_CUDA_TRY(cudaGetLastError());
   CPM_API_END

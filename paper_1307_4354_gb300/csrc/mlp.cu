@@ -78,6 +78,7 @@ struct MlpFwdArgs {
   float dx2;
   float* du;             // out: correction ...
   float* u;              // ... or u += correction
+  const uint32_t* uslot; // u's slots (brick-dense u), or null (band order)
   // training outputs
   __nv_bfloat16* Xs;     // nB x 32
   __nv_bfloat16* H1;     // nB x 64
@@ -236,12 +237,12 @@ __global__ void __launch_bounds__(kFwdWarps * 32, MODE == 2 ? 2 : 3) k_mlp_forwa
       const int64_t r0 = p0 + g, r1 = p0 + g + 8;
       if (r0 < A.nB) {
         const float d = sw[g] * A.dx2 * (y0 + b3);
-        if (MODE == 1) A.u[r0] += d; else A.du[r0] = d;
+        if (MODE == 1) A.u[A.uslot ? A.uslot[r0] : r0] += d; else A.du[r0] = d;
         if (MODE == 2 && A.S) A.S[r0] = sw[g];
       }
       if (r1 < A.nB) {
         const float d = sw[g + 8] * A.dx2 * (y1 + b3);
-        if (MODE == 1) A.u[r1] += d; else A.du[r1] = d;
+        if (MODE == 1) A.u[A.uslot ? A.uslot[r1] : r1] += d; else A.du[r1] = d;
         if (MODE == 2 && A.S) A.S[r1] = sw[g + 8];
       }
     }
@@ -678,7 +679,7 @@ void MlpLevelData::build(const Level& lev, const double* diagM, cudaStream_t st)
 }
 
 void mlp_forward(const float* params, const MlpLevelData& D, const float* r, float dx2, float* du,
-                 float* u_add, const MlpTrainBuffers* tb, cudaStream_t st) {
+                 float* u_add, const uint32_t* uslot, const MlpTrainBuffers* tb, cudaStream_t st) {
   MlpFwdArgs a{};
   a.params = params;
   a.r = r;
@@ -688,6 +689,7 @@ void mlp_forward(const float* params, const MlpLevelData& D, const float* r, flo
   a.dx2 = dx2;
   a.du = du;
   a.u = u_add;
+  a.uslot = uslot;
   if (tb) {
     a.Xs = tb->Xs.get();
     a.H1 = tb->H1.get();
@@ -739,11 +741,12 @@ void mlp_loss_grad(const float* params, const MlpLevelData& D, const LevelView<f
   CPM_CUDA_TRY(cudaFuncSetAttribute(k_mlp_backward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)sizeof(BwdShared)));
   tb.ensure(nB, L.nplus, ((int64_t)DL.nbricks + 1) << (2 * DL.dim));
-  mlp_forward(params, D, r, dx2, tb.du.get(), nullptr, &tb, st);
+  mlp_forward(params, D, r, dx2, tb.du.get(), nullptr, nullptr, &tb, st);
   // M du (extension over B+ then the stencil)
   const Vec32<const float> du{nullptr, tb.du.get()};
-  launch_extend32(DL, du, tb.w.get(), st);
-  launch_lap32(DL, LAP_APPLY, du, tb.w.get(), nullptr, 0.f, Vec32<float>{nullptr, tb.Mdu.get()}, nullptr, st);
+  launch_extend32(DL, DL.all, du, tb.w.get(), st);
+  launch_lap32(DL, LAP_APPLY, du, tb.w.get(), nullptr, 0.f, Vec32<float>{nullptr, tb.Mdu.get()}, nullptr,
+               all_rows(DL), st);
   const int nb256 = (int)((nB + 255) / 256);
   k_mlp_resid<<<nb256, 256, 0, st>>>(r, tb.du.get(), tb.Mdu.get(), cvec, cval, nB, tb.z.get(),
                                       tb.lpart.get());

@@ -36,10 +36,10 @@ struct MlpTrainBuffers {
   void ensure(int32_t nB, int64_t nplus, int64_t slots);
 };
 
-// du = network correction of residual r (u_add != null: u_add += du instead);
-// tb != null also stores the activations for the backward pass.
+// du = network correction of residual r (u_add != null: u_add += du instead, at
+// the slots uslot where given); tb != null also stores the activations for the backward pass.
 void mlp_forward(const float* params, const MlpLevelData& D, const float* r, float dx2, float* du,
-                 float* u_add, const MlpTrainBuffers* tb, cudaStream_t st);
+                 float* u_add, const uint32_t* uslot, const MlpTrainBuffers* tb, cudaStream_t st);
 // Loss ||r - A du||^2 / ||r||^2 (tb.loss: [||z||^2, ||r||^2]) and gradient (tb.grad).
 void mlp_loss_grad(const float* params, const MlpLevelData& D, const LevelView<float>& L,
                    const DenseView& DL, const float* cvec, float cval, const float* r, MlpTrainBuffers& tb,
