@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "dense32.cuh"
+#include "pdl.cuh"
 
 namespace cpm {
 
@@ -251,10 +252,10 @@ __device__ __forceinline__ float4 load_row_ordered(const DenseView& L, const flo
   const uint64_t m = __ldg(L.bmask + brick);
   const uint32_t nib = (uint32_t)(m >> (4 * row)) & 15u;
   const float* p = u + __ldg(L.bstart + brick) + __popcll(m & ((1ull << (4 * row)) - 1ull));
-  if (nib & 1u) v.x = __ldg(p);
-  if (nib & 2u) v.y = __ldg(p + (nib & 1u));
-  if (nib & 4u) v.z = __ldg(p + __popc(nib & 3u));
-  if (nib & 8u) v.w = __ldg(p + __popc(nib & 7u));
+  if (nib & 1u) v.x = ld_prior(p);
+  if (nib & 2u) v.y = ld_prior(p + (nib & 1u));
+  if (nib & 4u) v.z = ld_prior(p + __popc(nib & 3u));
+  if (nib & 8u) v.w = ld_prior(p + __popc(nib & 7u));
   return v;
 }
 
@@ -279,6 +280,7 @@ __global__ void __launch_bounds__(32 * WARPS, kExtThreadsSM / (32 * WARPS))
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* win = box[warp];
   const int32_t tile = blockIdx.x * WARPS + warp;
+  release_next();
   if (tile >= S.ntiles) return;
   const uint32_t hdr = __ldg(S.tiles + (size_t)tile * kTileWords + min(lane, kTileWords - 1));
     const uint32_t tbox = __shfl_sync(0xffffffffu, hdr, kTileBox);
@@ -290,6 +292,7 @@ __global__ void __launch_bounds__(32 * WARPS, kExtThreadsSM / (32 * WARPS))
       ra = __ldg(S.pts[0] + k);
       rb = __ldg(S.pts[1] + k);
     }
+    wait_prior();
     // row r = lane + 32 h of the 2^(d-1) columns of bricks along x: column r / 4^(d-1),
     // row r mod 4^(d-1) of its bricks
     const int xhi = (tbox >> 2) & 3;
@@ -311,8 +314,8 @@ __global__ void __launch_bounds__(32 * WARPS, kExtThreadsSM / (32 * WARPS))
         lo[h] = load_row_ordered<DIM>(L, u, blo, row);
         if (xhi > 0) hi[h] = load_row_ordered<DIM>(L, u, bhi, row);
       } else {
-        lo[h] = __ldg(reinterpret_cast<const float4*>(u + ((size_t)blo << (2 * DIM))) + row);
-        if (xhi > 0) hi[h] = __ldg(reinterpret_cast<const float4*>(u + ((size_t)bhi << (2 * DIM))) + row);
+        lo[h] = ld_prior(reinterpret_cast<const float4*>(u + ((size_t)blo << (2 * DIM))) + row);
+        if (xhi > 0) hi[h] = ld_prior(reinterpret_cast<const float4*>(u + ((size_t)bhi << (2 * DIM))) + row);
       }
     }
 #pragma unroll
@@ -399,11 +402,11 @@ static void extend_units(const DenseView& L, const UnitsView& S, int variant, co
                          int32_t npts, cudaStream_t st) {
   if (S.ntiles <= 0) return;
   if (variant == 2)
-    k_extend_units<DIM, CIN, COUT, 4><<<nblk(S.ntiles, 4), 128, 0, st>>>(L, S, u, w, npts);
+    launch_pdl(k_extend_units<DIM, CIN, COUT, 4>, nblk(S.ntiles, 4), 128, st, L, S, u, w, npts);
   else if (variant == 1)
-    k_extend_units<DIM, CIN, COUT, 2><<<nblk(S.ntiles, 2), 64, 0, st>>>(L, S, u, w, npts);
+    launch_pdl(k_extend_units<DIM, CIN, COUT, 2>, nblk(S.ntiles, 2), 64, st, L, S, u, w, npts);
   else
-    k_extend_units<DIM, CIN, COUT, 1><<<S.ntiles, 32, 0, st>>>(L, S, u, w, npts);
+    launch_pdl(k_extend_units<DIM, CIN, COUT, 1>, S.ntiles, 32, st, L, S, u, w, npts);
 }
 
 static void extend32(const DenseView& L, const UnitsView& S, int variant, Vec32<const float> u, float* w,
@@ -472,26 +475,28 @@ __global__ void __launch_bounds__(256) k_lap_rows(DenseView L, const float* u, c
                                                   float* __restrict__ fd, RowsView rows) {
   constexpr int ROWS = DIM == 3 ? 16 : 4, SH = 2 * DIM;
   uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  release_next();
   if (t >= rows.n) return;
   if (rows.list) t = __ldg(rows.list + t);
   const int32_t b = (int32_t)(t / ROWS);
   const int row = (int)(t % ROWS);
   const int y = row & 3, z = row >> 2;
   const size_t s0 = ((size_t)b << SH) + 4 * row;
-  auto load4 = [](const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); };
+  auto load4 = [](const float* p) { return ld_prior(reinterpret_cast<const float4*>(p)); };
   const int4 fa = __ldg(L.bface + 2 * (int64_t)b);
   const int4 fb = DIM == 3 ? __ldg(L.bface + 2 * (int64_t)b + 1) : make_int4(0, 0, 0, 0);
   const bool ordered = CIN || !out.dense;  // band-order data on either side
   const uint64_t m = ordered ? __ldg(L.bmask + b) : 0ull;
   const int32_t start = ordered ? __ldg(L.bstart + b) : 0;
-  const float4 w0 = load4(w + s0);
   float4 uu, ff = make_float4(0.f, 0.f, 0.f, 0.f), dd = ff, cc = make_float4(cval, cval, cval, cval);
+  if (MODE != LAP_APPLY && MODE != LAP_RESID) dd = __ldg(reinterpret_cast<const float4*>(L.dA + s0));
+  if (MODE != LAP_APPLY && L.c) cc = __ldg(reinterpret_cast<const float4*>(L.c + s0));
+  wait_prior();
+  const float4 w0 = load4(w + s0);
   if (!CIN) {
-    uu = *reinterpret_cast<const float4*>(u + s0);
+    uu = load4(u + s0);
     if (MODE != LAP_APPLY) ff = load4(f + s0);
   }
-  if (MODE != LAP_APPLY && MODE != LAP_RESID) dd = load4(L.dA + s0);
-  if (MODE != LAP_APPLY && L.c) cc = load4(L.c + s0);
   auto row4 = [&](int32_t bb, int rr) { return load4(w + ((size_t)bb << SH) + 4 * rr); };
   const float4 ym = row4(y > 0 ? b : fa.z, y > 0 ? row - 1 : row + 3);
   const float4 yp = row4(y < 3 ? b : fa.w, y < 3 ? row + 1 : row - 3);
@@ -500,8 +505,8 @@ __global__ void __launch_bounds__(256) k_lap_rows(DenseView L, const float* u, c
     zm = row4(z > 0 ? b : fb.x, z > 0 ? row - 4 : row + 12);
     zp = row4(z < 3 ? b : fb.y, z < 3 ? row + 4 : row - 12);
   }
-  const float xm = __ldg(w + ((size_t)fa.x << SH) + 4 * row + 3);
-  const float xp = __ldg(w + ((size_t)fa.y << SH) + 4 * row);
+  const float xm = ld_prior(w + ((size_t)fa.x << SH) + 4 * row + 3);
+  const float xp = ld_prior(w + ((size_t)fa.y << SH) + 4 * row);
   const uint32_t nib = (uint32_t)(m >> (4 * row)) & 15u;
   const int32_t i0 = start + __popcll(m & ((1ull << (4 * row)) - 1ull));
   const int32_t off[4] = {0, (int)(nib & 1u), __popc(nib & 3u), __popc(nib & 7u)};
@@ -510,8 +515,8 @@ __global__ void __launch_bounds__(256) k_lap_rows(DenseView L, const float* u, c
 #pragma unroll
     for (int a = 0; a < 4; ++a)
       if ((nib >> a) & 1u) {
-        a4[a] = u[i0 + off[a]];
-        if (MODE != LAP_APPLY) b4[a] = __ldg(f + i0 + off[a]);
+        a4[a] = ld_prior(u + i0 + off[a]);
+        if (MODE != LAP_APPLY) b4[a] = ld_prior(f + i0 + off[a]);
       }
     uu = make_float4(a4[0], a4[1], a4[2], a4[3]);
     ff = make_float4(b4[0], b4[1], b4[2], b4[3]);
@@ -555,11 +560,11 @@ static void lap32(const DenseView& L, Vec32<const float> u, const float* w, cons
   if (rows.n == 0) return;
   const unsigned g = nblk(rows.n, 256);
   if (L.dim == 3) {
-    if (u.dense) k_lap_rows<3, MODE, false><<<g, 256, 0, st>>>(L, u.dense, w, f, cval, out, nullptr, rows);
-    else k_lap_rows<3, MODE, true><<<g, 256, 0, st>>>(L, u.compact, w, f, cval, out, fd, rows);
+    if (u.dense) launch_pdl(k_lap_rows<3, MODE, false>, g, 256, st, L, u.dense, w, f, cval, out, (float*)nullptr, rows);
+    else launch_pdl(k_lap_rows<3, MODE, true>, g, 256, st, L, u.compact, w, f, cval, out, fd, rows);
   } else {
-    if (u.dense) k_lap_rows<2, MODE, false><<<g, 256, 0, st>>>(L, u.dense, w, f, cval, out, nullptr, rows);
-    else k_lap_rows<2, MODE, true><<<g, 256, 0, st>>>(L, u.compact, w, f, cval, out, fd, rows);
+    if (u.dense) launch_pdl(k_lap_rows<2, MODE, false>, g, 256, st, L, u.dense, w, f, cval, out, (float*)nullptr, rows);
+    else launch_pdl(k_lap_rows<2, MODE, true>, g, 256, st, L, u.compact, w, f, cval, out, fd, rows);
   }
   count_launch();
 }
@@ -577,14 +582,17 @@ void launch_lap32(const DenseView& L, LapMode mode, Vec32<const float> u, const 
 __global__ void __launch_bounds__(256) k_jacobi_zero(const float* __restrict__ f, const float* __restrict__ dA,
                                                      float* __restrict__ u, RowsView rows) {
   uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  release_next();
   if (t >= rows.n) return;
   if (rows.list) t = __ldg(rows.list + t);
-  const float4 a = __ldg(reinterpret_cast<const float4*>(f) + t), d = __ldg(reinterpret_cast<const float4*>(dA) + t);
+  const float4 d = __ldg(reinterpret_cast<const float4*>(dA) + t);
+  wait_prior();
+  const float4 a = ld_prior(reinterpret_cast<const float4*>(f) + t);
   reinterpret_cast<float4*>(u)[t] = make_float4(a.x * d.x, a.y * d.y, a.z * d.z, a.w * d.w);
 }
 void launch_jacobi_zero32(const DenseView& L, const float* f, float* u, const RowsView& rows, cudaStream_t st) {
   if (rows.n == 0) return;
-  k_jacobi_zero<<<nblk(rows.n, 256), 256, 0, st>>>(f, L.dA, u, rows);
+  launch_pdl(k_jacobi_zero, nblk(rows.n, 256), 256, st, f, L.dA, u, rows);
   count_launch();
 }
 
@@ -600,10 +608,12 @@ __global__ void __launch_bounds__(256) k_transfer_dense(const float4* __restrict
                                                         const int32_t* __restrict__ bfwd,
                                                         const float* __restrict__ src, float* __restrict__ out) {
   const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  release_next();
   if (j >= n) return;
   const float4 r = __ldg(rec + j);
   const uint32_t d = __ldg(dst + j);
-  const float old = ADD ? out[d] : 0.f;
+  wait_prior();
+  const float old = ADD ? ld_prior(out + d) : 0.f;
   const uint32_t s = __float_as_uint(r.x);
   const int32_t b = (int32_t)(s >> (2 * DIM));
   const int x = s & 3, y = (s >> 2) & 3, z = DIM == 3 ? (s >> 4) & 3 : 0;
@@ -618,8 +628,8 @@ __global__ void __launch_bounds__(256) k_transfer_dense(const float4* __restrict
       const int row = ((y + bb) & 3) * 4 + (DIM == 3 ? ((z + c) & 3) * 16 : 0);
       const int32_t b0 = q ? __ldg(bfwd + 8 * (int64_t)b + q) : b;
       const int32_t b1 = x == 3 ? __ldg(bfwd + 8 * (int64_t)b + q + 1) : b0;
-      const float v0 = __ldg(src + ((size_t)b0 << (2 * DIM)) + row + x);
-      const float v1 = __ldg(src + ((size_t)b1 << (2 * DIM)) + row + ((x + 1) & 3));
+      const float v0 = ld_prior(src + ((size_t)b0 << (2 * DIM)) + row + x);
+      const float v1 = ld_prior(src + ((size_t)b1 << (2 * DIM)) + row + ((x + 1) & 3));
       accy += wy[bb] * (wx[0] * v0 + wx[1] * v1);
     }
     acc += (DIM == 3 ? wz[c] : 1.f) * accy;
@@ -633,11 +643,11 @@ void launch_transfer32(const DenseTransfer& T, const DenseView& source, const fl
   const float4* r = T.rec.get();
   const uint32_t* d = T.dst.get();
   if (source.dim == 3) {
-    if (add) k_transfer_dense<3, true><<<g, 256, 0, st>>>(r, d, T.n, source.bfwd, src, out);
-    else k_transfer_dense<3, false><<<g, 256, 0, st>>>(r, d, T.n, source.bfwd, src, out);
+    if (add) launch_pdl(k_transfer_dense<3, true>, g, 256, st, r, d, T.n, source.bfwd, src, out);
+    else launch_pdl(k_transfer_dense<3, false>, g, 256, st, r, d, T.n, source.bfwd, src, out);
   } else {
-    if (add) k_transfer_dense<2, true><<<g, 256, 0, st>>>(r, d, T.n, source.bfwd, src, out);
-    else k_transfer_dense<2, false><<<g, 256, 0, st>>>(r, d, T.n, source.bfwd, src, out);
+    if (add) launch_pdl(k_transfer_dense<2, true>, g, 256, st, r, d, T.n, source.bfwd, src, out);
+    else launch_pdl(k_transfer_dense<2, false>, g, 256, st, r, d, T.n, source.bfwd, src, out);
   }
   count_launch();
 }
@@ -647,11 +657,13 @@ template <int DIM>
 __global__ void __launch_bounds__(256) k_prolong_coarsest(TransferView<float> tv, const uint32_t* __restrict__ slot,
                                                           const float* __restrict__ src, float* __restrict__ out) {
   const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  release_next();
   if (j >= tv.n) return;
   const float sx = __ldg(tv.fr + j), sy = __ldg(tv.fr + tv.n + j);
   const float sz = DIM == 3 ? __ldg(tv.fr + 2 * (int64_t)tv.n + j) : 0.f;
   const float wx[2] = {1.f - sx, sx}, wy[2] = {1.f - sy, sy}, wz[2] = {1.f - sz, sz};
   const uint32_t d = __ldg(slot + j);
+  wait_prior();
   float acc = 0.f;
 #pragma unroll
   for (int c = 0; c < (DIM == 3 ? 2 : 1); ++c) {
@@ -659,19 +671,19 @@ __global__ void __launch_bounds__(256) k_prolong_coarsest(TransferView<float> tv
 #pragma unroll
     for (int bb = 0; bb < 2; ++bb) {
       const int q = 4 * c + 2 * bb;
-      const float v0 = __ldg(src + __ldg(tv.idx + (int64_t)q * tv.n + j));
-      const float v1 = __ldg(src + __ldg(tv.idx + (int64_t)(q + 1) * tv.n + j));
+      const float v0 = ld_prior(src + __ldg(tv.idx + (int64_t)q * tv.n + j));
+      const float v1 = ld_prior(src + __ldg(tv.idx + (int64_t)(q + 1) * tv.n + j));
       accy += wy[bb] * (wx[0] * v0 + wx[1] * v1);
     }
     acc += (DIM == 3 ? wz[c] : 1.f) * accy;
   }
-  out[d] += acc;
+  out[d] = ld_prior(out + d) + acc;
 }
 void launch_prolong_coarsest32(const TransferView<float>& tv, const uint32_t* slot, const float* src, float* out,
                                cudaStream_t st) {
   if (tv.n <= 0) return;
-  if (tv.dim == 3) k_prolong_coarsest<3><<<nblk(tv.n, 256), 256, 0, st>>>(tv, slot, src, out);
-  else k_prolong_coarsest<2><<<nblk(tv.n, 256), 256, 0, st>>>(tv, slot, src, out);
+  if (tv.dim == 3) launch_pdl(k_prolong_coarsest<3>, nblk(tv.n, 256), 256, st, tv, slot, src, out);
+  else launch_pdl(k_prolong_coarsest<2>, nblk(tv.n, 256), 256, st, tv, slot, src, out);
   count_launch();
 }
 

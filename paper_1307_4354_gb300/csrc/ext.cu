@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "ops.cuh"
+#include "pdl.cuh"
 #include "pair.cuh"
 
 namespace cpm {
@@ -427,7 +428,8 @@ __device__ __forceinline__ T stage_box(const LevelView<T>& L, const T* __restric
   constexpr int RS = TileBox<T, DIM, REL>::RS;
   load_box_bricks(L.tile_mask, L.tile_bstart, tile, sm.mask, sm.start);
   __syncthreads();
-  const T ref = REL ? __ldg(u + sm.start[0][0]) : T(0);
+  wait_prior();
+  const T ref = REL ? ld_prior(u + sm.start[0][0]) : T(0);
   BoxRow b;
   for (int r = threadIdx.x; box_row(sm.mask, sm.start, tbox, DIM, r, b); r += NT) {
     T v[7];
@@ -438,7 +440,7 @@ __device__ __forceinline__ T stage_box(const LevelView<T>& L, const T* __restric
       if (x <= b.xhi + 3) {
         const bool hi = x >= 4;
         if (((hi ? b.rbb : b.rba) >> (x & 3)) & 1u) {
-          v[i] = __ldg(u + (hi ? b.cb++ : b.ca++));
+          v[i] = ld_prior(u + (hi ? b.cb++ : b.ca++));
           if (REL) v[i] -= ref;
         }
       }
@@ -464,6 +466,7 @@ __global__ void __launch_bounds__(kExtThreads) k_extend_tiles(LevelView<T> L, co
   constexpr int RS = kRS;
   __shared__ TileBox<T, DIM, REL> sm;
   const int32_t tile = blockIdx.x;
+  release_next();
   const uint32_t tbox = __ldg(L.tile_box + tile);
   const int32_t beg = __ldg(L.tile_start + tile);
   const int32_t end = with_ghost ? __ldg(L.tile_start + tile + 1) : __ldg(L.tile_mid + tile);
@@ -517,10 +520,11 @@ __device__ __forceinline__ float stage_box_pair(const LevelView<double>& L, cons
   load_box_bricks(L.tile_mask, L.tile_bstart, tile, sm.mask, sm.start);
   if (threadIdx.x == 0) sm.dmax = 0u;
   __syncthreads();
+  wait_prior();
   // brick 0 holds the tile's stencil bases, which are band nodes (checked when
   // the band is built); the clamp only keeps the index inside B regardless
   const int32_t last = min(max(sm.start[0][1] + __popc(sm.mask[0][1]) - 1, 0), L.nB - 1);
-  const float ref = (float)__ldg(u + last);
+  const float ref = (float)ld_prior(u + last);
   const double refd = (double)ref;
   float amax = 0.f;
   BoxRow b;
@@ -533,7 +537,7 @@ __device__ __forceinline__ float stage_box_pair(const LevelView<double>& L, cons
       if (x <= b.xhi + 3) {
         const bool hi = x >= 4;
         if (((hi ? b.rbb : b.rba) >> (x & 3)) & 1u) {
-          const float2 d = pair_split(__ldg(u + (hi ? b.cb++ : b.ca++)) - refd);
+          const float2 d = pair_split(ld_prior(u + (hi ? b.cb++ : b.ca++)) - refd);
           vh[i] = d.x;
           vl[i] = d.y;
           amax = fmaxf(amax, fabsf(d.x));
@@ -609,6 +613,7 @@ __global__ void __launch_bounds__(kExtThreads) k_extend_pair(LevelView<double> L
                                                              float* __restrict__ refv, uint32_t* dmax) {
   __shared__ PairBox<DIM> sm;
   const int32_t tile = blockIdx.x;
+  release_next();
   const uint32_t tbox = __ldg(L.tile_box + tile);
   const int32_t beg = __ldg(L.tile_start + tile), end = __ldg(L.tile_start + tile + 1);
   if (beg == end) return;
@@ -646,9 +651,9 @@ void launch_extend(const LevelView<double>& L, const double* u, double* w, int32
   if (npts <= 0 || L.ntiles <= 0) return;
   const bool with_ghost = npts > L.nB;
   if (L.dim == 3)
-    k_extend_tiles<double, 3><<<L.ntiles, kExtThreads, 0, st>>>(L, u, w, with_ghost, nullptr);
+    launch_pdl(k_extend_tiles<double, 3>, L.ntiles, kExtThreads, st, L, u, w, with_ghost, (double*)nullptr);
   else
-    k_extend_tiles<double, 2><<<L.ntiles, kExtThreads, 0, st>>>(L, u, w, with_ghost, nullptr);
+    launch_pdl(k_extend_tiles<double, 2>, L.ntiles, kExtThreads, st, L, u, w, with_ghost, (double*)nullptr);
   count_launch();
 }
 
@@ -657,9 +662,9 @@ void launch_extend_rel(const LevelView<T>& L, const T* u, T* delta, T* refv, cud
   const int32_t nt = L.ntiles;
   if (nt <= 0) return;
   if (L.dim == 3)
-    k_extend_tiles<T, 3, true><<<nt, kExtThreads, 0, st>>>(L, u, delta, true, refv);
+    launch_pdl(k_extend_tiles<T, 3, true>, nt, kExtThreads, st, L, u, delta, true, refv);
   else
-    k_extend_tiles<T, 2, true><<<nt, kExtThreads, 0, st>>>(L, u, delta, true, refv);
+    launch_pdl(k_extend_tiles<T, 2, true>, nt, kExtThreads, st, L, u, delta, true, refv);
   count_launch();
 }
 __global__ void k_pair_weights(const double* w, float2* wp, int64_t n) {
@@ -680,9 +685,9 @@ void launch_extend_pair(const LevelView<double>& L, const double* u, float2* del
   if (nt <= 0) return;
   CPM_CHECK(L.ewp != nullptr, CPM_ERR_ARG, "pair weights not built");
   if (L.dim == 3)
-    k_extend_pair<3><<<nt, kExtThreads, 0, st>>>(L, u, delta, refv, dmax);
+    launch_pdl(k_extend_pair<3>, nt, kExtThreads, st, L, u, delta, refv, dmax);
   else
-    k_extend_pair<2><<<nt, kExtThreads, 0, st>>>(L, u, delta, refv, dmax);
+    launch_pdl(k_extend_pair<2>, nt, kExtThreads, st, L, u, delta, refv, dmax);
   count_launch();
 }
 

@@ -9,6 +9,8 @@
 #pragma once
 #include <cstdint>
 
+#include "pdl.cuh"
+
 namespace cpm {
 
 constexpr int kGemvWarps = 8;
@@ -32,6 +34,8 @@ __global__ void __launch_bounds__(kGemvWarps * 32) k_dense_gemv(const M* __restr
                                                                 GemvVectors<T> v, int32_t n) {
   constexpr int kChunk = (4096 / NV) / 32 * 32;  // a multiple of 32
   __shared__ M sb[NV][kChunk];
+  release_next();
+  wait_prior();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int32_t row0 = blockIdx.x * kGemvRowsPerBlock + warp * kGemvRowsPerWarp;
   const M* a[kGemvRowsPerWarp];
@@ -49,7 +53,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32) k_dense_gemv(const M* __restr
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < NV; ++q)
-      for (int32_t j = threadIdx.x; j < cn; j += blockDim.x) sb[q][j] = (M)v.b[q][c0 + j];
+      for (int32_t j = threadIdx.x; j < cn; j += blockDim.x) sb[q][j] = (M)ld_prior(v.b[q] + c0 + j);
     __syncthreads();
 #pragma unroll 2
     for (int32_t j = lane; j < cn; j += 32) {
@@ -72,7 +76,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32) k_dense_gemv(const M* __restr
       M s = acc[r][q];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0 && ok[r]) v.x[q][row0 + r] = ADD ? v.x[q][row0 + r] + (T)s : (T)s;
+      if (lane == 0 && ok[r]) v.x[q][row0 + r] = ADD ? ld_prior(v.x[q] + row0 + r) + (T)s : (T)s;
     }
   }
 }
@@ -88,6 +92,8 @@ __global__ void __launch_bounds__(kGemvWarps * 32) k_dense_gemv_v4(const float* 
                                                                    GemvVectors<T> v, int32_t n) {
   constexpr int kChunk = (4096 / NV) / 128 * 128;  // a multiple of 128 columns
   __shared__ __align__(16) float sb[NV][kChunk];
+  release_next();
+  wait_prior();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int32_t row0 = blockIdx.x * kGemvRowsPerBlock + warp * kGemvRowsPerWarp;
   const float* a[kGemvRowsPerWarp];
@@ -106,7 +112,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32) k_dense_gemv_v4(const float* 
 #pragma unroll
     for (int q = 0; q < NV; ++q)
       for (int32_t j = threadIdx.x; j < cn; j += blockDim.x)
-        sb[q][j] = c0 + j < n ? (float)v.b[q][c0 + j] : 0.f;
+        sb[q][j] = c0 + j < n ? (float)ld_prior(v.b[q] + c0 + j) : 0.f;
     __syncthreads();
 #pragma unroll 4
     for (int32_t j = 4 * lane; j < cn; j += 128) {
@@ -130,7 +136,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32) k_dense_gemv_v4(const float* 
       float s = acc[r][q];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0 && ok[r]) v.x[q][row0 + r] = ADD ? v.x[q][row0 + r] + (T)s : (T)s;
+      if (lane == 0 && ok[r]) v.x[q][row0 + r] = ADD ? ld_prior(v.x[q] + row0 + r) + (T)s : (T)s;
     }
   }
 }
@@ -152,10 +158,10 @@ void launch_dense_gemv(const M* A, const T* const* b, T* const* x, int G, int32_
     }
     const unsigned grid = dense_gemv_blocks(n);
     switch (nv) {
-      case 1: k_dense_gemv<M, T, ADD, 1><<<grid, kGemvWarps * 32, 0, st>>>(A, v, n); break;
-      case 2: k_dense_gemv<M, T, ADD, 2><<<grid, kGemvWarps * 32, 0, st>>>(A, v, n); break;
-      case 3: k_dense_gemv<M, T, ADD, 3><<<grid, kGemvWarps * 32, 0, st>>>(A, v, n); break;
-      default: k_dense_gemv<M, T, ADD, 4><<<grid, kGemvWarps * 32, 0, st>>>(A, v, n); break;
+      case 1: launch_pdl(k_dense_gemv<M, T, ADD, 1>, grid, kGemvWarps * 32, st, A, v, n); break;
+      case 2: launch_pdl(k_dense_gemv<M, T, ADD, 2>, grid, kGemvWarps * 32, st, A, v, n); break;
+      case 3: launch_pdl(k_dense_gemv<M, T, ADD, 3>, grid, kGemvWarps * 32, st, A, v, n); break;
+      default: launch_pdl(k_dense_gemv<M, T, ADD, 4>, grid, kGemvWarps * 32, st, A, v, n); break;
     }
   }
 }
@@ -173,10 +179,10 @@ void launch_dense_gemv_v4(const float* A, int32_t ld, const T* const* b, T* cons
     }
     const unsigned grid = dense_gemv_blocks(n);
     switch (nv) {
-      case 1: k_dense_gemv_v4<T, ADD, 1><<<grid, kGemvWarps * 32, 0, st>>>(A, ld, v, n); break;
-      case 2: k_dense_gemv_v4<T, ADD, 2><<<grid, kGemvWarps * 32, 0, st>>>(A, ld, v, n); break;
-      case 3: k_dense_gemv_v4<T, ADD, 3><<<grid, kGemvWarps * 32, 0, st>>>(A, ld, v, n); break;
-      default: k_dense_gemv_v4<T, ADD, 4><<<grid, kGemvWarps * 32, 0, st>>>(A, ld, v, n); break;
+      case 1: launch_pdl(k_dense_gemv_v4<T, ADD, 1>, grid, kGemvWarps * 32, st, A, ld, v, n); break;
+      case 2: launch_pdl(k_dense_gemv_v4<T, ADD, 2>, grid, kGemvWarps * 32, st, A, ld, v, n); break;
+      case 3: launch_pdl(k_dense_gemv_v4<T, ADD, 3>, grid, kGemvWarps * 32, st, A, ld, v, n); break;
+      default: launch_pdl(k_dense_gemv_v4<T, ADD, 4>, grid, kGemvWarps * 32, st, A, ld, v, n); break;
     }
   }
 }

@@ -9,6 +9,7 @@
 #include "ops.cuh"
 #include "gemv.cuh"
 #include "pair.cuh"
+#include "pdl.cuh"
 
 #include <atomic>
 
@@ -67,72 +68,9 @@ __device__ inline void block_max_sum(double m, double s, double* part) {
 }
 
 // ----------------------------------------------------------------- M stencil
-// Stencil passes on B, one warp per brick (lane l handles nodes l and l + 32
-// of the 4x4x4 brick; in 2-D lanes 0..15 the 16 nodes of a 4x4 brick).  The
-// Laplacian neighbours of a node are found by brick addressing: a neighbour
-// inside the brick is a local position of the same brick, one across a face
-// is a local position of the face-neighbour brick, and its index in B+ is
-// start + popcount of the occupancy mask below it (band mask first, then
-// ghost mask).  The brick tables are warp-uniform loads, so the pass reads
-// no per-point index table: per point only u, f, diag and w (and writes the
-// result).
-// Occupancy masks and starts of one slot of a brick record.
-struct SlotTab {
-  uint64_t bm, gm;
-  int32_t bs, gs;
-};
-template <bool BAND_ONLY>
-__device__ __forceinline__ SlotTab slot_tab(const BrickRec* R, int q) {
-  SlotTab t;
-  t.bm = __ldg(&R->bm[q]);
-  t.bs = __ldg(&R->bs[q]);
-  t.gm = BAND_ONLY ? 0ull : __ldg(&R->gm[q]);
-  t.gs = BAND_ONLY ? 0 : __ldg(&R->gs[q]);
-  return t;
-}
-// Index in B+ (or in B only) of local node l of a brick, -1 if absent.
-__device__ __forceinline__ int32_t tab_index(const SlotTab& t, int l, int32_t nB) {
-  const uint64_t bit = 1ull << l;
-  if (t.bm & bit) return t.bs + __popcll(t.bm & (bit - 1ull));
-  if (t.gm & bit) return nB + t.gs + __popcll(t.gm & (bit - 1ull));
-  return -1;
-}
-// The 2d neighbours (-x, +x, -y, +y, -z, +z) of local node l: inside the
-// brick (its own tables, already in registers) or across a face (the tables
-// of record slot q + 1, loaded only for nodes on that face).
-template <int DIM, bool BAND_ONLY>
-__device__ __forceinline__ void brick_neighbours(const BrickRec* R, const SlotTab& own, int l,
-                                                 int32_t nB, int32_t k[6]) {
-  const int x = l & 3, y = (l >> 2) & 3, z = l >> 4;
-  const int step[3] = {1, 4, 16};
-  const int pos[3] = {x, y, z};
-#pragma unroll
-  for (int q = 0; q < 2 * DIM; ++q) {
-    const int a = q >> 1;
-    const bool up = q & 1;
-    const bool face = up ? pos[a] == 3 : pos[a] == 0;
-    const int ln = face ? (up ? l - 3 * step[a] : l + 3 * step[a]) : (up ? l + step[a] : l - step[a]);
-    k[q] = tab_index(face ? slot_tab<BAND_ONLY>(R, q + 1) : own, ln, nB);
-  }
-}
-
-// Threads per brick of the stencil passes: 64 (one node each) or 32 (two).
-#ifndef CPM_LAP_TPB
-#define CPM_LAP_TPB 64
-#endif
-constexpr int kLapTPB = CPM_LAP_TPB;
-static_assert(kLapTPB == 32 || kLapTPB == 64, "threads per brick");
-
-// Stencil passes over the per-point neighbour table (1) or by brick
-// addressing (0).
-#ifndef CPM_LAP_INDEXED
-#define CPM_LAP_INDEXED 1
-#endif
-constexpr bool kLapIndexed = CPM_LAP_INDEXED != 0;
-
 template <typename T>
 static unsigned lap_grid(const LevelView<T>& L) {
-  return kLapIndexed ? nblk(L.nB, 256) : nblk((int64_t)L.bv.nbricks * kLapTPB, 256);
+  return nblk(L.nB, 256);
 }
 int lap_blocks_f64(const LevelView<double>& L) { return (int)lap_grid(L); }
 
@@ -145,89 +83,8 @@ int lap_blocks_f64(const LevelView<double>& L) { return (int)lap_grid(L); }
 //           dropped): out = u + omega (f - (cI - L_B) u) / (c + gamma), or
 //           out = f - (cI - L_B) u
 constexpr int LAP_RM_JAC = 8, LAP_RM_RES = 9, LAP_BAND = 10, LAP_VARD = 11;
-template <typename T, int DIM, int MODE>
-__global__ void __launch_bounds__(256) k_lap(LevelView<T> L, const T* u, const T* __restrict__ w,
-                                             const T* __restrict__ f, const T* __restrict__ cvec,
-                                             T cval, const T* __restrict__ dA, T omega, T* out,
-                                             T* u_inout, double* part, const T* __restrict__ refv) {
-  constexpr bool RM = MODE == LAP_RM_JAC || MODE == LAP_RM_RES || MODE == LAP_BAND || MODE == LAP_VARD;
-  const int32_t b = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) / kLapTPB);
-  const int lane = threadIdx.x % kLapTPB;
-  double rm = 0.0, rs = 0.0;
-  const BrickRec* R = L.bv.brec + (b < L.bv.nbricks ? b : 0);
-  const uint64_t bm = b < L.bv.nbricks ? __ldg(&R->bm[0]) : 0ull;
-  if (bm) {
-    const SlotTab own = slot_tab<RM>(R, 0);
-    const int32_t bs = own.bs;
-#pragma unroll
-    for (int h = 0; h < (DIM == 3 ? 64 / kLapTPB : 1); ++h) {
-      const int l = lane + kLapTPB * h;
-      if ((DIM == 2 && l >= 16) || !((bm >> l) & 1ull)) continue;
-      if ((MODE == LAP_JAC_RED || MODE == LAP_JAC_BLACK) &&
-          node_colour_local(l) != (MODE == LAP_JAC_BLACK ? 1 : 0))
-        continue;
-      const int32_t i = bs + __popcll(bm & ((1ull << l) - 1ull));
-      int32_t k[6];
-      brick_neighbours<DIM, RM>(R, own, l, L.nB, k);
-      const T ui = u[i];
-      if (MODE == LAP_VARD) {  // out = L~ u, refv = the diffusion coefficient a
-        const T ai = refv[i];
-        T s = T(0);
-#pragma unroll
-        for (int q = 0; q < 2 * DIM; ++q)
-          if (k[q] >= 0) s += (T(0.5) * (ai + refv[k[q]])) * (u[k[q]] - ui);
-        out[i] = s * L.inv_h2;
-        continue;
-      }
-      if (RM) {
-        T s = T(0);
-#pragma unroll
-        for (int q = 0; q < 2 * DIM; ++q)
-          if (k[q] >= 0) s += u[k[q]];
-        if (MODE == LAP_BAND) {  // out = L_B u
-          out[i] = s * L.inv_h2 - L.gamma * ui;
-          continue;
-        }
-        const T c = cvec ? cvec[i] : cval;
-        const T diag = c + L.gamma;
-        const T r = f[i] - diag * ui + s * L.inv_h2;
-        out[i] = MODE == LAP_RM_JAC ? ui + omega * r / diag : r;
-        continue;
-      }
-      const T wi = w[i];
-      T s = T(0), Mu;
-      if (MODE == LAP_RESID_REL || MODE == LAP_JAC_REL) {
-        const T ri = refv[i];
-#pragma unroll
-        for (int q = 0; q < 2 * DIM; ++q) {
-          const int32_t kk = k[q] < 0 ? i : k[q];
-          s += (refv[kk] - ri) + (w[kk] - wi);
-        }
-        Mu = s * L.inv_h2 + L.gamma * ((ri - ui) + wi);
-      } else {
-#pragma unroll
-        for (int q = 0; q < 2 * DIM; ++q) s += w[k[q] < 0 ? i : k[q]] - wi;
-        Mu = s * L.inv_h2 + L.gamma * (wi - ui);
-      }
-      if (MODE == LAP_APPLY) {
-        out[i] = Mu;
-      } else {
-        const T c = cvec ? cvec[i] : cval;
-        const T r = f[i] - c * ui + Mu;
-        if (MODE == LAP_RESID || MODE == LAP_RESID_REL) {
-          out[i] = r;
-          rm = fmax(rm, fabs((double)r));
-          rs += (double)r * (double)r;
-        } else {
-          u_inout[i] = ui + r * dA[i];
-        }
-      }
-    }
-  }
-  if ((MODE == LAP_RESID || MODE == LAP_RESID_REL) && part) block_max_sum(rm, rs, part);
-}
 
-// The same passes with one thread per band point and its 2d neighbours read
+// Stencil passes on B, one thread per band point, its 2d neighbours read
 // from the per-point index table (B+ indices, the node itself where a
 // neighbour is missing).  Ruuth-Merriman modes drop ghost neighbours.
 template <typename T, int DIM, int MODE>
@@ -237,6 +94,7 @@ __global__ void __launch_bounds__(256) k_lap_idx(LevelView<T> L, const T* u, con
                                                  T* u_inout, double* part, const T* __restrict__ refv) {
   constexpr bool RM = MODE == LAP_RM_JAC || MODE == LAP_RM_RES || MODE == LAP_BAND || MODE == LAP_VARD;
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  release_next();
   double rm = 0.0, rs = 0.0;
   bool active = i < L.nB;
   if (active && (MODE == LAP_JAC_RED || MODE == LAP_JAC_BLACK)) {
@@ -247,51 +105,52 @@ __global__ void __launch_bounds__(256) k_lap_idx(LevelView<T> L, const T* u, con
     int32_t k[6];
 #pragma unroll
     for (int q = 0; q < 2 * DIM; ++q) k[q] = __ldg(L.nbr + (int64_t)q * L.nB + i);
-    const T ui = u[i];
+    wait_prior();
+    const T ui = ld_prior(u + i);
     if (MODE == LAP_VARD) {  // out = L~ u, refv = the diffusion coefficient a
-      const T ai = refv[i];
+      const T ai = ld_prior(refv + i);
       T s = T(0);
 #pragma unroll
       for (int q = 0; q < 2 * DIM; ++q)
-        if (k[q] < L.nB && k[q] != i) s += (T(0.5) * (ai + refv[k[q]])) * (u[k[q]] - ui);
+        if (k[q] < L.nB && k[q] != i) s += (T(0.5) * (ai + ld_prior(refv + k[q]))) * (ld_prior(u + k[q]) - ui);
       out[i] = s * L.inv_h2;
     } else if (RM) {
       T s = T(0);
 #pragma unroll
       for (int q = 0; q < 2 * DIM; ++q)
-        if (k[q] < L.nB && k[q] != i) s += u[k[q]];
+        if (k[q] < L.nB && k[q] != i) s += ld_prior(u + k[q]);
       if (MODE == LAP_BAND) {
         out[i] = s * L.inv_h2 - L.gamma * ui;
       } else {
-        const T c = cvec ? cvec[i] : cval;
+        const T c = cvec ? __ldg(cvec + i) : cval;
         const T diag = c + L.gamma;
-        const T r = f[i] - diag * ui + s * L.inv_h2;
+        const T r = ld_prior(f + i) - diag * ui + s * L.inv_h2;
         out[i] = MODE == LAP_RM_JAC ? ui + omega * r / diag : r;
       }
     } else {
-      const T wi = w[i];
+      const T wi = ld_prior(w + i);
       T s = T(0), Mu;
       if (MODE == LAP_RESID_REL || MODE == LAP_JAC_REL) {
-        const T ri = refv[i];
+        const T ri = ld_prior(refv + i);
 #pragma unroll
-        for (int q = 0; q < 2 * DIM; ++q) s += (refv[k[q]] - ri) + (w[k[q]] - wi);
+        for (int q = 0; q < 2 * DIM; ++q) s += (ld_prior(refv + k[q]) - ri) + (ld_prior(w + k[q]) - wi);
         Mu = s * L.inv_h2 + L.gamma * ((ri - ui) + wi);
       } else {
 #pragma unroll
-        for (int q = 0; q < 2 * DIM; ++q) s += w[k[q]] - wi;
+        for (int q = 0; q < 2 * DIM; ++q) s += ld_prior(w + k[q]) - wi;
         Mu = s * L.inv_h2 + L.gamma * (wi - ui);
       }
       if (MODE == LAP_APPLY) {
         out[i] = Mu;
       } else {
-        const T c = cvec ? cvec[i] : cval;
-        const T r = f[i] - c * ui + Mu;
+        const T c = cvec ? __ldg(cvec + i) : cval;
+        const T r = ld_prior(f + i) - c * ui + Mu;
         if (MODE == LAP_RESID || MODE == LAP_RESID_REL) {
           out[i] = r;
           rm = fabs((double)r);
           rs = (double)r * (double)r;
         } else {
-          u_inout[i] = ui + r * dA[i];
+          u_inout[i] = ui + r * __ldg(dA + i);
         }
       }
     }
@@ -303,12 +162,8 @@ template <int DIM, int MODE, typename T>
 static void lap_dispatch(const LevelView<T>& L, const T* u, const T* w, const T* f, const T* cvec,
                          T cval, const T* dA, T omega, T* out, T* u_inout, double* part,
                          const T* refv, cudaStream_t st) {
-  if (kLapIndexed)
-    k_lap_idx<T, DIM, MODE><<<lap_grid(L), 256, 0, st>>>(L, u, w, f, cvec, cval, dA, omega, out,
-                                                          u_inout, part, refv);
-  else
-    k_lap<T, DIM, MODE><<<lap_grid(L), 256, 0, st>>>(L, u, w, f, cvec, cval, dA, omega, out, u_inout,
-                                                      part, refv);
+  launch_pdl(k_lap_idx<T, DIM, MODE>, lap_grid(L), 256, st, L, u, w, f, cvec, cval, dA, omega, out, u_inout, part,
+             refv);
   count_launch();
 }
 
@@ -362,6 +217,9 @@ void launch_resid_rel(const LevelView<double>& L, const double* u, const double*
 // on the bit patterns of |r|).  Each thread takes kPairPts points (strided by
 // the block), so the block's norm reduction is shared by several points.
 constexpr int kPairPts = 4;
+// Fewer points than fill the chip that way take one point per thread (circle,
+// 2912 points: 7.7 us with four in a row).
+constexpr int64_t kPairSmall = 152 * 1024;
 
 // Largest |x| and sum of x^2 over the block into part[2 b], part[2 b + 1];
 // m holds the bit pattern of a non-negative double (ordered as an integer).
@@ -392,7 +250,7 @@ __device__ inline void block_maxbits_sum(unsigned long long m, double s, double*
   }
 }
 
-template <int DIM>
+template <int DIM, int PTS>
 __global__ void __launch_bounds__(256) k_resid_pair(LevelView<double> L, const double* __restrict__ u,
                                                     const float2* __restrict__ dp,
                                                     const float* __restrict__ rp,
@@ -402,20 +260,22 @@ __global__ void __launch_bounds__(256) k_resid_pair(LevelView<double> L, const d
                                                     double* part) {
   unsigned long long rm = 0ull;
   double rs = 0.0;
+  release_next();
+  wait_prior();
 #pragma unroll
-  for (int j = 0; j < kPairPts; ++j) {
-    const int32_t i = (blockIdx.x * kPairPts + j) * blockDim.x + threadIdx.x;
+  for (int j = 0; j < PTS; ++j) {
+    const int32_t i = (blockIdx.x * PTS + j) * blockDim.x + threadIdx.x;
     if (i >= L.nB) continue;  // (not break: the points' loads can then overlap)
     int32_t k[2 * DIM];
 #pragma unroll
     for (int q = 0; q < 2 * DIM; ++q) k[q] = __ldg(L.nbr + (int64_t)q * L.nB + i);
-    const float ri = __ldg(rp + i);
-    const float2 di = __ldg(dp + i);
+    const float ri = ld_prior(rp + i);
+    const float2 di = ld_prior(dp + i);
     float sh = 0.f, sl = 0.f;
 #pragma unroll
     for (int q = 0; q < 2 * DIM; ++q) {
-      const float rk = __ldg(rp + k[q]);
-      const float2 dk = __ldg(dp + k[q]);
+      const float rk = ld_prior(rp + k[q]);
+      const float2 dk = ld_prior(dp + k[q]);
       float ah, al, bh, bl, ch, cl, t;
       two_sum(rk, -ri, ah, al);
       two_sum(dk.x, -di.x, bh, bl);
@@ -427,14 +287,14 @@ __global__ void __launch_bounds__(256) k_resid_pair(LevelView<double> L, const d
     float Sh, Sl, lh, ll;
     fast_two_sum(sh, sl, Sh, Sl);
     pair_mul(Sh, Sl, ih2.x, ih2.y, lh, ll);             // S / dx^2
-    const double ui = u[i];
+    const double ui = ld_prior(u + i);
     const float2 e = pair_split(pair_f2d(ri) - ui);      // ref_i - u_i
     float th, tl, gh, gl, mh, ml;
     pair_add(e.x, e.y, di.x, di.y, th, tl);
     pair_mul(th, tl, gam.x, gam.y, gh, gl);             // gamma ((ref_i - u_i) + delta_i)
     pair_add(lh, ll, gh, gl, mh, ml);                   // M u_i
-    const double c = cvec ? cvec[i] : cval;
-    const double res = (f[i] - c * ui) + pair_to_f64(mh, ml);
+    const double c = cvec ? __ldg(cvec + i) : cval;
+    const double res = (ld_prior(f + i) - c * ui) + pair_to_f64(mh, ml);
     r[i] = res;
     rm = max(rm, (unsigned long long)__double_as_longlong(res) & 0x7FFFFFFFFFFFFFFFull);  // |res|
     rs += res * res;
@@ -443,7 +303,8 @@ __global__ void __launch_bounds__(256) k_resid_pair(LevelView<double> L, const d
 }
 
 int resid_pair_blocks(const LevelView<double>& L) {
-  return (int)((L.nB + 256 * kPairPts - 1) / (256 * kPairPts));
+  const int pts = L.nB < kPairSmall ? 1 : kPairPts;
+  return (int)((L.nB + 256 * pts - 1) / (256 * pts));
 }
 
 void launch_resid_pair(const LevelView<double>& L, const double* u, const float2* delta,
@@ -455,10 +316,10 @@ void launch_resid_pair(const LevelView<double>& L, const double* u, const float2
   const float ih2h = (float)ih2, gamh = (float)gam;
   const float2 ih2p = make_float2(ih2h, (float)(ih2 - (double)ih2h));
   const float2 gamp = make_float2(gamh, (float)(gam - (double)gamh));
-  if (L.dim == 3)
-    k_resid_pair<3><<<nb, 256, 0, st>>>(L, u, delta, refv, f, cvec, cval, ih2p, gamp, r, part);
-  else
-    k_resid_pair<2><<<nb, 256, 0, st>>>(L, u, delta, refv, f, cvec, cval, ih2p, gamp, r, part);
+  const bool small = L.nB < kPairSmall;
+  auto kernel = L.dim == 3 ? (small ? k_resid_pair<3, 1> : k_resid_pair<3, kPairPts>)
+                           : (small ? k_resid_pair<2, 1> : k_resid_pair<2, kPairPts>);
+  launch_pdl(kernel, nb, 256, st, L, u, delta, refv, f, cvec, cval, ih2p, gamp, r, part);
   count_launch();
 }
 
@@ -682,6 +543,7 @@ template <typename T, int DIM>
 __global__ void __launch_bounds__(256) k_transfer(TransferView<T> tv, const T* __restrict__ src,
                                                   T* __restrict__ dst, bool add) {
   const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  release_next();
   if (j >= tv.n) return;
   const T sx = __ldg(tv.fr + j), sy = __ldg(tv.fr + tv.n + j);
   const T sz = DIM == 3 ? __ldg(tv.fr + 2 * tv.n + j) : T(0);
@@ -693,6 +555,7 @@ __global__ void __launch_bounds__(256) k_transfer(TransferView<T> tv, const T* _
     y = (int)((kb >> 16) & 0xffffu);
     z = (int)((kb >> 32) & 0xffffu);
   }
+  wait_prior();
   T acc = T(0);
 #pragma unroll
   for (int c = 0; c < (DIM == 3 ? 2 : 1); ++c) {
@@ -703,13 +566,13 @@ __global__ void __launch_bounds__(256) k_transfer(TransferView<T> tv, const T* _
       const int32_t i0 = tv.idx ? __ldg(tv.idx + (int64_t)q * tv.n + j) : band_index(tv.src, x, y + bb, z + c);
       const int32_t i1 = tv.idx ? __ldg(tv.idx + (int64_t)(q + 1) * tv.n + j)
                                 : band_index(tv.src, x + 1, y + bb, z + c);
-      const T v0 = __ldg(src + (i0 < 0 ? 0 : i0));
-      const T v1 = __ldg(src + (i1 < 0 ? 0 : i1));
+      const T v0 = ld_prior(src + (i0 < 0 ? 0 : i0));
+      const T v1 = ld_prior(src + (i1 < 0 ? 0 : i1));
       accy += wy[bb] * (wx[0] * v0 + wx[1] * v1);
     }
     acc += (DIM == 3 ? wz[c] : T(1)) * accy;
   }
-  dst[j] = add ? dst[j] + acc : acc;
+  dst[j] = add ? ld_prior(dst + j) + acc : acc;
 }
 
 // Cubic restriction / prolongation: degree-3 interpolation at the target's cp
@@ -752,8 +615,8 @@ void launch_transfer(const TransferView<T>& tv, const T* src, T* dst, bool add, 
     if (tv.dim == 3) k_transfer3<T, 3><<<nblk(tv.n, 256), 256, 0, st>>>(tv, src, dst, add);
     else k_transfer3<T, 2><<<nblk(tv.n, 256), 256, 0, st>>>(tv, src, dst, add);
   } else {
-    if (tv.dim == 3) k_transfer<T, 3><<<nblk(tv.n, 256), 256, 0, st>>>(tv, src, dst, add);
-    else k_transfer<T, 2><<<nblk(tv.n, 256), 256, 0, st>>>(tv, src, dst, add);
+    if (tv.dim == 3) launch_pdl(k_transfer<T, 3>, nblk(tv.n, 256), 256, st, tv, src, dst, add);
+    else launch_pdl(k_transfer<T, 2>, nblk(tv.n, 256), 256, st, tv, src, dst, add);
   }
   count_launch();
 }
@@ -780,41 +643,56 @@ void launch_norm_partials(const T* x, int64_t n, double* part, cudaStream_t st) 
 // out[0] = max|x|, out[1] = sum x^2, out[2] = 1 / max|x| (0 if max is 0);
 // out[3] = the largest of the kPairSlots float slots of dmax (non-negative,
 // compared as integers), which are reset to 0, or 0 without dmax.
-__global__ void k_norm_final(const double* part, int nblocks, double* out, uint32_t* dmax) {
-  __shared__ uint32_t dm;
-  if (threadIdx.x == 0) dm = 0u;
-  __syncthreads();
-  if (dmax) {
+__global__ void __launch_bounds__(1024) k_norm_final(const double* part, int nblocks, double* out, uint32_t* dmax) {
+  __shared__ double sm[32], ss[32];
+  __shared__ uint32_t sd[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  release_next();
+  wait_prior();
+  uint32_t dm = 0u;
+  if (dmax)
     for (int i = threadIdx.x; i < kPairSlots; i += blockDim.x) {
-      atomicMax(&dm, dmax[i]);
+      dm = max(dm, dmax[i]);
       dmax[i] = 0u;
     }
-  }
   double m = 0.0, s = 0.0;
   for (int i = threadIdx.x; i < nblocks; i += blockDim.x) {
-    m = fmax(m, part[2 * i]);
-    s += part[2 * i + 1];
+    m = fmax(m, ld_prior(part + 2 * i));
+    s += ld_prior(part + 2 * i + 1);
   }
-  __shared__ double sm[32], ss[32];
+#pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     s += __shfl_xor_sync(0xffffffffu, s, o);
   }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) { sm[wid] = m; ss[wid] = s; }
+  dm = __reduce_max_sync(0xffffffffu, dm);
+  if (lane == 0) {
+    sm[wid] = m;
+    ss[wid] = s;
+    sd[wid] = dm;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double M = 0.0, S = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) { M = fmax(M, sm[q]); S += ss[q]; }
-    out[0] = M;
-    out[1] = S;
-    out[2] = M > 0.0 ? 1.0 / M : 0.0;
-    out[3] = (double)__uint_as_float(dm);
+  if (wid == 0) {
+    const bool on = lane < (int)(blockDim.x >> 5);
+    m = on ? sm[lane] : 0.0;
+    s = on ? ss[lane] : 0.0;
+    dm = __reduce_max_sync(0xffffffffu, on ? sd[lane] : 0u);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+      s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    if (lane == 0) {
+      out[0] = m;
+      out[1] = s;
+      out[2] = m > 0.0 ? 1.0 / m : 0.0;
+      out[3] = (double)__uint_as_float(dm);
+    }
   }
 }
 
 void launch_norm_final(const double* part, int nblocks, double* out, cudaStream_t st, uint32_t* dmax) {
-  k_norm_final<<<1, 1024, 0, st>>>(part, nblocks, out, dmax);
+  launch_pdl(k_norm_final, 1, 1024, st, part, nblocks, out, dmax);
   count_launch();
 }
 
@@ -841,10 +719,12 @@ void launch_axpy_scaled(double* u, const float* d, const double* norms, int64_t 
 
 __global__ void k_axpy64(double* __restrict__ u, const double* __restrict__ d, int64_t n) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) u[i] += d[i];
+  release_next();
+  wait_prior();
+  if (i < n) u[i] = ld_prior(u + i) + ld_prior(d + i);
 }
 void launch_axpy64(double* u, const double* d, int64_t n, cudaStream_t st) {
-  k_axpy64<<<nblk(n, 256), 256, 0, st>>>(u, d, n);
+  launch_pdl(k_axpy64, nblk(n, 256), 256, st, u, d, n);
   count_launch();
 }
 

@@ -1,0 +1,59 @@
+// Programmatic dependent launch: a kernel launched with launch_pdl may start
+// while the kernel before it in the stream drains.  It reads its static inputs
+// (tables built with the hierarchy), then calls wait_prior() and only then
+// touches what earlier kernels wrote or still read.  Every kernel launched this
+// way calls wait_prior(), so that completion is transitive along the stream.
+// Values written by earlier kernels are read with ld_prior: a plain (coherent)
+// load that the compiler keeps behind the wait, which it need not do for
+// __ldg.  A V-cycle is some 80 kernels of 2 to 100 us, each of which otherwise
+// starts about 1 us after the one before it has ended.
+#pragma once
+
+#include "cpm_internal.cuh"
+
+namespace cpm {
+
+// Let the next kernel of the stream be scheduled as this one's blocks drain.
+__device__ __forceinline__ void release_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+// Wait until the kernels before this one are complete and their writes visible.
+__device__ __forceinline__ void wait_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ float ld_prior(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_prior(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_prior(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_prior(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p)
+               : "memory");
+  return v;
+}
+
+template <typename... P, typename... A>
+void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  CPM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
+}
+
+}  // namespace cpm
