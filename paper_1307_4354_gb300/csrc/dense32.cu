@@ -776,6 +776,38 @@ __global__ void k_row_emit(const uint64_t* mask, int64_t nrows, int per, const i
   if (t < nrows && ((mask[t / per] >> (4 * (t % per))) & 15ull)) rows[pos[t]] = (uint32_t)t;
 }
 
+// FP64 lists: flags of the marked points of B, flags of the kept E-order
+// positions, and their scatter.
+__global__ void k_list_flags(const uint32_t* slot, int32_t n, int dim, const uint64_t* mask, int64_t* flag) {
+  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const uint32_t s = slot[i];
+  flag[i] = (mask[s >> (2 * dim)] >> (s & ((1u << (2 * dim)) - 1u))) & 1ull;
+}
+__global__ void k_list_emit(const uint32_t* slot, int32_t n, int dim, const uint64_t* mask, const int64_t* pos,
+                            int32_t* list) {
+  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const uint32_t s = slot[i];
+  if ((mask[s >> (2 * dim)] >> (s & ((1u << (2 * dim)) - 1u))) & 1ull) list[pos[i]] = i;
+}
+__global__ void k_epos_flags(const uint32_t* erec, int64_t n, const uint8_t* keep, int64_t* flag) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n) flag[k] = keep[erec[k] >> 6];
+}
+__global__ void k_epos_emit(const uint32_t* erec, int64_t n, const uint8_t* keep, const int64_t* pos,
+                            uint32_t* epos) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n && keep[erec[k] >> 6]) epos[pos[k]] = (uint32_t)k;
+}
+__global__ void k_epos_starts(const int32_t* tile_start, int32_t ntiles, int64_t n, const int64_t* pos,
+                              int32_t total, int32_t* tstart) {
+  const int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t > ntiles) return;
+  const int32_t k = t < ntiles ? tile_start[t] : (int32_t)n;
+  tstart[t] = k < n ? (int32_t)pos[k] : total;
+}
+
 static void build_need(const Level& L, const Dense32& D, const uint64_t* mask, NeedSet& S, cudaStream_t st) {
   DBuf<uint8_t> keep(L.nplus());
   k_keep_near<<<nblk(L.nplus(), 256), 256, 0, st>>>(L.view(), L.key.get(), L.nplus(), L.dim, mask, keep.get());
@@ -788,6 +820,20 @@ static void build_need(const Level& L, const Dense32& D, const uint64_t* mask, N
   S.nrows = (int32_t)scan_exclusive_i64(pos.get(), nrows, st);
   S.rows.alloc((size_t)S.nrows);
   k_row_emit<<<nblk(nrows, 256), 256, 0, st>>>(mask, nrows, per, pos.get(), S.rows.get());
+  CPM_CUDA_TRY(cudaGetLastError());
+  const int64_t np = L.nplus();
+  DBuf<int64_t> lpos(np);
+  k_list_flags<<<nblk(L.nB, 256), 256, 0, st>>>(D.slot.get(), L.nB, L.dim, mask, lpos.get());
+  S.nlist = (int32_t)scan_exclusive_i64(lpos.get(), L.nB, st);
+  S.list.alloc((size_t)S.nlist);
+  k_list_emit<<<nblk(L.nB, 256), 256, 0, st>>>(D.slot.get(), L.nB, L.dim, mask, lpos.get(), S.list.get());
+  k_epos_flags<<<nblk(np, 256), 256, 0, st>>>(L.erec.get(), np, keep.get(), lpos.get());
+  const int32_t ne = (int32_t)scan_exclusive_i64(lpos.get(), np, st);
+  S.epos.alloc((size_t)ne);
+  S.tstart.alloc((size_t)L.ntiles + 1);
+  k_epos_emit<<<nblk(np, 256), 256, 0, st>>>(L.erec.get(), np, keep.get(), lpos.get(), S.epos.get());
+  k_epos_starts<<<nblk(L.ntiles + 1, 256), 256, 0, st>>>(L.tile_start.get(), L.ntiles, np, lpos.get(), ne,
+                                                         S.tstart.get());
   CPM_CUDA_TRY(cudaGetLastError());
   CPM_CUDA_TRY(cudaStreamSynchronize(st));  // the scratch arrays go out of scope
 }

@@ -61,6 +61,10 @@ struct NeedSet {
   ExtUnits units;
   DBuf<uint32_t> rows;
   int32_t nrows = 0;
+  // the same for FP64 passes in band order (PointSet)
+  DBuf<int32_t> list, tstart;
+  DBuf<uint32_t> epos;
+  int32_t nlist = 0;
 };
 // Brick-dense structures of one level.
 struct Dense32 {
@@ -89,6 +93,7 @@ struct DenseTransfer {
   int32_t n = 0;
 };
 UnitsView units_view(const ExtUnits& U);
+inline PointSet point_set(const NeedSet& S) { return {S.list.get(), S.nlist, S.tstart.get(), S.epos.get()}; }
 inline RowsView rows_view(const NeedSet& S) { return {S.rows.get(), (uint32_t)S.nrows}; }
 inline RowsView all_rows(const DenseView& L) { return {nullptr, (uint32_t)L.nbricks << (2 * (L.dim - 1))}; }
 // D.resid from the cells of the restriction to the next level; D.sweep too where

@@ -462,32 +462,37 @@ __device__ __forceinline__ T stage_box(const LevelView<T>& L, const T* __restric
 template <typename T, int DIM, bool REL = false>
 __global__ void __launch_bounds__(kExtThreads) k_extend_tiles(LevelView<T> L, const T* __restrict__ u,
                                                               T* __restrict__ w, bool with_ghost,
-                                                              T* __restrict__ refv) {
+                                                              T* __restrict__ refv, const int32_t* tstart,
+                                                              const uint32_t* epos) {
   constexpr int RS = kRS;
   __shared__ TileBox<T, DIM, REL> sm;
   const int32_t tile = blockIdx.x;
   release_next();
   const uint32_t tbox = __ldg(L.tile_box + tile);
-  const int32_t beg = __ldg(L.tile_start + tile);
-  const int32_t end = with_ghost ? __ldg(L.tile_start + tile + 1) : __ldg(L.tile_mid + tile);
-  if (beg == end) return;  // a tile of ghost points only, extension over B
+  // the tile's points: its range of the E order, or of a list of E-order positions
+  const int32_t beg = __ldg((tstart ? tstart : L.tile_start) + tile);
+  const int32_t end = tstart ? __ldg(tstart + tile + 1)
+                      : with_ghost ? __ldg(L.tile_start + tile + 1) : __ldg(L.tile_mid + tile);
+  if (beg == end) return;  // no point of the set in this tile
   // this thread's first point: issue its record loads before staging
-  int32_t k = beg + threadIdx.x;
+  int32_t q = beg + threadIdx.x;
   uint32_t rec = 0;
   PointWeights<T, DIM> pw;
-  if (k < end) {
+  if (q < end) {
+    const int32_t k = tstart ? (int32_t)__ldg(epos + q) : q;
     rec = __ldg(L.erec + k);
     pw.load(L, k);
   }
   const T ref = stage_box<T, DIM, REL, kExtThreads>(L, u, tile, tbox, sm);
-  for (; k < end; k += kExtThreads) {
+  for (; q < end; q += kExtThreads) {
     const T* base = sm.win + ((rec >> 4) & 3) * 7 * RS + ((rec >> 2) & 3) * RS + (rec & 3) * 4;
     w[rec >> 6] = contract<DIM>(base, pw);
     if (REL) refv[rec >> 6] = ref;
-    const int32_t kn = k + kExtThreads;
-    if (kn < end) {
-      rec = __ldg(L.erec + kn);
-      pw.load(L, kn);
+    const int32_t qn = q + kExtThreads;
+    if (qn < end) {
+      const int32_t k = tstart ? (int32_t)__ldg(epos + qn) : qn;
+      rec = __ldg(L.erec + k);
+      pw.load(L, k);
     }
   }
 }
@@ -651,9 +656,18 @@ void launch_extend(const LevelView<double>& L, const double* u, double* w, int32
   if (npts <= 0 || L.ntiles <= 0) return;
   const bool with_ghost = npts > L.nB;
   if (L.dim == 3)
-    launch_pdl(k_extend_tiles<double, 3>, L.ntiles, kExtThreads, st, L, u, w, with_ghost, (double*)nullptr);
+    launch_pdl(k_extend_tiles<double, 3>, L.ntiles, kExtThreads, st, L, u, w, with_ghost, (double*)nullptr,
+               (const int32_t*)nullptr, (const uint32_t*)nullptr);
   else
-    launch_pdl(k_extend_tiles<double, 2>, L.ntiles, kExtThreads, st, L, u, w, with_ghost, (double*)nullptr);
+    launch_pdl(k_extend_tiles<double, 2>, L.ntiles, kExtThreads, st, L, u, w, with_ghost, (double*)nullptr,
+               (const int32_t*)nullptr, (const uint32_t*)nullptr);
+  count_launch();
+}
+
+void launch_extend_set(const LevelView<double>& L, const PointSet& S, const double* u, double* w, cudaStream_t st) {
+  if (L.ntiles <= 0) return;
+  auto kernel = L.dim == 3 ? k_extend_tiles<double, 3> : k_extend_tiles<double, 2>;
+  launch_pdl(kernel, L.ntiles, kExtThreads, st, L, u, w, true, (double*)nullptr, S.tstart, S.epos);
   count_launch();
 }
 
@@ -662,9 +676,11 @@ void launch_extend_rel(const LevelView<T>& L, const T* u, T* delta, T* refv, cud
   const int32_t nt = L.ntiles;
   if (nt <= 0) return;
   if (L.dim == 3)
-    launch_pdl(k_extend_tiles<T, 3, true>, nt, kExtThreads, st, L, u, delta, true, refv);
+    launch_pdl(k_extend_tiles<T, 3, true>, nt, kExtThreads, st, L, u, delta, true, refv, (const int32_t*)nullptr,
+               (const uint32_t*)nullptr);
   else
-    launch_pdl(k_extend_tiles<T, 2, true>, nt, kExtThreads, st, L, u, delta, true, refv);
+    launch_pdl(k_extend_tiles<T, 2, true>, nt, kExtThreads, st, L, u, delta, true, refv, (const int32_t*)nullptr,
+               (const uint32_t*)nullptr);
   count_launch();
 }
 __global__ void k_pair_weights(const double* w, float2* wp, int64_t n) {

@@ -426,6 +426,26 @@ static void smooth32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* 
   }
 }
 
+// The same in FP64, band order: sweeps on the points of `need` only, if given,
+// from u = 0 if zero.
+static void sweeps64(cpm_hier_s* H, Workspace& W, int l, const double* f, double* u, int sweeps, bool zero,
+                     const NeedSet* need, cudaStream_t st) {
+  HLevel& lv = H->L[l];
+  const LevelView<double> v = lv.view<double>();
+  const PointSet set = need ? point_set(*need) : PointSet{};
+  double* w = W.w64[l].w.get();
+  for (int s = 0; s < sweeps; ++s) {
+    if (zero && s == 0) {
+      launch_jacobi_zero(v, need ? &set : nullptr, f, lv.dA64.get(), u, st);
+    } else if (need) {
+      launch_extend_set(v, set, u, w, st);
+      launch_lap_set(v, LAP_JACOBI, set, u, w, f, lv.c64.get(), H->c, lv.dA64.get(), nullptr, u, st);
+    } else {
+      mbr_op(H, W, l, LAP_JACOBI, f, u, nullptr, lv.dA64.get(), u, nullptr, st);
+    }
+  }
+}
+
 template <typename T>
 static void smooth(cpm_hier_s* H, Workspace& W, int l, const T* f, T* u, int sweeps,
                    cudaStream_t st) {
@@ -634,6 +654,45 @@ static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const flo
   }
 }
 
+// FP64 V-cycle of the same options, band order.  zero: u[g] is to be taken as 0
+// (it need not be set).
+static void vcycle64(cpm_hier_s* H, Workspace* const* W, int G, int l, const double* const* f, double* const* u,
+                     bool zero, cudaStream_t st) {
+  const int nl = (int)H->L.size();
+  HLevel& lv = H->L[l];
+  const LevelView<double> v = lv.view<double>();
+  const bool last = l + 1 == nl - 1;
+  const NeedSet* need = l > 0 ? &lv.dense.sweep : nullptr;
+  const PointSet rset = point_set(lv.dense.resid);
+  const double* cf[kMaxGroup];
+  double* cu[kMaxGroup];
+  for (int g = 0; g < G; ++g) {
+    Work<double>& w = W[g]->w64[l];
+    if (zero && H->opts.nu1 == 0) CPM_CUDA_TRY(cudaMemsetAsync(u[g], 0, sizeof(double) * v.nB, st));
+    sweeps64(H, *W[g], l, f[g], u[g], H->opts.nu1, zero, need, st);
+    const double* uu = u[g];
+    if (H->opts.residual_mode == 0) {  // the residual of E u
+      if (need) launch_extend_set(v, point_set(*need), u[g], w.tmp.get(), st);
+      else launch_extend(v, u[g], w.tmp.get(), v.nB, st);
+      uu = w.tmp.get();
+    }
+    launch_extend_set(v, rset, uu, w.w.get(), st);
+    launch_lap_set(v, LAP_RESID, rset, uu, w.w.get(), f[g], lv.c64.get(), H->c, nullptr, w.r.get(), nullptr, st);
+    Work<double>& cw = W[g]->w64[l + 1];
+    launch_transfer<double>(tview<double>(lv.R, v.dim), w.r.get(), cw.f.get(), false, st);
+    cf[g] = cw.f.get();
+    cu[g] = cw.u.get();
+  }
+  if (last)
+    coarse_solve<double>(H, W, G, cf, cu, st);
+  else
+    for (int q = 0; q < H->opts.cycle; ++q) vcycle64(H, W, G, l + 1, cf, cu, q == 0, st);
+  for (int g = 0; g < G; ++g) {
+    launch_transfer<double>(tview<double>(lv.P, v.dim), cu[g], u[g], true, st);
+    sweeps64(H, *W[g], l, f[g], u[g], H->opts.nu2, false, need, st);
+  }
+}
+
 // V-cycle of Algorithm 4.1 from level l for G systems in lockstep.
 template <typename T>
 static void vcycle_level(cpm_hier_s* H, Workspace* const* W, int G, int l, const T* const* f,
@@ -643,11 +702,10 @@ static void vcycle_level(cpm_hier_s* H, Workspace* const* W, int G, int l, const
     coarse_solve<T>(H, W, G, f, u, st);
     return;
   }
-  if constexpr (sizeof(T) == 4) {
-    if (H->dense_cycle && l == 0) {
-      vcycle32(H, W, G, 0, f, u, State32::compact, true, st);
-      return;
-    }
+  if (H->dense_cycle && l == 0) {
+    if constexpr (sizeof(T) == 4) vcycle32(H, W, G, 0, f, u, State32::compact, true, st);
+    else vcycle64(H, W, G, 0, f, u, false, st);
+    return;
   }
   HLevel& lv = H->L[l];
   HLevel& cv = H->L[l + 1];
@@ -747,12 +805,15 @@ static void outer_step(cpm_hier_s* H, Workspace* const* W, int G, int mode, int 
   if (mode == CPM_SOLVE_F64) {
     const double* r[kMaxGroup];
     double* d[kMaxGroup];
+    const bool zero_start = H->dense_cycle && !first_fmg;
     for (int g = 0; g < G; ++g) {
-      CPM_CUDA_TRY(cudaMemsetAsync(W[g]->d64.get(), 0, sizeof(double) * nB, st));
+      if (!zero_start) CPM_CUDA_TRY(cudaMemsetAsync(W[g]->d64.get(), 0, sizeof(double) * nB, st));
       r[g] = W[g]->r64.get();
       d[g] = W[g]->d64.get();
     }
-    if (first_fmg)
+    if (zero_start)
+      vcycle64(H, W, G, 0, r, d, true, st);
+    else if (first_fmg)
       for (int g = 0; g < G; ++g) fmg<double>(H, *W[g], r[g], d[g], st);
     else
       vcycle_level<double>(H, W, G, 0, r, d, st);

@@ -91,12 +91,14 @@ template <typename T, int DIM, int MODE>
 __global__ void __launch_bounds__(256) k_lap_idx(LevelView<T> L, const T* u, const T* __restrict__ w,
                                                  const T* __restrict__ f, const T* __restrict__ cvec,
                                                  T cval, const T* __restrict__ dA, T omega, T* out,
-                                                 T* u_inout, double* part, const T* __restrict__ refv) {
+                                                 T* u_inout, double* part, const T* __restrict__ refv,
+                                                 const int32_t* __restrict__ list, int32_t nlist) {
   constexpr bool RM = MODE == LAP_RM_JAC || MODE == LAP_RM_RES || MODE == LAP_BAND || MODE == LAP_VARD;
-  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   release_next();
   double rm = 0.0, rs = 0.0;
-  bool active = i < L.nB;
+  bool active = i < (list ? nlist : L.nB);
+  if (list && active) i = __ldg(list + i);
   if (active && (MODE == LAP_JAC_RED || MODE == LAP_JAC_BLACK)) {
     const uint64_t kk = __ldg(L.key + i);
     active = ((key_x(kk) + key_y(kk) + (DIM == 3 ? key_z(kk) : 0)) & 1) == (MODE == LAP_JAC_BLACK ? 1 : 0);
@@ -163,7 +165,7 @@ static void lap_dispatch(const LevelView<T>& L, const T* u, const T* w, const T*
                          T cval, const T* dA, T omega, T* out, T* u_inout, double* part,
                          const T* refv, cudaStream_t st) {
   launch_pdl(k_lap_idx<T, DIM, MODE>, lap_grid(L), 256, st, L, u, w, f, cvec, cval, dA, omega, out, u_inout, part,
-             refv);
+             refv, (const int32_t*)nullptr, 0);
   count_launch();
 }
 
@@ -188,6 +190,41 @@ void launch_lap(const LevelView<double>& L, LapMode mode, const double* u, const
   if (mode == LAP_JACOBI) lap_dim<LAP_JACOBI>(L, u, w, f, cvec, cval, dA, omega, out, u_inout, part, (const T*)nullptr, st);
   if (mode == LAP_JAC_RED) lap_dim<LAP_JAC_RED>(L, u, w, f, cvec, cval, dA, omega, out, u_inout, part, (const T*)nullptr, st);
   if (mode == LAP_JAC_BLACK) lap_dim<LAP_JAC_BLACK>(L, u, w, f, cvec, cval, dA, omega, out, u_inout, part, (const T*)nullptr, st);
+}
+
+template <int MODE>
+static void lap_set(const LevelView<double>& L, const PointSet& S, const double* u, const double* w,
+                    const double* f, const double* cvec, double cval, const double* dA, double* out,
+                    double* u_inout, cudaStream_t st) {
+  if (S.n <= 0) return;
+  auto kernel = L.dim == 3 ? k_lap_idx<double, 3, MODE> : k_lap_idx<double, 2, MODE>;
+  launch_pdl(kernel, nblk(S.n, 256), 256, st, L, u, w, f, cvec, cval, dA, 0.0, out, u_inout, (double*)nullptr,
+             (const double*)nullptr, S.list, S.n);
+  count_launch();
+}
+void launch_lap_set(const LevelView<double>& L, LapMode mode, const PointSet& S, const double* u, const double* w,
+                    const double* f, const double* cvec, double cval, const double* dA, double* out,
+                    double* u_inout, cudaStream_t st) {
+  if (mode == LAP_RESID) lap_set<LAP_RESID>(L, S, u, w, f, cvec, cval, dA, out, u_inout, st);
+  else lap_set<LAP_JACOBI>(L, S, u, w, f, cvec, cval, dA, out, u_inout, st);
+}
+
+__global__ void __launch_bounds__(256) k_jacobi_zero64(const double* __restrict__ f, const double* __restrict__ dA,
+                                                       const int32_t* __restrict__ list, int32_t n, double* u) {
+  int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  release_next();
+  if (i >= n) return;
+  if (list) i = __ldg(list + i);
+  const double d = __ldg(dA + i);
+  wait_prior();
+  u[i] = ld_prior(f + i) * d;
+}
+void launch_jacobi_zero(const LevelView<double>& L, const PointSet* S, const double* f, const double* dA, double* u,
+                        cudaStream_t st) {
+  const int32_t n = S ? S->n : L.nB;
+  if (n <= 0) return;
+  launch_pdl(k_jacobi_zero64, nblk(n, 256), 256, st, f, dA, S ? S->list : (const int32_t*)nullptr, n, u);
+  count_launch();
 }
 
 template <typename T>

@@ -32,6 +32,16 @@ struct LevelView {
   const int32_t* nbr;   // 2d x nB neighbour indices into B+
 };
 
+// A set of points that a pass visits (FP64, see the needed points in
+// dense32.cu): band indices for the stencil, and per extension tile a range of
+// E-order positions.
+struct PointSet {
+  const int32_t* list;    // band indices
+  int32_t n;
+  const int32_t* tstart;  // ntiles + 1 offsets into epos
+  const uint32_t* epos;   // E-order positions
+};
+
 // Transfer records: for each target point, the base node of its linear
 // (2^d) or cubic (4^d) stencil in the source grid (packed x | y << 16 | z << 32)
 // and the fractions (SoA, d x n).  The stencil nodes are located through the source
@@ -58,6 +68,8 @@ __host__ __device__ inline int node_colour_local(int l) { return ((l & 3) + ((l 
 // w = E u on the first npts points of B+ (npts = nB or nB + nG), FP64 (the FP32
 // extension is in dense32.cuh).
 void launch_extend(const LevelView<double>& L, const double* u, double* w, int32_t npts, cudaStream_t st);
+// w = E u at the points of S only.
+void launch_extend_set(const LevelView<double>& L, const PointSet& S, const double* u, double* w, cudaStream_t st);
 
 // Extension over B+ in relative form: delta_j = (E u)_j - ref_j with
 // ref_j = u at a reference node of j's tile (see k_extend_tiles).
@@ -86,6 +98,13 @@ void launch_resid_rel(const LevelView<double>& L, const double* u, const double*
 void launch_lap(const LevelView<double>& L, LapMode mode, const double* u, const double* w,
                 const double* f, const double* cvec, double cval, const double* dA, double omega,
                 double* out, double* u_inout, double* part, int nblocks_part, cudaStream_t st);
+// The RESID or JACOBI pass at the points of S only (no norm partials).
+void launch_lap_set(const LevelView<double>& L, LapMode mode, const PointSet& S, const double* u, const double* w,
+                    const double* f, const double* cvec, double cval, const double* dA, double* out,
+                    double* u_inout, cudaStream_t st);
+// u = f dA, the first Jacobi sweep from u = 0 (S null: every point of B).
+void launch_jacobi_zero(const LevelView<double>& L, const PointSet* S, const double* f, const double* dA, double* u,
+                        cudaStream_t st);
 
 // Number of blocks (2 partial doubles each) of a RESID / RESID_REL stencil pass.
 int lap_blocks_f64(const LevelView<double>& L);
