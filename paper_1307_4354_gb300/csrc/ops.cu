@@ -995,108 +995,6 @@ template void launch_assemble_A<double>(const LevelView<double>&, const double*,
 template void launch_assemble_A<float>(const LevelView<double>&, const double*, double, float*,
                                        cudaStream_t);
 
-// ----------------------------------------------------------------- setup: inverse
-// Gauss-Jordan with partial pivoting, in place: at step k the pivot row p
-// (max |A[i][k]|, i >= k) is swapped into row k, row k is scaled by the
-// reciprocal pivot (with A[k][k] replaced by 1 first), and every other row i
-// subtracts A[i][k] times row k (with A[i][k] replaced by 0 first).  Row
-// swaps permute the columns of the computed inverse; they are undone at the
-// end in reverse order.
-__global__ void k_gj_pivot(const double* A, int32_t n, int32_t k, int32_t* piv, int32_t* err) {
-  double best = -1.0;
-  int32_t arg = k;
-  for (int32_t i = k + threadIdx.x; i < n; i += blockDim.x) {
-    const double v = fabs(A[(size_t)i * n + k]);
-    if (v > best) { best = v; arg = i; }
-  }
-  __shared__ double sv[1024];
-  __shared__ int32_t si[1024];
-  sv[threadIdx.x] = best;
-  si[threadIdx.x] = arg;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      const double o = sv[threadIdx.x + s];
-      const int32_t oi = si[threadIdx.x + s];
-      if (o > sv[threadIdx.x] || (o == sv[threadIdx.x] && oi < si[threadIdx.x])) {
-        sv[threadIdx.x] = o;
-        si[threadIdx.x] = oi;
-      }
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    piv[k] = si[0];
-    if (!(sv[0] > 1e-300)) atomicOr(err, 1);
-  }
-}
-
-__global__ void k_gj_swap_scale(double* A, int32_t n, int32_t k, const int32_t* piv, double* col) {
-  const int32_t p = piv[k];
-  double* rk = A + (size_t)k * n;
-  if (p != k) {
-    double* rp = A + (size_t)p * n;
-    for (int32_t j = threadIdx.x; j < n; j += blockDim.x) {
-      const double t = rk[j];
-      rk[j] = rp[j];
-      rp[j] = t;
-    }
-    __syncthreads();
-  }
-  __shared__ double pivinv;
-  if (threadIdx.x == 0) {
-    const double a = rk[k];
-    pivinv = a != 0.0 ? 1.0 / a : 0.0;
-    rk[k] = 1.0;
-  }
-  __syncthreads();
-  for (int32_t j = threadIdx.x; j < n; j += blockDim.x) rk[j] *= pivinv;
-  (void)col;
-}
-
-__global__ void k_gj_save_col(const double* A, int32_t n, int32_t k, double* col) {
-  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) col[i] = A[(size_t)i * n + k];
-}
-
-__global__ void k_gj_eliminate(double* A, int32_t n, int32_t k, const double* __restrict__ col) {
-  const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int32_t i = blockIdx.y;
-  if (j >= n || i == k) return;
-  const double m = col[i];
-  if (m == 0.0) return;
-  const double akj = A[(size_t)k * n + j];
-  double* aij = A + (size_t)i * n + j;
-  *aij = (j == k ? 0.0 : *aij) - m * akj;
-}
-
-__global__ void k_gj_swap_cols(double* A, int32_t n, int32_t k, const int32_t* piv) {
-  const int32_t p = piv[k];
-  if (p == k) return;
-  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double* r = A + (size_t)i * n;
-  const double t = r[k];
-  r[k] = r[p];
-  r[p] = t;
-}
-
-void invert_dense(double* A, int32_t n, cudaStream_t st, int32_t* err) {
-  DBuf<int32_t> piv(n);
-  DBuf<double> col(n);
-  const dim3 eg(nblk(n, 256), n);
-  for (int32_t k = 0; k < n; ++k) {
-    k_gj_pivot<<<1, 1024, 0, st>>>(A, n, k, piv.get(), err);
-    k_gj_swap_scale<<<1, 1024, 0, st>>>(A, n, k, piv.get(), col.get());
-    k_gj_save_col<<<nblk(n, 256), 256, 0, st>>>(A, n, k, col.get());
-    k_gj_eliminate<<<eg, 256, 0, st>>>(A, n, k, col.get());
-  }
-  for (int32_t k = n - 1; k >= 0; --k)
-    k_gj_swap_cols<<<nblk(n, 256), 256, 0, st>>>(A, n, k, piv.get());
-  CPM_CUDA_TRY(cudaGetLastError());
-  CPM_CUDA_TRY(cudaStreamSynchronize(st));
-}
-
 // ----------------------------------------------------------------- instantiations
 #define CPM_INST(T)                                                                              \
   template void launch_rm_jacobi<T>(const LevelView<T>&, const T*, const T*, const T*, T, T, T*, \
