@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(kExtThreads) k_extend_pair(LevelView<double> L
     load_w(k);
   }
   const float ref = stage_box_pair<DIM>(L, u, tile, tbox, sm);
-  if (threadIdx.x == 0) atomicMax(dmax + (tile & (kPairSlots - 1)), sm.dmax);
+  if (threadIdx.x == 0 && dmax) atomicMax(dmax + (tile & (kPairSlots - 1)), sm.dmax);
   for (; k < end; k += kExtThreads) {
     const int o = ((rec >> 4) & 3) * 7 * kRS + ((rec >> 2) & 3) * kRS + (rec & 3) * 4;
     float dh, dl;

@@ -773,28 +773,29 @@ static void fmg(cpm_hier_s* H, Workspace& W, const T* f, T* u, cudaStream_t st) 
   }
 }
 
-// Outer residual r = f - A u on the finest level with norms into W.norms, in
+// Outer residual r = f - A u on the finest level with norms into W.norms (if wanted), in
 // the relative form (differences formed from exact inputs; its rounding floor
 // is far below that of w = E u followed by the stencil at fine dx), evaluated
 // in FP32 pairs on the FP32 pipe (default) or in FP64.
 static void outer_residual(cpm_hier_s* H, Workspace& W, const double* f, const double* u, double* r,
-                           cudaStream_t st, bool pair) {
+                           cudaStream_t st, bool pair, bool norms = true) {
   HLevel& lv = H->L[0];
   const LevelView<double> v = lv.view<double>();
+  double* part = norms ? W.part.get() : nullptr;
   if (H->opts.op_form != CPM_OP_MBR) {  // direct form of Eq. 3.3
-    level_op<double>(H, W, 0, LAP_RESID, f, u, r, W.part.get(), st);
-    launch_norm_final(W.part.get(), paper_blocks(v), W.norms, st);
+    level_op<double>(H, W, 0, LAP_RESID, f, u, r, part, st);
+    if (norms) launch_norm_final(W.part.get(), paper_blocks(v), W.norms, st);
     return;
   }
   if (pair && H->pair_resid) {
-    launch_extend_pair(v, u, W.dpair.get(), W.rpair.get(), W.dmax.get(), st);
-    launch_resid_pair(v, u, W.dpair.get(), W.rpair.get(), f, lv.c64.get(), H->c, r, W.part.get(), st);
-    launch_norm_final(W.part.get(), resid_pair_blocks(v), W.norms, st, W.dmax.get());
+    launch_extend_pair(v, u, W.dpair.get(), W.rpair.get(), norms ? W.dmax.get() : nullptr, st);
+    launch_resid_pair(v, u, W.dpair.get(), W.rpair.get(), f, lv.c64.get(), H->c, r, part, st);
+    if (norms) launch_norm_final(W.part.get(), resid_pair_blocks(v), W.norms, st, W.dmax.get());
     return;
   }
   launch_extend_rel(v, u, W.w64[0].w.get(), W.refv.get(), st);
-  launch_resid_rel(v, u, W.w64[0].w.get(), W.refv.get(), f, lv.c64.get(), H->c, r, W.part.get(), st);
-  launch_norm_final(W.part.get(), lap_blocks_f64(v), W.norms, st);
+  launch_resid_rel(v, u, W.w64[0].w.get(), W.refv.get(), f, lv.c64.get(), H->c, r, part, st);
+  if (norms) launch_norm_final(W.part.get(), lap_blocks_f64(v), W.norms, st);
 }
 
 // One outer iteration after the residual, for G systems of one hierarchy in
@@ -1342,7 +1343,7 @@ cpm_status cpm_vcycle(cpm_hier h, int32_t prec, const void* f, void* u, cpm_stre
 cpm_status cpm_residual(cpm_hier h, const double* f, const double* u, double* r, cpm_stream stream) {
   CPM_API_BEGIN
   CPM_CHECK(h != nullptr && u != nullptr && f != nullptr && r != nullptr, CPM_ERR_ARG, "NULL argument");
-  outer_residual(h, h->ws, f, u, r, (cudaStream_t)stream, h->pair_resid);
+  outer_residual(h, h->ws, f, u, r, (cudaStream_t)stream, h->pair_resid, false);
   CPM_CUDA_TRY(cudaGetLastError());
   CPM_API_END
 }
