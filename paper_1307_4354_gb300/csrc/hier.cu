@@ -393,6 +393,10 @@ static void level_op(cpm_hier_s* H, Workspace& W, int l, LapMode mode, const T* 
   T* u_inout = upd ? const_cast<T*>(u) : nullptr;
   if (H->opts.op_form == CPM_OP_PAPER || H->opts.op_form == CPM_OP_VARDIFF) {
     const T* a = H->opts.op_form == CPM_OP_VARDIFF ? avec_of<T>(lv) : nullptr;
+    if (!a && !part && u != out && (mode == LAP_APPLY || mode == LAP_RESID) && paper_fused<T>(v)) {
+      launch_paper_fused<T>(v, mode, u, f, lv.cvec<T>(), (T)H->c, nullptr, out, st);
+      return;
+    }
     if (a)
       launch_lap_vard<T>(v, u, a, w.v.get(), st);
     else
@@ -460,6 +464,16 @@ static void smooth(cpm_hier_s* H, Workspace& W, int l, const T* f, T* u, int swe
   Work<T>& w = W.work<T>(l);
   const T omega = (T)H->opts.omega;
   const T cval = (T)H->c;
+  if (H->opts.smoother == CPM_SMOOTH_JACOBI && H->opts.op_form == CPM_OP_PAPER && paper_fused<T>(v) && sweeps > 0) {
+    // sweeps between u and tmp; an odd last one is copied back
+    T* from = u;
+    T* to = w.tmp.get();
+    for (int s = 0; s < sweeps; ++s, std::swap(from, to))
+      launch_paper_fused<T>(v, LAP_JACOBI, from, f, lv.cvec<T>(), cval, lv.dA<T>(), to, st);
+    if (from != u)
+      CPM_CUDA_TRY(cudaMemcpyAsync(u, from, sizeof(T) * v.nB, cudaMemcpyDeviceToDevice, st));
+    return;
+  }
   for (int s = 0; s < sweeps; ++s) {
     if (H->opts.smoother == CPM_SMOOTH_RM) {
       launch_rm_jacobi<T>(v, u, f, lv.cvec<T>(), cval, omega, w.tmp.get(), st);

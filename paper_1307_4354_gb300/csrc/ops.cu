@@ -543,6 +543,133 @@ __global__ void __launch_bounds__(256) k_paper(LevelView<T> L, const T* u, const
   if (MODE == LAP_RESID && part) block_max_sum(rm, rs, part);
 }
 
+// The same operator in one pass over the extension tiles: E_1 L_B u at cp(x_i)
+// needs L_B u at the 2^d middle nodes of the cubic stencil, whose Laplacian
+// neighbours all lie in the stencil and so in B.  With linear weights l over
+// the middle nodes and their second differences e (weights l_0, l_1 - 2 l_0,
+// l_0 - 2 l_1, l_1 over the four nodes of an axis), E_1 L_B u is the sum over
+// the axes of the products with e on that axis and l on the others, so each
+// stencil row is contracted with the cubic weights, with l and with e.  Taken
+// for FP32, and in 2-D: in 3-D FP64 the extra products cost more FP64 time than
+// the two passes they save.  u and out must not overlap.  M u on a circle of 29
+// thousand points, FP64: one launch of 8.7 us against three of 10.5 us (a call
+// 16.6 against 23.6 us); on the unit sphere at dx = 1/256, FP32: 199 us against
+// 268 us.
+template <typename T, int DIM, int MODE>
+__global__ void __launch_bounds__(64) k_paper_tiles(LevelView<T> L, const T* __restrict__ u,
+                                                    const T* __restrict__ f, const T* __restrict__ cvec, T cval,
+                                                    const T* __restrict__ dA, T* __restrict__ out) {
+  constexpr int NZ = DIM == 3 ? 7 : 1, NC = DIM == 3 ? 4 : 1, RS = 9;
+  __shared__ T box[NZ * 7 * RS];
+  const int32_t tile = blockIdx.x;
+  release_next();
+  const int32_t beg = __ldg(L.tile_start + tile), end = __ldg(L.tile_mid + tile);
+  if (beg == end) return;  // ghost points only
+  // this thread's first point: its records are in flight while the box is staged
+  uint32_t rec = 0;
+  T s[3] = {T(0), T(0), T(0)}, w3[3][4];
+  auto load = [&](int32_t k) {
+    rec = __ldg(L.erec + k);
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+      if constexpr (sizeof(T) == 8) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w3[a][j] = __ldg(L.ew64 + (int64_t)(4 * a + j) * L.nplus + k);
+        s[a] = __ldg(L.fr + (int64_t)a * L.nplus + (rec >> 6));
+      } else {
+        s[a] = __ldg(L.efr + (int64_t)a * L.nplus + k);
+        cubic_w(s[a], w3[a]);
+      }
+    }
+  };
+  int32_t k = beg + threadIdx.x;
+  if (k < end) load(k);
+  wait_prior();
+  for (int q = threadIdx.x; q < NZ * 49; q += 64) {
+    const int x = q % 7, y = (q / 7) % 7, z = q / 49;
+    const int j = (x >> 2) | ((y >> 2) << 1) | ((z >> 2) << 2);
+    const uint64_t bit = 1ull << ((x & 3) | ((y & 3) << 2) | ((z & 3) << 4));
+    const uint64_t m = __ldg(L.tile_mask + 8 * (int64_t)tile + j);
+    T v = T(0);
+    if (m & bit) v = ld_prior(u + __ldg(L.tile_bstart + 8 * (int64_t)tile + j) + __popcll(m & (bit - 1ull)));
+    box[(z * 7 + y) * RS + x] = v;
+  }
+  __syncthreads();
+  for (; k < end; k += 64) {
+    const int32_t i = (int32_t)(rec >> 6);
+    const int bx = rec & 3, by = (rec >> 2) & 3, bz = (rec >> 4) & 3;
+    T l[3][4], e[3][4];
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+      const T l0 = T(1) - s[a], l1 = s[a];
+      l[a][0] = T(0);
+      l[a][1] = l0;
+      l[a][2] = l1;
+      l[a][3] = T(0);
+      e[a][0] = l0;
+      e[a][1] = l1 - T(2) * l0;
+      e[a][2] = l0 - T(2) * l1;
+      e[a][3] = l1;
+    }
+    T e3 = T(0), e1l = T(0);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const T* p = box + ((bz + c) * 7 + by + b) * RS + bx;
+        T v[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) v[a] = p[a];
+        const T x3 = w3[0][0] * v[0] + w3[0][1] * v[1] + w3[0][2] * v[2] + w3[0][3] * v[3];
+        e3 += (w3[1][b] * (DIM == 3 ? w3[2][c] : T(1))) * x3;
+        const bool my = b == 1 || b == 2, mz = DIM == 2 || c == 1 || c == 2;  // middle nodes
+        if (my || mz) {
+          const T xl = l[0][1] * v[1] + l[0][2] * v[2];
+          T g = DIM == 3 ? (mz ? e[1][b] * l[2][c] : T(0)) : e[1][b];
+          if (DIM == 3 && my) g += l[1][b] * e[2][c];
+          e1l += g * xl;
+        }
+        if (my && mz) {
+          const T xe = e[0][0] * v[0] + e[0][1] * v[1] + e[0][2] * v[2] + e[0][3] * v[3];
+          e1l += (l[1][b] * (DIM == 3 ? l[2][c] : T(1))) * xe;
+        }
+      }
+    }
+    const T ui = ld_prior(u + i);
+    const T Mu = e1l * L.inv_h2 - L.gamma * (ui - e3);
+    if (MODE == LAP_APPLY) {
+      out[i] = Mu;
+    } else {
+      const T cc = cvec ? __ldg(cvec + i) : cval;
+      const T r = ld_prior(f + i) - cc * ui + Mu;
+      out[i] = MODE == LAP_RESID ? r : ui + r * __ldg(dA + i);
+    }
+    if (k + 64 < end) load(k + 64);
+  }
+}
+
+template <typename T>
+bool paper_fused(const LevelView<T>& L) {
+  return sizeof(T) == 4 || L.dim == 2;
+}
+template <typename T>
+void launch_paper_fused(const LevelView<T>& L, LapMode mode, const T* u, const T* f, const T* cvec, T cval,
+                        const T* dA, T* out, cudaStream_t st) {
+  if (L.ntiles <= 0) return;
+  if (L.dim == 3) {
+    if constexpr (sizeof(T) == 4) {
+      auto k = mode == LAP_APPLY ? k_paper_tiles<T, 3, LAP_APPLY>
+               : mode == LAP_RESID ? k_paper_tiles<T, 3, LAP_RESID> : k_paper_tiles<T, 3, LAP_JACOBI>;
+      launch_pdl(k, L.ntiles, 64, st, L, u, f, cvec, cval, dA, out);
+    }
+  } else {
+    auto k = mode == LAP_APPLY ? k_paper_tiles<T, 2, LAP_APPLY>
+             : mode == LAP_RESID ? k_paper_tiles<T, 2, LAP_RESID> : k_paper_tiles<T, 2, LAP_JACOBI>;
+    launch_pdl(k, L.ntiles, 64, st, L, u, f, cvec, cval, dA, out);
+  }
+  count_launch();
+}
+
 int paper_blocks(const LevelView<double>& L) { return (int)nblk(L.nB, 256); }
 
 template <typename T>
@@ -1008,6 +1135,9 @@ template void launch_assemble_A<float>(const LevelView<double>&, const double*, 
   template void launch_paper<T>(const LevelView<T>&, LapMode, const T*, const T*, const T*,     \
                                 const T*, const T*, T, const T*, T*, T*, double*, const T*,      \
                                 cudaStream_t);                                                   \
+  template bool paper_fused<T>(const LevelView<T>&);                                            \
+  template void launch_paper_fused<T>(const LevelView<T>&, LapMode, const T*, const T*, const T*, T, const T*, \
+                                      T*, cudaStream_t);                                        \
   template void launch_lap_vard<T>(const LevelView<T>&, const T*, const T*, T*, cudaStream_t);  \
   template void launch_norm_partials<T>(const T*, int64_t, double*, cudaStream_t);               \
   template void launch_cast_to_f64<T>(const T*, double*, int64_t, cudaStream_t);                 \

@@ -145,6 +145,14 @@ template <typename T>
 void launch_paper(const LevelView<T>& L, LapMode mode, const T* u, const T* v, const T* w, const T* f,
                   const T* cvec, T cval, const T* dA, T* out, T* u_inout, double* part,
                   const T* avec, cudaStream_t st);
+// APPLY, RESID or JACOBI of the paper form (constant coefficient) in one pass,
+// where that is the faster way (paper_fused); out = u + (f - c u + M_p u) dA for
+// JACOBI.  u and out must not overlap.
+template <typename T>
+bool paper_fused(const LevelView<T>& L);
+template <typename T>
+void launch_paper_fused(const LevelView<T>& L, LapMode mode, const T* u, const T* f, const T* cvec, T cval,
+                        const T* dA, T* out, cudaStream_t st);
 // v = L~ u = sum over axes of D^b diag(A^f a) D^f u on B (band-restricted).
 template <typename T>
 void launch_lap_vard(const LevelView<T>& L, const T* u, const T* a, T* v, cudaStream_t st);

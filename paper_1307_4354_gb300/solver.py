@@ -109,12 +109,16 @@ class Hierarchy:
         self.band = band
         self.handle = capi.cpm_build_hierarchy(band.handle, o, _stream(stream))
         self.n_levels, self.nb = capi.cpm_hier_info(self.handle, 0)
+        self._sizes = [capi.cpm_hier_info(self.handle, l)[1] for l in range(self.n_levels)]
 
     def ext_tuning(self, level: int = 0):
         """(FP32 extension launch shape chosen for the level, ms of each candidate)."""
         return capi.cpm_hier_ext_tuning(self.handle, level)
 
     def level_size(self, level: int) -> int:
+        # sizes do not change after the build; a bad level is the library's error
+        if 0 <= level < self.n_levels:
+            return self._sizes[level]
         return capi.cpm_hier_info(self.handle, level)[1]
 
     def apply(self, u: torch.Tensor, level: int = 0, out: torch.Tensor | None = None, stream=None):
