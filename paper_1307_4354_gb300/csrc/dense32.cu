@@ -268,7 +268,7 @@ __device__ __forceinline__ float4 load_row_ordered(const DenseView& L, const flo
 //
 // Bound by the L1 data pipe (73 % of its peak: the 16 row loads of a unit, the
 // window stores, the staging) with issue slots at 52 %.  Unit sphere,
-// dx = 1/256, 8.16 M points: 74 us, against 108 us for one thread per point on
+// dx = 1/256, 8.16 M points: 73 us, against 108 us for one thread per point on
 // boxes gathered value by value from band order (16 row loads per point).
 // Chunks of up to six points whose 64 values stay in registers halve the row
 // loads again but leave 13 warps on an SM: 111 us.
@@ -467,7 +467,7 @@ int tune_extend32(const DenseView& L, const float* u, float* w, cudaStream_t st,
 //
 // Bound by HBM and by the latency of its one round of loads: 31 bytes per point
 // at two thirds of the slots used, against 44 with a table of six neighbour
-// indices.  Unit sphere, dx = 1/256, 6.8 M points: 47 us a Jacobi sweep (53 us
+// indices.  Unit sphere, dx = 1/256, 6.8 M points: 45 us a Jacobi sweep (53 us
 // with the table).
 template <int DIM, int MODE, bool CIN>
 __global__ void __launch_bounds__(256) k_lap_rows(DenseView L, const float* u, const float* __restrict__ w,

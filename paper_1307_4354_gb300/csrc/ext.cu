@@ -534,20 +534,25 @@ __device__ __forceinline__ float stage_box_pair(const LevelView<double>& L, cons
   float amax = 0.f;
   BoxRow b;
   for (int r = threadIdx.x; box_row(sm.mask, sm.start, tbox, DIM, r, b); r += kExtThreads) {
-    float vh[7], vl[7];
+    // all of the row's loads before any is used (an absent node takes the
+    // reference, so that its difference is zero)
+    double du[7];
 #pragma unroll
     for (int i = 0; i < 7; ++i) {
       const int x = b.xlo + i;
-      vh[i] = vl[i] = 0.f;
+      du[i] = refd;
       if (x <= b.xhi + 3) {
         const bool hi = x >= 4;
-        if (((hi ? b.rbb : b.rba) >> (x & 3)) & 1u) {
-          const float2 d = pair_split(ld_prior(u + (hi ? b.cb++ : b.ca++)) - refd);
-          vh[i] = d.x;
-          vl[i] = d.y;
-          amax = fmaxf(amax, fabsf(d.x));
-        }
+        if (((hi ? b.rbb : b.rba) >> (x & 3)) & 1u) du[i] = ld_prior(u + (hi ? b.cb++ : b.ca++));
       }
+    }
+    float vh[7], vl[7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+      const float2 d = pair_split(du[i] - refd);
+      vh[i] = d.x;
+      vl[i] = d.y;
+      amax = fmaxf(amax, fabsf(d.x));
     }
     const int o = (b.z * 7 + b.y) * kRS;
 #pragma unroll

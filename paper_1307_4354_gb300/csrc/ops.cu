@@ -253,9 +253,9 @@ void launch_resid_rel(const LevelView<double>& L, const double* u, const double*
 // f - c u_i and the sum with M u_i, and r^2 for the norm (the maximum is taken
 // on the bit patterns of |r|).  Each thread takes kPairPts points (strided by
 // the block), so the block's norm reduction is shared by several points.
-constexpr int kPairPts = 4;
+constexpr int kPairPts = 2;
 // Fewer points than fill the chip that way take one point per thread (circle,
-// 2912 points: 7.7 us with four in a row).
+// 2912 points: 7.7 us with four in a row, 140 us at 8.5 M points with two, 147 with four).
 constexpr int64_t kPairSmall = 152 * 1024;
 
 // Largest |x| and sum of x^2 over the block into part[2 b], part[2 b + 1];
@@ -308,11 +308,19 @@ __global__ void __launch_bounds__(256) k_resid_pair(LevelView<double> L, const d
     for (int q = 0; q < 2 * DIM; ++q) k[q] = __ldg(L.nbr + (int64_t)q * L.nB + i);
     const float ri = ld_prior(rp + i);
     const float2 di = ld_prior(dp + i);
+    const double ui = ld_prior(u + i), fi = ld_prior(f + i);
+    float rn[2 * DIM];
+    float2 dn[2 * DIM];
+#pragma unroll
+    for (int q = 0; q < 2 * DIM; ++q) {
+      rn[q] = ld_prior(rp + k[q]);
+      dn[q] = ld_prior(dp + k[q]);
+    }
     float sh = 0.f, sl = 0.f;
 #pragma unroll
     for (int q = 0; q < 2 * DIM; ++q) {
-      const float rk = ld_prior(rp + k[q]);
-      const float2 dk = ld_prior(dp + k[q]);
+      const float rk = rn[q];
+      const float2 dk = dn[q];
       float ah, al, bh, bl, ch, cl, t;
       two_sum(rk, -ri, ah, al);
       two_sum(dk.x, -di.x, bh, bl);
@@ -324,14 +332,13 @@ __global__ void __launch_bounds__(256) k_resid_pair(LevelView<double> L, const d
     float Sh, Sl, lh, ll;
     fast_two_sum(sh, sl, Sh, Sl);
     pair_mul(Sh, Sl, ih2.x, ih2.y, lh, ll);             // S / dx^2
-    const double ui = ld_prior(u + i);
     const float2 e = pair_split(pair_f2d(ri) - ui);      // ref_i - u_i
     float th, tl, gh, gl, mh, ml;
     pair_add(e.x, e.y, di.x, di.y, th, tl);
     pair_mul(th, tl, gam.x, gam.y, gh, gl);             // gamma ((ref_i - u_i) + delta_i)
     pair_add(lh, ll, gh, gl, mh, ml);                   // M u_i
     const double c = cvec ? __ldg(cvec + i) : cval;
-    const double res = (ld_prior(f + i) - c * ui) + pair_to_f64(mh, ml);
+    const double res = (fi - c * ui) + pair_to_f64(mh, ml);
     r[i] = res;
     rm = max(rm, (unsigned long long)__double_as_longlong(res) & 0x7FFFFFFFFFFFFFFFull);  // |res|
     if (part) rs += res * res;
