@@ -537,29 +537,7 @@ __global__ void k_neighbours(BrickView v, const uint64_t* key, int32_t nB, int d
   }
 }
 
-// 9. Brick records: masks and starts of every occupied brick and of its face
-// neighbours (order -x, +x, -y, +y, -z, +z).
-__global__ void k_brick_recs(BrickView v, const uint32_t* bcoord, int dim, BrickRec* rec) {
-  const int32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= v.nbricks) return;
-  const uint32_t c = bcoord[b];
-  const int bx = (int)(c & 1023), by = (int)((c >> 10) & 1023), bz = (int)((c >> 20) & 1023);
-  const int d[7][3] = {{0, 0, 0}, {-1, 0, 0}, {1, 0, 0}, {0, -1, 0}, {0, 1, 0}, {0, 0, -1}, {0, 0, 1}};
-  BrickRec r;
-  for (int q = 0; q < 7; ++q) {
-    const int x = bx + d[q][0], y = by + d[q][1], z = bz + d[q][2];
-    int32_t nb = -1;
-    if (q <= 2 * dim && x >= 0 && y >= 0 && z >= 0 && x < v.nbx && y < v.nby && z < v.nbz)
-      nb = v.map[((size_t)z * v.nby + y) * v.nbx + x];
-    r.bm[q] = nb >= 0 ? v.bmask[nb] : 0ull;
-    r.gm[q] = nb >= 0 ? v.gmask[nb] : 0ull;
-    r.bs[q] = nb >= 0 ? v.bstart[nb] : 0;
-    r.gs[q] = nb >= 0 ? v.gstart[nb] : 0;
-  }
-  rec[b] = r;
-}
-
-// 10. Table 4.1 counts: per band point the number of its 2d Laplacian
+// 9. Table 4.1 counts: per band point the number of its 2d Laplacian
 // neighbours inside B (the band-restricted L) and whether the node lies outside
 // its own cubic stencil (an extra diagonal entry of M = E_1 L - gamma (I - E_3)).
 __global__ void k_band_counts(BrickView v, const uint64_t* key, int32_t nB, int dim,
@@ -691,8 +669,6 @@ void build_level(const cpm_surface& surf, double lo, double dx, int n, double la
   L.gstart.alloc(nocc);
   k_copy_i64_to_i32<<<blocks_for(nocc, 256), 256, 0, st>>>(bcount.get(), L.bstart.get(), nocc);
   k_copy_i64_to_i32<<<blocks_for(nocc, 256), 256, 0, st>>>(gcount.get(), L.gstart.get(), nocc);
-  L.brec.alloc(nocc);
-  k_brick_recs<<<blocks_for(nocc, 256), 256, 0, st>>>(L.view(), L.bcoord.get(), dim, L.brec.get());
   CPM_CUDA_TRY(cudaGetLastError());
 
   // 6. points

@@ -91,16 +91,6 @@ __host__ __device__ inline int key_ox(uint64_t k) { return (int)((k >> 48) & 15u
 __host__ __device__ inline int key_oy(uint64_t k) { return (int)((k >> 52) & 15u) - 8; }
 __host__ __device__ inline int key_oz(uint64_t k) { return (int)((k >> 56) & 15u) - 8; }
 
-// ----------------------------------------------------------------- brick records
-// Per brick, the occupancy masks and starts of the brick itself (slot 0) and
-// of its face neighbours (slots 1..6: -x, +x, -y, +y, -z, +z; zero masks where
-// there is none), so that a stencil pass finds every Laplacian neighbour with
-// loads addressed by the brick number alone.
-struct BrickRec {
-  uint64_t bm[7], gm[7];
-  int32_t bs[7], gs[7];
-};
-
 // ----------------------------------------------------------------- brick view
 // Plain-pointer view of a level's brick tables, passed by value to kernels.
 struct BrickView {
@@ -109,7 +99,6 @@ struct BrickView {
   const uint64_t* gmask;  // ghost occupancy
   const int32_t* bstart;  // first band index of the brick
   const int32_t* gstart;  // first ghost index of the brick (relative to nB)
-  const BrickRec* brec;   // nbricks brick records
   int nbx, nby, nbz;
   int n;                  // nodes per axis
   int32_t nB;
@@ -159,7 +148,6 @@ struct Level {
   DBuf<uint64_t> bmask, gmask;
   DBuf<int32_t> bstart, gstart;
   DBuf<uint32_t> bcoord;  // packed brick coordinates bx | by << 10 | bz << 20 (<= 1023 each)
-  DBuf<BrickRec> brec;    // per brick: masks and starts of it and its face neighbours
   // per point of B+
   DBuf<uint64_t> key;
   DBuf<double> cp;    // d x (nB+nG), SoA
@@ -185,7 +173,7 @@ struct Level {
   BrickView view() const {
     BrickView v;
     v.map = map.get(); v.bmask = bmask.get(); v.gmask = gmask.get();
-    v.bstart = bstart.get(); v.gstart = gstart.get(); v.brec = brec.get();
+    v.bstart = bstart.get(); v.gstart = gstart.get();
     v.nbx = nbx; v.nby = nby; v.nbz = nbz; v.n = n; v.nB = nB; v.nbricks = nbricks;
     return v;
   }

@@ -1005,7 +1005,7 @@ static void copy_level(const Level& a, Level& b, cudaStream_t st) {
                                    cudaMemcpyDeviceToDevice, st));
   };
   cp(b.map, a.map); cp(b.bmask, a.bmask); cp(b.gmask, a.gmask); cp(b.bstart, a.bstart);
-  cp(b.gstart, a.gstart); cp(b.bcoord, a.bcoord); cp(b.brec, a.brec); cp(b.key, a.key); cp(b.cp, a.cp);
+  cp(b.gstart, a.gstart); cp(b.bcoord, a.bcoord); cp(b.key, a.key); cp(b.cp, a.cp);
   cp(b.fr64, a.fr64); cp(b.fr32, a.fr32);
   b.ntiles = a.ntiles;
   cp(b.tile_brick, a.tile_brick); cp(b.tile_box, a.tile_box); cp(b.tile_mask, a.tile_mask); cp(b.tile_bstart, a.tile_bstart); cp(b.tile_start, a.tile_start); cp(b.tile_mid, a.tile_mid); cp(b.erec, a.erec);

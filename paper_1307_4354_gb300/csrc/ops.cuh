@@ -60,10 +60,6 @@ struct TransferView {
 enum LapMode { LAP_APPLY = 0, LAP_RESID = 1, LAP_JACOBI = 2, LAP_RESID_REL = 3,
                LAP_JAC_RED = 4, LAP_JAC_BLACK = 5,  // Jacobi update of one colour only
                LAP_JAC_REL = 6 };                    // Jacobi update from the relative extension
-// Red (0) / black (1): parity of the sum of the grid coordinates.  Bricks start
-// at multiples of 4, so the parity of the local coordinates inside a brick is
-// that of the global ones.
-__host__ __device__ inline int node_colour_local(int l) { return ((l & 3) + ((l >> 2) & 3) + (l >> 4)) & 1; }
 
 // w = E u on the first npts points of B+ (npts = nB or nB + nG), FP64 (the FP32
 // extension is in dense32.cuh).
