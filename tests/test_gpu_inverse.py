@@ -17,7 +17,7 @@ import synth
 pytestmark = pytest.mark.gpu
 
 CASES = [("circle", (0.8,), 1 / 6), ("circle", (1.0,), 1 / 7), ("circle", (1.0,), 1 / 8),
-         ("circle", (0.9,), 1 / 9), ("circle", (1.0,), 1 / 13), ("sphere", (1.0,), 1 / 6)]
+         ("circle", (0.9,), 1 / 9), ("circle", (1.0,), 1 / 13), ("sphere", (1.0,), 1 / 6), ("sphere", (1.0,), 1 / 9)]
 
 
 @pytest.mark.parametrize("kind,params,dx", CASES)
