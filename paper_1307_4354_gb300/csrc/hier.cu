@@ -340,6 +340,9 @@ static void alloc_workspace(const cpm_hier_s& H, Workspace& W, double* norms_slo
     W.gm64.alloc(nc, kGmresMaxM);
     W.gm32.alloc(nc, kGmresMaxM);
   }
+  // the clears above are complete before a stream that does not wait for the
+  // default stream uses the vectors
+  CPM_CUDA_TRY(cudaStreamSynchronize(nullptr));
   CPM_CUDA_TRY(cudaStreamCreateWithFlags(&W.hs, cudaStreamNonBlocking));
   CPM_CUDA_TRY(cudaEventCreateWithFlags(&W.ev, cudaEventDisableTiming));
   CPM_CUDA_TRY(cudaMallocHost(&W.pinned, 8 * sizeof(double)));
