@@ -64,6 +64,18 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], uint32
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+template <bool TRANS>
+__device__ __forceinline__ void ldmatrix4(uint32_t (&d)[4], const __nv_bfloat16* p) {
+  if (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+
 constexpr int kFwdWarps = 8;
 constexpr int kW1S = 40;  // padded row (k) stride of the transposed W1 in shared memory (bf16)
 constexpr int kW2S = 72;  // same for W2
@@ -87,14 +99,16 @@ struct MlpFwdArgs {
 };
 
 // MODE: 0 du = correction, 1 u += correction, 2 du and the training outputs.
-// Bound by the latency of the feature gather (27 indices, then 27 values, all in
-// flight per lane): 1.63 M points 113 us with a point per lane and three CTAs
-// on an SM, against 170 us with a point per lane of a half warp.
+// Bound by the feature gather (27 indices, then 27 values, all in flight per
+// lane) and the L1 data pipe, which also carries the weights: a warp reads each
+// weight fragment once (ldmatrix) for its 32 points.  1.63 M points: 106 us with
+// a point per lane and three CTAs on an SM; 113 us with the weights read once per
+// 16 points, 170 us with a point per lane of a half warp.
 template <int MODE>
 __global__ void __launch_bounds__(kFwdWarps * 32, MODE == 2 ? 2 : 3) k_mlp_forward(MlpFwdArgs A) {
   __shared__ __align__(16) __nv_bfloat16 w1t[64 * kW1S];  // w1t[n][k] = W1[k][n]
   __shared__ __align__(16) __nv_bfloat16 w2t[64 * kW2S];
-  __shared__ float bias1[64], bias2[64], w3s[64];
+  __shared__ __align__(8) float bias1[64], bias2[64], w3s[64];
   __shared__ __align__(16) __nv_bfloat16 xs[kFwdWarps][32 * kXS];
   __shared__ float ss[kFwdWarps][32];
   for (int q = threadIdx.x; q < 64 * 32; q += blockDim.x) {
@@ -111,15 +125,13 @@ __global__ void __launch_bounds__(kFwdWarps * 32, MODE == 2 ? 2 : 3) k_mlp_forwa
     w3s[q] = A.params[kOffW3 + q];
   }
   __syncthreads();
-  const float b3 = A.params[kOffB3];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
-  const int64_t nsteps = ((int64_t)A.nB + 31) / 32;
-  for (int64_t step = (int64_t)blockIdx.x * kFwdWarps + warp; step < nsteps;
-       step += (int64_t)gridDim.x * kFwdWarps) {
+  const int32_t nsteps = (A.nB + 31) / 32;
+  for (int32_t step = (int32_t)blockIdx.x * kFwdWarps + warp; step < nsteps; step += (int32_t)gridDim.x * kFwdWarps) {
     // features: one point per lane
     {
-      const int64_t p = step * 32 + lane;
+      const int32_t p = step * 32 + lane;
       __nv_bfloat16* xw = xs[warp];
       float f[32];
       float smax = 0.f;
@@ -149,103 +161,88 @@ __global__ void __launch_bounds__(kFwdWarps * 32, MODE == 2 ? 2 : 3) k_mlp_forwa
         v.z = pack_bf16(f[q + 4], f[q + 5]);
         v.w = pack_bf16(f[q + 6], f[q + 7]);
         *reinterpret_cast<uint4*>(&xw[lane * kXS + q]) = v;
-        if (MODE == 2 && A.Xs && p < A.nB) reinterpret_cast<uint4*>(A.Xs + p * 32)[q / 8] = v;
+        if (MODE == 2 && A.Xs && p < A.nB) reinterpret_cast<uint4*>(A.Xs + (int64_t)p * 32)[q / 8] = v;
       }
       ss[warp][lane] = smax;
     }
     __syncwarp();
-#pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-    const int64_t p0 = step * 32 + 16 * half;
-    const __nv_bfloat16* xw = xs[warp] + 16 * half * kXS;
-    const float* sw = ss[warp] + 16 * half;
-    // layer 1: [16 x 32] x [32 x 64]
-    uint32_t a[2][4];
+    const int32_t p0 = step * 32 + g;  // this lane's rows: p0 + 8 q, q = 0 .. 3
+    // layer 1: [32 x 32] x [32 x 64]
+    uint32_t a[2][2][4];
 #pragma unroll
-    for (int kc = 0; kc < 2; ++kc) {
-      a[kc][0] = *reinterpret_cast<const uint32_t*>(&xw[g * kXS + kc * 16 + 2 * t]);
-      a[kc][1] = *reinterpret_cast<const uint32_t*>(&xw[(g + 8) * kXS + kc * 16 + 2 * t]);
-      a[kc][2] = *reinterpret_cast<const uint32_t*>(&xw[g * kXS + kc * 16 + 8 + 2 * t]);
-      a[kc][3] = *reinterpret_cast<const uint32_t*>(&xw[(g + 8) * kXS + kc * 16 + 8 + 2 * t]);
-    }
-    float h[8][4];
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+      for (int kc = 0; kc < 2; ++kc)
+        ldmatrix4<false>(a[m][kc], &xs[warp][(16 * m + (lane & 15)) * kXS + kc * 16 + (lane >> 4) * 8]);
+    // relu(h1) as the A operand of layer 2 (C tiles 2j, 2j+1 form k-chunk j)
+    uint32_t a2[2][4][4];
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-      const int n = nt * 8 + 2 * t;
-      h[nt][0] = h[nt][2] = bias1[n];
-      h[nt][1] = h[nt][3] = bias1[n + 1];
+      uint32_t wb[4];
+      ldmatrix4<false>(wb, &w1t[(nt * 8 + (lane & 7)) * kW1S + (lane >> 3) * 8]);
+      const float2 bb = *reinterpret_cast<const float2*>(&bias1[nt * 8 + 2 * t]);
 #pragma unroll
-      for (int kc = 0; kc < 2; ++kc) {
-        const __nv_bfloat16* wb = &w1t[(nt * 8 + g) * kW1S + kc * 16 + 2 * t];
-        mma_bf16(h[nt], a[kc], *reinterpret_cast<const uint32_t*>(wb),
-                 *reinterpret_cast<const uint32_t*>(wb + 8));
+      for (int m = 0; m < 2; ++m) {
+        float h[4] = {bb.x, bb.y, bb.x, bb.y};
+#pragma unroll
+        for (int kc = 0; kc < 2; ++kc) mma_bf16(h, a[m][kc], wb[2 * kc], wb[2 * kc + 1]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) h[e] = fmaxf(h[e], 0.f);
+        a2[m][nt / 2][2 * (nt & 1)] = pack_bf16(h[0], h[1]);
+        a2[m][nt / 2][2 * (nt & 1) + 1] = pack_bf16(h[2], h[3]);
       }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) h[nt][e] = fmaxf(h[nt][e], 0.f);
-    }
-    // relu(h1) as the A operand of layer 2 (C tiles 2j, 2j+1 form k-chunk j)
-    uint32_t a2[4][4];
-#pragma unroll
-    for (int kc = 0; kc < 4; ++kc) {
-      a2[kc][0] = pack_bf16(h[2 * kc][0], h[2 * kc][1]);
-      a2[kc][1] = pack_bf16(h[2 * kc][2], h[2 * kc][3]);
-      a2[kc][2] = pack_bf16(h[2 * kc + 1][0], h[2 * kc + 1][1]);
-      a2[kc][3] = pack_bf16(h[2 * kc + 1][2], h[2 * kc + 1][3]);
     }
     if (MODE == 2 && A.H1) {
 #pragma unroll
-      for (int kc = 0; kc < 4; ++kc) {
-        const int64_t r0 = p0 + g, r1 = p0 + g + 8;
-        const int c0 = kc * 16 + 2 * t;
-        if (r0 < A.nB) {
-          *reinterpret_cast<uint32_t*>(A.H1 + r0 * 64 + c0) = a2[kc][0];
-          *reinterpret_cast<uint32_t*>(A.H1 + r0 * 64 + c0 + 8) = a2[kc][2];
-        }
-        if (r1 < A.nB) {
-          *reinterpret_cast<uint32_t*>(A.H1 + r1 * 64 + c0) = a2[kc][1];
-          *reinterpret_cast<uint32_t*>(A.H1 + r1 * 64 + c0 + 8) = a2[kc][3];
-        }
+      for (int q = 0; q < 4; ++q) {
+        const int32_t r = p0 + 8 * q;
+        if (r < A.nB)
+#pragma unroll
+          for (int nt = 0; nt < 8; ++nt)
+            *reinterpret_cast<uint32_t*>(A.H1 + (int64_t)r * 64 + nt * 8 + 2 * t) = a2[q / 2][nt / 2][2 * (nt & 1) + (q & 1)];
       }
     }
-    // layer 2: [16 x 64] x [64 x 64], then relu and the dot with w3
-    float y0 = 0.f, y1 = 0.f;
-#pragma unroll
+    // layer 2: [32 x 64] x [64 x 64], then relu and the dot with w3
+    float y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
     for (int nt = 0; nt < 8; ++nt) {
       const int n = nt * 8 + 2 * t;
-      float c[4] = {bias2[n], bias2[n + 1], bias2[n], bias2[n + 1]};
+      uint32_t wb[2][4];
 #pragma unroll
-      for (int kc = 0; kc < 4; ++kc) {
-        const __nv_bfloat16* wb = &w2t[(nt * 8 + g) * kW2S + kc * 16 + 2 * t];
-        mma_bf16(c, a2[kc], *reinterpret_cast<const uint32_t*>(wb),
-                 *reinterpret_cast<const uint32_t*>(wb + 8));
-      }
+      for (int k2 = 0; k2 < 2; ++k2)
+        ldmatrix4<false>(wb[k2], &w2t[(nt * 8 + (lane & 7)) * kW2S + 32 * k2 + (lane >> 3) * 8]);
+      const float2 bb = *reinterpret_cast<const float2*>(&bias2[n]), w3 = *reinterpret_cast<const float2*>(&w3s[n]);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) c[e] = fmaxf(c[e], 0.f);
-      if (MODE == 2 && A.H2) {
-        const int64_t r0 = p0 + g, r1 = p0 + g + 8;
-        if (r0 < A.nB) *reinterpret_cast<uint32_t*>(A.H2 + r0 * 64 + n) = pack_bf16(c[0], c[1]);
-        if (r1 < A.nB) *reinterpret_cast<uint32_t*>(A.H2 + r1 * 64 + n) = pack_bf16(c[2], c[3]);
-      }
-      y0 += c[0] * w3s[n] + c[1] * w3s[n + 1];
-      y1 += c[2] * w3s[n] + c[3] * w3s[n + 1];
-    }
-    y0 += __shfl_xor_sync(0xffffffffu, y0, 1);
-    y0 += __shfl_xor_sync(0xffffffffu, y0, 2);
-    y1 += __shfl_xor_sync(0xffffffffu, y1, 1);
-    y1 += __shfl_xor_sync(0xffffffffu, y1, 2);
-    if (t == 0) {
-      const int64_t r0 = p0 + g, r1 = p0 + g + 8;
-      if (r0 < A.nB) {
-        const float d = sw[g] * A.dx2 * (y0 + b3);
-        if (MODE == 1) A.u[A.uslot ? A.uslot[r0] : r0] += d; else A.du[r0] = d;
-        if (MODE == 2 && A.S) A.S[r0] = sw[g];
-      }
-      if (r1 < A.nB) {
-        const float d = sw[g + 8] * A.dx2 * (y1 + b3);
-        if (MODE == 1) A.u[A.uslot ? A.uslot[r1] : r1] += d; else A.du[r1] = d;
-        if (MODE == 2 && A.S) A.S[r1] = sw[g + 8];
+      for (int m = 0; m < 2; ++m) {
+        float c[4] = {bb.x, bb.y, bb.x, bb.y};
+#pragma unroll
+        for (int kc = 0; kc < 4; ++kc) mma_bf16(c, a2[m][kc], wb[kc / 2][2 * (kc & 1)], wb[kc / 2][2 * (kc & 1) + 1]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c[e] = fmaxf(c[e], 0.f);
+        if (MODE == 2 && A.H2) {
+          const int32_t r0 = p0 + 16 * m, r1 = r0 + 8;
+          if (r0 < A.nB) *reinterpret_cast<uint32_t*>(A.H2 + (int64_t)r0 * 64 + n) = pack_bf16(c[0], c[1]);
+          if (r1 < A.nB) *reinterpret_cast<uint32_t*>(A.H2 + (int64_t)r1 * 64 + n) = pack_bf16(c[2], c[3]);
+        }
+        y[2 * m] += c[0] * w3.x + c[1] * w3.y;
+        y[2 * m + 1] += c[2] * w3.x + c[3] * w3.y;
       }
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      y[q] += __shfl_xor_sync(0xffffffffu, y[q], 1);
+      y[q] += __shfl_xor_sync(0xffffffffu, y[q], 2);
+    }
+    // lane t of a row's four writes row p0 + 8 t
+    {
+      const int32_t r = p0 + 8 * t;
+      const float yt = t == 0 ? y[0] : t == 1 ? y[1] : t == 2 ? y[2] : y[3];
+      if (r < A.nB) {
+        const float sc = ss[warp][8 * t + g];
+        const float d = sc * A.dx2 * (yt + __ldg(A.params + kOffB3));
+        if (MODE == 1) A.u[A.uslot ? A.uslot[r] : r] += d; else A.du[r] = d;
+        if (MODE == 2 && A.S) A.S[r] = sc;
+      }
     }
     __syncwarp();
   }
@@ -294,18 +291,6 @@ __device__ __forceinline__ void copy16_or_zero(void* smem, const void* gmem, boo
                "l"(gmem), "r"(n)
                : "memory");
 }
-template <bool TRANS>
-__device__ __forceinline__ void ldmatrix4(uint32_t (&d)[4], const __nv_bfloat16* p) {
-  if (TRANS)
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
-                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
-  else
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
-                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
-}
-
 // Copies of one group (zero rows past the last point).
 __device__ __forceinline__ void bwd_fetch(BwdStage& s, const float* dy, const __nv_bfloat16* Xs,
                                           const __nv_bfloat16* H1, const __nv_bfloat16* H2, int64_t p0,
