@@ -661,7 +661,7 @@ void launch_extend(const LevelView<double>& L, const double* u, double* w, int32
   if (npts <= 0 || L.ntiles <= 0) return;
   const bool with_ghost = npts > L.nB;
   if (L.dim == 3)
-    launch_pdl(k_extend_tiles<double, 3>, L.ntiles, kExtThreads, st, L, u, w, with_ghost, (double*)nullptr,
+    launch_dep(false, k_extend_tiles<double, 3>, L.ntiles, kExtThreads, st, L, u, w, with_ghost, (double*)nullptr,
                (const int32_t*)nullptr, (const uint32_t*)nullptr);
   else
     launch_pdl(k_extend_tiles<double, 2>, L.ntiles, kExtThreads, st, L, u, w, with_ghost, (double*)nullptr,
@@ -672,7 +672,7 @@ void launch_extend(const LevelView<double>& L, const double* u, double* w, int32
 void launch_extend_set(const LevelView<double>& L, const PointSet& S, const double* u, double* w, cudaStream_t st) {
   if (L.ntiles <= 0) return;
   auto kernel = L.dim == 3 ? k_extend_tiles<double, 3> : k_extend_tiles<double, 2>;
-  launch_pdl(kernel, L.ntiles, kExtThreads, st, L, u, w, true, (double*)nullptr, S.tstart, S.epos);
+  launch_dep(L.dim == 2, kernel, L.ntiles, kExtThreads, st, L, u, w, true, (double*)nullptr, S.tstart, S.epos);
   count_launch();
 }
 

@@ -157,11 +157,15 @@ void launch_dense_gemv(const M* A, const T* const* b, T* const* x, int G, int32_
       v.x[q] = x[g0 + q];
     }
     const unsigned grid = dense_gemv_blocks(n);
+    // Between FP64 passes the product starts after the kernel before it (see
+    // launch_dep); between FP32 passes an early start gains (a mixed solve on
+    // the sphere at dx = 1/12: 0.88 ms, 0.96 without).
+    constexpr bool kEarly = sizeof(T) == 4;
     switch (nv) {
-      case 1: launch_pdl(k_dense_gemv<M, T, ADD, 1>, grid, kGemvWarps * 32, st, A, v, n); break;
-      case 2: launch_pdl(k_dense_gemv<M, T, ADD, 2>, grid, kGemvWarps * 32, st, A, v, n); break;
-      case 3: launch_pdl(k_dense_gemv<M, T, ADD, 3>, grid, kGemvWarps * 32, st, A, v, n); break;
-      default: launch_pdl(k_dense_gemv<M, T, ADD, 4>, grid, kGemvWarps * 32, st, A, v, n); break;
+      case 1: launch_dep(kEarly, k_dense_gemv<M, T, ADD, 1>, grid, kGemvWarps * 32, st, A, v, n); break;
+      case 2: launch_dep(kEarly, k_dense_gemv<M, T, ADD, 2>, grid, kGemvWarps * 32, st, A, v, n); break;
+      case 3: launch_dep(kEarly, k_dense_gemv<M, T, ADD, 3>, grid, kGemvWarps * 32, st, A, v, n); break;
+      default: launch_dep(kEarly, k_dense_gemv<M, T, ADD, 4>, grid, kGemvWarps * 32, st, A, v, n); break;
     }
   }
 }

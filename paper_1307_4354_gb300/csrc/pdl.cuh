@@ -49,8 +49,15 @@ __device__ __forceinline__ float4 ld_prior(const float4* p) {
   return v;
 }
 
+// early: the kernel's blocks may be placed while the kernel before it drains.
+// They then go where that one leaves room, unevenly, which costs a kernel of
+// about one wave of blocks that is bound by the FP64 pipe more than its start:
+// with the 3-D FP64 extension and the FP64 GEMV placed early, FP64 solves took
+// 9.6 ms (unit sphere, dx = 1/32), 31.7 ms (1/96), 1.28 ms (circle, 1/64), else
+// 5.6, 29.5 and 1.21 ms.  The FP32 extension gains from it (an FP32 V-cycle at
+// dx = 1/128 0.56 ms, 0.62 without).
 template <typename... P, typename... A>
-void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st, A... args) {
+void launch_dep(bool early, void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st, A... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -59,8 +66,12 @@ void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_
   cfg.blockDim = dim3(block);
   cfg.stream = st;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   CPM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
+}
+template <typename... P, typename... A>
+void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st, A... args) {
+  launch_dep(true, kernel, grid, block, st, args...);
 }
 
 }  // namespace cpm
