@@ -494,7 +494,7 @@ def run_cpm(args, world, rank, local):
                                     "frac": ach_res / pk.get("hbm_gbs", 6800.0), "traffic": None,
                                     "algorithmic_bytes": bytes_res, "ms": resid_ms,
                                     "note": "the pair extension is FP32-pipe and latency bound "
-                                            "(pair arithmetic, 72 registers); see profiles"},
+                                            "(pair arithmetic, 70 registers); see profiles"},
         "clocks": clk.summary(),
     }
     if cpu:
