@@ -22,8 +22,13 @@
 // integers and added to A with one FP64 operation per entry.  56 bits of every
 // operand enter, below the rounding of an FP64 product relative to the largest
 // entry of the row and the column: direct solves on 16 levels (circles 312 ..
-// 4536 points, spheres 4358 .. 7190, an ellipsoid) are 0.66 to 1.41 times as
-// far from the solution as with FP64 elimination, 0.97 in the mean.
+// 4536 points, spheres 4358 .. 7190, an ellipsoid; constant coefficients) are
+// 0.66 to 1.41 times as far from the solution as with FP64 elimination, 0.97 in
+// the mean.
+//
+// An entry far below its row's and its column's largest keeps few of those 56
+// bits, so the slices serve matrices whose rows have one scale (kMaxSpread).
+// Others (a diffusion coefficient or a c over decades) take the products in FP64.
 //
 // 7190 rows: 0.15 s (product 86 ms, panels 33 ms, panel updates 18 ms), against
 // 1.36 s for 7190 rank-one steps over the matrix in HBM.
@@ -31,6 +36,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "ops.cuh"
 
@@ -43,6 +49,14 @@ static unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 constexpr int kBlk = 128;   // columns per block (the K of the product)
 constexpr int kPan = 16;    // columns eliminated by one panel kernel
 constexpr int kSlices = 7;
+// Largest ratio of the rows' scales (largest magnitude off the diagonal) and of
+// the diagonal's magnitudes for the sliced products.  Row-wise backward error of
+// direct solves in units of 2^-53, circles of 360 to 712 points, slices against
+// FP64 products.  Ratio off the diagonal (a over decades) 13 to 17: 1116, 605 at
+// worst; 27: 870, 246; 140: 2200, 240; 1.5e4: 9819, 26; 1.9e6: 498425, 90.  On
+// the diagonal (c over decades) 8: 61, 41; 22: 125, 31; 2e3: 500, 21.  Levels
+// with constant coefficients have ratios of 1.3 to 8.8.
+constexpr double kMaxSpread = 16.0;
 
 // ----------------------------------------------------------------- panels
 // One cluster eliminates `steps` <= kPan columns c0 .. of Q (n rows of kBlk
@@ -251,6 +265,45 @@ __global__ void k_gj_put(double* A, int32_t n, int32_t k0, int b, const double* 
   if (e >= (int64_t)n * kBlk) return;
   const int c = (int)(e % kBlk);
   if (c < b) A[(e / kBlk) * n + k0 + c] = Q[e];
+}
+
+// ----------------------------------------------------------------- row scales
+// out[0], out[1]: the smallest and the largest row scale (largest magnitude off
+// the diagonal, as bits; zeros are left out), out[2], out[3]: the same of the
+// diagonal.  One warp per row.
+__global__ void __launch_bounds__(256) k_row_scales(const double* __restrict__ A, int32_t n,
+                                                    unsigned long long* out) {
+  const int32_t i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (i >= n) return;
+  double m = 0.0;
+  for (int32_t j = lane; j < n; j += 32)
+    if (j != i) m = fmax(m, fabs(A[(size_t)i * n + j]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane > 1) return;
+  const double x = lane == 0 ? m : fabs(A[(size_t)i * n + i]);
+  if (x > 0.0) {
+    atomicMin(out + 2 * lane, (unsigned long long)__double_as_longlong(x));
+    atomicMax(out + 2 * lane + 1, (unsigned long long)__double_as_longlong(x));
+  }
+}
+// Whether the products of an inverse of A may be sliced.  Synchronous.
+static bool sliced_products(const double* A, int32_t n, cudaStream_t st) {
+  DBuf<unsigned long long> d(4);
+  unsigned long long h[4] = {~0ull, 0ull, ~0ull, 0ull};
+  CPM_CUDA_TRY(cudaMemcpyAsync(d.get(), h, sizeof(h), cudaMemcpyHostToDevice, st));
+  k_row_scales<<<nblk(n, 8), 256, 0, st>>>(A, n, d.get());
+  CPM_CUDA_TRY(cudaGetLastError());
+  CPM_CUDA_TRY(cudaMemcpyAsync(h, d.get(), sizeof(h), cudaMemcpyDeviceToHost, st));
+  CPM_CUDA_TRY(cudaStreamSynchronize(st));
+  auto one_scale = [&](int k) {
+    double lo, hi;
+    std::memcpy(&lo, &h[k], sizeof(lo));
+    std::memcpy(&hi, &h[k + 1], sizeof(hi));
+    return h[k + 1] == 0 || hi <= kMaxSpread * lo;
+  };
+  return one_scale(0) && one_scale(2);
 }
 
 // ----------------------------------------------------------------- slices
@@ -470,6 +523,58 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_gj_product(double* A, int32
   }
 }
 
+// The same in FP64: R the pivot rows as they were (kBlk rows of n doubles, zero
+// beyond b).  64 x 64 entries per block, 4 x 4 per thread.  Bound by the FP64
+// pipe (2 n^3 flops in all: 7190 rows 0.61 s; a build with them 0.68 s, with the
+// slices 0.15 s, with rank-one steps 1.35 s).
+constexpr int kP64 = 64, kP64K = 16;
+__global__ void k_gj_rows(const double* A, int32_t n, const int32_t* rows, int b, double* R) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= (int64_t)n * kBlk) return;
+  const int j = (int)(e / n);
+  R[e] = j < b ? A[(size_t)rows[j] * n + e % n] : 0.0;
+}
+__global__ void __launch_bounds__(256) k_gj_product64(double* A, int32_t n, int32_t k0, int b,
+                                                      const double* __restrict__ Q, const double* __restrict__ R,
+                                                      const int32_t* __restrict__ owner) {
+  __shared__ double qs[kP64K][kP64 + 1], rs[kP64K][kP64];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int32_t i0 = blockIdx.y * kP64, c0 = blockIdx.x * kP64;
+  double acc[4][4] = {};
+  for (int j0 = 0; j0 < kBlk; j0 += kP64K) {
+    for (int e = tid; e < kP64 * kP64K; e += 256) {
+      const int32_t i = i0 + e / kP64K, c = c0 + e % kP64;
+      qs[e % kP64K][e / kP64K] = i < n ? Q[(size_t)i * kBlk + j0 + e % kP64K] : 0.0;
+      rs[e / kP64][e % kP64] = c < n ? R[(size_t)(j0 + e / kP64) * n + c] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kP64K; ++j) {
+      double q[4], r[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        q[k] = qs[j][ty + 16 * k];
+        r[k] = rs[j][tx + 16 * k];
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[a][c] += q[a] * r[c];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int32_t i = i0 + ty + 16 * a, c = c0 + tx + 16 * k;
+      if (i >= n || c >= n || (c >= k0 && c < k0 + b)) continue;
+      const int32_t o = owner[i];
+      double* x = A + (size_t)i * n + c;
+      *x = (o >= k0 && o < k0 + b ? 0.0 : *x) + acc[a][k];
+    }
+}
+
 // out[k][rows[j]] = A[rows[k]][j].
 __global__ void k_gj_unpermute(const double* A, int32_t n, const int32_t* rows, double* out) {
   const int32_t per = (n + blockDim.x - 1) / blockDim.x;  // blocks per row
@@ -479,9 +584,16 @@ __global__ void k_gj_unpermute(const double* A, int32_t n, const int32_t* rows, 
 
 void invert_dense(DBuf<double>& A, int32_t n, cudaStream_t st, int32_t* err) {
   if (n <= 0) return;
-  DBuf<double> Q((size_t)n * kBlk), U(kPan * kBlk);
-  DBuf<__nv_bfloat16> QS((size_t)kSlices * n * kBlk), US((size_t)kSlices * n * kBlk);
+  DBuf<double> Q((size_t)n * kBlk), U(kPan * kBlk), R;
+  DBuf<__nv_bfloat16> QS, US;
   DBuf<int32_t> qe(n), ue(n), owner(n), rows(n);
+  const bool sliced = n > kBlk && sliced_products(A.get(), n, st);
+  if (sliced) {
+    QS.alloc((size_t)kSlices * n * kBlk);
+    US.alloc((size_t)kSlices * n * kBlk);
+  } else if (n > kBlk) {  // (one block has no product)
+    R.alloc((size_t)n * kBlk);
+  }
   CPM_CUDA_TRY(cudaMemsetAsync(owner.get(), 0xff, sizeof(int32_t) * n, st));
   CPM_CUDA_TRY(cudaFuncSetAttribute(k_gj_product, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)sizeof(GjShared)));
@@ -521,11 +633,15 @@ void invert_dense(DBuf<double>& A, int32_t n, cudaStream_t st, int32_t* err) {
                                       owner.get(), U.get(), err));
       k_gj_inner<<<nblk(n, kInnerRows), 256, 0, st>>>(Q.get(), n, c0, steps, k0 + c0, owner.get(), U.get());
     }
-    if (b < n) {
+    if (sliced) {
       k_slice_rows<<<nblk(n, 8), 256, 0, st>>>(Q.get(), n, QS.get(), qe.get());
       k_slice_cols<<<nblk(n, kSliceCols), 256, 0, st>>>(A.get(), n, rows.get() + k0, b, US.get(), ue.get());
       k_gj_product<<<grid, kProdThreads, sizeof(GjShared), st>>>(A.get(), n, k0, b, QS.get(), qe.get(), US.get(), ue.get(),
                                                         owner.get(), ntm, ntn);
+    } else if (n > kBlk) {
+      const dim3 g64(nblk(n, kP64), nblk(n, kP64));
+      k_gj_rows<<<nblk(nq, 256), 256, 0, st>>>(A.get(), n, rows.get() + k0, b, R.get());
+      k_gj_product64<<<g64, 256, 0, st>>>(A.get(), n, k0, b, Q.get(), R.get(), owner.get());
     }
     k_gj_put<<<nblk(nq, 256), 256, 0, st>>>(A.get(), n, k0, b, Q.get());
     CPM_CUDA_TRY(cudaGetLastError());
