@@ -65,3 +65,15 @@ def test_backward_error_of_the_direct_solve(radius, dx, form, da, wave, dc):
         res = np.abs(f.astype(np.longdouble) - A.astype(np.longdouble) @ uo)
         err = float((res / (np.abs(A) @ np.abs(uo) + np.abs(f))).max())
         assert err <= 4 * ob.nb * 2.0 ** -53, (ob.nb, seed, err * 2.0 ** 53)
+
+
+@pytest.mark.parametrize("kind,dx", [("circle", 1 / 6), ("circle", 1 / 16)])
+def test_a_nan_in_the_matrix_is_refused(kind, dx):
+    """One NaN in c: the elimination is left with a row of NaNs, which has no
+    pivot, whatever the number of column blocks (272 and 712 rows)."""
+    torch, pkg = require_cuda()
+    g = pkg.Band(kind, (), dx)
+    c = torch.ones(g.nb, dtype=torch.float64, device="cuda")
+    c[g.nb // 3] = float("nan")
+    with pytest.raises(pkg.capi.CpmError, match="singular"):
+        pkg.Hierarchy(g, coarsest_dx=dx, c_device=c)
