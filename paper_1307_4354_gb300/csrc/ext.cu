@@ -681,8 +681,8 @@ void launch_extend_rel(const LevelView<T>& L, const T* u, T* delta, T* refv, cud
   const int32_t nt = L.ntiles;
   if (nt <= 0) return;
   if (L.dim == 3)
-    launch_pdl(k_extend_tiles<T, 3, true>, nt, kExtThreads, st, L, u, delta, true, refv, (const int32_t*)nullptr,
-               (const uint32_t*)nullptr);
+    launch_dep(sizeof(T) == 4, k_extend_tiles<T, 3, true>, nt, kExtThreads, st, L, u, delta, true, refv,
+               (const int32_t*)nullptr, (const uint32_t*)nullptr);
   else
     launch_pdl(k_extend_tiles<T, 2, true>, nt, kExtThreads, st, L, u, delta, true, refv, (const int32_t*)nullptr,
                (const uint32_t*)nullptr);

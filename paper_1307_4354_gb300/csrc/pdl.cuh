@@ -54,8 +54,10 @@ __device__ __forceinline__ float4 ld_prior(const float4* p) {
 // about one wave of blocks that is bound by the FP64 pipe more than its start:
 // with the 3-D FP64 extension and the FP64 GEMV placed early, FP64 solves took
 // 9.6 ms (unit sphere, dx = 1/32), 31.7 ms (1/96), 1.28 ms (circle, 1/64), else
-// 5.6, 29.5 and 1.21 ms.  The FP32 extension gains from it (an FP32 V-cycle at
-// dx = 1/128 0.56 ms, 0.62 without).
+// 5.6, 29.5 and 1.21 ms.  The 3-D FP64 extension in relative form is the same
+// kernel (relative-form FP64 solves at dx = 1/32 9.4 ms, else 7.6; a torus at 1/44
+// 24.2 and 22.4).  The FP32 extension gains from it (an FP32 V-cycle at dx = 1/128
+// 0.56 ms, 0.62 without).
 template <typename... P, typename... A>
 void launch_dep(bool early, void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st, A... args) {
   cudaLaunchAttribute at{};
