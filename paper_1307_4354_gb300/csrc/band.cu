@@ -291,6 +291,22 @@ __global__ void k_scan_add(int64_t* d, int64_t n, const int64_t* tile_offsets) {
     if (base + i < n) d[base + i] += add;
 }
 
+size_t scan_scratch(int64_t n) {
+  size_t sum = 0;
+  for (int64_t t = n; t > 1;) sum += (size_t)(t = (t + kScanTile - 1) / kScanTile);
+  return sum + 1;
+}
+void scan_exclusive_async(int64_t* d, int64_t n, int64_t* scratch, cudaStream_t st) {
+  if (n <= 0) return;
+  const int64_t tiles = (n + kScanTile - 1) / kScanTile;
+  k_scan_tiles<<<(unsigned)tiles, kScanThreads, 0, st>>>(d, n, scratch);
+  if (tiles > 1) {
+    scan_exclusive_async(scratch, tiles, scratch + tiles, st);
+    k_scan_add<<<(unsigned)tiles, kScanThreads, 0, st>>>(d, n, scratch);
+  }
+  CPM_CUDA_TRY(cudaGetLastError());
+}
+
 int64_t scan_exclusive_i64(int64_t* d, int64_t n, cudaStream_t st) {
   if (n <= 0) return 0;
   const int64_t tiles = (n + kScanTile - 1) / kScanTile;

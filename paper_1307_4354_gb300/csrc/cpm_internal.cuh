@@ -166,7 +166,7 @@ struct Level {
   DBuf<float> efr32;          // d x (nB+nG) fractions in E order
   DBuf<double> ew64;          // 4d x (nB+nG) FP64 cubic weights in E order
   DBuf<float2> ewp;           // the same as FP32 pairs (built on demand: build_pair_weights)
-  int ext_variant = 0;        // FP32 extension's launch shape, chosen by timing (ExtVariant)
+  int ext_variant = 0;        // FP32 extension's launch shape (tune_extend32)
   float ext_ms[3] = {0.f, 0.f, 0.f};
   DBuf<int32_t> nbr;          // 2d x nB: B+ index of the Laplacian neighbours of B
 
@@ -198,6 +198,9 @@ void set_capturing(bool on);
 
 // Exclusive scan of int64 values in place; returns the total (band.cu).
 int64_t scan_exclusive_i64(int64_t* d, int64_t n, cudaStream_t st);
+// The same without the total and without a wait; scratch: scan_scratch(n) elements.
+size_t scan_scratch(int64_t n);
+void scan_exclusive_async(int64_t* d, int64_t n, int64_t* scratch, cudaStream_t st);
 
 // Surface descriptor as passed to kernels.
 struct SurfaceDev {

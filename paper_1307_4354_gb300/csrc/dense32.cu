@@ -8,7 +8,7 @@
 // them share each base on a smooth surface.  A unit is up to two points with
 // one base: a thread that evaluates both needs each of the base's 4^(d-1) rows
 // once, half the shared-memory loads that bound the pass.
-#include <algorithm>
+#include <vector>
 
 #include "dense32.cuh"
 #include "pdl.cuh"
@@ -101,9 +101,9 @@ __global__ void __launch_bounds__(32) k_units_emit(BrickView v, const uint32_t* 
                                                    const uint32_t* tile_box, const int32_t* tile_start,
                                                    const uint32_t* erec, const float* efr, int64_t nplus,
                                                    int dim, const uint8_t* keep, const uint32_t* slot,
-                                                   const int64_t* unit0, const int64_t* tile0,
-                                                   const int32_t* bfwd, uint32_t* tiles, float4* pts0,
-                                                   float4* pts1, uint32_t* cidx0, uint32_t* cidx1) {
+                                                   const int64_t* unit0, int64_t ubase,
+                                                   const int64_t* tile0, int64_t tbase, const int32_t* bfwd,
+                                                   uint32_t* tiles, float4* pts0, float4* pts1, uint32_t* cidx0, uint32_t* cidx1) {
   __shared__ int hist[64], key[64], start[64];
   const int lane = threadIdx.x;
   const int32_t tile = blockIdx.x;
@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(32) k_units_emit(BrickView v, const uint32_t* 
   const uint32_t tb = tile_brick[tile];
   const int bx = tb & 1023, by = (tb >> 10) & 1023, bz = (tb >> 20) & 1023;
   const int32_t home = v.map[((size_t)bz * v.nby + by) * v.nbx + bx];
-  uint32_t* hdr = tiles + tile0[tile] * kTileWords;
-  const int64_t u0 = unit0[tile];
+  uint32_t* hdr = tiles + (tile0[tile] - tbase) * kTileWords;
+  const int64_t u0 = unit0[tile] - ubase;
   if (lane < kTileWords) {
     uint32_t word = 0;
     if (lane < 8) word = (uint32_t)bfwd[8 * (int64_t)home + lane];
@@ -154,55 +154,22 @@ __global__ void __launch_bounds__(32) k_units_emit(BrickView v, const uint32_t* 
     const float fx = efr[k], fy = efr[nplus + k], fz = dim == 3 ? efr[2 * nplus + k] : 0.f;
     if (!(r & 1)) {
       pts0[p] = make_float4(__uint_as_float(s | ((b & 7u) << kSlotBits)), fx, fy, fz);
-      cidx0[p] = idx;
+      if (cidx0) cidx0[p] = idx;
     }
     if ((r & 1) || r == hist[b] - 1) {  // (an odd count's last unit repeats its point)
       pts1[p] = make_float4(__uint_as_float(s | ((b >> 3) << kSlotBits)), fx, fy, fz);
-      cidx1[p] = idx;
+      if (cidx1) cidx1[p] = idx;
     }
   }
-}
-
-static void build_units(const Level& L, const Dense32& D, const uint8_t* keep, ExtUnits& out, cudaStream_t st) {
-  const int64_t nt = L.ntiles;
-  out.ntiles = 0;
-  if (nt <= 0) return;
-  DBuf<int64_t> nu(nt), used(nt);
-  k_units_count<<<(unsigned)nt, 32, 0, st>>>(L.tile_start.get(), L.erec.get(), keep, nu.get(), used.get());
-  CPM_CUDA_TRY(cudaGetLastError());
-  const int64_t nunits = scan_exclusive_i64(nu.get(), nt, st);
-  out.ntiles = (int32_t)scan_exclusive_i64(used.get(), nt, st);
-  out.tiles.alloc((size_t)out.ntiles * kTileWords);
-  for (int h = 0; h < 2; ++h) {
-    out.pts[h].alloc((size_t)nunits);
-    out.cidx[h].alloc((size_t)nunits);
-  }
-  k_units_emit<<<(unsigned)nt, 32, 0, st>>>(L.view(), L.tile_brick.get(), L.tile_box.get(), L.tile_start.get(),
-                                            L.erec.get(), L.efr32.get(), L.nplus(), L.dim, keep, D.slot.get(),
-                                            nu.get(), used.get(), D.bfwd.get(), out.tiles.get(), out.pts[0].get(),
-                                            out.pts[1].get(), out.cidx[0].get(), out.cidx[1].get());
-  CPM_CUDA_TRY(cudaGetLastError());
-}
-
-void build_dense32(const Level& L, Dense32& D, cudaStream_t st) {
-  CPM_CHECK((int64_t)dense_size(L) <= (int64_t)kSlotMask, CPM_ERR_ARG, "too many bricks on one level");
-  D.bface.alloc((size_t)2 * L.nbricks);
-  D.bfwd.alloc((size_t)8 * L.nbricks);
-  D.slot.alloc((size_t)L.nplus());
-  k_dense_bricks<<<nblk(L.nbricks, 256), 256, 0, st>>>(L.view(), L.bcoord.get(), L.dim, D.bface.get(),
-                                                       D.bfwd.get());
-  k_dense_slots<<<nblk(L.nplus(), 256), 256, 0, st>>>(L.view(), L.key.get(), L.nplus(), L.dim, D.slot.get());
-  CPM_CUDA_TRY(cudaGetLastError());
-  build_units(L, D, nullptr, D.all, st);
 }
 
 UnitsView units_view(const ExtUnits& U) {
   UnitsView v;
-  v.tiles = U.tiles.get();
+  v.tiles = U.tiles;
   v.ntiles = U.ntiles;
   for (int h = 0; h < 2; ++h) {
-    v.pts[h] = U.pts[h].get();
-    v.cidx[h] = U.cidx[h].get();
+    v.pts[h] = U.pts[h];
+    v.cidx[h] = U.cidx[h];
   }
   return v;
 }
@@ -640,8 +607,8 @@ void launch_transfer32(const DenseTransfer& T, const DenseView& source, const fl
                        cudaStream_t st) {
   if (T.n <= 0) return;
   const unsigned g = nblk(T.n, 256);
-  const float4* r = T.rec.get();
-  const uint32_t* d = T.dst.get();
+  const float4* r = T.rec;
+  const uint32_t* d = T.dst;
   if (source.dim == 3) {
     if (add) launch_pdl(k_transfer_dense<3, true>, g, 256, st, r, d, T.n, source.bfwd, src, out);
     else launch_pdl(k_transfer_dense<3, false>, g, 256, st, r, d, T.n, source.bfwd, src, out);
@@ -771,9 +738,10 @@ __global__ void k_row_flags(const uint64_t* mask, int64_t nrows, int per, int64_
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < nrows) flag[t] = ((mask[t / per] >> (4 * (t % per))) & 15ull) != 0;
 }
-__global__ void k_row_emit(const uint64_t* mask, int64_t nrows, int per, const int64_t* pos, uint32_t* rows) {
+__global__ void k_row_emit(const uint64_t* mask, int64_t nrows, int per, const int64_t* pos, int64_t base,
+                           uint32_t* rows) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < nrows && ((mask[t / per] >> (4 * (t % per))) & 15ull)) rows[pos[t]] = (uint32_t)t;
+  if (t < nrows && ((mask[t / per] >> (4 * (t % per))) & 15ull)) rows[pos[t] - base] = (uint32_t)t;
 }
 
 // FP64 lists: flags of the marked points of B, flags of the kept E-order
@@ -785,78 +753,27 @@ __global__ void k_list_flags(const uint32_t* slot, int32_t n, int dim, const uin
   flag[i] = (mask[s >> (2 * dim)] >> (s & ((1u << (2 * dim)) - 1u))) & 1ull;
 }
 __global__ void k_list_emit(const uint32_t* slot, int32_t n, int dim, const uint64_t* mask, const int64_t* pos,
-                            int32_t* list) {
+                            int64_t base, int32_t* list) {
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t s = slot[i];
-  if ((mask[s >> (2 * dim)] >> (s & ((1u << (2 * dim)) - 1u))) & 1ull) list[pos[i]] = i;
+  if ((mask[s >> (2 * dim)] >> (s & ((1u << (2 * dim)) - 1u))) & 1ull) list[pos[i] - base] = i;
 }
 __global__ void k_epos_flags(const uint32_t* erec, int64_t n, const uint8_t* keep, int64_t* flag) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n) flag[k] = keep[erec[k] >> 6];
 }
-__global__ void k_epos_emit(const uint32_t* erec, int64_t n, const uint8_t* keep, const int64_t* pos,
+__global__ void k_epos_emit(const uint32_t* erec, int64_t n, const uint8_t* keep, const int64_t* pos, int64_t base,
                             uint32_t* epos) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n && keep[erec[k] >> 6]) epos[pos[k]] = (uint32_t)k;
+  if (k < n && keep[erec[k] >> 6]) epos[pos[k] - base] = (uint32_t)k;
 }
-__global__ void k_epos_starts(const int32_t* tile_start, int32_t ntiles, int64_t n, const int64_t* pos,
+__global__ void k_epos_starts(const int32_t* tile_start, int32_t ntiles, int64_t n, const int64_t* pos, int64_t base,
                               int32_t total, int32_t* tstart) {
   const int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t > ntiles) return;
   const int32_t k = t < ntiles ? tile_start[t] : (int32_t)n;
-  tstart[t] = k < n ? (int32_t)pos[k] : total;
-}
-
-static void build_need(const Level& L, const Dense32& D, const uint64_t* mask, NeedSet& S, cudaStream_t st) {
-  DBuf<uint8_t> keep(L.nplus());
-  k_keep_near<<<nblk(L.nplus(), 256), 256, 0, st>>>(L.view(), L.key.get(), L.nplus(), L.dim, mask, keep.get());
-  CPM_CUDA_TRY(cudaGetLastError());
-  build_units(L, D, keep.get(), S.units, st);
-  const int per = L.dim == 3 ? 16 : 4;
-  const int64_t nrows = (int64_t)L.nbricks * per;
-  DBuf<int64_t> pos(nrows);
-  k_row_flags<<<nblk(nrows, 256), 256, 0, st>>>(mask, nrows, per, pos.get());
-  S.nrows = (int32_t)scan_exclusive_i64(pos.get(), nrows, st);
-  S.rows.alloc((size_t)S.nrows);
-  k_row_emit<<<nblk(nrows, 256), 256, 0, st>>>(mask, nrows, per, pos.get(), S.rows.get());
-  CPM_CUDA_TRY(cudaGetLastError());
-  const int64_t np = L.nplus();
-  DBuf<int64_t> lpos(np);
-  k_list_flags<<<nblk(L.nB, 256), 256, 0, st>>>(D.slot.get(), L.nB, L.dim, mask, lpos.get());
-  S.nlist = (int32_t)scan_exclusive_i64(lpos.get(), L.nB, st);
-  S.list.alloc((size_t)S.nlist);
-  k_list_emit<<<nblk(L.nB, 256), 256, 0, st>>>(D.slot.get(), L.nB, L.dim, mask, lpos.get(), S.list.get());
-  k_epos_flags<<<nblk(np, 256), 256, 0, st>>>(L.erec.get(), np, keep.get(), lpos.get());
-  const int32_t ne = (int32_t)scan_exclusive_i64(lpos.get(), np, st);
-  S.epos.alloc((size_t)ne);
-  S.tstart.alloc((size_t)L.ntiles + 1);
-  k_epos_emit<<<nblk(np, 256), 256, 0, st>>>(L.erec.get(), np, keep.get(), lpos.get(), S.epos.get());
-  k_epos_starts<<<nblk(L.ntiles + 1, 256), 256, 0, st>>>(L.tile_start.get(), L.ntiles, np, lpos.get(), ne,
-                                                         S.tstart.get());
-  CPM_CUDA_TRY(cudaGetLastError());
-  CPM_CUDA_TRY(cudaStreamSynchronize(st));  // the scratch arrays go out of scope
-}
-
-void build_need_sets(const Level& L, Dense32& D, const TransferCells* restrict_from, const TransferCells* prolong_from,
-                     cudaStream_t st) {
-  DBuf<uint64_t> mr(L.nbricks), mu(L.nbricks);
-  const size_t bytes = sizeof(uint64_t) * L.nbricks;
-  CPM_CUDA_TRY(cudaMemsetAsync(mr.get(), 0, bytes, st));
-  k_mark_cells<<<nblk(restrict_from->n, 256), 256, 0, st>>>(restrict_from->base, restrict_from->n, L.dim, L.view(),
-                                                            mr.get());
-  build_need(L, D, mr.get(), D.resid, st);
-  if (prolong_from) {  // a coarse level: its sweeps can be restricted too
-    CPM_CUDA_TRY(cudaMemsetAsync(mu.get(), 0, bytes, st));
-    k_mark_cells<<<nblk(prolong_from->n, 256), 256, 0, st>>>(prolong_from->base, prolong_from->n, L.dim, L.view(),
-                                                             mu.get());
-    k_mark_stencils<<<L.ntiles, 32, 0, st>>>(L.view(), L.tile_brick.get(), L.tile_start.get(), L.erec.get(), L.dim,
-                                             D.bfwd.get(), mu.get());
-    k_or_masks<<<nblk(L.nbricks, 256), 256, 0, st>>>(mu.get(), mr.get(), L.nbricks);
-    build_need(L, D, mu.get(), D.sweep, st);
-    D.mask_sweep = std::move(mu);
-  }
-  CPM_CUDA_TRY(cudaGetLastError());
+  tstart[t] = k < n ? (int32_t)(pos[k] - base) : total;
 }
 
 // flag[j]: target j (a point of B of the target level) is wanted
@@ -868,7 +785,7 @@ __global__ void k_target_flags(const uint32_t* slot, int32_t n, int dim, const u
 }
 __global__ void k_transfer_emit(const uint64_t* base, const float* fr, int32_t n, int dim, BrickView src,
                                 const uint32_t* slot, bool dense_dst, const uint64_t* mask, const int64_t* pos,
-                                float4* rec, uint32_t* dst) {
+                                int64_t base0, float4* rec, uint32_t* dst) {
   const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const uint32_t sj = slot[j];
@@ -877,25 +794,218 @@ __global__ void k_transfer_emit(const uint64_t* base, const float* fr, int32_t n
   const int x = (int)(k & 0xffffu), y = (int)((k >> 16) & 0xffffu), z = (int)((k >> 32) & 0xffffu);
   const int32_t b = src.map[((size_t)(z >> 2) * src.nby + (y >> 2)) * src.nbx + (x >> 2)];
   const uint32_t s = ((uint32_t)max(b, 0) << (2 * dim)) | (uint32_t)((x & 3) | ((y & 3) << 2) | ((z & 3) << 4));
-  const int64_t p = pos[j];
+  const int64_t p = pos[j] - base0;
   rec[p] = make_float4(__uint_as_float(s), fr[j], fr[n + j], dim == 3 ? fr[2 * (int64_t)n + j] : 0.f);
   dst[p] = dense_dst ? sj : (uint32_t)j;
 }
 
-void build_transfer32(const Level& target, const Dense32& TD, const Level& source, const TransferCells& cells,
-                      bool dense_dst, bool pruned, DenseTransfer& T, cudaStream_t st) {
-  const uint64_t* mask = pruned ? TD.mask_sweep.get() : nullptr;
-  DBuf<int64_t> pos(cells.n);
-  k_target_flags<<<nblk(cells.n, 256), 256, 0, st>>>(TD.slot.get(), cells.n, target.dim, mask, pos.get());
+// ----------------------------------------------------------------- build
+// out[q] = d[at[q]]
+struct ScanMarks {
+  static constexpr int kMax = 16;
+  int64_t at[kMax];
+};
+__global__ void k_pick(const int64_t* d, ScanMarks m, int n, int64_t* out) {
+  if ((int)threadIdx.x < n) out[threadIdx.x] = d[m.at[threadIdx.x]];
+}
+
+// At least n elements of scratch (what was there is lost).
+template <typename T>
+static void grow(DBuf<T>& d, size_t n, cudaStream_t st) {
+  if (d.n >= n) return;
+  CPM_CUDA_TRY(cudaStreamSynchronize(st));  // the old block may be in use
+  d.alloc(n);
+}
+
+// The counts of all of a level's sets are scanned in one go, so that a level
+// costs one wait of the host.  With a scan, its scratch and a wait per set and
+// list, hierarchies without a dense inverse took 14.0 ms to build (sphere at
+// dx = 1/96), 9.3 (circle at 1/640), 5.1 (sphere at 1/32), so 10.4, 6.3 and 4.1 ms.
+class CountScan {
+ public:
+  CountScan(DBuf<int64_t>& d, cudaStream_t st) : d_(d), st_(st) {}
+  // A segment of n > 0 counts; data(q) once all segments are known.
+  int segment(int64_t n) {
+    CPM_CHECK(n > 0 && begin_.size() + 1 < ScanMarks::kMax, CPM_ERR_ARG, "bad scan segment");
+    begin_.push_back(total_);
+    total_ += n;
+    return (int)begin_.size() - 1;
+  }
+  void allocate() {  // the counts, the entry that receives their sum, the picked values, the scan's scratch
+    grow(d_, (size_t)(total_ + 1 + ScanMarks::kMax) + scan_scratch(total_ + 1), st_);
+  }
+  int64_t* data(int q) { return d_.get() + begin_[q]; }
+  // Exclusive scan over all segments; synchronous.
+  void run() {
+    const int n = (int)begin_.size();
+    int64_t* picked = d_.get() + total_ + 1;
+    CPM_CUDA_TRY(cudaMemsetAsync(d_.get() + total_, 0, sizeof(int64_t), st_));
+    scan_exclusive_async(d_.get(), total_ + 1, picked + ScanMarks::kMax, st_);
+    ScanMarks m{};
+    for (int q = 0; q < n; ++q) m.at[q] = begin_[q];
+    m.at[n] = total_;
+    k_pick<<<1, 32, 0, st_>>>(d_.get(), m, n + 1, picked);
+    CPM_CUDA_TRY(cudaGetLastError());
+    base_.resize(n + 1);
+    CPM_CUDA_TRY(cudaMemcpyAsync(base_.data(), picked, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, st_));
+    CPM_CUDA_TRY(cudaStreamSynchronize(st_));
+  }
+  int64_t base(int q) const { return base_[q]; }                  // scanned value where segment q starts
+  int64_t count(int q) const { return base_[q + 1] - base_[q]; }  // sum of segment q
+
+ private:
+  DBuf<int64_t>& d_;
+  cudaStream_t st_;
+  int64_t total_ = 0;
+  std::vector<int64_t> begin_, base_;
+};
+
+// One set of a level: segments of its counts, and where its lists go.
+namespace {
+struct SetBuild {
+  const uint64_t* mask = nullptr;  // null: every point of B+
+  uint8_t* keep = nullptr;
+  ExtUnits* units = nullptr;
+  NeedSet* need = nullptr;
+  int units_seg = 0, tiles_seg = 0, rows_seg = 0, list_seg = 0, epos_seg = 0;
+};
+}  // namespace
+
+static void alloc_units(ExtUnits& U, int64_t ntiles, int64_t nunits, bool with_band) {
+  U.ntiles = (int32_t)ntiles;
+  // records of both points, band indices (two words each per unit), headers
+  const size_t words = (size_t)(with_band ? 2 * nunits : 0) + (size_t)ntiles * kTileWords;
+  U.data.alloc((size_t)(2 * nunits) + (words + 3) / 4);
+  U.pts[0] = U.data.get();
+  U.pts[1] = U.pts[0] + nunits;
+  uint32_t* w = reinterpret_cast<uint32_t*>(U.pts[1] + nunits);
+  for (int h = 0; h < 2; ++h) U.cidx[h] = with_band ? w + h * nunits : nullptr;
+  U.tiles = w + (with_band ? 2 * nunits : 0);
+}
+
+static void alloc_need(NeedSet& S, int64_t nrows, int64_t nlist, int64_t ne, int64_t ntiles) {
+  S.nrows = (int32_t)nrows;
+  S.nlist = (int32_t)nlist;
+  S.data.alloc((size_t)(nrows + nlist + ne + ntiles + 1));
+  S.rows = S.data.get();
+  S.list = reinterpret_cast<int32_t*>(S.rows + nrows);
+  S.epos = S.rows + nrows + nlist;
+  S.tstart = reinterpret_cast<int32_t*>(S.epos + ne);
+}
+
+void build_dense32(const Level& L, Dense32& D, const CycleCells* cyc, DenseScratch& sc, cudaStream_t st) {
+  CPM_CHECK((int64_t)dense_size(L) <= (int64_t)kSlotMask, CPM_ERR_ARG, "too many bricks on one level");
+  const int64_t nt = L.ntiles, np = L.nplus(), nB = L.nB;
+  const int per = L.dim == 3 ? 16 : 4;
+  const int64_t nrows = (int64_t)L.nbricks * per;
+  D.bface.alloc((size_t)2 * L.nbricks);
+  D.bfwd.alloc((size_t)8 * L.nbricks);
+  D.slot.alloc((size_t)np);
+  k_dense_bricks<<<nblk(L.nbricks, 256), 256, 0, st>>>(L.view(), L.bcoord.get(), L.dim, D.bface.get(),
+                                                       D.bfwd.get());
+  k_dense_slots<<<nblk(np, 256), 256, 0, st>>>(L.view(), L.key.get(), np, L.dim, D.slot.get());
   CPM_CUDA_TRY(cudaGetLastError());
-  T.n = (int32_t)scan_exclusive_i64(pos.get(), cells.n, st);
-  T.rec.alloc((size_t)T.n);
-  T.dst.alloc((size_t)T.n);
-  k_transfer_emit<<<nblk(cells.n, 256), 256, 0, st>>>(cells.base, cells.fr, cells.n, target.dim, source.view(),
-                                                      TD.slot.get(), dense_dst, mask, pos.get(), T.rec.get(),
-                                                      T.dst.get());
+  if (nt <= 0) return;
+
+  // masks of the needed nodes, and the points of B+ whose w they take
+  SetBuild set[3];
+  int nset = 1;
+  set[0].units = &D.all;
+  const uint64_t* sweep_mask = nullptr;
+  if (cyc && cyc->restrict_from.n > 0) {
+    grow(sc.mask, (size_t)2 * L.nbricks, st);
+    grow(sc.keep, (size_t)(2 * np), st);
+    uint64_t *mr = sc.mask.get(), *mu = mr + L.nbricks;
+    CPM_CUDA_TRY(cudaMemsetAsync(mr, 0, sizeof(uint64_t) * 2 * L.nbricks, st));
+    const TransferCells &r = cyc->restrict_from, &p = cyc->prolong_from;
+    k_mark_cells<<<nblk(r.n, 256), 256, 0, st>>>(r.base, r.n, L.dim, L.view(), mr);
+    set[nset].mask = mr;
+    set[nset].units = &D.resid.units;
+    set[nset++].need = &D.resid;
+    if (p.n > 0) {  // a coarse level: its sweeps can be restricted too
+      k_mark_cells<<<nblk(p.n, 256), 256, 0, st>>>(p.base, p.n, L.dim, L.view(), mu);
+      k_mark_stencils<<<(unsigned)nt, 32, 0, st>>>(L.view(), L.tile_brick.get(), L.tile_start.get(), L.erec.get(),
+                                                   L.dim, D.bfwd.get(), mu);
+      k_or_masks<<<nblk(L.nbricks, 256), 256, 0, st>>>(mu, mr, L.nbricks);
+      sweep_mask = mu;
+      set[nset].mask = mu;
+      set[nset].units = &D.sweep.units;
+      set[nset++].need = &D.sweep;
+    }
+    for (int q = 1; q < nset; ++q) {
+      set[q].keep = sc.keep.get() + (q - 1) * np;
+      k_keep_near<<<nblk(np, 256), 256, 0, st>>>(L.view(), L.key.get(), np, L.dim, set[q].mask, set[q].keep);
+    }
+    CPM_CUDA_TRY(cudaGetLastError());
+  }
+
+  // counts of everything, one scan
+  CountScan scan(sc.counts, st);
+  for (int q = 0; q < nset; ++q) {
+    set[q].units_seg = scan.segment(nt);
+    set[q].tiles_seg = scan.segment(nt);
+    if (!set[q].need) continue;
+    set[q].rows_seg = scan.segment(nrows);
+    set[q].list_seg = scan.segment(nB);
+    set[q].epos_seg = scan.segment(np);
+  }
+  const TransferIn* in[2] = {nullptr, nullptr};
+  int in_seg[2] = {0, 0};
+  for (int q = 0; cyc && q < 2; ++q)
+    if (cyc->in[q].out && cyc->in[q].cells.n > 0) {
+      in[q] = &cyc->in[q];
+      in_seg[q] = scan.segment(in[q]->cells.n);
+    }
+  scan.allocate();
+  for (int q = 0; q < nset; ++q) {
+    const SetBuild& s = set[q];
+    k_units_count<<<(unsigned)nt, 32, 0, st>>>(L.tile_start.get(), L.erec.get(), s.keep, scan.data(s.units_seg),
+                                               scan.data(s.tiles_seg));
+    if (!s.need) continue;
+    k_row_flags<<<nblk(nrows, 256), 256, 0, st>>>(s.mask, nrows, per, scan.data(s.rows_seg));
+    k_list_flags<<<nblk(nB, 256), 256, 0, st>>>(D.slot.get(), L.nB, L.dim, s.mask, scan.data(s.list_seg));
+    k_epos_flags<<<nblk(np, 256), 256, 0, st>>>(L.erec.get(), np, s.keep, scan.data(s.epos_seg));
+  }
+  for (int q = 0; q < 2; ++q)
+    if (in[q])
+      k_target_flags<<<nblk(in[q]->cells.n, 256), 256, 0, st>>>(
+          D.slot.get(), in[q]->cells.n, L.dim, in[q]->pruned ? sweep_mask : nullptr, scan.data(in_seg[q]));
   CPM_CUDA_TRY(cudaGetLastError());
-  CPM_CUDA_TRY(cudaStreamSynchronize(st));
+  scan.run();
+
+  for (int q = 0; q < nset; ++q) {
+    const SetBuild& s = set[q];
+    alloc_units(*s.units, scan.count(s.tiles_seg), scan.count(s.units_seg), s.need == nullptr);
+    k_units_emit<<<(unsigned)nt, 32, 0, st>>>(
+        L.view(), L.tile_brick.get(), L.tile_box.get(), L.tile_start.get(), L.erec.get(), L.efr32.get(), np, L.dim,
+        s.keep, D.slot.get(), scan.data(s.units_seg), scan.base(s.units_seg), scan.data(s.tiles_seg),
+        scan.base(s.tiles_seg), D.bfwd.get(), s.units->tiles, s.units->pts[0], s.units->pts[1], s.units->cidx[0],
+        s.units->cidx[1]);
+    if (!s.need) continue;
+    const int64_t ne = scan.count(s.epos_seg);
+    alloc_need(*s.need, scan.count(s.rows_seg), scan.count(s.list_seg), ne, nt);
+    k_row_emit<<<nblk(nrows, 256), 256, 0, st>>>(s.mask, nrows, per, scan.data(s.rows_seg), scan.base(s.rows_seg),
+                                                 s.need->rows);
+    k_list_emit<<<nblk(nB, 256), 256, 0, st>>>(D.slot.get(), L.nB, L.dim, s.mask, scan.data(s.list_seg),
+                                               scan.base(s.list_seg), s.need->list);
+    k_epos_emit<<<nblk(np, 256), 256, 0, st>>>(L.erec.get(), np, s.keep, scan.data(s.epos_seg),
+                                               scan.base(s.epos_seg), s.need->epos);
+    k_epos_starts<<<nblk(nt + 1, 256), 256, 0, st>>>(L.tile_start.get(), L.ntiles, np, scan.data(s.epos_seg),
+                                                     scan.base(s.epos_seg), (int32_t)ne, s.need->tstart);
+  }
+  for (int q = 0; q < 2; ++q) {
+    if (!in[q]) continue;
+    const TransferCells& c = in[q]->cells;
+    DenseTransfer& T = *in[q]->out;
+    T.n = (int32_t)scan.count(in_seg[q]);
+    T.data.alloc((size_t)T.n + (T.n + 3) / 4);
+    T.rec = T.data.get();
+    T.dst = reinterpret_cast<uint32_t*>(T.rec + T.n);
+    k_transfer_emit<<<nblk(c.n, 256), 256, 0, st>>>(c.base, c.fr, c.n, L.dim, in[q]->source->view(), D.slot.get(),
+                                                    in[q]->dense_dst, in[q]->pruned ? sweep_mask : nullptr,
+                                                    scan.data(in_seg[q]), scan.base(in_seg[q]), T.rec, T.dst);
+  }
+  CPM_CUDA_TRY(cudaGetLastError());
 }
 
 // ----------------------------------------------------------------- layout changes

@@ -51,20 +51,22 @@ struct DenseView {
 // Units of the extension (dense32.cu) over a set of points.
 struct ExtUnits {
   int32_t ntiles = 0;
-  DBuf<uint32_t> tiles;  // header words of the tiles that hold points of the set
-  DBuf<float4> pts[2];   // a unit's first and second point: slot (bits) and cp fractions
-  DBuf<uint32_t> cidx[2];  // their band indices
+  uint32_t* tiles = nullptr;               // header words of the tiles that hold points of the set
+  float4* pts[2] = {nullptr, nullptr};     // a unit's first and second point: slot (bits) and cp fractions
+  uint32_t* cidx[2] = {nullptr, nullptr};  // their band indices (Dense32::all only)
+  DBuf<float4> data;                       // holds them all
 };
 // The nodes of a level that a pass inside a cycle has to visit: rows of the
 // stencil, and the points whose w = E u they take (dense32.cu).
 struct NeedSet {
   ExtUnits units;
-  DBuf<uint32_t> rows;
+  uint32_t* rows = nullptr;
   int32_t nrows = 0;
   // the same for FP64 passes in band order (PointSet)
-  DBuf<int32_t> list, tstart;
-  DBuf<uint32_t> epos;
+  int32_t *list = nullptr, *tstart = nullptr;
+  uint32_t* epos = nullptr;
   int32_t nlist = 0;
+  DBuf<uint32_t> data;  // holds them all
 };
 // Brick-dense structures of one level.
 struct Dense32 {
@@ -73,39 +75,55 @@ struct Dense32 {
   DBuf<uint32_t> slot;
   ExtUnits all;          // every point of B+
   DBuf<float> dA, c;     // brick-dense omega / diag(A) and c
-  // levels of a V-cycle (build_need_sets)
+  // levels of a V-cycle
   NeedSet resid;         // residual that is restricted (every level but the coarsest)
   NeedSet sweep;         // sweeps (levels between the finest and the coarsest)
-  DBuf<uint64_t> mask_sweep;
 };
 // Targets of a linear transfer: base nodes of their cells in the source grid
 // (packed), fractions (SoA, d x n).
 struct TransferCells {
-  const uint64_t* base;
-  const float* fr;
-  int32_t n;
+  const uint64_t* base = nullptr;
+  const float* fr = nullptr;
+  int32_t n = 0;
 };
 // Linear transfer from a brick-dense source: per target the slot (bits) of the
 // cell's first node and the fractions, and where the result goes.
 struct DenseTransfer {
-  DBuf<float4> rec;
-  DBuf<uint32_t> dst;
+  float4* rec = nullptr;
+  uint32_t* dst = nullptr;
   int32_t n = 0;
+  DBuf<float4> data;  // holds both
 };
 UnitsView units_view(const ExtUnits& U);
-inline PointSet point_set(const NeedSet& S) { return {S.list.get(), S.nlist, S.tstart.get(), S.epos.get()}; }
-inline RowsView rows_view(const NeedSet& S) { return {S.rows.get(), (uint32_t)S.nrows}; }
+inline PointSet point_set(const NeedSet& S) { return {S.list, S.nlist, S.tstart, S.epos}; }
+inline RowsView rows_view(const NeedSet& S) { return {S.rows, (uint32_t)S.nrows}; }
 inline RowsView all_rows(const DenseView& L) { return {nullptr, (uint32_t)L.nbricks << (2 * (L.dim - 1))}; }
-// D.resid from the cells of the restriction to the next level; D.sweep too where
-// the level is prolonged from (prolong_from: the cells of the finer level's points).
-void build_need_sets(const Level& L, Dense32& D, const TransferCells* restrict_from,
-                     const TransferCells* prolong_from, cudaStream_t st);
-// Records of a transfer to the points of B of `target` (only those in its sweep set if
-// pruned), written brick-dense or in band order.
-void build_transfer32(const Level& target, const Dense32& TD, const Level& source, const TransferCells& cells,
-                      bool dense_dst, bool pruned, DenseTransfer& T, cudaStream_t st);
+// A transfer to the points of B of a level, from the cells of all of them:
+// written brick-dense or in band order, only to the level's sweep set if pruned.
+struct TransferIn {
+  TransferCells cells;
+  const Level* source = nullptr;
+  bool dense_dst = false, pruned = false;
+  DenseTransfer* out = nullptr;  // null: none
+};
+// What a level's part in a cycle follows from: the cells of the restriction to
+// the next level (none: the coarsest level), those of the finer level's points
+// in this one (none: the finest level), and the transfers into this level.
+struct CycleCells {
+  TransferCells restrict_from, prolong_from;
+  TransferIn in[2];
+};
+// Scratch of build_dense32, kept from level to level.
+struct DenseScratch {
+  DBuf<int64_t> counts;
+  DBuf<uint64_t> mask;
+  DBuf<uint8_t> keep;
+};
 inline size_t dense_size(const Level& L) { return (size_t)(L.nbricks + 1) << (2 * L.dim); }
-void build_dense32(const Level& L, Dense32& D, cudaStream_t st);
+// Everything of D but dA and c; with cyc also the needed sets (D.resid where there
+// is a restriction, D.sweep where the level is prolonged from too) and the
+// transfers into the level.  The scratch is in use until st has caught up.
+void build_dense32(const Level& L, Dense32& D, const CycleCells* cyc, DenseScratch& sc, cudaStream_t st);
 // D.dA (and D.c) from the band-order vectors.
 void dense_static(const Level& L, Dense32& D, const float* dA, const float* c, cudaStream_t st);
 DenseView dense_view(const Level& L, const Dense32& D);
@@ -139,7 +157,9 @@ void launch_scatter32(const DenseView& L, const float* x, float* d, cudaStream_t
 void launch_gather32(const DenseView& L, const float* d, float* x, cudaStream_t st);
 void launch_scale_dense(const DenseView& L, const double* r, const double* norms, float* fd, cudaStream_t st);
 void launch_axpy_dense(const DenseView& L, double* u, const float* d, const double* norms, cudaStream_t st);
-// Time the extension's launch shapes (as tune_extension).
+// The fastest of the extension's launch shapes on a level (over B+, one warm-up
+// and three timed launches each, events on st); ms[v] gets each shape's time.
+// u, w: brick-dense scratch.
 int tune_extend32(const DenseView& L, const float* u, float* w, cudaStream_t st, float ms[3]);
 
 }  // namespace cpm

@@ -1141,7 +1141,6 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
   CPM_CHECK(o.coarse_gmres >= 0 && o.coarse_gmres <= 1000, CPM_ERR_ARG, "bad coarse_gmres");
   CPM_CHECK(o.residual_mode == 0 || o.residual_mode == 1, CPM_ERR_ARG, "bad residual_mode");
 
-  for (auto& lv : H->L) build_dense32(*lv.lev, lv.dense, st);
   DBuf<int32_t> err(1);
   CPM_CUDA_TRY(cudaMemsetAsync(err.get(), 0, sizeof(int32_t), st));
   for (int l = 0; l + 1 < nl; ++l) {
@@ -1150,19 +1149,24 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
   }
   H->dense_cycle = o.op_form == CPM_OP_MBR && o.smoother == CPM_SMOOTH_JACOBI && !o.relative &&
                    o.transfer_deg == 1 && nl > 1;
-  if (H->dense_cycle) {
+  {
+    DenseScratch scratch;
     auto cells = [](const Transfer& t) { return TransferCells{t.base.get(), t.fr32.get(), t.n}; };
-    for (int l = 0; l + 1 < nl; ++l) {
-      const TransferCells r = cells(H->L[l].R);
-      const TransferCells p = l > 0 ? cells(H->L[l - 1].P) : TransferCells{};
-      build_need_sets(*H->L[l].lev, H->L[l].dense, &r, l > 0 ? &p : nullptr, st);
+    for (int l = 0; l < nl; ++l) {
+      HLevel& lv = H->L[l];
+      CycleCells cyc;
+      const bool last = l == nl - 1;
+      if (!last) {
+        cyc.restrict_from = cells(lv.R);
+        if (l + 1 < nl - 1) cyc.in[0] = {cells(lv.P), H->L[l + 1].lev.get(), true, l > 0, &lv.P32};
+      }
+      if (l > 0) {
+        cyc.prolong_from = cells(H->L[l - 1].P);
+        cyc.in[1] = {cells(H->L[l - 1].R), H->L[l - 1].lev.get(), !last, !last, &H->L[l - 1].R32};
+      }
+      build_dense32(*lv.lev, lv.dense, H->dense_cycle ? &cyc : nullptr, scratch, st);
     }
-    for (int l = 0; l + 1 < nl; ++l) {
-      const bool last = l + 1 == nl - 1;
-      HLevel &a = H->L[l], &b = H->L[l + 1];
-      build_transfer32(*b.lev, b.dense, *a.lev, cells(a.R), !last, !last, a.R32, st);
-      if (!last) build_transfer32(*a.lev, a.dense, *b.lev, cells(a.P), true, l > 0, a.P32, st);
-    }
+    CPM_CUDA_TRY(cudaStreamSynchronize(st));  // the scratch goes out of scope
   }
   // per-point c on every level (restricted from the finest band)
   if (o.c_device) {
