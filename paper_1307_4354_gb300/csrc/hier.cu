@@ -105,12 +105,12 @@ struct Transfer {
 template <typename T>
 struct Work {
   DBuf<T> u, f, r, w, tmp, v, refv;
-  void alloc(int64_t nB, int64_t nplus, bool paper, bool relative) {
+  void alloc(int64_t nB, int64_t nplus, bool paper, bool relative, bool extended) {
     if (relative) refv.alloc(nplus);  // reference values of the relative extension
     u.alloc(nB);
     f.alloc(nB);
     r.alloc(nB);
-    w.alloc(nplus);
+    if (extended) w.alloc(nplus);  // E u in band order
     tmp.alloc(nB);
     if (paper) v.alloc(nB);  // L_B u of the paper-form operator
   }
@@ -218,8 +218,14 @@ using namespace cpm;
 struct Workspace {
   std::vector<cpm::Work<double>> w64;
   std::vector<cpm::Work<float>> w32;
-  std::vector<cpm::DBuf<float>> ud, wd, fd, rd;  // brick-dense u, w = E u, f and r of the FP32 passes
-  std::vector<cpm::DBuf<float>> td;  // brick-dense E u where the residual of E u is restricted
+  // brick-dense u, w = E u, f and r of the FP32 passes, as far as the options
+  // use them (r also takes E u where the residual of E u is restricted)
+  struct Dense {
+    cpm::DBuf<float> data;
+    float *u = nullptr, *w = nullptr, *f = nullptr, *r = nullptr;
+    size_t slots = 0;
+  };
+  std::vector<Dense> dense;
   cpm::DBuf<double> part;   // norm partials (2 per block)
   int part_blocks = 0;
   cpm::DBuf<double> own_norms;  // [max, sumsq, 1/max, -] unless norms points elsewhere
@@ -292,24 +298,41 @@ namespace cpm {
 static void alloc_workspace(const cpm_hier_s& H, Workspace& W, double* norms_slot = nullptr) {
   W.w64.resize(H.L.size());
   W.w32.resize(H.L.size());
-  W.ud.resize(H.L.size());
-  W.wd.resize(H.L.size());
-  W.fd.resize(H.L.size());
-  W.rd.resize(H.L.size());
-  W.td.resize(H.L.size());
+  W.dense.resize(H.L.size());
+  // a batch's systems run the plain cycle only, which keeps FP32 vectors in band
+  // order on the coarsest level alone
+  const bool cycle_only = norms_slot != nullptr && H.dense_cycle;
+  const bool mbr = H.opts.op_form == CPM_OP_MBR, relative = H.opts.relative != 0;
+  const bool jacobi = mbr && H.opts.smoother == CPM_SMOOTH_JACOBI && !relative;
   for (size_t l = 0; l < H.L.size(); ++l) {
     const int64_t nB = H.L[l].lev->nB, np = H.L[l].lev->nplus();
-    const bool paper = H.opts.op_form != CPM_OP_MBR;
-    W.w64[l].alloc(nB, np, paper, H.opts.relative != 0);
-    W.w32[l].alloc(nB, np, paper, H.opts.relative != 0);
-    const size_t slots = dense_size(*H.L[l].lev);
-    for (auto* v : {&W.ud[l], &W.wd[l], &W.fd[l], &W.rd[l], &W.td[l]}) {
-      const bool cycle_only = v == &W.rd[l] || v == &W.td[l];
-      if (cycle_only && (!H.dense_cycle || l + 1 == H.L.size())) continue;
-      if (v == &W.td[l] && H.opts.residual_mode == 1) continue;
-      v->alloc(slots);
-      CPM_CUDA_TRY(cudaMemset(v->get(), 0, sizeof(float) * slots));
+    const bool last = l + 1 == H.L.size();
+    W.w64[l].alloc(nB, np, !mbr, relative, true);
+    if (!cycle_only) {
+      W.w32[l].alloc(nB, np, !mbr, relative, !mbr || relative);
+    } else if (last) {
+      W.w32[l].u.alloc(nB);
+      W.w32[l].f.alloc(nB);
     }
+    Workspace::Dense& D = W.dense[l];
+    D.slots = dense_size(*H.L[l].lev);
+    const bool uf = jacobi && !(cycle_only && last), r = H.dense_cycle && !last;
+    const size_t n = D.slots * ((mbr ? 1 : 0) + (uf ? 2 : 0) + (r ? 1 : 0));
+    if (n == 0) continue;
+    D.data.alloc(n);
+    CPM_CUDA_TRY(cudaMemsetAsync(D.data.get(), 0, sizeof(float) * n, nullptr));
+    float* p = D.data.get();
+    auto take = [&]() {
+      float* q = p;
+      p += D.slots;
+      return q;
+    };
+    if (mbr) D.w = take();
+    if (uf) {
+      D.u = take();
+      D.f = take();
+    }
+    if (r) D.r = take();
   }
   const int64_t nB0 = H.L[0].lev->nB;
   W.part_blocks = std::max<int>(std::max(lap_blocks_f64(H.L[0].view<double>()),
@@ -333,8 +356,10 @@ static void alloc_workspace(const cpm_hier_s& H, Workspace& W, double* norms_slo
     W.chk_count.alloc(1);
     W.chk_max.alloc(1);
   }
-  W.r32.alloc(nB0);
-  W.d32.alloc(nB0);
+  if (!cycle_only) {
+    W.r32.alloc(nB0);
+    W.d32.alloc(nB0);
+  }
   if (H.coarse_mode == 3) {
     const int64_t nc = H.L.back().lev->nB;
     W.gm64.alloc(nc, kGmresMaxM);
@@ -375,8 +400,8 @@ static void mbr_op(cpm_hier_s* H, Workspace& W, int l, LapMode mode, const float
   HLevel& lv = H->L[l];
   const DenseView v = lv.dview();
   const Vec32<const float> uv{nullptr, u};
-  launch_extend32(v, v.all, uv, W.wd[l].get(), st);
-  launch_lap32(v, mode, uv, W.wd[l].get(), f, (float)H->c, Vec32<float>{nullptr, u_inout ? u_inout : out},
+  launch_extend32(v, v.all, uv, W.dense[l].w, st);
+  launch_lap32(v, mode, uv, W.dense[l].w, f, (float)H->c, Vec32<float>{nullptr, u_inout ? u_inout : out},
                nullptr, all_rows(v), st);
 }
 
@@ -423,13 +448,13 @@ static void smooth32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* 
                      cudaStream_t st) {
   HLevel& lv = H->L[l];
   const DenseView v = lv.dview();
-  const Vec32<float> dense{W.ud[l].get(), nullptr}, compact{nullptr, u};
+  const Vec32<float> dense{W.dense[l].u, nullptr}, compact{nullptr, u};
   for (int s = 0; s < sweeps; ++s) {
     const Vec32<float> in = s == 0 ? compact : dense, out = s == sweeps - 1 ? compact : dense;
     const Vec32<const float> cin{in.dense, in.compact};
-    launch_extend32(v, v.all, cin, W.wd[l].get(), st);
-    launch_lap32(v, LAP_JACOBI, cin, W.wd[l].get(), s == 0 ? f : W.fd[l].get(), (float)H->c, out,
-                 sweeps > 1 ? W.fd[l].get() : nullptr, all_rows(v), st);
+    launch_extend32(v, v.all, cin, W.dense[l].w, st);
+    launch_lap32(v, LAP_JACOBI, cin, W.dense[l].w, s == 0 ? f : W.dense[l].f, (float)H->c, out,
+                 sweeps > 1 ? W.dense[l].f : nullptr, all_rows(v), st);
   }
 }
 
@@ -566,11 +591,11 @@ static void coarse_solve(cpm_hier_s* H, Workspace* const* W, int G, const T* con
 }
 
 // What a level's FP32 iterate is at a point of the cycle: zero, brick-dense (in
-// Workspace::ud) or in band order.
+// Workspace::Dense::u) or in band order.
 enum class State32 { zero, dense, compact };
 
-// Weighted Jacobi sweeps of level l on brick-dense vectors, f in Workspace::fd
-// (where u is in band order, so is f, and the first sweep fills fd).  Only the
+// Weighted Jacobi sweeps of level l on brick-dense vectors, f in Workspace::Dense::f
+// (where u is in band order, so is f, and the first sweep fills it).  Only the
 // rows and points of `need`, if given.  The last sweep writes u_out (band
 // order) where that is given.
 static void sweeps32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* u, State32& state, int sweeps,
@@ -578,19 +603,19 @@ static void sweeps32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* 
   const DenseView v = H->L[l].dview();
   const UnitsView units = need ? units_view(need->units) : v.all;
   const RowsView rows = need ? rows_view(*need) : all_rows(v);
-  float* ud = W.ud[l].get();
-  float* fd = W.fd[l].get();
+  float* ud = W.dense[l].u;
+  float* fd = W.dense[l].f;
   for (int s = 0; s < sweeps; ++s) {
     const Vec32<float> out = u_out && s == sweeps - 1 ? Vec32<float>{nullptr, u_out} : Vec32<float>{ud, nullptr};
     if (state == State32::zero && out.dense) {
       launch_jacobi_zero32(v, fd, ud, rows, st);
     } else {
       if (state == State32::zero)
-        CPM_CUDA_TRY(cudaMemsetAsync(ud, 0, W.ud[l].n * sizeof(float), st));
+        CPM_CUDA_TRY(cudaMemsetAsync(ud, 0, W.dense[l].slots * sizeof(float), st));
       const bool band = state == State32::compact;
       const Vec32<const float> in{band ? nullptr : ud, band ? u : nullptr};
-      launch_extend32(v, units, in, W.wd[l].get(), st);
-      launch_lap32(v, LAP_JACOBI, in, W.wd[l].get(), band ? f : fd, (float)H->c, out, band ? fd : nullptr, rows,
+      launch_extend32(v, units, in, W.dense[l].w, st);
+      launch_lap32(v, LAP_JACOBI, in, W.dense[l].w, band ? f : fd, (float)H->c, out, band ? fd : nullptr, rows,
                    st);
     }
     state = out.dense ? State32::dense : State32::compact;
@@ -600,8 +625,8 @@ static void sweeps32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* 
 // FP32 V-cycle of the MBR form with Jacobi smoothing and linear transfers, all
 // vectors brick-dense between the levels; the coarsest solve is in band order.
 // Level 0: state says how u[g] and f[g] come (zero and dense: f in
-// Workspace::fd; band order: u[g], f[g], and fd is filled); u_out, if given,
-// receives the result in band order, else it is left in Workspace::ud.  Below
+// Workspace::Dense::f; band order: u[g], f[g], and fd is filled); u_out, if given,
+// receives the result in band order, else it is left in Workspace::Dense::u.  Below
 // level 0 only the needed points are visited (NeedSet).
 static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const float* const* f, float* const* u,
                      State32 state0, bool band_out, cudaStream_t st) {
@@ -615,23 +640,23 @@ static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const flo
   float* cu[kMaxGroup];
   for (int g = 0; g < G; ++g) {
     Workspace& w = *W[g];
-    float* ud = w.ud[l].get();
-    float* fd = w.fd[l].get();
+    float* ud = w.dense[l].u;
+    float* fd = w.dense[l].f;
     state[g] = state0;
     int pre = H->opts.nu1;
     auto make_dense = [&]() {
-      if (state[g] == State32::zero) CPM_CUDA_TRY(cudaMemsetAsync(ud, 0, w.ud[l].n * sizeof(float), st));
+      if (state[g] == State32::zero) CPM_CUDA_TRY(cudaMemsetAsync(ud, 0, w.dense[l].slots * sizeof(float), st));
       if (state[g] == State32::compact) {
         launch_scatter32(v, u[g], ud, st);
         launch_scatter32(v, f[g], fd, st);
       }
       state[g] = State32::dense;
     };
-    if (l == 0 && H->learned_active && pre > 0) {
+    if (l == 0 && H->learned_active && pre > 0 && w.w32[0].r.n > 0) {  // (not a batch's workspace)
       // learned smoother in place of the first Jacobi sweep: r = f - A u, u += net(r)
       make_dense();
-      launch_extend32(v, v.all, {ud, nullptr}, w.wd[0].get(), st);
-      launch_lap32(v, LAP_RESID, {ud, nullptr}, w.wd[0].get(), fd, (float)H->c, {nullptr, w.w32[0].r.get()},
+      launch_extend32(v, v.all, {ud, nullptr}, w.dense[0].w, st);
+      launch_lap32(v, LAP_RESID, {ud, nullptr}, w.dense[0].w, fd, (float)H->c, {nullptr, w.w32[0].r.get()},
                    nullptr, all_rows(v), st);
       mlp_forward(H->mlp->params.get(), *H->mlpd, w.w32[0].r.get(), 1.f / v.inv_h2, nullptr, ud, v.slot, nullptr,
                   st);
@@ -643,15 +668,15 @@ static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const flo
     const NeedSet& rs = lv.dense.resid;
     const float* uu = ud;
     if (H->opts.residual_mode == 0) {
-      launch_extend32(v, need ? units_view(need->units) : v.all, {ud, nullptr}, w.td[l].get(), st);
-      uu = w.td[l].get();
+      launch_extend32(v, need ? units_view(need->units) : v.all, {ud, nullptr}, w.dense[l].r, st);
+      uu = w.dense[l].r;  // the residual takes its place row by row
     }
-    launch_extend32(v, units_view(rs.units), {uu, nullptr}, w.wd[l].get(), st);
-    launch_lap32(v, LAP_RESID, {uu, nullptr}, w.wd[l].get(), fd, (float)H->c, {w.rd[l].get(), nullptr}, nullptr,
+    launch_extend32(v, units_view(rs.units), {uu, nullptr}, w.dense[l].w, st);
+    launch_lap32(v, LAP_RESID, {uu, nullptr}, w.dense[l].w, fd, (float)H->c, {w.dense[l].r, nullptr}, nullptr,
                  rows_view(rs), st);
-    cf[g] = last ? w.w32[l + 1].f.get() : w.fd[l + 1].get();
+    cf[g] = last ? w.w32[l + 1].f.get() : w.dense[l + 1].f;
     cu[g] = w.w32[l + 1].u.get();
-    launch_transfer32(lv.R32, v, w.rd[l].get(), const_cast<float*>(cf[g]), false, st);
+    launch_transfer32(lv.R32, v, w.dense[l].r, const_cast<float*>(cf[g]), false, st);
   }
   if (last) {
     coarse_solve<float>(H, W, G, cf, cu, st);
@@ -663,11 +688,11 @@ static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const flo
   for (int g = 0; g < G; ++g) {
     Workspace& w = *W[g];
     if (last)
-      launch_prolong_coarsest32(tview<float>(lv.P, lv.lev->dim), v.slot, cu[g], w.ud[l].get(), st);
+      launch_prolong_coarsest32(tview<float>(lv.P, lv.lev->dim), v.slot, cu[g], w.dense[l].u, st);
     else
-      launch_transfer32(lv.P32, H->L[l + 1].dview(), w.ud[l + 1].get(), w.ud[l].get(), true, st);
+      launch_transfer32(lv.P32, H->L[l + 1].dview(), w.dense[l + 1].u, w.dense[l].u, true, st);
     sweeps32(H, w, l, nullptr, nullptr, state[g], H->opts.nu2, need, band_out ? u[g] : nullptr, st);
-    if (band_out && H->opts.nu2 == 0) launch_gather32(v, w.ud[l].get(), u[g], st);
+    if (band_out && H->opts.nu2 == 0) launch_gather32(v, w.dense[l].u, u[g], st);
   }
 }
 
@@ -839,11 +864,11 @@ static void outer_step(cpm_hier_s* H, Workspace* const* W, int G, int mode, int 
   } else if (H->dense_cycle && !first_fmg) {
     const DenseView v = H->L[0].dview();
     for (int g = 0; g < G; ++g)
-      launch_scale_dense(v, W[g]->r64.get(), W[g]->norms, W[g]->fd[0].get(), st);
+      launch_scale_dense(v, W[g]->r64.get(), W[g]->norms, W[g]->dense[0].f, st);
     for (int j = 0; j < inner; ++j)
       vcycle32(H, W, G, 0, nullptr, nullptr, j == 0 ? State32::zero : State32::dense, false, st);
     for (int g = 0; g < G; ++g)
-      launch_axpy_dense(v, W[g]->u_own.get(), W[g]->ud[0].get(), W[g]->norms, st);
+      launch_axpy_dense(v, W[g]->u_own.get(), W[g]->dense[0].u, W[g]->norms, st);
   } else {
     const float* r[kMaxGroup];
     float* d[kMaxGroup];
@@ -1215,7 +1240,7 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
     CPM_CUDA_TRY(cudaGetLastError());
     CPM_CUDA_TRY(cudaStreamSynchronize(st));
     lv.dM64 = std::move(dM);
-    dense_static(*lv.lev, lv.dense, lv.dA32.get(), lv.c32.get(), st);
+    if (o.op_form == CPM_OP_MBR) dense_static(*lv.lev, lv.dense, lv.dA32.get(), lv.c32.get(), st);
   }
   // coarsest: dense A = diag(c) - M, inverted in place (FP64)
   H->nc = cl.nB;
@@ -1261,12 +1286,25 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
 
   // solve buffers
   alloc_workspace(*H, H->ws);
-  // the launch shape of every level's FP32 extension, by timing
+  // the launch shape of every level's FP32 extension, by timing, on zeros
+  DBuf<float> probe;
   for (int l = 0; l < nl; ++l) {
     Level& lev = *H->L[l].lev;
-    lev.ext_variant = o.ext_variant > 0 ? o.ext_variant - 1
-                                        : tune_extend32(H->L[l].dview(), H->ws.ud[l].get(), H->ws.wd[l].get(),
-                                                        st, lev.ext_ms);
+    if (o.ext_variant > 0) {
+      lev.ext_variant = o.ext_variant - 1;
+      continue;
+    }
+    Workspace::Dense& D = H->ws.dense[l];
+    float *u = D.u, *w = D.w;
+    if (!u || !w) {  // forms whose passes are in band order
+      if (probe.n < 2 * D.slots) {
+        probe.alloc(2 * D.slots);
+        CPM_CUDA_TRY(cudaMemsetAsync(probe.get(), 0, sizeof(float) * probe.n, st));
+      }
+      u = probe.get();
+      w = u + D.slots;
+    }
+    lev.ext_variant = tune_extend32(H->L[l].dview(), u, w, st, lev.ext_ms);
   }
   *out = H.release();
   CPM_API_END
