@@ -1255,7 +1255,7 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
       launch_assemble_A<double>(H->L[nl - 1].view<double>(), H->L[nl - 1].c64.get(), H->c,
                                 H->Ainv.get(), st);
     CPM_CUDA_TRY(cudaGetLastError());
-    invert_dense(H->Ainv, H->nc, st, err.get());
+    invert_dense(H->Ainv.get(), H->nc, st, err.get());
     if (H->nc <= kCoarseF32CopyMax) {
       H->ld_f32 = (H->nc + 3) / 4 * 4;
       const int64_t np = (int64_t)H->nc * H->ld_f32;

@@ -582,22 +582,32 @@ __global__ void __launch_bounds__(256) k_gj_product64(double* A, int32_t n, int3
     }
 }
 
-// out[k][rows[j]] = A[rows[k]][j].
-__global__ void k_gj_unpermute(const double* A, int32_t n, const int32_t* rows, double* out) {
-  const int32_t per = (n + blockDim.x - 1) / blockDim.x;  // blocks per row
-  const int32_t k = blockIdx.x / per, j = (blockIdx.x % per) * blockDim.x + threadIdx.x;
-  if (j < n) out[(size_t)k * n + rows[j]] = A[(size_t)rows[k] * n + j];
+// The inverse is A[rows[k]][j] at row k and column rows[j].  In place, with a
+// buffer of b columns (rows moved) and then of b rows (columns moved) at a time: a
+// second matrix would double the memory of the build.  owner is the inverse
+// permutation of rows.  7190 rows: a build takes 150.7 ms, with a second matrix
+// 150.4; with b = 128 151.7.
+__global__ void k_gj_copy_columns(const double* A, int32_t n, int32_t k0, int b, double* buf) {
+  const int c = blockIdx.y * blockDim.x + threadIdx.x;
+  if (c < b) buf[(size_t)blockIdx.x * b + c] = A[(size_t)blockIdx.x * n + k0 + c];
+}
+__global__ void k_gj_move_rows(double* A, int32_t n, int32_t k0, int b, const double* buf, const int32_t* rows) {
+  const int c = blockIdx.y * blockDim.x + threadIdx.x;
+  if (c < b) A[(size_t)blockIdx.x * n + k0 + c] = buf[(size_t)rows[blockIdx.x] * b + c];
+}
+__global__ void k_gj_move_columns(double* A, int32_t n, int32_t i0, const double* buf, const int32_t* owner) {
+  const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < n) A[(size_t)(i0 + blockIdx.y) * n + j] = buf[(size_t)blockIdx.y * n + owner[j]];
 }
 
-void invert_dense(DBuf<double>& A, int32_t n, cudaStream_t st, int32_t* err) {
+void invert_dense(double* A, int32_t n, cudaStream_t st, int32_t* err) {
   if (n <= 0) return;
   DBuf<double> Q((size_t)n * kBlk), U(kPan * kBlk), R;
-  DBuf<__nv_bfloat16> QS, US;
+  DBuf<__nv_bfloat16> S;  // slices of Q, then of U
   DBuf<int32_t> qe(n), ue(n), owner(n), rows(n);
-  const bool sliced = n > kBlk && sliced_products(A.get(), n, st);
+  const bool sliced = n > kBlk && sliced_products(A, n, st);
   if (sliced) {
-    QS.alloc((size_t)kSlices * n * kBlk);
-    US.alloc((size_t)kSlices * n * kBlk);
+    S.alloc((size_t)2 * kSlices * n * kBlk);
   } else if (n > kBlk) {  // (one block has no product)
     R.alloc((size_t)n * kBlk);
   }
@@ -629,11 +639,12 @@ void invert_dense(DBuf<double>& A, int32_t n, cudaStream_t st, int32_t* err) {
     cudaGetLastError();
   }
   const int64_t nq = (int64_t)n * kBlk;
+  __nv_bfloat16 *QS = S.get(), *US = sliced ? QS + (size_t)kSlices * n * kBlk : nullptr;
   const int32_t ntm = (n + kTM - 1) / kTM, ntn = (n + kTN - 1) / kTN;
   const unsigned grid = (unsigned)std::min<int64_t>((int64_t)ntm * ntn, 152);
   for (int32_t k0 = 0; k0 < n; k0 += kBlk) {
     const int b = std::min(kBlk, n - k0);
-    k_gj_gather<<<nblk(nq, 256), 256, 0, st>>>(A.get(), n, k0, b, Q.get());
+    k_gj_gather<<<nblk(nq, 256), 256, 0, st>>>(A, n, k0, b, Q.get());
     for (int c0 = 0; c0 < b; c0 += kPan) {
       const int steps = std::min(kPan, b - c0);
       CPM_CUDA_TRY(cudaLaunchKernelEx(&cfg, panel, Q.get(), n, c0, steps, k0 + c0, rows.get() + k0,
@@ -641,23 +652,34 @@ void invert_dense(DBuf<double>& A, int32_t n, cudaStream_t st, int32_t* err) {
       k_gj_inner<<<nblk(n, kInnerRows), 256, 0, st>>>(Q.get(), n, c0, steps, k0 + c0, owner.get(), U.get());
     }
     if (sliced) {
-      k_slice_rows<<<nblk(n, 8), 256, 0, st>>>(Q.get(), n, QS.get(), qe.get());
-      k_slice_cols<<<nblk(n, kSliceCols), 256, 0, st>>>(A.get(), n, rows.get() + k0, b, US.get(), ue.get());
-      k_gj_product<<<grid, kProdThreads, sizeof(GjShared), st>>>(A.get(), n, k0, b, QS.get(), qe.get(), US.get(), ue.get(),
+      k_slice_rows<<<nblk(n, 8), 256, 0, st>>>(Q.get(), n, QS, qe.get());
+      k_slice_cols<<<nblk(n, kSliceCols), 256, 0, st>>>(A, n, rows.get() + k0, b, US, ue.get());
+      k_gj_product<<<grid, kProdThreads, sizeof(GjShared), st>>>(A, n, k0, b, QS, qe.get(), US, ue.get(),
                                                         owner.get(), ntm, ntn);
     } else if (n > kBlk) {
       const dim3 g64(nblk(n, kP64), nblk(n, kP64));
-      k_gj_rows<<<nblk(nq, 256), 256, 0, st>>>(A.get(), n, rows.get() + k0, b, R.get());
-      k_gj_product64<<<g64, 256, 0, st>>>(A.get(), n, k0, b, Q.get(), R.get(), owner.get());
+      k_gj_rows<<<nblk(nq, 256), 256, 0, st>>>(A, n, rows.get() + k0, b, R.get());
+      k_gj_product64<<<g64, 256, 0, st>>>(A, n, k0, b, Q.get(), R.get(), owner.get());
     }
-    k_gj_put<<<nblk(nq, 256), 256, 0, st>>>(A.get(), n, k0, b, Q.get());
+    k_gj_put<<<nblk(nq, 256), 256, 0, st>>>(A, n, k0, b, Q.get());
     CPM_CUDA_TRY(cudaGetLastError());
   }
-  DBuf<double> out((size_t)n * n);
-  k_gj_unpermute<<<nblk(n, 256) * (unsigned)n, 256, 0, st>>>(A.get(), n, rows.get(), out.get());
+  // (the slices' space holds 448 columns of doubles)
+  double* buf = sliced ? reinterpret_cast<double*>(S.get()) : Q.get();
+  const int wide = sliced ? 2 * kSlices * kBlk / 4 : kBlk;
+  for (int32_t k0 = 0; k0 < n; k0 += wide) {
+    const int b = std::min(wide, n - k0);
+    const dim3 g(n, nblk(b, 256));
+    k_gj_copy_columns<<<g, 256, 0, st>>>(A, n, k0, b, buf);
+    k_gj_move_rows<<<g, 256, 0, st>>>(A, n, k0, b, buf, rows.get());
+  }
+  for (int32_t i0 = 0; i0 < n; i0 += wide) {
+    const int b = std::min(wide, n - i0);
+    CPM_CUDA_TRY(cudaMemcpyAsync(buf, A + (size_t)i0 * n, sizeof(double) * b * n, cudaMemcpyDeviceToDevice, st));
+    k_gj_move_columns<<<dim3(nblk(n, 256), b), 256, 0, st>>>(A, n, i0, buf, owner.get());
+  }
   CPM_CUDA_TRY(cudaGetLastError());
   CPM_CUDA_TRY(cudaStreamSynchronize(st));
-  A = std::move(out);
 }
 
 }  // namespace cpm

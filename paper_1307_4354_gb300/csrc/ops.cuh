@@ -216,7 +216,7 @@ void launch_diag_M(const LevelView<double>& L, double* diagM, cudaStream_t st);
 template <typename M>
 void launch_assemble_A(const LevelView<double>& L, const double* cvec, double cval, M* A,
                        cudaStream_t st);
-// A (row-major n x n) := its inverse (inverse.cu).  Synchronous.
-void invert_dense(DBuf<double>& A, int32_t n, cudaStream_t st, int32_t* err);
+// A (row-major n x n) := its inverse, in place (inverse.cu).  Synchronous.
+void invert_dense(double* A, int32_t n, cudaStream_t st, int32_t* err);
 
 }  // namespace cpm

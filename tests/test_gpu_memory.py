@@ -1,5 +1,8 @@
-"""Device memory of workspaces, as the free memory of the device shows it (run by
-itself: other processes on the same device would be counted too)."""
+"""Device memory of workspaces and of the coarsest level's inverse, as the free
+memory of the device shows it (run by itself: other processes on the same device
+would be counted too)."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -49,3 +52,25 @@ def test_batch_workspace_holds_what_its_cycle_uses(opts):
     used = (before - _free(torch)) / n
     B.close()
     assert used <= 1.15 * expected, (used / g.nb, expected / g.nb)
+
+
+def test_inverse_needs_no_second_matrix():
+    """While a hierarchy with an FP64 inverse of 10136 rows (822 MB) is built, the
+    device never holds half a matrix more than afterwards."""
+    torch, pkg = require_cuda()
+    g = pkg.Band("sphere", (0.8,), 1 / 12)
+    kw = dict(coarsest_dx=1 / 12)
+    pkg.Hierarchy(g, **kw).close()  # (modules and kernels are loaded)
+    low, stop = [_free(torch)], threading.Event()
+
+    def watch():
+        while not stop.is_set():
+            low[0] = min(low[0], torch.cuda.mem_get_info()[0])
+
+    t = threading.Thread(target=watch)
+    t.start()
+    H = pkg.Hierarchy(g, **kw)
+    stop.set()
+    t.join()
+    assert g.nb > 10000 and H.n_levels == 1
+    assert _free(torch) - low[0] <= 4 * g.nb ** 2, (_free(torch) - low[0], g.nb)
