@@ -670,7 +670,7 @@ void launch_extend(const LevelView<double>& L, const double* u, double* w, int32
 }
 
 void launch_extend_set(const LevelView<double>& L, const PointSet& S, const double* u, double* w, cudaStream_t st) {
-  if (L.ntiles <= 0) return;
+  if (L.ntiles <= 0 || S.n <= 0) return;  // (blocks of tiles without points do not wait, see pdl.cuh)
   auto kernel = L.dim == 3 ? k_extend_tiles<double, 3> : k_extend_tiles<double, 2>;
   launch_dep(L.dim == 2, kernel, L.ntiles, kExtThreads, st, L, u, w, true, (double*)nullptr, S.tstart, S.epos);
   count_launch();

@@ -1,8 +1,10 @@
 // Programmatic dependent launch: a kernel launched with launch_pdl may start
 // while the kernel before it in the stream drains.  It reads its static inputs
 // (tables built with the hierarchy), then calls wait_prior() and only then
-// touches what earlier kernels wrote or still read.  Every kernel launched this
-// way calls wait_prior(), so that completion is transitive along the stream.
+// touches what earlier kernels wrote or still read.  Completion has to be
+// transitive along the stream: a grid completes only after the one before it if
+// at least one of its threads calls wait_prior().  Threads without work return
+// before that, so nothing is launched this way over an empty set.
 // Values written by earlier kernels are read with ld_prior: a plain (coherent)
 // load that the compiler keeps behind the wait, which it need not do for
 // __ldg.  A V-cycle is some 80 kernels of 2 to 100 us, each of which otherwise
