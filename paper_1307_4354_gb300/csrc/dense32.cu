@@ -26,9 +26,6 @@ constexpr int kRowStride = 20, kPlaneStride = 144;
 #define CPM_EXT_THREADS_SM 896
 #endif
 constexpr int kExtThreadsSM = CPM_EXT_THREADS_SM;
-#ifndef CPM_EXT_WARPS
-#define CPM_EXT_WARPS 2
-#endif
 
 // A tile's header words: 0..7 brick numbers of the box (index i + 2 j + 4 k,
 // the number of bricks if absent), 8 the range of base positions (2 bits lo,
@@ -101,9 +98,10 @@ __global__ void __launch_bounds__(32) k_units_emit(BrickView v, const uint32_t* 
                                                    const uint32_t* tile_box, const int32_t* tile_start,
                                                    const uint32_t* erec, const float* efr, int64_t nplus,
                                                    int dim, const uint8_t* keep, const uint32_t* slot,
-                                                   const int64_t* unit0, int64_t ubase,
-                                                   const int64_t* tile0, int64_t tbase, const int32_t* bfwd,
-                                                   uint32_t* tiles, float4* pts0, float4* pts1, uint32_t* cidx0, uint32_t* cidx1) {
+                                                   const int64_t* unit0, int64_t ubase, const int64_t* tile0,
+                                                   int64_t tbase, const int32_t* bfwd, uint32_t* tiles,
+                                                   float4* pts0, float4* pts1, uint32_t* cidx0,
+                                                   uint32_t* cidx1) {
   __shared__ int hist[64], key[64], start[64];
   const int lane = threadIdx.x;
   const int32_t tile = blockIdx.x;
@@ -250,56 +248,56 @@ __global__ void __launch_bounds__(32 * WARPS, kExtThreadsSM / (32 * WARPS))
   release_next();
   if (tile >= S.ntiles) return;
   const uint32_t hdr = __ldg(S.tiles + (size_t)tile * kTileWords + min(lane, kTileWords - 1));
-    const uint32_t tbox = __shfl_sync(0xffffffffu, hdr, kTileBox);
-    const int32_t beg = (int32_t)__shfl_sync(0xffffffffu, hdr, kTileBeg);
-    const int32_t end = (int32_t)__shfl_sync(0xffffffffu, hdr, kTileEnd);
-    int32_t k = beg + lane;
-    float4 ra, rb;
-    if (k < end) {
-      ra = __ldg(S.pts[0] + k);
-      rb = __ldg(S.pts[1] + k);
-    }
-    wait_prior();
-    // row r = lane + 32 h of the 2^(d-1) columns of bricks along x: column r / 4^(d-1),
-    // row r mod 4^(d-1) of its bricks
-    const int xhi = (tbox >> 2) & 3;
-    const uint32_t ylo = (tbox >> 4) & 3, ny = ((tbox >> 6) & 3) + 3 - ylo;
-    const uint32_t zlo = (tbox >> 8) & 3, nz = ((tbox >> 10) & 3) + 3 - zlo;
-    float4 lo[NH], hi[NH];
-    bool in[NH];
+  const uint32_t tbox = __shfl_sync(0xffffffffu, hdr, kTileBox);
+  const int32_t beg = (int32_t)__shfl_sync(0xffffffffu, hdr, kTileBeg);
+  const int32_t end = (int32_t)__shfl_sync(0xffffffffu, hdr, kTileEnd);
+  int32_t k = beg + lane;
+  float4 ra, rb;
+  if (k < end) {
+    ra = __ldg(S.pts[0] + k);
+    rb = __ldg(S.pts[1] + k);
+  }
+  wait_prior();
+  // row r = lane + 32 h of the 2^(d-1) columns of bricks along x: column r / 4^(d-1),
+  // row r mod 4^(d-1) of its bricks
+  const int xhi = (tbox >> 2) & 3;
+  const uint32_t ylo = (tbox >> 4) & 3, ny = ((tbox >> 6) & 3) + 3 - ylo;
+  const uint32_t zlo = (tbox >> 8) & 3, nz = ((tbox >> 10) & 3) + 3 - zlo;
+  float4 lo[NH], hi[NH];
+  bool in[NH];
 #pragma unroll
-    for (int h = 0; h < NH; ++h) {
+  for (int h = 0; h < NH; ++h) {
+    const int q = DIM == 3 ? 2 * h + (lane >> 4) : (lane >> 2) & 1;
+    const int row = DIM == 3 ? lane & 15 : lane & 3;
+    const int32_t blo = (int32_t)__shfl_sync(0xffffffffu, hdr, 2 * q);
+    const int32_t bhi = (int32_t)__shfl_sync(0xffffffffu, hdr, 2 * q + 1);
+    const uint32_t y = 4 * (q & 1) + (row & 3), z = 4 * (q >> 1) + (row >> 2);
+    in[h] = y - ylo <= ny && (DIM == 3 ? z - zlo <= nz : lane < 8);
+    hi[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!in[h]) continue;
+    if constexpr (CIN) {
+      lo[h] = load_row_ordered<DIM>(L, u, blo, row);
+      if (xhi > 0) hi[h] = load_row_ordered<DIM>(L, u, bhi, row);
+    } else {
+      lo[h] = ld_prior(reinterpret_cast<const float4*>(u + ((size_t)blo << (2 * DIM))) + row);
+      if (xhi > 0) hi[h] = ld_prior(reinterpret_cast<const float4*>(u + ((size_t)bhi << (2 * DIM))) + row);
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < NH; ++h)
+    if (in[h]) {
       const int q = DIM == 3 ? 2 * h + (lane >> 4) : (lane >> 2) & 1;
       const int row = DIM == 3 ? lane & 15 : lane & 3;
-      const int32_t blo = (int32_t)__shfl_sync(0xffffffffu, hdr, 2 * q);
-      const int32_t bhi = (int32_t)__shfl_sync(0xffffffffu, hdr, 2 * q + 1);
-      const uint32_t y = 4 * (q & 1) + (row & 3), z = 4 * (q >> 1) + (row >> 2);
-      in[h] = y - ylo <= ny && (DIM == 3 ? z - zlo <= nz : lane < 8);
-      hi[h] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!in[h]) continue;
-      if constexpr (CIN) {
-        lo[h] = load_row_ordered<DIM>(L, u, blo, row);
-        if (xhi > 0) hi[h] = load_row_ordered<DIM>(L, u, bhi, row);
-      } else {
-        lo[h] = ld_prior(reinterpret_cast<const float4*>(u + ((size_t)blo << (2 * DIM))) + row);
-        if (xhi > 0) hi[h] = ld_prior(reinterpret_cast<const float4*>(u + ((size_t)bhi << (2 * DIM))) + row);
-      }
+      float4* o = reinterpret_cast<float4*>(win + (4 * (q & 1) + (row & 3)) * RS +
+                                            (4 * (q >> 1) + (row >> 2)) * kPlaneStride);
+      o[0] = lo[h];
+      if (xhi > 0) o[1] = make_float4(lo[h].y, lo[h].z, lo[h].w, hi[h].x);
+      if (xhi > 1) o[2] = make_float4(lo[h].z, lo[h].w, hi[h].x, hi[h].y);
+      if (xhi > 2) o[3] = make_float4(lo[h].w, hi[h].x, hi[h].y, hi[h].z);
     }
-#pragma unroll
-    for (int h = 0; h < NH; ++h)
-      if (in[h]) {
-        const int q = DIM == 3 ? 2 * h + (lane >> 4) : (lane >> 2) & 1;
-        const int row = DIM == 3 ? lane & 15 : lane & 3;
-        float4* o = reinterpret_cast<float4*>(win + (4 * (q & 1) + (row & 3)) * RS +
-                                              (4 * (q >> 1) + (row >> 2)) * kPlaneStride);
-        o[0] = lo[h];
-        if (xhi > 0) o[1] = make_float4(lo[h].y, lo[h].z, lo[h].w, hi[h].x);
-        if (xhi > 1) o[2] = make_float4(lo[h].z, lo[h].w, hi[h].x, hi[h].y);
-        if (xhi > 2) o[3] = make_float4(lo[h].w, hi[h].x, hi[h].y, hi[h].z);
-      }
-    __syncwarp();
+  __syncwarp();
 #pragma unroll 1
-    for (; k < end; k += 32) {
+  for (; k < end; k += 32) {
     const uint32_t sa = __float_as_uint(ra.x), sb = __float_as_uint(rb.x);
     const int px = (sa >> kSlotBits) & 3, py = ((sa >> 31) & 1) | ((sb >> (kSlotBits - 1)) & 2), pz = sb >> 30;
     float2 wa[4], wb[4], wz[4];  // (x, y) weights of either point, z weights of both
@@ -360,7 +358,7 @@ __global__ void __launch_bounds__(32 * WARPS, kExtThreadsSM / (32 * WARPS))
       ra = __ldg(S.pts[0] + k + 32);
       rb = __ldg(S.pts[1] + k + 32);
     }
-    }
+  }
 }
 
 // Launch shapes (variant 0, 1, 2): one, two or four tiles (warps) per CTA.
