@@ -556,17 +556,20 @@ __global__ void __launch_bounds__(256) k_paper(LevelView<T> L, const T* u, const
 // the middle nodes and their second differences e (weights l_0, l_1 - 2 l_0,
 // l_0 - 2 l_1, l_1 over the four nodes of an axis), E_1 L_B u is the sum over
 // the axes of the products with e on that axis and l on the others, so each
-// stencil row is contracted with the cubic weights, with l and with e.  Taken
-// for FP32, and in 2-D: in 3-D FP64 the extra products cost more FP64 time than
+// stencil row is contracted with the cubic weights, with l and with e.  In 3-D the
+// sums are ordered for their rounding: the cubic part axis by axis, the small terms
+// of the outer planes and rows before the large ones.  FP32 M u on spheres and tori
+// has 0.94 to 0.98 of the rms error of the three passes (1.12 to 1.14 with one sum
+// over the products of two weights).  Taken for FP32, and in 2-D: in 3-D FP64 the extra products cost more FP64 time than
 // the two passes they save.  u and out must not overlap.  M u on a circle of 29
 // thousand points, FP64: one launch of 8.7 us against three of 10.5 us (a call
-// 16.6 against 23.6 us); on the unit sphere at dx = 1/256, FP32: 199 us against
+// 16.6 against 23.6 us); on the unit sphere at dx = 1/256, FP32: 197 us against
 // 268 us.
 template <typename T, int DIM, int MODE>
 __global__ void __launch_bounds__(64) k_paper_tiles(LevelView<T> L, const T* __restrict__ u,
                                                     const T* __restrict__ f, const T* __restrict__ cvec, T cval,
                                                     const T* __restrict__ dA, T* __restrict__ out) {
-  constexpr int NZ = DIM == 3 ? 7 : 1, NC = DIM == 3 ? 4 : 1, RS = 9;
+  constexpr int NZ = DIM == 3 ? 7 : 1, RS = 9;
   __shared__ T box[NZ * 7 * RS];
   const int32_t tile = blockIdx.x;
   release_next();
@@ -619,28 +622,60 @@ __global__ void __launch_bounds__(64) k_paper_tiles(LevelView<T> L, const T* __r
       e[a][3] = l1;
     }
     T e3 = T(0), e1l = T(0);
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
+    if constexpr (DIM == 2) {
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
-        const T* p = box + ((bz + c) * 7 + by + b) * RS + bx;
+        const T* row = box + (by + b) * RS + bx;
         T v[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) v[a] = p[a];
+        for (int a = 0; a < 4; ++a) v[a] = row[a];
         const T x3 = w3[0][0] * v[0] + w3[0][1] * v[1] + w3[0][2] * v[2] + w3[0][3] * v[3];
-        e3 += (w3[1][b] * (DIM == 3 ? w3[2][c] : T(1))) * x3;
-        const bool my = b == 1 || b == 2, mz = DIM == 2 || c == 1 || c == 2;  // middle nodes
-        if (my || mz) {
-          const T xl = l[0][1] * v[1] + l[0][2] * v[2];
-          T g = DIM == 3 ? (mz ? e[1][b] * l[2][c] : T(0)) : e[1][b];
-          if (DIM == 3 && my) g += l[1][b] * e[2][c];
-          e1l += g * xl;
-        }
-        if (my && mz) {
+        e3 += w3[1][b] * x3;
+        const T xl = l[0][1] * v[1] + l[0][2] * v[2];
+        e1l += e[1][b] * xl;
+        if (b == 1 || b == 2) {
           const T xe = e[0][0] * v[0] + e[0][1] * v[1] + e[0][2] * v[2] + e[0][3] * v[3];
-          e1l += (l[1][b] * (DIM == 3 ? l[2][c] : T(1))) * xe;
+          e1l += l[1][b] * xe;
         }
       }
+    } else {  // FP32
+      float2 q01, q23;  // contracted in y and z, by x
+      float mid[2];     // the middle planes' sums over x and y
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) {
+        const int c = cc == 0 ? 0 : cc == 1 ? 3 : cc - 1;  // the outer planes first
+        const bool mz = c == 1 || c == 2;
+        float2 p01, p23;
+        float xl[4], xe[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float* row = box + ((bz + c) * 7 + by + b) * RS + bx;
+          float v[4];
+#pragma unroll
+          for (int a = 0; a < 4; ++a) v[a] = row[a];
+          const float2 wy = make_float2(w3[1][b], w3[1][b]), v01 = make_float2(v[0], v[1]), v23 = make_float2(v[2], v[3]);
+          p01 = b == 0 ? __fmul2_rn(wy, v01) : __ffma2_rn(wy, v01, p01);
+          p23 = b == 0 ? __fmul2_rn(wy, v23) : __ffma2_rn(wy, v23, p23);
+          const bool my = b == 1 || b == 2;
+          if (my || mz) xl[b] = l[0][1] * v[1] + l[0][2] * v[2];
+          if (my && mz) xe[b] = e[0][0] * v[0] + e[0][1] * v[1] + e[0][2] * v[2] + e[0][3] * v[3];
+        }
+        const float2 wz = make_float2(w3[2][c], w3[2][c]);
+        q01 = cc == 0 ? __fmul2_rn(wz, p01) : __ffma2_rn(wz, p01, q01);
+        q23 = cc == 0 ? __fmul2_rn(wz, p23) : __ffma2_rn(wz, p23, q23);
+        e1l += e[2][c] * (l[1][1] * xl[1] + l[1][2] * xl[2]);
+        if (mz) {
+          float m = e[1][0] * xl[0] + e[1][3] * xl[3];
+          m += e[1][1] * xl[1];
+          m += e[1][2] * xl[2];
+          m += l[1][1] * xe[1];
+          m += l[1][2] * xe[2];
+          mid[c - 1] = m;
+        }
+      }
+      e1l += l[2][1] * mid[0];
+      e1l += l[2][2] * mid[1];
+      e3 = (w3[0][0] * q01.x + w3[0][2] * q23.x) + (w3[0][1] * q01.y + w3[0][3] * q23.y);
     }
     const T ui = ld_prior(u + i);
     const T Mu = e1l * L.inv_h2 - L.gamma * (ui - e3);
