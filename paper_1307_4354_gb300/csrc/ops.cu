@@ -556,14 +556,15 @@ __global__ void __launch_bounds__(256) k_paper(LevelView<T> L, const T* u, const
 // the middle nodes and their second differences e (weights l_0, l_1 - 2 l_0,
 // l_0 - 2 l_1, l_1 over the four nodes of an axis), E_1 L_B u is the sum over
 // the axes of the products with e on that axis and l on the others, so each
-// stencil row is contracted with the cubic weights, with l and with e.  In 3-D the
-// sums are ordered for their rounding: the cubic part axis by axis, the small terms
-// of the outer planes and rows before the large ones.  FP32 M u on spheres and tori
-// has 0.94 to 0.98 of the rms error of the three passes (1.12 to 1.14 with one sum
-// over the products of two weights).  Taken for FP32, and in 2-D: in 3-D FP64 the extra products cost more FP64 time than
-// the two passes they save.  u and out must not overlap.  M u on a circle of 29
-// thousand points, FP64: one launch of 8.7 us against three of 10.5 us (a call
-// 16.6 against 23.6 us); on the unit sphere at dx = 1/256, FP32: 197 us against
+// stencil row is contracted with the cubic weights, with l and with e.  In 3-D
+// the sums are ordered for their rounding: the cubic part axis by axis, the
+// small terms of the outer planes and rows before the large ones.  FP32 M u on
+// spheres and tori has 0.94 to 0.98 of the rms error of the three passes (1.12
+// to 1.14 with one sum over the products of two weights).  Taken for FP32, and
+// in 2-D: in 3-D FP64 the extra products cost more FP64 time than the two passes
+// they save.  u and out must not overlap.  M u on a circle of 29 thousand
+// points, FP64: one launch of 8.7 us against three of 10.5 us (a call 16.6
+// against 23.6 us); on the unit sphere at dx = 1/256, FP32: 197 us against
 // 268 us.
 template <typename T, int DIM, int MODE>
 __global__ void __launch_bounds__(64) k_paper_tiles(LevelView<T> L, const T* __restrict__ u,
