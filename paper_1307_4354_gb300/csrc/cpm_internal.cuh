@@ -81,6 +81,25 @@ struct DBuf {
   T* get() const { return p; }
 };
 
+// A part of a device block, and what deals out a block's parts: run once without
+// a block, for its size, then again with it.  (An allocation costs some 10 us.)
+template <typename T>
+struct Part {
+  T* p = nullptr;
+  size_t n = 0;
+  T* get() const { return p; }
+};
+struct Carver {
+  unsigned char* block = nullptr;
+  size_t used = 0;
+  template <typename T>
+  void operator()(Part<T>& part, size_t n) {
+    part.n = n;
+    part.p = block && n ? reinterpret_cast<T*>(block + used) : nullptr;
+    used += (n * sizeof(T) + 511) / 512 * 512;  // (aligned like a block of its own)
+  }
+};
+
 // ----------------------------------------------------------------- key packing
 // key = x | y << 16 | z << 32 | (ox + 8) << 48 | (oy + 8) << 52 | (oz + 8) << 56
 // (o = cubic stencil base - node coordinate, in [-8, 7]).

@@ -400,24 +400,28 @@ int tune_extend32(const DenseView& L, const float* u, float* w, cudaStream_t st,
   int best = 0;
   for (int v = 0; v < 3; ++v) ms[v] = 0.f;
   if (L.all.ntiles <= 0) return best;
-  cudaEvent_t e0, e1;
-  CPM_CUDA_TRY(cudaEventCreate(&e0));
-  CPM_CUDA_TRY(cudaEventCreate(&e1));
+  struct Events {
+    cudaEvent_t e[6] = {};
+    ~Events() {
+      for (cudaEvent_t q : e)
+        if (q) cudaEventDestroy(q);
+    }
+  } ev;
+  for (cudaEvent_t& q : ev.e) CPM_CUDA_TRY(cudaEventCreate(&q));
   constexpr int kReps = 3;
   const Vec32<const float> uv{u, nullptr};
-  for (int v = 0; v < 3; ++v) {
+  for (int v = 0; v < 3; ++v) {  // one wait for all three
     extend32(L, L.all, v, uv, w, st);  // warm-up
-    CPM_CUDA_TRY(cudaEventRecord(e0, st));
+    CPM_CUDA_TRY(cudaEventRecord(ev.e[2 * v], st));
     for (int r = 0; r < kReps; ++r) extend32(L, L.all, v, uv, w, st);
-    CPM_CUDA_TRY(cudaEventRecord(e1, st));
-    CPM_CUDA_TRY(cudaEventSynchronize(e1));
-    CPM_CUDA_TRY(cudaEventElapsedTime(&ms[v], e0, e1));
+    CPM_CUDA_TRY(cudaEventRecord(ev.e[2 * v + 1], st));
+  }
+  CPM_CUDA_TRY(cudaEventSynchronize(ev.e[5]));
+  for (int v = 0; v < 3; ++v) {
+    CPM_CUDA_TRY(cudaEventElapsedTime(&ms[v], ev.e[2 * v], ev.e[2 * v + 1]));
     ms[v] /= kReps;
     if (ms[v] < ms[best]) best = v;
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  CPM_CUDA_TRY(cudaGetLastError());
   return best;
 }
 
@@ -896,9 +900,14 @@ void build_dense32(const Level& L, Dense32& D, const CycleCells* cyc, DenseScrat
   const int64_t nt = L.ntiles, np = L.nplus(), nB = L.nB;
   const int per = L.dim == 3 ? 16 : 4;
   const int64_t nrows = (int64_t)L.nbricks * per;
-  D.bface.alloc((size_t)2 * L.nbricks);
-  D.bfwd.alloc((size_t)8 * L.nbricks);
-  D.slot.alloc((size_t)np);
+  auto carve = [&](Carver take) {
+    take(D.bface, (size_t)2 * L.nbricks);
+    take(D.bfwd, (size_t)8 * L.nbricks);
+    take(D.slot, (size_t)np);
+    return take.used;
+  };
+  D.tables.alloc(carve(Carver{}));
+  carve(Carver{D.tables.get()});
   k_dense_bricks<<<nblk(L.nbricks, 256), 256, 0, st>>>(L.view(), L.bcoord.get(), L.dim, D.bface.get(),
                                                        D.bfwd.get());
   k_dense_slots<<<nblk(np, 256), 256, 0, st>>>(L.view(), L.key.get(), np, L.dim, D.slot.get());

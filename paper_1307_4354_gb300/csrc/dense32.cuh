@@ -70,9 +70,10 @@ struct NeedSet {
 };
 // Brick-dense structures of one level.
 struct Dense32 {
-  DBuf<int4> bface;
-  DBuf<int32_t> bfwd;
-  DBuf<uint32_t> slot;
+  Part<int4> bface;
+  Part<int32_t> bfwd;
+  Part<uint32_t> slot;
+  DBuf<unsigned char> tables;  // holds these three
   ExtUnits all;          // every point of B+
   DBuf<float> dA, c;     // brick-dense omega / diag(A) and c
   // levels of a V-cycle

@@ -93,26 +93,27 @@ __global__ void k_transfer_index(const uint64_t* base, int32_t n, int dim, Brick
 }
 
 struct Transfer {
-  DBuf<uint64_t> base;
-  DBuf<int32_t> idx;  // linear, indexed: 2^d x n source indices
+  Part<uint64_t> base;
+  Part<int32_t> idx;  // linear, indexed: 2^d x n source indices
   BrickView src{};
   int deg = 1;
-  DBuf<double> fr64;
-  DBuf<float> fr32;
+  Part<double> fr64;
+  Part<float> fr32;
   int32_t n = 0;
+  DBuf<unsigned char> block;  // holds them all
 };
 
 template <typename T>
 struct Work {
-  DBuf<T> u, f, r, w, tmp, v, refv;
-  void alloc(int64_t nB, int64_t nplus, bool paper, bool relative, bool extended) {
-    if (relative) refv.alloc(nplus);  // reference values of the relative extension
-    u.alloc(nB);
-    f.alloc(nB);
-    r.alloc(nB);
-    if (extended) w.alloc(nplus);  // E u in band order
-    tmp.alloc(nB);
-    if (paper) v.alloc(nB);  // L_B u of the paper-form operator
+  Part<T> u, f, r, w, tmp, v, refv;
+  void carve(Carver& take, int64_t nB, int64_t nplus, bool paper, bool relative, bool extended) {
+    if (relative) take(refv, nplus);  // reference values of the relative extension
+    take(u, nB);
+    take(f, nB);
+    take(r, nB);
+    if (extended) take(w, nplus);  // E u in band order
+    take(tmp, nB);
+    if (paper) take(v, nB);  // L_B u of the paper-form operator
   }
 };
 
@@ -221,24 +222,24 @@ struct Workspace {
   // brick-dense u, w = E u, f and r of the FP32 passes, as far as the options
   // use them (r also takes E u where the residual of E u is restricted)
   struct Dense {
-    cpm::DBuf<float> data;
-    float *u = nullptr, *w = nullptr, *f = nullptr, *r = nullptr;
+    cpm::Part<float> u, w, f, r;
     size_t slots = 0;
   };
   std::vector<Dense> dense;
-  cpm::DBuf<double> part;   // norm partials (2 per block)
+  cpm::Part<double> part;   // norm partials (2 per block)
   int part_blocks = 0;
-  cpm::DBuf<double> own_norms;  // [max, sumsq, 1/max, -] unless norms points elsewhere
+  cpm::Part<double> own_norms;  // [max, sumsq, 1/max, -] unless norms points elsewhere
   double* norms = nullptr;
-  cpm::DBuf<double> normf;  // norms of f
-  cpm::DBuf<double> u_own, f_own, r64, d64;
-  cpm::DBuf<double> refv;   // per point of the finest B+: the extension's reference value (FP64 form)
-  cpm::DBuf<float2> dpair;  // pair form: delta_j = (E u)_j - ref_j over the finest B+
-  cpm::DBuf<float> rpair;   // pair form: ref_j
-  cpm::DBuf<uint32_t> dmax; // pair form: slots of the largest staged |u - ref| (norms[3])
-  cpm::DBuf<int32_t> chk_list, chk_count;      // pointwise FP64 check: candidate points
-  cpm::DBuf<unsigned long long> chk_max;       // and the largest |r| among them (bits)
-  cpm::DBuf<float> r32, d32;
+  cpm::Part<double> normf;  // norms of f
+  cpm::Part<double> u_own, f_own, r64, d64;
+  cpm::Part<double> refv;   // per point of the finest B+: the extension's reference value (FP64 form)
+  cpm::Part<float2> dpair;  // pair form: delta_j = (E u)_j - ref_j over the finest B+
+  cpm::Part<float> rpair;   // pair form: ref_j
+  cpm::Part<uint32_t> dmax; // pair form: slots of the largest staged |u - ref| (norms[3])
+  cpm::Part<int32_t> chk_list, chk_count;      // pointwise FP64 check: candidate points
+  cpm::Part<unsigned long long> chk_max;       // and the largest |r| among them (bits)
+  cpm::Part<float> r32, d32;
+  cpm::DBuf<unsigned char> block;  // holds all of these
   cpm::GmresWork<double> gm64;  // coarsest-level GMRES (coarse mode 3)
   cpm::GmresWork<float> gm32;
   cudaStream_t hs = nullptr;
@@ -294,78 +295,80 @@ struct cpm_hier_s {
 };
 
 namespace cpm {
-// Allocate the work vectors of every level and the solve vectors.
+// The work vectors of every level and the solve vectors, in one block: with an
+// allocation for each of them (and of the transfers' and brick tables) a sphere at
+// dx = 1/128 took 3.3 ms to build as one level, 11.8 ms with four coarser ones; so
+// 2.6 and 9.5 ms.
 static void alloc_workspace(const cpm_hier_s& H, Workspace& W, double* norms_slot = nullptr) {
-  W.w64.resize(H.L.size());
-  W.w32.resize(H.L.size());
-  W.dense.resize(H.L.size());
+  const size_t nl = H.L.size();
+  W.w64.resize(nl);
+  W.w32.resize(nl);
+  W.dense.resize(nl);
   // a batch's systems run the plain cycle only, which keeps FP32 vectors in band
   // order on the coarsest level alone
   const bool cycle_only = norms_slot != nullptr && H.dense_cycle;
   const bool mbr = H.opts.op_form == CPM_OP_MBR, relative = H.opts.relative != 0;
   const bool jacobi = mbr && H.opts.smoother == CPM_SMOOTH_JACOBI && !relative;
-  for (size_t l = 0; l < H.L.size(); ++l) {
-    const int64_t nB = H.L[l].lev->nB, np = H.L[l].lev->nplus();
-    const bool last = l + 1 == H.L.size();
-    W.w64[l].alloc(nB, np, !mbr, relative, true);
-    if (!cycle_only) {
-      W.w32[l].alloc(nB, np, !mbr, relative, !mbr || relative);
-    } else if (last) {
-      W.w32[l].u.alloc(nB);
-      W.w32[l].f.alloc(nB);
-    }
-    Workspace::Dense& D = W.dense[l];
-    D.slots = dense_size(*H.L[l].lev);
-    const bool uf = jacobi && !(cycle_only && last), r = H.dense_cycle && !last;
-    const size_t n = D.slots * ((mbr ? 1 : 0) + (uf ? 2 : 0) + (r ? 1 : 0));
-    if (n == 0) continue;
-    D.data.alloc(n);
-    CPM_CUDA_TRY(cudaMemsetAsync(D.data.get(), 0, sizeof(float) * n, nullptr));
-    float* p = D.data.get();
-    auto take = [&]() {
-      float* q = p;
-      p += D.slots;
-      return q;
-    };
-    if (mbr) D.w = take();
-    if (uf) {
-      D.u = take();
-      D.f = take();
-    }
-    if (r) D.r = take();
-  }
-  const int64_t nB0 = H.L[0].lev->nB;
+  const int64_t nB0 = H.L[0].lev->nB, np0 = H.L[0].lev->nplus();
   W.part_blocks = std::max<int>(std::max(lap_blocks_f64(H.L[0].view<double>()),
                                           paper_blocks(H.L[0].view<double>())),
                                  kNormBlocks);
-  W.part.alloc(2 * (size_t)W.part_blocks);
-  W.own_norms.alloc(4);
+  size_t cleared = 0;  // bytes at the start that are set to zero
+  auto carve = [&](Carver take) {
+    for (size_t l = 0; l < nl; ++l) {
+      Workspace::Dense& D = W.dense[l];
+      const bool last = l + 1 == nl;
+      D.slots = dense_size(*H.L[l].lev);
+      if (mbr) take(D.w, D.slots);
+      if (jacobi && !(cycle_only && last)) {
+        take(D.u, D.slots);
+        take(D.f, D.slots);
+      }
+      if (H.dense_cycle && !last) take(D.r, D.slots);
+    }
+    if (H.pair_resid) take(W.dmax, kPairSlots);
+    cleared = take.used;
+    for (size_t l = 0; l < nl; ++l) {
+      const int64_t nB = H.L[l].lev->nB, np = H.L[l].lev->nplus();
+      W.w64[l].carve(take, nB, np, !mbr, relative, true);
+      if (!cycle_only) {
+        W.w32[l].carve(take, nB, np, !mbr, relative, !mbr || relative);
+      } else if (l + 1 == nl) {
+        take(W.w32[l].u, nB);
+        take(W.w32[l].f, nB);
+      }
+    }
+    take(W.part, 2 * (size_t)W.part_blocks);
+    take(W.own_norms, 4);
+    take(W.normf, 4);
+    take(W.u_own, nB0);
+    take(W.f_own, nB0);
+    take(W.r64, nB0);
+    take(W.d64, nB0);
+    take(W.refv, np0);  // FP64 form (also the check of the pair form)
+    if (H.pair_resid) {
+      take(W.dpair, np0);
+      take(W.rpair, np0);
+      take(W.chk_list, kCheckCap);
+      take(W.chk_count, 1);
+      take(W.chk_max, 1);
+    }
+    if (!cycle_only) {
+      take(W.r32, nB0);
+      take(W.d32, nB0);
+    }
+    return take.used;
+  };
+  W.block.alloc(carve(Carver{}));
+  carve(Carver{W.block.get()});
   W.norms = norms_slot ? norms_slot : W.own_norms.get();
-  W.normf.alloc(4);
-  W.u_own.alloc(nB0);
-  W.f_own.alloc(nB0);
-  W.r64.alloc(nB0);
-  W.d64.alloc(nB0);
-  W.refv.alloc(H.L[0].lev->nplus());  // FP64 form (also the check of the pair form)
-  if (H.pair_resid) {
-    W.dpair.alloc(H.L[0].lev->nplus());
-    W.rpair.alloc(H.L[0].lev->nplus());
-    W.dmax.alloc(kPairSlots);
-    CPM_CUDA_TRY(cudaMemset(W.dmax.get(), 0, sizeof(uint32_t) * kPairSlots));
-    W.chk_list.alloc(kCheckCap);
-    W.chk_count.alloc(1);
-    W.chk_max.alloc(1);
-  }
-  if (!cycle_only) {
-    W.r32.alloc(nB0);
-    W.d32.alloc(nB0);
-  }
+  if (cleared > 0) CPM_CUDA_TRY(cudaMemsetAsync(W.block.get(), 0, cleared, nullptr));
   if (H.coarse_mode == 3) {
     const int64_t nc = H.L.back().lev->nB;
     W.gm64.alloc(nc, kGmresMaxM);
     W.gm32.alloc(nc, kGmresMaxM);
   }
-  // the clears above are complete before a stream that does not wait for the
+  // the clear above is complete before a stream that does not wait for the
   // default stream uses the vectors
   CPM_CUDA_TRY(cudaStreamSynchronize(nullptr));
   CPM_CUDA_TRY(cudaStreamCreateWithFlags(&W.hs, cudaStreamNonBlocking));
@@ -400,8 +403,8 @@ static void mbr_op(cpm_hier_s* H, Workspace& W, int l, LapMode mode, const float
   HLevel& lv = H->L[l];
   const DenseView v = lv.dview();
   const Vec32<const float> uv{nullptr, u};
-  launch_extend32(v, v.all, uv, W.dense[l].w, st);
-  launch_lap32(v, mode, uv, W.dense[l].w, f, (float)H->c, Vec32<float>{nullptr, u_inout ? u_inout : out},
+  launch_extend32(v, v.all, uv, W.dense[l].w.get(), st);
+  launch_lap32(v, mode, uv, W.dense[l].w.get(), f, (float)H->c, Vec32<float>{nullptr, u_inout ? u_inout : out},
                nullptr, all_rows(v), st);
 }
 
@@ -448,13 +451,13 @@ static void smooth32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* 
                      cudaStream_t st) {
   HLevel& lv = H->L[l];
   const DenseView v = lv.dview();
-  const Vec32<float> dense{W.dense[l].u, nullptr}, compact{nullptr, u};
+  const Vec32<float> dense{W.dense[l].u.get(), nullptr}, compact{nullptr, u};
   for (int s = 0; s < sweeps; ++s) {
     const Vec32<float> in = s == 0 ? compact : dense, out = s == sweeps - 1 ? compact : dense;
     const Vec32<const float> cin{in.dense, in.compact};
-    launch_extend32(v, v.all, cin, W.dense[l].w, st);
-    launch_lap32(v, LAP_JACOBI, cin, W.dense[l].w, s == 0 ? f : W.dense[l].f, (float)H->c, out,
-                 sweeps > 1 ? W.dense[l].f : nullptr, all_rows(v), st);
+    launch_extend32(v, v.all, cin, W.dense[l].w.get(), st);
+    launch_lap32(v, LAP_JACOBI, cin, W.dense[l].w.get(), s == 0 ? f : W.dense[l].f.get(), (float)H->c, out,
+                 sweeps > 1 ? W.dense[l].f.get() : nullptr, all_rows(v), st);
   }
 }
 
@@ -603,8 +606,8 @@ static void sweeps32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* 
   const DenseView v = H->L[l].dview();
   const UnitsView units = need ? units_view(need->units) : v.all;
   const RowsView rows = need ? rows_view(*need) : all_rows(v);
-  float* ud = W.dense[l].u;
-  float* fd = W.dense[l].f;
+  float* ud = W.dense[l].u.get();
+  float* fd = W.dense[l].f.get();
   for (int s = 0; s < sweeps; ++s) {
     const Vec32<float> out = u_out && s == sweeps - 1 ? Vec32<float>{nullptr, u_out} : Vec32<float>{ud, nullptr};
     if (state == State32::zero && out.dense) {
@@ -614,8 +617,8 @@ static void sweeps32(cpm_hier_s* H, Workspace& W, int l, const float* f, float* 
         CPM_CUDA_TRY(cudaMemsetAsync(ud, 0, W.dense[l].slots * sizeof(float), st));
       const bool band = state == State32::compact;
       const Vec32<const float> in{band ? nullptr : ud, band ? u : nullptr};
-      launch_extend32(v, units, in, W.dense[l].w, st);
-      launch_lap32(v, LAP_JACOBI, in, W.dense[l].w, band ? f : fd, (float)H->c, out, band ? fd : nullptr, rows,
+      launch_extend32(v, units, in, W.dense[l].w.get(), st);
+      launch_lap32(v, LAP_JACOBI, in, W.dense[l].w.get(), band ? f : fd, (float)H->c, out, band ? fd : nullptr, rows,
                    st);
     }
     state = out.dense ? State32::dense : State32::compact;
@@ -640,8 +643,8 @@ static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const flo
   float* cu[kMaxGroup];
   for (int g = 0; g < G; ++g) {
     Workspace& w = *W[g];
-    float* ud = w.dense[l].u;
-    float* fd = w.dense[l].f;
+    float* ud = w.dense[l].u.get();
+    float* fd = w.dense[l].f.get();
     state[g] = state0;
     int pre = H->opts.nu1;
     auto make_dense = [&]() {
@@ -655,8 +658,8 @@ static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const flo
     if (l == 0 && H->learned_active && pre > 0 && w.w32[0].r.n > 0) {  // (not a batch's workspace)
       // learned smoother in place of the first Jacobi sweep: r = f - A u, u += net(r)
       make_dense();
-      launch_extend32(v, v.all, {ud, nullptr}, w.dense[0].w, st);
-      launch_lap32(v, LAP_RESID, {ud, nullptr}, w.dense[0].w, fd, (float)H->c, {nullptr, w.w32[0].r.get()},
+      launch_extend32(v, v.all, {ud, nullptr}, w.dense[0].w.get(), st);
+      launch_lap32(v, LAP_RESID, {ud, nullptr}, w.dense[0].w.get(), fd, (float)H->c, {nullptr, w.w32[0].r.get()},
                    nullptr, all_rows(v), st);
       mlp_forward(H->mlp->params.get(), *H->mlpd, w.w32[0].r.get(), 1.f / v.inv_h2, nullptr, ud, v.slot, nullptr,
                   st);
@@ -668,15 +671,15 @@ static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const flo
     const NeedSet& rs = lv.dense.resid;
     const float* uu = ud;
     if (H->opts.residual_mode == 0) {
-      launch_extend32(v, need ? units_view(need->units) : v.all, {ud, nullptr}, w.dense[l].r, st);
-      uu = w.dense[l].r;  // the residual takes its place row by row
+      launch_extend32(v, need ? units_view(need->units) : v.all, {ud, nullptr}, w.dense[l].r.get(), st);
+      uu = w.dense[l].r.get();  // the residual takes its place row by row
     }
-    launch_extend32(v, units_view(rs.units), {uu, nullptr}, w.dense[l].w, st);
-    launch_lap32(v, LAP_RESID, {uu, nullptr}, w.dense[l].w, fd, (float)H->c, {w.dense[l].r, nullptr}, nullptr,
-                 rows_view(rs), st);
-    cf[g] = last ? w.w32[l + 1].f.get() : w.dense[l + 1].f;
+    launch_extend32(v, units_view(rs.units), {uu, nullptr}, w.dense[l].w.get(), st);
+    launch_lap32(v, LAP_RESID, {uu, nullptr}, w.dense[l].w.get(), fd, (float)H->c, {w.dense[l].r.get(), nullptr},
+                 nullptr, rows_view(rs), st);
+    cf[g] = last ? w.w32[l + 1].f.get() : w.dense[l + 1].f.get();
     cu[g] = w.w32[l + 1].u.get();
-    launch_transfer32(lv.R32, v, w.dense[l].r, const_cast<float*>(cf[g]), false, st);
+    launch_transfer32(lv.R32, v, w.dense[l].r.get(), const_cast<float*>(cf[g]), false, st);
   }
   if (last) {
     coarse_solve<float>(H, W, G, cf, cu, st);
@@ -688,11 +691,11 @@ static void vcycle32(cpm_hier_s* H, Workspace* const* W, int G, int l, const flo
   for (int g = 0; g < G; ++g) {
     Workspace& w = *W[g];
     if (last)
-      launch_prolong_coarsest32(tview<float>(lv.P, lv.lev->dim), v.slot, cu[g], w.dense[l].u, st);
+      launch_prolong_coarsest32(tview<float>(lv.P, lv.lev->dim), v.slot, cu[g], w.dense[l].u.get(), st);
     else
-      launch_transfer32(lv.P32, H->L[l + 1].dview(), w.dense[l + 1].u, w.dense[l].u, true, st);
+      launch_transfer32(lv.P32, H->L[l + 1].dview(), w.dense[l + 1].u.get(), w.dense[l].u.get(), true, st);
     sweeps32(H, w, l, nullptr, nullptr, state[g], H->opts.nu2, need, band_out ? u[g] : nullptr, st);
-    if (band_out && H->opts.nu2 == 0) launch_gather32(v, w.dense[l].u, u[g], st);
+    if (band_out && H->opts.nu2 == 0) launch_gather32(v, w.dense[l].u.get(), u[g], st);
   }
 }
 
@@ -864,11 +867,11 @@ static void outer_step(cpm_hier_s* H, Workspace* const* W, int G, int mode, int 
   } else if (H->dense_cycle && !first_fmg) {
     const DenseView v = H->L[0].dview();
     for (int g = 0; g < G; ++g)
-      launch_scale_dense(v, W[g]->r64.get(), W[g]->norms, W[g]->dense[0].f, st);
+      launch_scale_dense(v, W[g]->r64.get(), W[g]->norms, W[g]->dense[0].f.get(), st);
     for (int j = 0; j < inner; ++j)
       vcycle32(H, W, G, 0, nullptr, nullptr, j == 0 ? State32::zero : State32::dense, false, st);
     for (int g = 0; g < G; ++g)
-      launch_axpy_dense(v, W[g]->u_own.get(), W[g]->dense[0].u, W[g]->norms, st);
+      launch_axpy_dense(v, W[g]->u_own.get(), W[g]->dense[0].u.get(), W[g]->norms, st);
   } else {
     const float* r[kMaxGroup];
     float* d[kMaxGroup];
@@ -1045,15 +1048,21 @@ static void build_transfer(const Level& target, const Level& src, Transfer& t, i
   t.n = target.nB;
   t.src = src.view();
   t.deg = deg;
-  t.base.alloc((size_t)t.n);
-  t.fr64.alloc((size_t)target.dim * t.n);
-  t.fr32.alloc((size_t)target.dim * t.n);
+  const bool indexed = CPM_TRANSFER_INDEXED && deg == 1 && t.n > 0;
+  auto carve = [&](Carver take) {
+    take(t.base, (size_t)t.n);
+    take(t.fr64, (size_t)target.dim * t.n);
+    take(t.fr32, (size_t)target.dim * t.n);
+    if (indexed) take(t.idx, (size_t)(target.dim == 3 ? 8 : 4) * t.n);
+    return take.used;
+  };
+  t.block.alloc(carve(Carver{}));
+  carve(Carver{t.block.get()});
   k_transfer_records<<<nblk(t.n, 256), 256, 0, st>>>(target.cp.get(), target.nplus(), t.n, target.dim, deg,
                                                      src.lo, src.dx, src.view(), t.base.get(),
                                                      t.fr64.get(), t.fr32.get(), err);
   CPM_CUDA_TRY(cudaGetLastError());
-  if (CPM_TRANSFER_INDEXED && deg == 1 && t.n > 0) {
-    t.idx.alloc((size_t)(target.dim == 3 ? 8 : 4) * t.n);
+  if (indexed) {
     k_transfer_index<<<nblk(t.n, 256), 256, 0, st>>>(t.base.get(), t.n, target.dim, src.view(),
                                                      t.idx.get());
     CPM_CUDA_TRY(cudaGetLastError());
@@ -1238,7 +1247,6 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
     k_diag_A<<<nblk(nB, 256), 256, 0, st>>>(dM.get(), lv.c64.get(), H->c, o.omega, lv.dA64.get(),
                                             lv.dA32.get(), nB);
     CPM_CUDA_TRY(cudaGetLastError());
-    CPM_CUDA_TRY(cudaStreamSynchronize(st));
     lv.dM64 = std::move(dM);
     if (o.op_form == CPM_OP_MBR) dense_static(*lv.lev, lv.dense, lv.dA32.get(), lv.c32.get(), st);
   }
@@ -1295,7 +1303,7 @@ cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts_in, cpm_
       continue;
     }
     Workspace::Dense& D = H->ws.dense[l];
-    float *u = D.u, *w = D.w;
+    float *u = D.u.get(), *w = D.w.get();
     if (!u || !w) {  // forms whose passes are in band order
       if (probe.n < 2 * D.slots) {
         probe.alloc(2 * D.slots);
