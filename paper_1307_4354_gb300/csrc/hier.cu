@@ -313,21 +313,8 @@ static void alloc_workspace(const cpm_hier_s& H, Workspace& W, double* norms_slo
   W.part_blocks = std::max<int>(std::max(lap_blocks_f64(H.L[0].view<double>()),
                                           paper_blocks(H.L[0].view<double>())),
                                  kNormBlocks);
-  size_t cleared = 0;  // bytes at the start that are set to zero
+  size_t cleared_from = 0;  // the parts from here on are set to zero
   auto carve = [&](Carver take) {
-    for (size_t l = 0; l < nl; ++l) {
-      Workspace::Dense& D = W.dense[l];
-      const bool last = l + 1 == nl;
-      D.slots = dense_size(*H.L[l].lev);
-      if (mbr) take(D.w, D.slots);
-      if (jacobi && !(cycle_only && last)) {
-        take(D.u, D.slots);
-        take(D.f, D.slots);
-      }
-      if (H.dense_cycle && !last) take(D.r, D.slots);
-    }
-    if (H.pair_resid) take(W.dmax, kPairSlots);
-    cleared = take.used;
     for (size_t l = 0; l < nl; ++l) {
       const int64_t nB = H.L[l].lev->nB, np = H.L[l].lev->nplus();
       W.w64[l].carve(take, nB, np, !mbr, relative, true);
@@ -357,12 +344,26 @@ static void alloc_workspace(const cpm_hier_s& H, Workspace& W, double* norms_slo
       take(W.r32, nB0);
       take(W.d32, nB0);
     }
+    cleared_from = take.used;
+    for (size_t l = 0; l < nl; ++l) {
+      Workspace::Dense& D = W.dense[l];
+      const bool last = l + 1 == nl;
+      D.slots = dense_size(*H.L[l].lev);
+      if (mbr) take(D.w, D.slots);
+      if (jacobi && !(cycle_only && last)) {
+        take(D.u, D.slots);
+        take(D.f, D.slots);
+      }
+      if (H.dense_cycle && !last) take(D.r, D.slots);
+    }
+    if (H.pair_resid) take(W.dmax, kPairSlots);
     return take.used;
   };
   W.block.alloc(carve(Carver{}));
   carve(Carver{W.block.get()});
   W.norms = norms_slot ? norms_slot : W.own_norms.get();
-  if (cleared > 0) CPM_CUDA_TRY(cudaMemsetAsync(W.block.get(), 0, cleared, nullptr));
+  if (W.block.n > cleared_from)
+    CPM_CUDA_TRY(cudaMemsetAsync(W.block.get() + cleared_from, 0, W.block.n - cleared_from, nullptr));
   if (H.coarse_mode == 3) {
     const int64_t nc = H.L.back().lev->nB;
     W.gm64.alloc(nc, kGmresMaxM);
