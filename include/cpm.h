@@ -234,7 +234,8 @@ typedef struct cpm_hier_s* cpm_hier;
  * the restriction and prolongation records, diag(A) on every level and the
  * inverse of the coarsest-level matrix (FP64, for the direct solve of
  * Algorithm 4.1 step 2).  The finest band is copied; `finest` may be
- * destroyed afterwards.  Synchronous.
+ * destroyed afterwards.  Device memory: about 900 bytes per finest band point
+ * (CPM_OP_PAPER 680) and the coarsest level's inverse.  Synchronous.
  * Errors: CPM_ERR_ARG (bad options), CPM_ERR_REACH, CPM_ERR_SINGULAR.
  */
 cpm_status cpm_build_hierarchy(cpm_band finest, const cpm_mg_opts* opts,
@@ -492,7 +493,7 @@ typedef struct cpm_batch_s* cpm_batch;
  * uneven): n_hier hierarchies, each with n_rhs right-hand sides; system
  * s = i * n_rhs + k uses hierarchy i (n_hier * n_rhs <= CPM_BATCH_MAX_SYSTEMS).
  * Every system gets its own workspace (work vectors of every level, about
- * 130 bytes per finest band point); the hierarchies' static data is shared,
+ * 155 bytes per finest band point, 180 with relative sweeps); the hierarchies' static data is shared,
  * not owned by the batch, and must outlive it.  tune_cache: optional path of a
  * text file ("<batch key> <K>" per line) in which the autotuner keeps the
  * concurrency it chose for a batch of this shape (NULL: no file).  No

@@ -18,8 +18,8 @@ namespace cpm {
 // Let the next kernel of the stream be scheduled as this one's blocks drain.
 // Not for the largest grids: there the signal of every block costs more than
 // the overlap gives (extension over 78 thousand tiles: 82 us with it, 73 us
-// without; a mixed solve at dx = 1/256 25.3 ms with this limit, 25.9 without),
-// and the next kernel follows the last block's end.
+// without; a mixed solve of five outer iterations at dx = 1/256 25.3 ms with this
+// limit, 25.9 without), and the next kernel follows the last block's end.
 constexpr unsigned kReleaseBlocks = 32768;
 __device__ __forceinline__ void release_next() {
   if (gridDim.x <= kReleaseBlocks) asm volatile("griddepcontrol.launch_dependents;");
