@@ -822,7 +822,8 @@ static void grow(DBuf<T>& d, size_t n, cudaStream_t st) {
 // The counts of all of a level's sets are scanned in one go, so that a level
 // costs one wait of the host.  With a scan, its scratch and a wait per set and
 // list, hierarchies without a dense inverse took 14.0 ms to build (sphere at
-// dx = 1/96), 9.3 (circle at 1/640), 5.1 (sphere at 1/32), so 10.4, 6.3 and 4.1 ms.
+// dx = 1/96), 9.3 (circle at 1/640), 5.1 (sphere at 1/32), so 10.4, 6.3 and 4.1 ms
+// (7.9, 5.5 and 3.3 since workspaces and tables share blocks of memory).
 class CountScan {
  public:
   CountScan(DBuf<int64_t>& d, cudaStream_t st) : d_(d), st_(st) {}
